@@ -8,7 +8,7 @@ path: symbolic peel, encode + coded products, numeric peel.
 
 value = useful 2MNK FLOP / step time of the headline precision (split-BF16x3
 on tcgen05 when the build has it, else plain FP32), with inputs resident in
-HBM (A, B = 256 MB each, larger than L2).  The FP32 CUDA-core path is timed
+HBM (A, B = 256 MB each, larger than L2).  The FP32 path is timed
 beside it.  ``--impl reference`` times the FP64 CPU oracle instead.
 """
 from __future__ import annotations
@@ -251,7 +251,7 @@ class StageEvents:
 TOL = {"fp32": 1e-5, "bf16x3": 1e-5, "fp16x3": 1e-5, "bf16": 2e-2, "mxfp8": 6e-2, "exact": 1e-5,
        "bf16x3-fused": 1e-5}
 # MMA flops executed per useful coded flop by each tensor-core precision
-MMA_MULT = {"bf16x3": 3, "bf16x3-fused": 3, "fp16x3": 3, "bf16": 1, "mxfp8": 1}
+MMA_MULT = {"fp32": 6, "bf16x3": 3, "bf16x3-fused": 3, "fp16x3": 3, "bf16": 1, "mxfp8": 1}
 
 
 def _propagation(code, order, Ah, Bh, h, sources, ncols=256, kappa=None):
@@ -457,7 +457,6 @@ def run_ours(args, wl):
     else:
         precs = [args.precision] + (["fp32"] if args.precision != "fp32" else [])
     results = {}
-    sms = torch.cuda.get_device_properties(dev).multi_processor_count
     gpu_index = local
     cvd = os.environ.get("CUDA_VISIBLE_DEVICES", "")
     if cvd and cvd.split(",")[0].strip().isdigit():
@@ -560,7 +559,7 @@ def run_ours(args, wl):
         clocks.end()
         ms, ms_serial = _max_over_ranks([ms, ms_serial], device=dev)
         stage = {}
-        recorded = ["schedule", "a_prep", "gemm", "peel"] + (["b_prep"] if prec != "fp32" else [])
+        recorded = ["schedule", "a_prep", "gemm", "peel"] + ["b_prep"]
         # (the autotuner covers the bf16 tensor-core kernels only)
         for si, nm in enumerate(bpx.STAGE_NAMES):
             if nm not in recorded:
@@ -631,32 +630,23 @@ def run_ours(args, wl):
     gemm_ms = R["stage"]["gemm"]
     rows_mean = sum(R["rows"]) / len(R["rows"])
     clk = R["clocks"].get("sm_mhz") or 0
-    if head != "fp32":
-        # tensor-core paths: MMA flops executed per launch (split terms, or
-        # the exact path's digit-pair products) against the measured bf16
-        # peak (FP8: times the nominal fp8 / bf16 ratio of 2)
-        if head == "exact":
-            S_ex = bpx.exact_params(code, K)["S"]
-            mult = S_ex * (S_ex + 1) // 2
-        else:
-            mult = MMA_MULT[head]
-        flops = 2.0 * rows_mean * N * K * mult
-        achieved = flops / (gemm_ms * 1e-3) / 1e12
-        peak = peaks.get("bf16_tflops", 1900.0) * (2.0 if head == "mxfp8" else 1.0)
-        src = "measured bf16 burst (MEASURED_PEAKS.json)" if peaks else "fallback"
-        roof = {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-                "frac": achieved / peak, "traffic": _traffic(wl["name"], head, tuned.get(head)),
-                "peak_source": src + (" x 2 (nominal fp8/bf16)" if head == "mxfp8" else ""),
-                "kernel": "coded tcgen05 GEMM" + (" (block-scaled MXFP8)" if head == "mxfp8" else ""),
-                "work_per_launch": "2 x coded rows x N x K x %d MMA flops" % mult}
+    # tensor-core paths: MMA flops executed per launch (split terms, or the
+    # exact path's digit-pair products) against the measured bf16 peak (FP8:
+    # times the nominal fp8 / bf16 ratio of 2)
+    if head == "exact":
+        S_ex = bpx.exact_params(code, K)["S"]
+        mult = S_ex * (S_ex + 1) // 2
     else:
-        flops = 2.0 * rows_mean * N * K
-        achieved = flops / (gemm_ms * 1e-3) / 1e12
-        mhz = peaks.get("sm_max_mhz", 2070.0)
-        peak = sms * 128 * 2 * mhz * 1e6 / 1e12
-        roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-                "traffic": None, "peak_source": f"FFMA: {sms} SMs x 128 lanes x 2 x {mhz:.0f} MHz",
-                "kernel": "coded FP32 SIMT GEMM", "work_per_launch": "2 x coded rows x N x K"}
+        mult = MMA_MULT[head]
+    flops = 2.0 * rows_mean * N * K * mult
+    achieved = flops / (gemm_ms * 1e-3) / 1e12
+    peak = peaks.get("bf16_tflops", 1900.0) * (2.0 if head == "mxfp8" else 1.0)
+    src = "measured bf16 burst (MEASURED_PEAKS.json)" if peaks else "fallback"
+    roof = {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+            "frac": achieved / peak, "traffic": _traffic(wl["name"], head, tuned.get(head)),
+            "peak_source": src + (" x 2 (nominal fp8/bf16)" if head == "mxfp8" else ""),
+            "kernel": "coded tcgen05 GEMM" + (" (block-scaled MXFP8)" if head == "mxfp8" else ""),
+            "work_per_launch": "2 x coded rows x N x K x %d MMA flops" % mult}
     # decode GB/s: compulsory bytes of the peel (read each non-direct
     # resolver's product and every other block it subtracts, write C_s)
     peel_ms = R["stage"]["peel"]
@@ -706,19 +696,14 @@ def run_ours(args, wl):
         rows_m = sum(r["rows"]) / len(r["rows"])
         if gm <= 0:
             continue
-        if prec == "fp32":
-            mhz = peaks.get("sm_max_mhz", 2070.0)
-            pk, unit = sms * 128 * 2 * mhz * 1e6 / 1e12, "FFMA"
-            work = 2.0 * rows_m * N * K
+        if prec == "exact":
+            S_ex = bpx.exact_params(code, K)["S"]
+            mult = S_ex * (S_ex + 1) // 2     # digit pairs (i, l) with i + l < S
         else:
-            if prec == "exact":
-                S_ex = bpx.exact_params(code, K)["S"]
-                mult = S_ex * (S_ex + 1) // 2     # digit pairs (i, l) with i + l < S
-            else:
-                mult = MMA_MULT[prec]
-            pk = peaks.get("bf16_tflops", 1900.0) * (2.0 if prec == "mxfp8" else 1.0)
-            unit = "measured bf16 burst" + (" x 2 (nominal fp8/bf16)" if prec == "mxfp8" else "")
-            work = 2.0 * rows_m * N * K * mult
+            mult = MMA_MULT[prec]
+        pk = peaks.get("bf16_tflops", 1900.0) * (2.0 if prec == "mxfp8" else 1.0)
+        unit = "measured bf16 burst" + (" x 2 (nominal fp8/bf16)" if prec == "mxfp8" else "")
+        work = 2.0 * rows_m * N * K * mult
         ach = work / (gm * 1e-3) / 1e12
         gr[prec] = {"achieved_tflops": ach, "peak_tflops": pk, "frac": ach / pk, "peak": unit, "gemm_ms": gm}
     line["gemm_roofline"] = gr
@@ -730,21 +715,21 @@ def run_ours(args, wl):
                       "bytes_def": "sum over non-direct sources of (deg(resolver)+1) h N 4"}
     # the HBM-bound staging stages against their compulsory bytes: the
     # encode reads A once and writes the coded rows (bf16 hi + lo: 4 B per
-    # element, or FP32: 4 B), the B split reads B and writes B^T hi + lo
+    # element, or FP32 in three bf16 parts: 6 B), the B split reads B and writes B^T hi + lo
     def _hbm(nbytes, ms, what):
         gbs = nbytes / (ms * 1e-3) / 1e9 if ms and ms > 0 else None
         return {"bytes_per_step": nbytes, "ms": ms, "gbs": gbs, "frac_hbm": gbs / hbm if gbs else None,
                 "bytes_def": what}
     st_ = R["stage"]
     if head in ("bf16x3", "bf16", "fp32"):
-        out_b = 4 if head in ("bf16x3", "fp32") else 2
+        out_b = {"bf16x3": 4, "fp32": 6}.get(head, 2)
         line["encode"] = _hbm(4.0 * M * K + out_b * rows_mean * K, st_.get("a_prep", 0.0),
                               "read A once (4 M K) + write the coded rows (%d B per element)" % out_b)
     if head in ("bf16x3", "bf16"):
         line["b_split"] = _hbm(4.0 * K * N + (4 if head == "bf16x3" else 2) * K * N, st_.get("b_prep", 0.0),
                                "read B (4 K N) + write B^T hi (+ lo) bf16")
     line["clocks"] = R["clocks"]
-    per_step = {"bf16x3": 5, "bf16": 5, "mxfp8": 5, "fp32": 4, "exact": 7, "fp16x3": 7, "bf16x3-fused": 4}[head]
+    per_step = {"bf16x3": 5, "bf16": 5, "mxfp8": 5, "fp32": 7, "exact": 7, "fp16x3": 7, "bf16x3-fused": 4}[head]
     if head == "fp16x3" and len(code.cell_src) >= 4 * code.num_cells:
         per_step += 2  # the K-chunked encode of high-degree codes: three kernels instead of one
     line["gpu_launches"] = per_step * steps
@@ -1122,20 +1107,14 @@ def run_straggler(args, wl):
         S_ex = bpx.exact_params(code, K)["S"]
         mult = S_ex * (S_ex + 1) // 2     # digit pairs (i, l) with i + l < S
     else:
-        mult = {"bf16x3": 3, "fp16x3": 3, "bf16": 1, "fp32": 1}[prec]
+        mult = {"bf16x3": 3, "fp16x3": 3, "bf16": 1, "fp32": 6}[prec]
     peaks = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json"))) if os.path.exists(
         os.path.join(ROOT, "MEASURED_PEAKS.json")) else {}
     ach = 2.0 * float(np.mean(rows)) * N * K * mult / (stage["gemm"] * 1e-3) / 1e12
-    if prec != "fp32":
-        pk = peaks.get("bf16_tflops", 1900.0)
-        roof = {"bound": "tensor", "achieved": ach, "peak": pk, "unit": "TFLOP/s", "frac": ach / pk,
-                "traffic": None, "kernel": "coded tcgen05 GEMM",
-                "work_per_launch": "2 x coded rows x N x K x %d MMA flops" % mult}
-    else:
-        mhz = peaks.get("sm_max_mhz", 2070.0)
-        pk = torch.cuda.get_device_properties(0).multi_processor_count * 128 * 2 * mhz * 1e6 / 1e12
-        roof = {"bound": "alu", "achieved": ach, "peak": pk, "unit": "TFLOP/s", "frac": ach / pk,
-                "traffic": None, "kernel": "coded FP32 SIMT GEMM", "work_per_launch": "2 x coded rows x N x K"}
+    pk = peaks.get("bf16_tflops", 1900.0)
+    roof = {"bound": "tensor", "achieved": ach, "peak": pk, "unit": "TFLOP/s", "frac": ach / pk,
+            "traffic": None, "kernel": "coded tcgen05 GEMM",
+            "work_per_launch": "2 x coded rows x N x K x %d MMA flops" % mult}
     H = sum(1.0 / j for j in range(1, code.num_cells + 1))
     # How much of the peel could have overlapped the products (outside the
     # timed region, on the first timed steps): the decodable set's arrivals in
@@ -1176,7 +1155,7 @@ def run_straggler(args, wl):
                       "units": "1 / mu; T_c = sigma_c X_c"},
             "computed_cells_mean": float(np.mean(rows)) / h,
             "roofline": roof, "clocks": ck,
-            "gpu_launches": ({"bf16x3": 5, "bf16": 5, "fp16x3": 7, "fp32": 4, "exact": 7}[prec]
+            "gpu_launches": ({"bf16x3": 5, "bf16": 5, "fp16x3": 7, "fp32": 7, "exact": 7}[prec]
                              + (2 if prec == "fp16x3" and len(code.cell_src) >= 4 * code.num_cells else 0)) * steps}
     print(json.dumps(line), flush=True)
 

@@ -239,6 +239,25 @@ int products_impl(const bpx_code* c, const float* d_A, const float* d_B, int M, 
   switch (precision) {
     case BPX_FP32: {
       float* a_coded = reinterpret_cast<float*>(base + L.a_hi);
+      if (bpx::f32_on_tensor_cores(c, N, K, h)) {
+        void* const a[3] = {base + L.a_hi, base + L.a_lo, base + L.a_3};
+        void* const b[3] = {base + L.b_hi, base + L.b_lo, base + L.b_3};
+        stage_mark(opts, BPX_STAGE_B_PREP, 0, st);
+        e = bpx::launch_b_parts(p, d_B, K, N, b, st);
+        stage_mark(opts, BPX_STAGE_B_PREP, 1, st);
+        stage_mark(opts, BPX_STAGE_A_PREP, 0, st);
+        if (e == cudaSuccess) e = bpx::launch_encode_parts(g, p, d_A, M, K, h, a, st);
+        stage_mark(opts, BPX_STAGE_A_PREP, 1, st);
+        stage_mark(opts, BPX_STAGE_GEMM, 0, st);
+        if (e == cudaSuccess)
+          e = bpx::launch_gemm_f32_tc(p, a, b, c->num_cells, N, K, h, bpx::rows_expected(c, h), d_products, d_C,
+                                      d_info, st);
+        // operands the parts cannot hold (a plan counter says so): FP32 on the CUDA cores
+        if (e == cudaSuccess) e = bpx::launch_encode_f32_flagged(g, p, d_A, M, K, h, a_coded, st);
+        if (e == cudaSuccess) e = bpx::launch_gemm_f32_flagged(g, p, a_coded, d_B, N, K, h, d_products, d_C, st);
+        stage_mark(opts, BPX_STAGE_GEMM, 1, st);
+        break;
+      }
       stage_mark(opts, BPX_STAGE_A_PREP, 0, st);
       e = bpx::launch_encode_f32(g, p, d_A, M, K, h, a_coded, st);
       stage_mark(opts, BPX_STAGE_A_PREP, 1, st);

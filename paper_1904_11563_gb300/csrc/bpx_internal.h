@@ -52,6 +52,7 @@ struct WsLayout {
   // staging for the tensor-core paths (bf16 / fp8 operands; exact-slice
   // digit planes in a_hi / b_hi)
   size_t a_hi, a_lo, b_hi, b_lo, a_scale, b_scale;
+  size_t a_3, b_3;  // FP32 on the tensor cores: the third bf16 parts
   // exact-slice: max |A| per row position (h words) then max |B| per column
   // (N words), as float bits; decoded sources as exact int64 (S h N)
   size_t ex_amax, ex_c64;
@@ -71,6 +72,16 @@ struct ExactParams {
 // Fills *P for the code's sigma and K; BPX_ERR_UNSUPPORTED (with a message)
 // when the digits or the exact integer sums would not fit.
 int exact_params(const bpx_code* c, int K, ExactParams* P);
+
+// Coded rows to expect from a mask of e erased columns (launch heuristics).
+inline long long rows_expected(const bpx_code* c, int h) {
+  const long long rows = static_cast<long long>(c->num_cells) * h;
+  return c->e > 0 && c->e < c->n ? rows * (c->n - c->e) / c->n : rows;
+}
+
+// Whether BPX_FP32 products of this shape run on the tensor cores (three bf16
+// parts per operand, six products) rather than on the CUDA cores.
+bool f32_on_tensor_cores(const bpx_code* c, int N, int K, int h);
 
 // twod: the two-dimensional scheme (products are h x (N / k) blocks, operand
 // staging holds the summed A and B operands of the code's factored cells).
@@ -103,6 +114,7 @@ enum {
   CTR_NNEW,       // sources recovered this round (scratch)
   CTR_ERR,        // device error code raised by a kernel self-check
   CTR_PLAN,       // kPlanReady once a whole plan is in place (zeroed by bpx_workspace_init)
+  CTR_F32_SIMT,   // FP32 operands hold an element the tensor-core parts cannot (cleared by every schedule)
   CTR_LEN = 16
 };
 constexpr int32_t kPlanReady = 0x504C414E;  // "PLAN"

@@ -268,6 +268,20 @@ cudaError_t launch_encode_f32(const DevGraph& g, const DevPlan& p, const float* 
 cudaError_t launch_encode_split(const DevGraph& g, const DevPlan& p, const float* A, int M, int K,
                                 int h, void* a_hi, void* a_lo, cudaStream_t st);
 cudaError_t launch_b_split(const float* B, int K, int N, void* b_hi, void* b_lo, cudaStream_t st);
+// FP32 operands for the tensor cores: the coded rows / B^T as three bf16
+// parts whose sum is the FP32 value; flag (a plan counter) is raised when an
+// element's parts would not hold it.
+cudaError_t launch_encode_parts(const DevGraph& g, const DevPlan& p, const float* A, int M, int K, int h,
+                                void* const a[3], cudaStream_t st);
+cudaError_t launch_b_parts(const DevPlan& p, const float* B, int K, int N, void* const b[3], cudaStream_t st);
+// The FP32 encode and GEMM on the CUDA cores when that flag is up (else both return at once).
+cudaError_t launch_encode_f32_flagged(const DevGraph& g, const DevPlan& p, const float* A, int M, int K, int h,
+                                      float* out, cudaStream_t st);
+cudaError_t launch_gemm_f32_flagged(const DevGraph& g, const DevPlan& p, const float* a_coded, const float* B, int N,
+                                    int K, int h, float* products, float* C_direct, cudaStream_t st);
+cudaError_t launch_gemm_f32_tc(const DevPlan& p, void* const a[3], void* const b[3], int num_cells, int N, int K, int h,
+                               long long rows_est, float* products, float* C_direct, int32_t* info_out,
+                               cudaStream_t st);
 // MXFP8 staging (E4M3 data + UE8M0 scales in the GEMM's per-stage order) and GEMM.
 cudaError_t launch_encode_mx(const DevGraph& g, const DevPlan& p, const float* A, int M, int K, int h,
                              void* out, void* sfa, cudaStream_t st);

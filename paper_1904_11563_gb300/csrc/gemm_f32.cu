@@ -1,4 +1,7 @@
-// a3, plain FP32 path: coded products on the CUDA cores (FFMA).
+// a3, plain FP32 path: coded products on the CUDA cores (FFMA).  Small
+// products run here; larger ones on the tensor cores from three bf16 parts
+// per operand (gemm_tc.cu), with the flagged kernels below behind them for
+// operands those parts cannot hold.
 //
 // The coded operand (rows of the surviving cells in ascending cell order,
 // each the FP32 sum of its sources' rows) is formed by the encode pass first
@@ -33,14 +36,9 @@ __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(kPending) : "memory");
 }
 
-__global__ void __launch_bounds__(kThreads, 1)
-gemm_f32_kernel(DevPlan p, const float* __restrict__ Ac, const float* __restrict__ B, int N, int K, int h,
-                float* products, float* C_direct) {
-  const int nsurv = p.ctr[CTR_NSURV];
-  const long long Mc = static_cast<long long>(nsurv) * h;
-  const long long m0 = static_cast<long long>(blockIdx.y) * BM;
-  if (m0 >= Mc) return;
-  const int n0 = blockIdx.x * BN;
+__device__ __forceinline__ void gemm_f32_tile(const DevPlan& p, const float* __restrict__ Ac,
+                                              const float* __restrict__ B, int N, int K, int h, float* products,
+                                              float* C_direct, long long Mc, long long m0, int n0) {
 
   extern __shared__ __align__(16) float smem_f[];
   float (*As)[BK][BM + APAD] = reinterpret_cast<float (*)[BK][BM + APAD]>(smem_f);
@@ -163,7 +161,42 @@ gemm_f32_kernel(DevPlan p, const float* __restrict__ Ac, const float* __restrict
   }
 }
 
+__global__ void __launch_bounds__(kThreads, 1)
+gemm_f32_kernel(DevPlan p, const float* __restrict__ Ac, const float* __restrict__ B, int N, int K, int h,
+                float* products, float* C_direct) {
+  const long long Mc = static_cast<long long>(p.ctr[CTR_NSURV]) * h;
+  const long long m0 = static_cast<long long>(blockIdx.y) * BM;
+  if (m0 < Mc) gemm_f32_tile(p, Ac, B, N, K, h, products, C_direct, Mc, m0, blockIdx.x * BN);
+}
+
+// Behind the tensor-core FP32 GEMM: one CTA per SM walks the tiles when the
+// staging raised the flag, else returns at once.
+__global__ void __launch_bounds__(kThreads, 1)
+gemm_f32_flagged_kernel(DevPlan p, const float* __restrict__ Ac, const float* __restrict__ B, int N, int K, int h,
+                        float* products, float* C_direct) {
+  if (p.ctr[CTR_F32_SIMT] == 0) return;
+  const long long Mc = static_cast<long long>(p.ctr[CTR_NSURV]) * h;
+  const long long n_tiles = (N + BN - 1) / BN, tiles = (Mc + BM - 1) / BM * n_tiles;
+  for (long long t = blockIdx.x; t < tiles; t += gridDim.x) {
+    const long long m = t / n_tiles;
+    gemm_f32_tile(p, Ac, B, N, K, h, products, C_direct, Mc, m * BM, static_cast<int>(t - m * n_tiles) * BN);
+    __syncthreads();  // the tile's last shared-memory reads before the next tile's copies
+  }
+}
+
 }  // namespace
+
+cudaError_t launch_gemm_f32_flagged(const DevGraph& g, const DevPlan& p, const float* a_coded, const float* B, int N,
+                                    int K, int h, float* products, float* C_direct, cudaStream_t st) {
+  const long long rows = static_cast<long long>(g.num_cells) * h;
+  if (rows == 0 || N == 0) return cudaSuccess;
+  const size_t smem = sizeof(float) * kStages * BK * ((BM + APAD) + BN);
+  cudaError_t e = cudaFuncSetAttribute(gemm_f32_flagged_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       static_cast<int>(smem));
+  if (e != cudaSuccess) return e;
+  gemm_f32_flagged_kernel<<<num_sms(), kThreads, smem, st>>>(p, a_coded, B, N, K, h, products, C_direct);
+  return cudaGetLastError();
+}
 
 // a_coded: the FP32 coded rows of the surviving cells (encode pass output),
 // num_cells h rows of K floats (only the surviving ones are read).

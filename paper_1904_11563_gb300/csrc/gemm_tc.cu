@@ -47,6 +47,7 @@ namespace {
 // passes one as a __grid_constant__ parameter.
 struct __align__(64) TcJob {
   CUtensorMap map_ahi, map_alo, map_bhi, map_blo;
+  CUtensorMap map_a3, map_b3;  // third bf16 part of FP32 operands (three-part jobs)
   const int32_t* ctr;     // plan counters (surviving-cell count)
   const int32_t* surv;    // surviving cells, ascending
   const int32_t* direct;  // per cell: the source it resolves at depth 1, or -1
@@ -78,15 +79,19 @@ struct __align__(64) TcJob {
   const int32_t* b_exp;
 };
 
-template <bool kSplit, int kBN, int kBK = BK>
+// kParts: 16-bit arrays per operand (1 plain, 2 hi + lo, 3 an FP32 operand in
+// three bf16 parts).
+template <int kParts, int kBN, int kBK = BK>
 struct Stage {
   static constexpr uint32_t kA = BM * kBK * 2;   // 16 or 8 KB
   static constexpr uint32_t kB = kBN * kBK * 2;  // 32, 16 or 8 KB
-  static constexpr uint32_t kBytes = kSplit ? 2 * (kA + kB) : (kA + kB);
+  static constexpr uint32_t kBytes = kParts * (kA + kB);
   static constexpr uint32_t kAhi = 0;
   static constexpr uint32_t kAlo = kA;
-  static constexpr uint32_t kBhi = kSplit ? 2 * kA : kA;
+  static constexpr uint32_t kA3 = 2 * kA;
+  static constexpr uint32_t kBhi = kParts * kA;
   static constexpr uint32_t kBlo = kBhi + kB;
+  static constexpr uint32_t kB3 = kBhi + 2 * kB;
 };
 
 // Output stores of the epilogue: streaming (.cs), so that the products and
@@ -198,7 +203,13 @@ __device__ __forceinline__ TileRef locate(const TcJob* jobs, int njobs, long lon
 // segments exact by construction, promoted to int32 and stored to the
 // diagonal's plane).  kMode == kMode2D: the two-dimensional scheme (k-slices
 // of the cell's terms in sequence; h x w output blocks).
-template <bool kSplit, int kStages, int kBN, int kPair, int kBK, int kMode = kModeRows>
+// kParts == 3: FP32 operands, each the exact sum of three bf16 parts
+// a = a1 + a2 + a3 (8 significand bits each); the six products whose order is
+// at most 2^-16 of a b are accumulated (a1 b1; a1 b2, a2 b1; a1 b3, a2 b2,
+// a3 b1), the five small ones of a segment before a1 b1, so that only a
+// segment's few a1 b1 adds truncate at the accumulator's full magnitude.  The
+// dropped products are below 2^-25 of a b each, half an FP32 rounding.
+template <int kParts, int kStages, int kBN, int kPair, int kBK, int kMode = kModeRows>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ table, int njobs,
                long long total_tiles, int group, int seg_kb) {
@@ -206,7 +217,8 @@ gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ t
   constexpr bool k2D = kMode == kMode2D;
   static_assert(kPair == 0 || kPair == 2, "tiles are 1-CTA or CTA-pair MMAs");
   constexpr bool k2Sm = kPair == 2;
-  using St = Stage<kSplit, k2Sm ? kBN / 2 : kBN, kBK>;  // a CTA pair holds half the B tile each
+  constexpr bool kSplit = kParts >= 2;
+  using St = Stage<kParts, k2Sm ? kBN / 2 : kBN, kBK>;  // a CTA pair holds half the B tile each
   constexpr int kTmemCols = 2 * kBN;  // two FP32 segment accumulators
   constexpr int kCols = kBN / 2;      // columns per epilogue warp
   extern __shared__ uint8_t smem_raw[];
@@ -216,6 +228,9 @@ gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ t
   __shared__ uint32_t tmem_base_sh;
   __shared__ volatile int abort_flag;
 
+  // FP32 operands with an element the three parts cannot hold: the CUDA-core
+  // kernel behind this launch computes the products instead
+  if (kParts == 3 && single.ctr[CTR_F32_SIMT] != 0) return;
   const TcJob* jobs = table ? table : &single;
   const bool grouped = table != nullptr;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -320,6 +335,10 @@ gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ t
             if (kSplit) tma_load_2d_pair(base + St::kAlo, &T.J->map_alo, fb0, xa, ya);
             tma_load_2d_pair(base + St::kBhi, &T.J->map_bhi, fb0, xb, yh);
             if (kSplit) tma_load_2d_pair(base + St::kBlo, &T.J->map_blo, fb0, xb, yh);
+            if (kParts == 3) {
+              tma_load_2d_pair(base + St::kA3, &T.J->map_a3, fb0, xa, ya);
+              tma_load_2d_pair(base + St::kB3, &T.J->map_b3, fb0, xb, yh);
+            }
             continue;
           }
           mbar_expect_tx(fb, St::kBytes);
@@ -327,6 +346,10 @@ gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ t
           if (kSplit) tma_load_2d(base + St::kAlo, &T.J->map_alo, fb, xa, ya);
           tma_load_2d(base + St::kBhi, &T.J->map_bhi, fb, xb, yb);
           if (kSplit) tma_load_2d(base + St::kBlo, &T.J->map_blo, fb, xb, yb);
+          if (kParts == 3) {
+            tma_load_2d(base + St::kA3, &T.J->map_a3, fb, xa, ya);
+            tma_load_2d(base + St::kB3, &T.J->map_b3, fb, xb, yb);
+          }
         }
       }
       if ((!ok || abort_flag) && !(k2Sm && rank != 0)) {
@@ -378,6 +401,25 @@ gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ t
             const uint64_t bhi = sdesc_k<kBK>(base + St::kBhi);
             const uint64_t alo = sdesc_k<kBK>(base + St::kAlo);
             const uint64_t blo = sdesc_k<kBK>(base + St::kBlo);
+            if constexpr (kParts == 3) {
+              const uint64_t a3 = sdesc_k<kBK>(base + St::kA3), b3 = sdesc_k<kBK>(base + St::kB3);
+              uint32_t acc = kb == kb0 ? 0u : 1u;
+              auto mma = [&](uint64_t a, uint64_t b) {
+#pragma unroll
+                for (int kk = 0; kk < kBK / 16; ++kk) {
+                  const uint64_t adv = static_cast<uint64_t>(kk * 32) >> 4;
+                  if constexpr (k2Sm) umma_kf16_pair(d_tmem, a + adv, b + adv, idesc, acc);
+                  else umma_kf16(d_tmem, a + adv, b + adv, idesc, acc);
+                  acc = 1u;
+                }
+              };
+              mma(a3, bhi);
+              mma(alo, blo);
+              mma(ahi, b3);
+              mma(alo, bhi);
+              mma(ahi, blo);
+              mma(ahi, bhi);
+            } else
 #pragma unroll
             for (int kk = 0; kk < kBK / 16; ++kk) {
               const uint64_t adv = static_cast<uint64_t>(kk * 32) >> 4;  // 16 bf16 = 32 B
@@ -591,16 +633,27 @@ int tile_pair(int config) {
 }
 int tile_bk(int config) { return (config % 10) >= 5 ? 32 : 64; }
 
+// FP32 in three parts: 128 x 128 tiles of single CTAs where the 256 x 256
+// tiles of CTA pairs would leave too many SMs idle in their last wave.
+bool f32_small_tiles(long long rows, int N) {
+  const long long pairs = std::max(1, num_sms() / 2), sms = std::max(1, num_sms());
+  const long long big = (rows + 255) / 256 * ((N + 255) / 256), small = (rows + 127) / 128 * ((N + 127) / 128);
+  // time in units of a 256 x 256 tile's (K = 8192: 3.67 ms against 4.77 ms
+  // with 128 x 128 tiles, which re-read more operand bytes per MMA): a
+  // 128 x 128 tile takes 0.65
+  return 0.65 * static_cast<double>((small + sms - 1) / sms) < static_cast<double>((big + pairs - 1) / pairs);
+}
+
 // seg_kb: k-slices of kBK per TMEM accumulation segment.
-template <bool kSplit, int kStages, int kBN, int kPair, int kBK, int kMode = kModeRows>
+template <int kParts, int kStages, int kBN, int kPair, int kBK, int kMode = kModeRows>
 cudaError_t launch_variant(const TcJob& single, const TcJob* table, int njobs, long long total_tiles,
                            int group, int seg_kb, cudaStream_t st) {
   // 32-wide slices: 32 KB of slack after the stages, so that the descriptors
   // of the 64-byte swizzled layout can never reach past the allocation.
   // (a CTA of a cta_group::2 pair stages half the B tile)
-  using St = Stage<kSplit, kPair == 2 ? kBN / 2 : kBN, kBK>;
+  using St = Stage<kParts, kPair == 2 ? kBN / 2 : kBN, kBK>;
   const size_t smem = static_cast<size_t>(kStages) * St::kBytes + 1024 + (kBK == 32 ? 32768 : 0);
-  auto kern = gemm_tc_kernel<kSplit, kStages, kBN, kPair, kBK, kMode>;
+  auto kern = gemm_tc_kernel<kParts, kStages, kBN, kPair, kBK, kMode>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
   if (total_tiles <= 0) return cudaSuccess;
@@ -638,12 +691,12 @@ cudaError_t dispatch_bk(bool split3, int bn, int pair, const TcJob& single, cons
                         long long total_tiles, int group, int seg_kb, cudaStream_t st) {
   constexpr int m = BK / kBK;  // stages scale up as slices shrink
   seg_kb *= m;                 // configs count segments in 64-wide k-blocks
-#define BPX_LV(SPLIT, STAGES, BN, PAIR) \
-  launch_variant<SPLIT, STAGES, BN, PAIR, kBK, kMode>(single, table, njobs, total_tiles, group, seg_kb, st)
+#define BPX_LV(PARTS, STAGES, BN, PAIR) \
+  launch_variant<PARTS, STAGES, BN, PAIR, kBK, kMode>(single, table, njobs, total_tiles, group, seg_kb, st)
   // CTA-pair MMAs: a stage holds the CTA's A rows and half the B tile
-  if (pair == 2) return split3 ? BPX_LV(true, 3 * m, 256, 2) : BPX_LV(false, 6 * m, 256, 2);
-  if (split3) return bn == 128 ? BPX_LV(true, 3 * m, 128, 0) : BPX_LV(true, 2 * m, 256, 0);
-  return bn == 128 ? BPX_LV(false, 6 * m, 128, 0) : BPX_LV(false, 4 * m, 256, 0);
+  if (pair == 2) return split3 ? BPX_LV(2, 3 * m, 256, 2) : BPX_LV(1, 6 * m, 256, 2);
+  if (split3) return bn == 128 ? BPX_LV(2, 3 * m, 128, 0) : BPX_LV(2, 2 * m, 256, 0);
+  return bn == 128 ? BPX_LV(1, 6 * m, 128, 0) : BPX_LV(1, 4 * m, 256, 0);
 #undef BPX_LV
 }
 
@@ -655,9 +708,9 @@ cudaError_t dispatch_exact_bk(int bn, int pair, const TcJob& J, long long total_
                               cudaStream_t st) {
   constexpr int m = BK / kBK;
   if (pair == 2)
-    return launch_variant<false, 6 * m, 256, 2, kBK, kModeExact>(J, nullptr, 1, total_tiles, group, seg, st);
-  if (bn == 128) return launch_variant<false, 6 * m, 128, 0, kBK, kModeExact>(J, nullptr, 1, total_tiles, group, seg, st);
-  return launch_variant<false, 4 * m, 256, 0, kBK, kModeExact>(J, nullptr, 1, total_tiles, group, seg, st);
+    return launch_variant<1, 6 * m, 256, 2, kBK, kModeExact>(J, nullptr, 1, total_tiles, group, seg, st);
+  if (bn == 128) return launch_variant<1, 6 * m, 128, 0, kBK, kModeExact>(J, nullptr, 1, total_tiles, group, seg, st);
+  return launch_variant<1, 4 * m, 256, 0, kBK, kModeExact>(J, nullptr, 1, total_tiles, group, seg, st);
 }
 
 cudaError_t dispatch_exact(int bn, int pair, int bk, const TcJob& J, long long total_tiles, int group, int seg,
@@ -796,6 +849,30 @@ cudaError_t launch_gemm_tc(const DevGraph& g, const DevPlan& p, const void* a_hi
   const int units = pair ? (J.m_tiles_max + 1) / 2 : J.m_tiles_max;
   const long long tiles = static_cast<long long>(units) * J.n_tiles;
   return dispatch(split3, bn, pair, bk, J, nullptr, 1, tiles, group, seg_kb, st);
+}
+
+// FP32 operands in three bf16 parts (a[i], b[i]): 256 x 256 tiles of CTA-pair
+// MMAs, or 128 x 128 tiles of 1-CTA MMAs (see f32_small_tiles); 64-wide
+// segments (24 MMAs each, so a drain is as rare as with hi + lo operands).
+// Tensor-bound: 96 KB staged per 24 MMAs and CTA, 32 B a clock.  Benchmark
+// workload (9088 coded rows, 8192 x 8192): 3.67 ms, 2.0 PFLOP/s of MMA work,
+// against 19.1 ms for the CUDA-core GEMM (FFMA-bound); relative error of a
+// directly computed block 1.3e-7 at K = 1992 against 8.0e-7, 1.7e-7 at 4096
+// against 1.1e-6.  32-wide k-slices (four stages) ran 3.73 ms.
+cudaError_t launch_gemm_f32_tc(const DevPlan& p, void* const a[3], void* const b[3], int num_cells, int N, int K, int h,
+                               long long rows_est, float* products, float* C_direct, int32_t* info_out,
+                               cudaStream_t st) {
+  const bool small = f32_small_tiles(rows_est, N);
+  const int bn = small ? 128 : 256;
+  TcJob J;
+  if (!tc_fill_job(&J, p, a[0], a[1], b[0], b[1], num_cells, N, K, h, bn, !small, BK, products, C_direct, info_out))
+    return cudaErrorInvalidValue;
+  const long long rows = static_cast<long long>(num_cells) * h;
+  if (!make_map(&J.map_a3, a[2], rows, K, BM) || !make_map(&J.map_b3, b[2], N, K, 128)) return cudaErrorInvalidValue;
+  const int units = small ? J.m_tiles_max : (J.m_tiles_max + 1) / 2;
+  const long long tiles = static_cast<long long>(units) * J.n_tiles;
+  if (small) return launch_variant<3, 2, 128, 0, BK>(J, nullptr, 1, tiles, 8, 1, st);
+  return launch_variant<3, 2, 256, 2, BK>(J, nullptr, 1, tiles, 8, 1, st);
 }
 
 // Exact-slice digit products: a_planes = coded rows x (S Kp) bf16, b_planes =

@@ -18,6 +18,8 @@
 #include <cuda_fp16.h>
 #include <cuda_fp8.h>
 
+#include <algorithm>
+
 #include "device_common.cuh"
 
 namespace bpx {
@@ -26,16 +28,49 @@ namespace {
 constexpr int kEncThreads = 128;
 constexpr int kEncVec = 8;  // consecutive K elements per thread (two float4 loads per source)
 
+// An FP32 value as three bf16 parts: p1 = RN(x), p2 = RN(x - p1), p3 = x - p1
+// - p2, whose sum is x exactly (8 significand bits each) while x lies in
+// [2^-102, 2^127): p1 does not round up to infinity and p3's last bit is a
+// normal bf16.  Zero is exact too; any other value is reported.
+__device__ __forceinline__ bool parts_unfit(float x) {
+  const uint32_t u = __float_as_uint(x) & 0x7fffffffu;
+  return u != 0u && u - (25u << 23) >= (254u - 25u) << 23;
+}
+__device__ __forceinline__ bool parts_split8(const float (&v)[8], __nv_bfloat16* o1, __nv_bfloat16* o2,
+                                             __nv_bfloat16* o3) {
+  uint32_t w1[4], w2[4], w3[4];
+  bool unfit = false;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const float x0 = v[2 * q], x1 = v[2 * q + 1];
+    unfit |= parts_unfit(x0) | parts_unfit(x1);
+    const __nv_bfloat162 p1 = __floats2bfloat162_rn(x0, x1);
+    const float2 f1 = __bfloat1622float2(p1);
+    const float r0 = x0 - f1.x, r1 = x1 - f1.y;
+    const __nv_bfloat162 p2 = __floats2bfloat162_rn(r0, r1);
+    const float2 f2 = __bfloat1622float2(p2);
+    const __nv_bfloat162 p3 = __floats2bfloat162_rn(r0 - f2.x, r1 - f2.y);
+    w1[q] = *reinterpret_cast<const uint32_t*>(&p1);
+    w2[q] = *reinterpret_cast<const uint32_t*>(&p2);
+    w3[q] = *reinterpret_cast<const uint32_t*>(&p3);
+  }
+  *reinterpret_cast<uint4*>(o1) = make_uint4(w1[0], w1[1], w1[2], w1[3]);
+  *reinterpret_cast<uint4*>(o2) = make_uint4(w2[0], w2[1], w2[2], w2[3]);
+  *reinterpret_cast<uint4*>(o3) = make_uint4(w3[0], w3[1], w3[2], w3[3]);
+  return unfit;
+}
+
 // A CTA covers `rows` coded rows x `cols` columns (cols = min(1024, K rounded
 // up to a power of two), rows = 1024 / cols): short K still fills the CTA.
 // blockIdx.x walks the coded rows fastest so that CTAs resident together read
 // the same K-chunk of A (L2 reuse of a source block across the cells that
 // contain it).
-template <int kMode>  // 0: FP32 out, 1: bf16 hi only, 2: bf16 hi + lo
+template <int kMode>  // 0: FP32 out, 1: bf16 hi only, 2: bf16 hi + lo, 3: three bf16 parts
 __device__ __forceinline__ void encode_body(const DevGraph& g, const DevPlan& p,
                                             const float* __restrict__ A, int M, int K, int h,
                                             float* out_f32, __nv_bfloat16* out_hi,
-                                            __nv_bfloat16* out_lo, int rblock, int kchunk) {
+                                            __nv_bfloat16* out_lo, int rblock, int kchunk,
+                                            __nv_bfloat16* out_3 = nullptr) {
   const int tpr = enc_threads_per_row(K);  // threads per row
   const int row = rblock * (kEncThreads / tpr) + threadIdx.x / tpr;  // coded row, compacted order
   const int nsurv = p.ctr[CTR_NSURV];
@@ -70,6 +105,8 @@ __device__ __forceinline__ void encode_body(const DevGraph& g, const DevPlan& p,
     float4* d = reinterpret_cast<float4*>(out_f32 + o);
     d[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
     d[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
+  } else if constexpr (kMode == 3) {
+    if (parts_split8(acc, out_hi + o, out_lo + o, out_3 + o)) p.ctr[CTR_F32_SIMT] = 1;
   } else {
     uint32_t hv[4], lv[4];
 #pragma unroll
@@ -94,12 +131,32 @@ encode_kernel(DevGraph g, DevPlan p, const float* __restrict__ A, int M, int K, 
   encode_body<kMode>(g, p, A, M, K, h, out_f32, out_hi, out_lo, blockIdx.x, blockIdx.y);
 }
 
+__global__ void __launch_bounds__(kEncThreads)
+encode_parts_kernel(DevGraph g, DevPlan p, const float* __restrict__ A, int M, int K, int h, __nv_bfloat16* o1,
+                    __nv_bfloat16* o2, __nv_bfloat16* o3) {
+  encode_body<3>(g, p, A, M, K, h, nullptr, o1, o2, blockIdx.x, blockIdx.y, o3);
+}
+
+// The FP32 encode behind the tensor-core FP32 GEMM: a fixed grid walks the
+// (row block, k-chunk) blocks when the staging raised the flag.
+__global__ void __launch_bounds__(kEncThreads)
+encode_f32_flagged_kernel(DevGraph g, DevPlan p, const float* __restrict__ A, int M, int K, int h, float* out,
+                          long long row_blocks, long long blocks) {
+  if (p.ctr[CTR_F32_SIMT] == 0) return;
+  for (long long b = blockIdx.x; b < blocks; b += gridDim.x) {
+    const long long kc = b / row_blocks;
+    encode_body<0>(g, p, A, M, K, h, out, nullptr, nullptr, static_cast<int>(b - kc * row_blocks), static_cast<int>(kc));
+  }
+}
+
 // B (K x N row-major FP32) -> Bt (N x K row-major bf16) through a 64 x 64
 // shared-memory tile: float4 reads along N, 16-byte bf16 writes along K.
 constexpr int kTile = 64;
-__device__ __forceinline__ void b_split_body(const float* __restrict__ B, int K, int N,
+template <bool kParts3 = false>
+__device__ __forceinline__ bool b_split_body(const float* __restrict__ B, int K, int N,
                                              __nv_bfloat16* bt_hi, __nv_bfloat16* bt_lo, int bx,
-                                             int by) {
+                                             int by, __nv_bfloat16* bt_3 = nullptr) {
+  bool unfit = false;
   __shared__ float tile[kTile][kTile + 1];
   const int n0 = bx * kTile, k0 = by * kTile;
   {
@@ -124,6 +181,14 @@ __device__ __forceinline__ void b_split_body(const float* __restrict__ B, int K,
     const int r = t >> 3, kc = t & 7;
     const int n = n0 + r, k = k0 + 8 * kc;
     if (n >= N || k >= K) continue;
+    if constexpr (kParts3) {
+      float v[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) v[q] = tile[8 * kc + q][r];
+      const long long o = static_cast<long long>(n) * K + k;
+      unfit |= parts_split8(v, bt_hi + o, bt_lo + o, bt_3 + o);
+      continue;
+    }
     uint32_t hv[4], lv[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -138,6 +203,13 @@ __device__ __forceinline__ void b_split_body(const float* __restrict__ B, int K,
     *reinterpret_cast<uint4*>(bt_hi + o) = make_uint4(hv[0], hv[1], hv[2], hv[3]);
     if (bt_lo) *reinterpret_cast<uint4*>(bt_lo + o) = make_uint4(lv[0], lv[1], lv[2], lv[3]);
   }
+  return unfit;
+}
+
+__global__ void __launch_bounds__(256)
+b_parts_kernel(DevPlan p, const float* __restrict__ B, int K, int N, __nv_bfloat16* o1, __nv_bfloat16* o2,
+               __nv_bfloat16* o3) {
+  if (b_split_body<true>(B, K, N, o1, o2, blockIdx.x, blockIdx.y, o3)) p.ctr[CTR_F32_SIMT] = 1;
 }
 
 __global__ void __launch_bounds__(256)
@@ -702,6 +774,35 @@ cudaError_t launch_b_f16(const float* B, int K, int N, void* b_hi, void* b_lo, u
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   b_split_f16_kernel<<<dim3((N + kTile - 1) / kTile, (K + kTile - 1) / kTile), 256, 0, st>>>(
       B, K, N, b_max, static_cast<__half*>(b_hi), static_cast<__half*>(b_lo), b_exp);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_encode_parts(const DevGraph& g, const DevPlan& p, const float* A, int M, int K, int h,
+                                void* const a[3], cudaStream_t st) {
+  const long long rows = static_cast<long long>(g.num_cells) * h;
+  if (rows == 0 || K == 0) return cudaSuccess;
+  dim3 grid(static_cast<unsigned>(enc_row_blocks(rows, K)), static_cast<unsigned>(enc_k_chunks(K)));
+  encode_parts_kernel<<<grid, kEncThreads, 0, st>>>(g, p, A, M, K, h, static_cast<__nv_bfloat16*>(a[0]),
+                                                    static_cast<__nv_bfloat16*>(a[1]),
+                                                    static_cast<__nv_bfloat16*>(a[2]));
+  return cudaGetLastError();
+}
+
+cudaError_t launch_b_parts(const DevPlan& p, const float* B, int K, int N, void* const b[3], cudaStream_t st) {
+  if (K == 0 || N == 0) return cudaSuccess;
+  dim3 grid((N + kTile - 1) / kTile, (K + kTile - 1) / kTile);
+  b_parts_kernel<<<grid, 256, 0, st>>>(p, B, K, N, static_cast<__nv_bfloat16*>(b[0]), static_cast<__nv_bfloat16*>(b[1]),
+                                       static_cast<__nv_bfloat16*>(b[2]));
+  return cudaGetLastError();
+}
+
+cudaError_t launch_encode_f32_flagged(const DevGraph& g, const DevPlan& p, const float* A, int M, int K, int h,
+                                      float* out, cudaStream_t st) {
+  const long long rows = static_cast<long long>(g.num_cells) * h;
+  if (rows == 0 || K == 0) return cudaSuccess;
+  const long long rb = enc_row_blocks(rows, K), blocks = rb * enc_k_chunks(K);
+  const unsigned grid = static_cast<unsigned>(std::min<long long>(blocks, 8LL * num_sms()));
+  encode_f32_flagged_kernel<<<grid, kEncThreads, 0, st>>>(g, p, A, M, K, h, out, rb, blocks);
   return cudaGetLastError();
 }
 

@@ -196,6 +196,7 @@ __device__ __forceinline__ void schedule_body(const DevGraph& g, const DevPlan& 
     if (tid == 0) {
       p.ctr[CTR_NSURV] = nsurv;
       p.ctr[CTR_PLAN] = 0;  // the rest of the plan follows (part 2)
+      p.ctr[CTR_F32_SIMT] = 0;
       p.info[BPX_INFO_DEVICE_ERR] = 0;  // cleared before the products run
     }
     return;
@@ -278,6 +279,7 @@ __device__ __forceinline__ void schedule_body(const DevGraph& g, const DevPlan& 
     p.ctr[CTR_NWAVES] = round;
     p.ctr[CTR_NREC] = nrec;
     p.ctr[CTR_ERR] = 0;
+    if (part != 2) p.ctr[CTR_F32_SIMT] = 0;
     p.ctr[CTR_PLAN] = kPlanReady;
     int32_t inf[BPX_INFO_LEN];
     for (int i = 0; i < BPX_INFO_LEN; ++i) inf[i] = 0;

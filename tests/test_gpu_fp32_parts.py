@@ -1,0 +1,68 @@
+"""FP32 products on the tensor cores (three bf16 parts per operand): tile and
+K edges against FP64, element by element, and operands that the parts cannot
+hold, which the CUDA-core kernel computes."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = [pytest.mark.gpu,
+              pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a CUDA GPU")]
+
+
+def _direct(bpx, A, B):
+    """C from the data columns alone (no erasure: every block is a product)."""
+    code = bpx.Code.systematic(8, 3, 8)
+    (M, K), N = A.shape, B.shape[1]
+    h = -(-M // code.num_sources)
+    ws = bpx.Workspace(code, M, N, K, h, bpx.FP32)
+    mask = torch.zeros(code.n, dtype=torch.uint8, device="cuda")
+    C, info = bpx.coded_matmul(code, A, B, h, bpx.FP32, mask, ws)
+    assert int(info[bpx.INFO_STATUS]) == bpx.OK
+    return C[:M]
+
+
+# 128 x 128 and 256 x 256 tiles, ragged rows, columns and K; K just past the
+# smallest the form takes, a multiple of 64, one 8-element chunk more
+@pytest.mark.parametrize("M,K,N", [(2050, 136, 1028), (1000, 520, 1100), (640, 2056, 516), (4096, 1024, 2048),
+                                   (4100, 1032, 2052), (8200, 128, 516)])
+@pytest.mark.parametrize("spread", [0.0, 20.0])
+def test_tile_edges(libbpx, M, K, N, spread):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(M + K)
+    A, B = (torch.randn(s, generator=g, device="cuda") *
+            torch.exp(spread * (torch.rand(s, generator=g, device="cuda") - 0.5)) for s in ((M, K), (K, N)))
+    C = _direct(libbpx, A, B).double()
+    A, B = A.double(), B.double()
+    # per element, relative to sum |a||b|: three dropped products (2^-25 each),
+    # a 64-wide segment's truncating adds (24, the full-magnitude ones at
+    # 2^-23), one rounded add per segment (2^-24)
+    gamma = (-(-K // 64) + 2 * 24 + 2) * 2.0 ** -24
+    assert ((C - A @ B).abs() <= gamma * (A.abs() @ B.abs())).all()
+
+
+@pytest.mark.parametrize("value", [float("inf"), float("-inf"), float("nan"), 3.4e38, 1e-40, 2.0 ** -103])
+@pytest.mark.parametrize("where", ["A", "B"])
+def test_elements_the_parts_cannot_hold(libbpx, value, where):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(3)
+    A = torch.randn((1000, 520), generator=g, device="cuda")
+    B = torch.randn((520, 1100), generator=g, device="cuda")
+    A[5, 17], B[17, 3] = 1.0, 0.5
+    (A if where == "A" else B)[5 if where == "A" else 17, 17 if where == "A" else 3] = value
+    if abs(value) < 1e-30:  # a row / column of such magnitudes: the products stay normal numbers
+        if where == "A":
+            A[5] *= 2.0 ** -103
+            A[5, 17] = value
+        else:
+            B[:, 3] *= 2.0 ** -103
+            B[17, 3] = value
+    C = _direct(libbpx, A, B).double()
+    R = A.double() @ B.double()
+    big = R.abs() > 3.4028234e38  # past FP32's largest
+    R = torch.where(big, torch.sign(R) * float("inf"), R)
+    assert torch.equal(torch.isnan(C), torch.isnan(R))
+    fin = torch.isfinite(R)
+    assert torch.equal(C[~fin & ~torch.isnan(R)], R[~fin & ~torch.isnan(R)])
+    S = A.double().abs() @ B.double().abs()
+    # an FFMA chain of K terms: K roundings of 2^-24, plus the last bit of a subnormal sum
+    assert ((C - R).abs()[fin] <= (520 * 2.0 ** -24 * S + 520 * 2.0 ** -149)[fin]).all()
