@@ -262,7 +262,7 @@ int products_impl(const bpx_code* c, const float* d_A, const float* d_B, int M, 
       e = bpx::launch_encode_f32(g, p, d_A, M, K, h, a_coded, st);
       stage_mark(opts, BPX_STAGE_A_PREP, 1, st);
       stage_mark(opts, BPX_STAGE_GEMM, 0, st);
-      if (e == cudaSuccess) e = bpx::launch_gemm_f32(g, p, a_coded, d_B, N, K, h, d_products, d_C, st);
+      if (e == cudaSuccess) e = bpx::launch_gemm_f32(g, p, a_coded, d_B, N, K, h, bpx::rows_expected(c, h), d_products, d_C, st);
       stage_mark(opts, BPX_STAGE_GEMM, 1, st);
       break;
     }

@@ -351,14 +351,16 @@ int exact_params(const bpx_code* c, int K, ExactParams* P) {
   return BPX_OK;
 }
 
-// The line between the two FP32 forms (whole calls, 128 x 256 CUDA-core tiles):
-// 1024 x 512 x 512 109 against 54 us, 512 x 768 x 512 148 against 58 us.
+// The line between the two FP32 forms.  Staging of B and GEMM, CUDA cores
+// against tensor cores (coded rows x K x N): 568 x 768 x 512 (0.22 G
+// multiply-adds) 27 against 37 us, 1136 x 512 x 512 (0.30 G) 27 against 32,
+// 1136 x 1024 x 1024 (1.2 G) 88 against 42.
 // Thin products (N K <= 65536) stay on the CUDA cores, so that their
 // workspace, mostly coded operands, stays below split-BF16's.
 bool f32_on_tensor_cores(const bpx_code* c, int N, int K, int h) {
   if (N <= 0 || K <= 0 || h <= 0) return false;
   return K >= 128 && static_cast<long long>(N) * K > 65536 &&
-         static_cast<double>(rows_expected(c, h)) * N * K >= 134217728.0;
+         static_cast<double>(rows_expected(c, h)) * N * K >= 4e8;
 }
 
 WsLayout ws_layout(const bpx_code* c, int M, int N, int K, int h, int precision, bool twod) {

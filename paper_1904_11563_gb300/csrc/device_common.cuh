@@ -291,7 +291,7 @@ cudaError_t launch_gemm_mx(const DevPlan& p, const void* a8, const void* sfa, co
                            int32_t* info_out, cudaStream_t st);
 // Plain FP32 coded GEMM over the encode pass's FP32 coded rows.
 cudaError_t launch_gemm_f32(const DevGraph& g, const DevPlan& p, const float* a_coded, const float* B, int N, int K,
-                            int h, float* products, float* C_direct, cudaStream_t st);
+                            int h, long long rows_est, float* products, float* C_direct, cudaStream_t st);
 // Tensor-core coded GEMM over the staged bf16 operands (split or plain).
 // The encode fused into the GEMM's operand load (BPX_BF16 / BPX_BF16X3,
 // CTA-pair 256 x 256 tiles): the coded rows are summed from A and split on

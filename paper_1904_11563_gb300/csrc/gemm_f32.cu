@@ -169,6 +169,98 @@ gemm_f32_kernel(DevPlan p, const float* __restrict__ Ac, const float* __restrict
   if (m0 < Mc) gemm_f32_tile(p, Ac, B, N, K, h, products, C_direct, Mc, m0, blockIdx.x * BN);
 }
 
+// Small products: BM x BN tiles, TM x 4 outputs a thread, so that a few
+// hundred rows still spread over the SMs.  Both operands arrive by cp.async
+// (A as it lies, k fastest; a thread reads four k of a row in one 16-byte
+// load) into a ring of kSmallStages 32-wide k-steps.  Each output is one FMA
+// chain over ascending k, the bits of the 128 x 256 kernel.
+constexpr int kSmallBK = 32, kSmallStages = 3;
+
+template <int SM, int SN, int TM>
+__global__ void __launch_bounds__((SM / TM) * (SN / 4))
+gemm_f32_small_kernel(DevPlan p, const float* __restrict__ Ac, const float* __restrict__ B, int N, int K, int h,
+                      float* products, float* C_direct) {
+  constexpr int kThr = (SM / TM) * (SN / 4), kLd = kSmallBK + 4;
+  __shared__ __align__(16) float As[kSmallStages][SM][kLd];
+  __shared__ __align__(16) float Bs[kSmallStages][kSmallBK][SN];
+  const long long Mc = static_cast<long long>(p.ctr[CTR_NSURV]) * h;
+  const long long m0 = static_cast<long long>(blockIdx.y) * SM;
+  if (m0 >= Mc) return;
+  const int n0 = blockIdx.x * SN;
+  const int tx = threadIdx.x % (SN / 4), ty = threadIdx.x / (SN / 4);
+  auto load = [&](int buf, int k0) {
+    for (int i = threadIdx.x; i < SM * (kSmallBK / 4); i += kThr) {
+      const int r = i / (kSmallBK / 4), k = k0 + 4 * (i % (kSmallBK / 4));
+      const bool v = m0 + r < Mc && k < K;
+      cp_async16(&As[buf][r][k - k0], v ? Ac + (m0 + r) * K + k : Ac, v);
+    }
+    for (int i = threadIdx.x; i < kSmallBK * (SN / 4); i += kThr) {
+      const int k = k0 + i / (SN / 4), n = n0 + 4 * (i % (SN / 4));
+      const bool v = k < K && n < N;
+      cp_async16(&Bs[buf][k - k0][n - n0], v ? B + static_cast<long long>(k) * N + n : B, v);
+    }
+  };
+  float acc[TM][4];
+#pragma unroll
+  for (int i = 0; i < TM; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+  const int ktiles = (K + kSmallBK - 1) / kSmallBK;
+#pragma unroll
+  for (int s = 0; s < kSmallStages - 1; ++s) {
+    if (s < ktiles) load(s, s * kSmallBK);
+    cp_async_commit();
+  }
+  for (int kt = 0; kt < ktiles; ++kt) {
+    const int buf = kt % kSmallStages;
+    cp_async_wait<kSmallStages - 2>();
+    __syncthreads();
+    const int nx = kt + kSmallStages - 1;
+    if (nx < ktiles) load(nx % kSmallStages, nx * kSmallBK);
+    cp_async_commit();
+#pragma unroll
+    for (int kk = 0; kk < kSmallBK; kk += 4) {
+      float4 a[TM];
+#pragma unroll
+      for (int i = 0; i < TM; ++i) a[i] = *reinterpret_cast<const float4*>(&As[buf][ty * TM + i][kk]);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float4 b = *reinterpret_cast<const float4*>(&Bs[buf][kk + q][tx * 4]);
+#pragma unroll
+        for (int i = 0; i < TM; ++i) {
+          const float av = q == 0 ? a[i].x : q == 1 ? a[i].y : q == 2 ? a[i].z : a[i].w;
+          acc[i][0] = fmaf(av, b.x, acc[i][0]);
+          acc[i][1] = fmaf(av, b.y, acc[i][1]);
+          acc[i][2] = fmaf(av, b.z, acc[i][2]);
+          acc[i][3] = fmaf(av, b.w, acc[i][3]);
+        }
+      }
+    }
+  }
+  cp_async_wait<0>();
+  const int n = n0 + tx * 4;
+  if (n >= N) return;
+#pragma unroll
+  for (int i = 0; i < TM; ++i) {
+    const long long r = m0 + ty * TM + i;
+    if (r >= Mc) continue;
+    const int ci = static_cast<int>(r / h), j = static_cast<int>(r - static_cast<long long>(ci) * h);
+    const int cell = p.surv[ci];
+    const int ds = C_direct ? p.direct[cell] : -1;
+    float* dst = ds >= 0 ? C_direct + (static_cast<long long>(ds) * h + j) * N
+                         : products + (static_cast<long long>(cell) * h + j) * N;
+    *reinterpret_cast<float4*>(dst + n) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+  }
+}
+
+template <int SM, int SN, int TM>
+cudaError_t launch_small(const DevPlan& p, const float* a_coded, const float* B, long long rows, int N, int K, int h,
+                         float* products, float* C_direct, cudaStream_t st) {
+  const dim3 grid((N + SN - 1) / SN, static_cast<unsigned>((rows + SM - 1) / SM));
+  gemm_f32_small_kernel<SM, SN, TM><<<grid, (SM / TM) * (SN / 4), 0, st>>>(p, a_coded, B, N, K, h, products, C_direct);
+  return cudaGetLastError();
+}
+
 // Behind the tensor-core FP32 GEMM: one CTA per SM walks the tiles when the
 // staging raised the flag, else returns at once.
 __global__ void __launch_bounds__(kThreads, 1)
@@ -199,11 +291,25 @@ cudaError_t launch_gemm_f32_flagged(const DevGraph& g, const DevPlan& p, const f
 }
 
 // a_coded: the FP32 coded rows of the surviving cells (encode pass output),
-// num_cells h rows of K floats (only the surviving ones are read).
+// num_cells h rows of K floats (only the surviving ones are read); rows_est:
+// the coded rows to expect.
 cudaError_t launch_gemm_f32(const DevGraph& g, const DevPlan& p, const float* a_coded, const float* B, int N, int K,
-                            int h, float* products, float* C_direct, cudaStream_t st) {
+                            int h, long long rows_est, float* products, float* C_direct, cudaStream_t st) {
   const long long rows = static_cast<long long>(g.num_cells) * h;
   if (rows == 0 || N == 0) return cudaSuccess;
+  // The smallest tile that still gives every SM one: 128 x 256 tiles of a few
+  // hundred rows leave most SMs idle.  GEMM time, 128 x 256 against the form
+  // chosen (coded rows x K x N): 568 x 256 x 128 49.1 -> 10.5 us (32 x 32),
+  // 568 x 768 x 512 127 -> 26.6 (32 x 64), 1136 x 512 x 512 88 -> 26.9 and
+  // 9088 x 256 x 256 49.1 -> 36.8 (64 x 64); with 144 tiles of 128 x 256
+  // (2272 x 64 x 2048) those keep: 18.7 against 24.5.
+  const long long sms = num_sms();
+  auto tiles = [&](int m, int n) { return (rows_est + m - 1) / m * ((N + n - 1) / n); };
+  if ((rows + 31) / 32 <= 65535 && 10 * tiles(BM, BN) < 9 * sms) {
+    if (2 * tiles(32, 64) <= sms) return launch_small<32, 32, 2>(p, a_coded, B, rows, N, K, h, products, C_direct, st);
+    if (tiles(32, 64) <= sms) return launch_small<32, 64, 4>(p, a_coded, B, rows, N, K, h, products, C_direct, st);
+    return launch_small<64, 64, 8>(p, a_coded, B, rows, N, K, h, products, C_direct, st);
+  }
   const size_t smem = sizeof(float) * kStages * BK * ((BM + APAD) + BN);
   cudaError_t e = cudaFuncSetAttribute(gemm_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(smem));

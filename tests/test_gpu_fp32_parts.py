@@ -1,6 +1,6 @@
-"""FP32 products on the tensor cores (three bf16 parts per operand): tile and
-K edges against FP64, element by element, and operands that the parts cannot
-hold, which the CUDA-core kernel computes."""
+"""FP32 products against FP64, element by element: on the tensor cores (three
+bf16 parts per operand) at tile and K edges, with operands that the parts
+cannot hold, and on the CUDA cores at the edges of each tile size."""
 import numpy as np
 import pytest
 
@@ -23,7 +23,7 @@ def _direct(bpx, A, B):
 
 # 128 x 128 and 256 x 256 tiles, ragged rows, columns and K; K just past the
 # smallest the form takes, a multiple of 64, one 8-element chunk more
-@pytest.mark.parametrize("M,K,N", [(2050, 136, 1028), (1000, 520, 1100), (640, 2056, 516), (4096, 1024, 2048),
+@pytest.mark.parametrize("M,K,N", [(2050, 136, 1540), (1000, 520, 1100), (640, 2056, 516), (4096, 1024, 2048),
                                    (4100, 1032, 2052), (8200, 128, 516)])
 @pytest.mark.parametrize("spread", [0.0, 20.0])
 def test_tile_edges(libbpx, M, K, N, spread):
@@ -66,3 +66,17 @@ def test_elements_the_parts_cannot_hold(libbpx, value, where):
     S = A.double().abs() @ B.double().abs()
     # an FFMA chain of K terms: K roundings of 2^-24, plus the last bit of a subnormal sum
     assert ((C - R).abs()[fin] <= (520 * 2.0 ** -24 * S + 520 * 2.0 ** -149)[fin]).all()
+
+
+# 32 x 32, 32 x 64, 64 x 64 and 128 x 256 tiles: ragged rows, columns and K
+@pytest.mark.parametrize("M,K,N", [(512, 256, 128), (200, 264, 132), (65, 8, 4), (130, 40, 68), (520, 776, 516),
+                                   (1000, 1000, 200), (8200, 264, 244), (2050, 72, 2052)])
+def test_cuda_core_tile_edges(libbpx, M, K, N):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(M + K)
+    A = torch.randn((M, K), generator=g, device="cuda")
+    B = torch.randn((K, N), generator=g, device="cuda")
+    C = _direct(libbpx, A, B).double()
+    A, B = A.double(), B.double()
+    # one FMA chain of K terms
+    assert ((C - A @ B).abs() <= K * 2.0 ** -24 * (A.abs() @ B.abs())).all()
