@@ -117,6 +117,12 @@ extern "C" int bpx_workspace_init(const bpx_code* c, void* ws, size_t ws_bytes, 
   }
   cudaError_t e = cudaMemsetAsync(base + L.p_info, 0, L.plan_end - L.p_info, S(stream));
   if (e != cudaSuccess) return cuda_fail(e, "bpx_workspace_init: memset");
+  // the schedule's tables, in plan arrays it then leaves alone
+  if (!c->word0.empty())
+    e = cudaMemcpyAsync(base + L.p_word, c->word0.data(), c->word0.size() * 4, cudaMemcpyHostToDevice, S(stream));
+  if (e == cudaSuccess && !c->affine.empty())
+    e = cudaMemcpyAsync(base + L.p_cursor, c->affine.data(), c->affine.size() * 4, cudaMemcpyHostToDevice, S(stream));
+  if (e != cudaSuccess) return cuda_fail(e, "bpx_workspace_init: copy");
   e = cudaStreamSynchronize(S(stream));
   if (e != cudaSuccess) return cuda_fail(e, "bpx_workspace_init: sync");
   return BPX_OK;

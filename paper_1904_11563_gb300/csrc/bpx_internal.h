@@ -25,6 +25,12 @@ struct bpx_code {
   // decreasing term count (ties by id); gray2 counts cells with > 1 term.
   std::vector<int32_t> t2_ptr, t2_a, t2_b, a2_ptr, a2_blk, b2_ptr, b2_blk, t2_order;
   int gray2 = 0;
+  // Schedule: every cell's initial word (count and id sum, sched_count_bits;
+  // empty when 32 bits do not hold them), and for a projection grid -- each
+  // source (z, l) in one cell of every column j, cell = affine[j] + affine[n
+  // + j] z + affine[2 n + j] l -- that table (else empty).
+  std::vector<uint32_t> word0;
+  std::vector<int32_t> affine;
 };
 
 namespace bpx {
@@ -44,7 +50,7 @@ struct WsLayout {
   size_t g_t2_ptr, g_t2_a, g_t2_b, g_a2_ptr, g_a2_blk, g_b2_ptr, g_b2_blk, g_t2_order;
   // plan (int32)
   size_t p_info, p_ctr, p_cnt, p_surv, p_direct, p_front0, p_front1, p_word;
-  size_t p_depth, p_resolver, p_order, p_wave_ptr, p_cursor;
+  size_t p_depth, p_resolver, p_order, p_wave_ptr, p_cursor;  // p_word, p_cursor: also uploaded (word0, affine)
   size_t p_pl_res, p_pl_ptr, p_pl_list;  // peel list: resolver and subtrahends per order entry
   size_t plan_end;
   // products (float, num_cells * h * N)
@@ -94,6 +100,27 @@ WsLayout ws_layout(const bpx_code* code, int M, int N, int K, int h, int precisi
 // empty.
 void finish_code(bpx_code* c, const std::vector<std::vector<int32_t>>& cells,
                  const std::vector<int32_t>& col_of_cell);
+
+// The schedule's per-cell word holds the cell's unknown-source count in its
+// low sched_count_bits (the top one of them marks an erased cell) and the sum
+// of its unknown sources' ids + 1 (values 1 .. S) above, modulo the word: when
+// one source is left, the sum is its id + 1.  sched_id_bits: the bits of S; a
+// 32-bit word (kept in shared memory) fits when both fields do, else the plan
+// keeps 64-bit words in global memory.
+constexpr int sched_id_bits(int S) {
+  int b = 0;
+  while (b < 31 && (S >> b) != 0) ++b;
+  return b;
+}
+constexpr bool sched_packable32(int S, int sigma) {
+  const int b = sched_id_bits(S);
+  return b <= 30 && sigma < (1 << (31 - b));
+}
+
+constexpr int sched_count_bits(int sigma) { return sched_id_bits(sigma) + 1; }
+
+// Fills the code's schedule tables (word0, affine).
+void build_schedule_tables(bpx_code* c);
 
 // Factors every cell for the two-dimensional scheme (fills the t2_* / a2_* /
 // b2_* arrays of the code).

@@ -76,6 +76,36 @@ void finish_code(bpx_code* c, const std::vector<std::vector<int32_t>>& cells,
   for (int j = 0; j < c->n - c->e; ++j) tot += hs[j];
   c->eps = static_cast<double>(tot) / (static_cast<double>(c->k) * c->b) - 1.0;
   build_terms_2d(c);
+  build_schedule_tables(c);
+}
+
+// word0 and affine (see bpx_code).
+void build_schedule_tables(bpx_code* c) {
+  c->word0.clear();
+  c->affine.clear();
+  if (sched_packable32(c->S, c->sigma)) {
+    const int cbits = sched_count_bits(c->sigma);
+    for (int i = 0; i < c->num_cells; ++i) {
+      uint32_t sum = 0;
+      for (int e = c->cell_ptr[i]; e < c->cell_ptr[i + 1]; ++e) sum += static_cast<uint32_t>(c->cell_src[e]) + 1u;
+      c->word0.push_back((sum << cbits) | static_cast<uint32_t>(c->cell_ptr[i + 1] - c->cell_ptr[i]));
+    }
+  }
+  const long long n = c->n;
+  if (c->S != static_cast<long long>(c->k) * c->b || c->num_edges != n * c->S || 3 * n > c->S + 2) return;
+  for (int s = 0; s <= c->S; ++s)
+    if (c->src_ptr[s] != n * s) return;
+  std::vector<int32_t> t(3 * n, 0);
+  for (int j = 0; j < n; ++j) {
+    t[j] = c->src_cell[j];
+    if (c->b > 1) t[n + j] = c->src_cell[n * c->k + j] - t[j];
+    if (c->k > 1) t[2 * n + j] = c->src_cell[n + j] - t[j];
+  }
+  for (int z = 0; z < c->b; ++z)
+    for (int l = 0; l < c->k; ++l)
+      for (int j = 0; j < n; ++j)
+        if (c->src_cell[n * (static_cast<long long>(z) * c->k + l) + j] != t[j] + t[n + j] * z + t[2 * n + j] * l) return;
+  c->affine = t;
 }
 
 }  // namespace bpx

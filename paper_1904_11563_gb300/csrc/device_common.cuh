@@ -27,6 +27,7 @@ struct DevGraph {
   const int32_t* t2_order;
   int n, S, num_cells, num_edges, sigma;
   int k, EA, EB;  // grid width (B blocks), A and B operand counts
+  int affine;     // the plan holds an affine cell table (bpx_code::affine)
 };
 
 // Peel plan written by the schedule kernel.
@@ -38,12 +39,13 @@ struct DevPlan {
   int32_t* direct;    // per cell: the source it resolves at depth 1, or -1
   int32_t* front0;    // frontier scratch
   int32_t* front1;
-  unsigned long long* word;  // per cell: unknown count << 32 | XOR of unknown ids + 1 (large codes)
+  unsigned long long* word;  // per cell: sum of the unknown sources' ids + 1 << 32 | their count (large
+                             // codes; else 32-bit initial words, uploaded with the graph)
   int32_t* depth;     // per source: round of recovery (0 = not recovered)
   int32_t* resolver;  // per source: resolving cell (INT32_MAX = none)
   int32_t* order;     // recovered sources sorted by (depth, source)
   int32_t* wave_ptr;  // order[wave_ptr[d-1] .. wave_ptr[d]) = sources of depth d
-  int32_t* cursor;    // placement cursors (scratch)
+  const int32_t* affine;  // projection grids: per column the first cell and its steps in z and l (3 n words)
   // Peel list, one entry per position i of `order`: the resolver of order[i]
   // and, in pl_list[pl_ptr[i] .. pl_ptr[i+1]), the other sources of that
   // resolver in ascending id (the blocks subtracted from its product).
@@ -51,21 +53,6 @@ struct DevPlan {
   int32_t* pl_ptr;
   int32_t* pl_list;
 };
-
-// The schedule's per-cell word holds the cell's unknown-source count above
-// the XOR of its unknown sources' ids + 1 (values 1 .. S).  sched_id_bits:
-// the bits of S; a 32-bit word (kept in shared memory) fits when the largest
-// cell degree stays below the remaining 31 - bits (the top bit marks an
-// erased cell), else the plan keeps 64-bit words in global memory.
-inline __host__ __device__ int sched_id_bits(int S) {
-  int b = 0;
-  while (b < 31 && (S >> b) != 0) ++b;
-  return b;
-}
-inline __host__ __device__ bool sched_packable32(int S, int sigma) {
-  const int b = sched_id_bits(S);
-  return b <= 30 && sigma < (1 << (31 - b));
-}
 
 inline DevGraph make_graph(const bpx_code* c, const void* ws, const WsLayout& L) {
   auto base = static_cast<const char*>(ws);
@@ -91,6 +78,7 @@ inline DevGraph make_graph(const bpx_code* c, const void* ws, const WsLayout& L)
   g.num_cells = c->num_cells;
   g.num_edges = c->num_edges;
   g.sigma = c->sigma;
+  g.affine = c->affine.empty() ? 0 : 1;
   return g;
 }
 
@@ -110,7 +98,7 @@ inline DevPlan make_plan(const void* ws, const WsLayout& L) {
   p.resolver = at(L.p_resolver);
   p.order = at(L.p_order);
   p.wave_ptr = at(L.p_wave_ptr);
-  p.cursor = at(L.p_cursor);
+  p.affine = at(L.p_cursor);
   p.pl_res = at(L.p_pl_res);
   p.pl_ptr = at(L.p_pl_ptr);
   p.pl_list = at(L.p_pl_list);

@@ -187,21 +187,21 @@ __device__ __forceinline__ bool b_split_body(const float* __restrict__ B, int K,
       for (int q = 0; q < 8; ++q) v[q] = tile[8 * kc + q][r];
       const long long o = static_cast<long long>(n) * K + k;
       unfit |= parts_split8(v, bt_hi + o, bt_lo + o, bt_3 + o);
-      continue;
-    }
-    uint32_t hv[4], lv[4];
+    } else {
+      uint32_t hv[4], lv[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const float x0 = tile[8 * kc + 2 * q][r], x1 = tile[8 * kc + 2 * q + 1][r];
-      const __nv_bfloat162 hh = __floats2bfloat162_rn(x0, x1);
-      hv[q] = *reinterpret_cast<const uint32_t*>(&hh);
-      const float2 f = __bfloat1622float2(hh);
-      const __nv_bfloat162 ll = __floats2bfloat162_rn(x0 - f.x, x1 - f.y);
-      lv[q] = *reinterpret_cast<const uint32_t*>(&ll);
+      for (int q = 0; q < 4; ++q) {
+        const float x0 = tile[8 * kc + 2 * q][r], x1 = tile[8 * kc + 2 * q + 1][r];
+        const __nv_bfloat162 hh = __floats2bfloat162_rn(x0, x1);
+        hv[q] = *reinterpret_cast<const uint32_t*>(&hh);
+        const float2 f = __bfloat1622float2(hh);
+        const __nv_bfloat162 ll = __floats2bfloat162_rn(x0 - f.x, x1 - f.y);
+        lv[q] = *reinterpret_cast<const uint32_t*>(&ll);
+      }
+      const long long o = static_cast<long long>(n) * K + k;
+      *reinterpret_cast<uint4*>(bt_hi + o) = make_uint4(hv[0], hv[1], hv[2], hv[3]);
+      if (bt_lo) *reinterpret_cast<uint4*>(bt_lo + o) = make_uint4(lv[0], lv[1], lv[2], lv[3]);
     }
-    const long long o = static_cast<long long>(n) * K + k;
-    *reinterpret_cast<uint4*>(bt_hi + o) = make_uint4(hv[0], hv[1], hv[2], hv[3]);
-    if (bt_lo) *reinterpret_cast<uint4*>(bt_lo + o) = make_uint4(lv[0], lv[1], lv[2], lv[3]);
   }
   return unfit;
 }
