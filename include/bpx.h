@@ -510,7 +510,8 @@ int bpx_group_autotune(bpx_group* group, const int* configs, int nconfigs, bpx_s
  * (cta_group::2; each CTA of the cluster holds 128 rows of A and half of
  * the B tile) with 64- / 32-wide k-slices; seg_kb = k-blocks of 64 per TMEM
  * accumulation segment, band = m-tiles (or m-tile pairs) per rasterisation
- * band.  gemm_config 0 = the default, 8080.  Precisions BPX_BF16,
+ * band.  gemm_config 0 = the default: 8080, or 128-wide or narrower tiles of
+ * one CTA for products that fill few CTA pairs.  Precisions BPX_BF16,
  * BPX_BF16X3 and BPX_EXACT (which uses the tile shape, pairing, k-slice and
  * band, with its own exact segment length; its default is also 8080).
  * Tile codes 3, 4, 7 and 8 name no kernel (BPX_ERR_INVAL).  No kernel loads

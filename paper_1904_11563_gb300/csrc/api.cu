@@ -291,7 +291,7 @@ int products_impl(const bpx_code* c, const float* d_A, const float* d_B, int M, 
                                    d_info, st);
       else if (e == cudaSuccess)
         e = bpx::launch_gemm_tc(g, p, a_hi, a_lo, b_hi, b_lo, c->num_cells, N, K, h, split,
-                                d_products, d_C, config, d_info, st);
+                                bpx::rows_expected(c, h), d_products, d_C, config, d_info, st);
       stage_mark(opts, BPX_STAGE_GEMM, 1, st);
       if (e == cudaErrorNotSupported)
         return fail(BPX_ERR_UNSUPPORTED, "bf16 tensor-core path not available in this build");
@@ -313,8 +313,8 @@ int products_impl(const bpx_code* c, const float* d_A, const float* d_B, int M, 
       stage_mark(opts, BPX_STAGE_A_PREP, 1, st);
       stage_mark(opts, BPX_STAGE_GEMM, 0, st);
       if (e == cudaSuccess)
-        e = bpx::launch_gemm_tc(g, p, a_hi, a_lo, b_hi, b_lo, c->num_cells, N, K, h, true, d_products, d_C, config,
-                                d_info, st, a_exp, b_exp);
+        e = bpx::launch_gemm_tc(g, p, a_hi, a_lo, b_hi, b_lo, c->num_cells, N, K, h, true, bpx::rows_expected(c, h),
+                                d_products, d_C, config, d_info, st, a_exp, b_exp);
       stage_mark(opts, BPX_STAGE_GEMM, 1, st);
       break;
     }

@@ -287,11 +287,12 @@ cudaError_t launch_gemm_f32(const DevGraph& g, const DevPlan& p, const float* a_
 cudaError_t launch_gemm_fused(const DevGraph& g, const DevPlan& p, const float* A, int M, const void* b_hi,
                               const void* b_lo, int num_cells, int N, int K, int h, bool split3, float* products,
                               float* C_direct, int config, int32_t* info_out, cudaStream_t st);
+// rows_est: the coded rows to expect (chooses the tile when config is 0).
 // a_exp / b_exp non-null: the split-fp16 operands of BPX_FP16X3 (a_lo and
 // b_lo required), unscaled by 2^-(a_exp[row] + b_exp[col]) in the epilogue.
 cudaError_t launch_gemm_tc(const DevGraph& g, const DevPlan& p, const void* a_hi, const void* a_lo,
                            const void* b_hi, const void* b_lo, int num_cells, int N, int K, int h,
-                           bool split3, float* products, float* C_direct, int config,
+                           bool split3, long long rows_est, float* products, float* C_direct, int config,
                            int32_t* info_out, cudaStream_t st, const int32_t* a_exp = nullptr,
                            const int32_t* b_exp = nullptr);
 

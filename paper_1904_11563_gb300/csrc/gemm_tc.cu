@@ -633,15 +633,35 @@ int tile_pair(int config) {
 }
 int tile_bk(int config) { return (config % 10) >= 5 ? 32 : 64; }
 
-// FP32 in three parts: 128 x 128 tiles of single CTAs where the 256 x 256
-// tiles of CTA pairs would leave too many SMs idle in their last wave.
-bool f32_small_tiles(long long rows, int N) {
-  const long long pairs = std::max(1, num_sms() / 2), sms = std::max(1, num_sms());
-  const long long big = (rows + 255) / 256 * ((N + 255) / 256), small = (rows + 127) / 128 * ((N + 127) / 128);
-  // time in units of a 256 x 256 tile's (K = 8192: 3.67 ms against 4.77 ms
-  // with 128 x 128 tiles, which re-read more operand bytes per MMA): a
-  // 128 x 128 tile takes 0.65
-  return 0.65 * static_cast<double>((small + sms - 1) / sms) < static_cast<double>((big + pairs - 1) / pairs);
+// The tile of a product whose caller names none (gemm_config 0): 256 x 256 of
+// a CTA pair, or 128 x 128 / 128 x 64 of one CTA where the pairs would leave
+// SMs idle (the same K segments, so the same bits).  Time = waves x k-blocks x
+// time per k-block + the last tile's drain, in units of a pair tile's
+// k-block.  Measured, split bf16, us per k-block of one tile on every SM and
+// drain: 1.03 and 8 (pair), 0.675 and 5.5 (128), 0.67 and 3.5 (64): a narrower
+// tile reads as much of A from shared memory per MMA.  GEMM, pair against the
+// tile chosen (coded rows x K x N): 568 x 256 x 128 16.3 -> 10.2 us, 1136 x
+// 1416 x 1100 32.8 -> 26.6, 4544 x 4096 x 512 67.5 -> 49.3; 2272 x 1992 x 2044
+// keeps pairs, 44 against 60.
+int auto_bn(int parts, long long rows, int N, int K) {
+  const long long sms = std::max(1, num_sms());
+  const int kb = (K + BK - 1) / BK;
+  const double scale = parts == 1 ? 2.0 : parts == 3 ? 0.5 : 1.0;  // drains against a k-block's MMAs
+  const int bn[3] = {256, 128, 64};
+  const double step[3] = {1.0, 0.655, parts == 1 ? 0.68 : 0.65}, drain[3] = {7.8 * scale, 5.3 * scale, 3.4 * scale};
+  int best = 0;
+  double least = 0.0;
+  for (int i = 0; i < 3; ++i) {
+    const int m = i == 0 ? 256 : 128;
+    const long long slots = i == 0 ? std::max(1LL, sms / 2) : sms;
+    const long long tiles = (rows + m - 1) / m * ((N + bn[i] - 1) / bn[i]);
+    const double t = static_cast<double>((tiles + slots - 1) / slots) * kb * step[i] + drain[i];
+    if (i == 0 || t < least) {
+      least = t;
+      best = i;
+    }
+  }
+  return bn[best];
 }
 
 // seg_kb: k-slices of kBK per TMEM accumulation segment.
@@ -693,6 +713,10 @@ cudaError_t dispatch_bk(bool split3, int bn, int pair, const TcJob& single, cons
   seg_kb *= m;                 // configs count segments in 64-wide k-blocks
 #define BPX_LV(PARTS, STAGES, BN, PAIR) \
   launch_variant<PARTS, STAGES, BN, PAIR, kBK, kMode>(single, table, njobs, total_tiles, group, seg_kb, st)
+  // (64-wide tiles: only as the default's choice for a small product)
+  if constexpr (kBK == BK && kMode == kModeRows) {
+    if (bn == 64) return split3 ? BPX_LV(2, 4, 64, 0) : BPX_LV(1, 8, 64, 0);
+  }
   // CTA-pair MMAs: a stage holds the CTA's A rows and half the B tile
   if (pair == 2) return split3 ? BPX_LV(2, 3 * m, 256, 2) : BPX_LV(1, 6 * m, 256, 2);
   if (split3) return bn == 128 ? BPX_LV(2, 3 * m, 128, 0) : BPX_LV(2, 2 * m, 256, 0);
@@ -828,7 +852,7 @@ bool gemm_config_ok(int config) { return tile_valid(config); }
 
 cudaError_t launch_gemm_tc(const DevGraph& g, const DevPlan& p, const void* a_hi, const void* a_lo,
                            const void* b_hi, const void* b_lo, int num_cells, int N, int K, int h,
-                           bool split3, float* products, float* C_direct, int config,
+                           bool split3, long long rows_est, float* products, float* C_direct, int config,
                            int32_t* info_out, cudaStream_t st, const int32_t* a_exp, const int32_t* b_exp) {
   if (!tile_valid(config)) return cudaErrorInvalidValue;
   if ((a_exp != nullptr) != (b_exp != nullptr) || (a_exp && !split3)) return cudaErrorInvalidValue;
@@ -842,6 +866,10 @@ cudaError_t launch_gemm_tc(const DevGraph& g, const DevPlan& p, const void* a_hi
   // 5.6e-7 (GEMM 2.05 / 2.10 / 2.27 ms), and on its worst peel chains
   // (propagation factor 32) 256-wide segments 9.2e-6, 128-wide 7.9e-6.
   if (a_exp && config == 0) seg_kb = 2;
+  if (config == 0) {
+    bn = auto_bn(split3 ? 2 : 1, rows_est, N, K);
+    pair = bn == 256 ? 2 : 0;
+  }
   TcJob J;
   if (!tc_fill_job(&J, p, a_hi, split3 ? a_lo : nullptr, b_hi, split3 ? b_lo : nullptr, num_cells, N, K, h,
                    bn, pair, bk, products, C_direct, info_out, a_exp, b_exp))
@@ -851,8 +879,7 @@ cudaError_t launch_gemm_tc(const DevGraph& g, const DevPlan& p, const void* a_hi
   return dispatch(split3, bn, pair, bk, J, nullptr, 1, tiles, group, seg_kb, st);
 }
 
-// FP32 operands in three bf16 parts (a[i], b[i]): 256 x 256 tiles of CTA-pair
-// MMAs, or 128 x 128 tiles of 1-CTA MMAs (see f32_small_tiles); 64-wide
+// FP32 operands in three bf16 parts (a[i], b[i]), the tile by auto_bn; 64-wide
 // segments (24 MMAs each, so a drain is as rare as with hi + lo operands).
 // Tensor-bound: 96 KB staged per 24 MMAs and CTA, 32 B a clock.  Benchmark
 // workload (9088 coded rows, 8192 x 8192): 3.67 ms, 2.0 PFLOP/s of MMA work,
@@ -862,15 +889,16 @@ cudaError_t launch_gemm_tc(const DevGraph& g, const DevPlan& p, const void* a_hi
 cudaError_t launch_gemm_f32_tc(const DevPlan& p, void* const a[3], void* const b[3], int num_cells, int N, int K, int h,
                                long long rows_est, float* products, float* C_direct, int32_t* info_out,
                                cudaStream_t st) {
-  const bool small = f32_small_tiles(rows_est, N);
-  const int bn = small ? 128 : 256;
+  const int bn = auto_bn(3, rows_est, N, K);
+  const bool small = bn < 256;
   TcJob J;
   if (!tc_fill_job(&J, p, a[0], a[1], b[0], b[1], num_cells, N, K, h, bn, !small, BK, products, C_direct, info_out))
     return cudaErrorInvalidValue;
   const long long rows = static_cast<long long>(num_cells) * h;
-  if (!make_map(&J.map_a3, a[2], rows, K, BM) || !make_map(&J.map_b3, b[2], N, K, 128)) return cudaErrorInvalidValue;
+  if (!make_map(&J.map_a3, a[2], rows, K, BM) || !make_map(&J.map_b3, b[2], N, K, bn == 64 ? 64 : 128)) return cudaErrorInvalidValue;
   const int units = small ? J.m_tiles_max : (J.m_tiles_max + 1) / 2;
   const long long tiles = static_cast<long long>(units) * J.n_tiles;
+  if (bn == 64) return launch_variant<3, 3, 64, 0, BK>(J, nullptr, 1, tiles, 8, 1, st);
   if (small) return launch_variant<3, 2, 128, 0, BK>(J, nullptr, 1, tiles, 8, 1, st);
   return launch_variant<3, 2, 256, 2, BK>(J, nullptr, 1, tiles, 8, 1, st);
 }

@@ -80,3 +80,23 @@ def test_cuda_core_tile_edges(libbpx, M, K, N):
     A, B = A.double(), B.double()
     # one FMA chain of K terms
     assert ((C - A @ B).abs() <= K * 2.0 ** -24 * (A.abs() @ B.abs())).all()
+
+
+# the tile that a default call takes (256 x 256 of a CTA pair, 128 x 128,
+# 128 x 64) does not change a bit: against the pair tile asked for by name
+@pytest.mark.parametrize("M,K,N", [(512, 256, 128), (1000, 1416, 1100), (4096, 4096, 512), (130, 72, 36)])
+@pytest.mark.parametrize("prec,pair", [("bf16", 8080), ("bf16x3", 8080), ("fp16x3", 8020)])
+def test_default_tile_same_bits(libbpx, M, K, N, prec, pair):
+    bpx = libbpx
+    code = bpx.Code.systematic(8, 3, 8)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(M + K)
+    A = torch.randn((M, K), generator=g, device="cuda")
+    B = torch.randn((K, N), generator=g, device="cuda")
+    h = -(-M // code.num_sources)
+    ws = bpx.Workspace(code, M, N, K, h, bpx.PRECISIONS[prec])
+    mask = torch.zeros(code.n, dtype=torch.uint8, device="cuda")
+    mask[[0, 9]] = 1
+    C = [bpx.coded_matmul(code, A, B, h, bpx.PRECISIONS[prec], mask, ws, opts=bpx.default_opts(gemm_config=c))[0]
+         for c in (0, pair)]
+    assert torch.equal(C[0], C[1])
