@@ -66,9 +66,16 @@ struct CellWord<false> {
   using T = unsigned long long;
 };
 
-// Ints of dynamic shared memory a plan takes with its whole graph in it.
-__host__ __device__ inline long long sched_local_ints(int cells, int S, int edges) {
-  return 2LL * cells + 5LL * S + 2LL * edges + 2;
+// Ints of dynamic shared memory a plan takes with its whole graph in it, and
+// whether it is worth copying there: always for a small one, else only where
+// the rounds would read the cells from tables (32 columns of a 24 x 9 grid,
+// computed cells, two rounds: the copy of its 27000 words costs 10 us).
+__host__ __device__ inline long long sched_local_ints(const DevGraph& g) {
+  return 2LL * g.num_cells + 5LL * g.S + 2LL * g.num_edges + 2;
+}
+__host__ __device__ inline bool sched_local(const DevGraph& g, long long smem_ints) {
+  const long long ints = sched_local_ints(g);
+  return ints <= smem_ints && (ints <= 8192 || !g.affine);
 }
 
 // One position of the peel list: its resolver's sources but s, ascending.
@@ -108,7 +115,7 @@ __device__ __forceinline__ void schedule_body(const DevGraph& g, const DevPlan& 
   const W cmask = (W(1) << cbits) - 1, gone = W(1) << (cbits - 1);
   W* word = kSmem ? reinterpret_cast<W*>(dyn_smem) : reinterpret_cast<W*>(p.word);
   int32_t* depth = kSmem ? dyn_smem + C : p.depth;
-  const bool local = kSmem && sched_local_ints(C, S, g.num_edges) <= smem_ints;
+  const bool local = kSmem && sched_local(g, smem_ints);
   // the recovered sources in the order of their claims: all of them in the
   // plan's scratch, and in a ring (a power of two) the rounds of at most half of it
   int32_t* ring = dyn_smem + C + S;
@@ -539,8 +546,7 @@ cudaError_t launch_schedule(const DevGraph& g, const DevPlan& p, const uint8_t* 
   const bool fill_later = g.S >= kFillSources && part != 1;
   cudaError_t e;
   if (sched_packable32(g.S, g.sigma) && state <= room) {
-    const long long local = sched_local_ints(g.num_cells, g.S, g.num_edges);
-    const long long ints = local <= room ? local : std::min(room, state + 2LL * g.S);
+    const long long ints = sched_local(g, room) ? sched_local_ints(g) : std::min(room, state + 2LL * g.S);
     if ((e = cudaFuncSetAttribute(schedule_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   static_cast<int>(kSmemMax))) != cudaSuccess)
       return e;
