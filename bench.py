@@ -254,6 +254,17 @@ TOL = {"fp32": 1e-5, "bf16x3": 1e-5, "fp16x3": 1e-5, "bf16": 2e-2, "mxfp8": 6e-2
 MMA_MULT = {"fp32": 6, "bf16x3": 3, "bf16x3-fused": 3, "fp16x3": 3, "bf16": 1, "mxfp8": 1}
 
 
+def _exact_mult(bpx, code, K):
+    """Digit products of the whole exact path: the pairs (i, l) with i + l < S,
+    or, for digits of at most 4 bits whose sums fit int32, A digits times pairs
+    of B's digits (include/bpx.h, exact slices)."""
+    P = bpx.exact_params(code, K)
+    S, w, half = P["S"], P["w"], 1 << (P["w"] - 1)
+    if w <= 4 and S % 2 == 0 and S * P["Kp"] * code.sigma * half * half * (2 * half + 1) < 2 ** 31:
+        return S // 2 * (S // 2 + 1)
+    return S * (S + 1) // 2
+
+
 def _propagation(code, order, Ah, Bh, h, sources, ncols=256, kappa=None):
     """nu_s = sqrt(sum_c coef_{s,c}^2 ||P_c||^2) / ||C_s|| for the sampled
     sources: coef from the peel recurrence over the library's plan (each
@@ -634,8 +645,7 @@ def run_ours(args, wl):
     # exact path's digit-pair products) against the measured bf16 peak (FP8:
     # times the nominal fp8 / bf16 ratio of 2)
     if head == "exact":
-        S_ex = bpx.exact_params(code, K)["S"]
-        mult = S_ex * (S_ex + 1) // 2
+        mult = _exact_mult(bpx, code, K)
     else:
         mult = MMA_MULT[head]
     flops = 2.0 * rows_mean * N * K * mult
@@ -697,8 +707,7 @@ def run_ours(args, wl):
         if gm <= 0:
             continue
         if prec == "exact":
-            S_ex = bpx.exact_params(code, K)["S"]
-            mult = S_ex * (S_ex + 1) // 2     # digit pairs (i, l) with i + l < S
+            mult = _exact_mult(bpx, code, K)
         else:
             mult = MMA_MULT[prec]
         pk = peaks.get("bf16_tflops", 1900.0) * (2.0 if prec == "mxfp8" else 1.0)
@@ -1104,8 +1113,7 @@ def run_straggler(args, wl):
     useful = 2.0 * M * N * K
     rows = [int((p_["mask"] == 0).sum().item()) * h for p_ in timed]
     if prec == "exact":
-        S_ex = bpx.exact_params(code, K)["S"]
-        mult = S_ex * (S_ex + 1) // 2     # digit pairs (i, l) with i + l < S
+        mult = _exact_mult(bpx, code, K)
     else:
         mult = {"bf16x3": 3, "fp16x3": 3, "bf16": 1, "fp32": 6}[prec]
     peaks = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json"))) if os.path.exists(

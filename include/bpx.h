@@ -348,7 +348,8 @@ int bpx_peel_decode(const bpx_code* code, const float* d_products, const uint8_t
  * The only errors are the fixed-point rounding of A and B and the dropped
  * pairs, both about 2^-24 relative to max|A row j| max|B column n| per K term.
  * Products cost S (S+1) / 2 bf16 MMAs per k-step (sigma 2: 6; sigma 8: 10;
- * sigma 24: 21) and the staged planes S times the bf16 operand bytes. */
+ * sigma 24: 21; bpx_coded_matmul pairs B's digits when w <= 4 and the int32
+ * sums allow, 12 at sigma 24, with the same integers) and the staged planes S times the bf16 operand bytes. */
 
 /* out[5] = { w, S, bits, K elements per exact FP32 segment, K padded to 64 }
  * for this code and K (host only).  BPX_ERR_UNSUPPORTED when sigma > 64 (digits

@@ -218,7 +218,7 @@ namespace {
 
 int products_impl(const bpx_code* c, const float* d_A, const float* d_B, int M, int N, int K,
                   int h, int precision, void* ws, size_t ws_bytes, float* d_products, float* d_C,
-                  const bpx_opts* opts, int32_t* d_info, cudaStream_t st) {
+                  const bpx_opts* opts, int32_t* d_info, cudaStream_t st, bool pair_digits = false) {
   if (!c || (!d_A && M > 0) || !d_B || !ws || !d_products)  // A unused when M = 0
     return fail(BPX_ERR_INVAL, "bpx_coded_products: NULL argument");
   if (int rc = check_shapes(c, M, N, K, h)) return rc;
@@ -339,11 +339,12 @@ int products_impl(const bpx_code* c, const float* d_A, const float* d_B, int M, 
     case BPX_EXACT: {
       bpx::ExactParams P;
       if (int rc = bpx::exact_params(c, K, &P)) return rc;
+      if (pair_digits) bpx::exact_pair_digits(c, &P);
       uint32_t* amax = reinterpret_cast<uint32_t*>(base + L.ex_amax);  // h words (A), then N (B)
       void* a_pl = base + L.a_hi;
       void* b_pl = base + L.b_hi;
       stage_mark(opts, BPX_STAGE_B_PREP, 0, st);
-      e = bpx::launch_exact_b(d_B, K, N, P, amax + h, b_pl, st);
+      e = bpx::launch_exact_b(d_B, K, N, P, amax + h, amax, h, b_pl, st);
       stage_mark(opts, BPX_STAGE_B_PREP, 1, st);
       stage_mark(opts, BPX_STAGE_A_PREP, 0, st);
       if (e == cudaSuccess)
@@ -363,14 +364,16 @@ int products_impl(const bpx_code* c, const float* d_A, const float* d_B, int M, 
   return BPX_OK;
 }
 
+// K > 0: the planes are the whole path's for this K (digit pairs of B where it takes them).
 int peel_exact_impl(const bpx_code* c, const int32_t* d_planes, int N, int h, float* d_C, const bpx_opts* opts,
-                    void* ws, size_t ws_bytes, cudaStream_t st) {
+                    void* ws, size_t ws_bytes, cudaStream_t st, int K = 0) {
   if (!c || !d_planes || !d_C || !ws) return fail(BPX_ERR_INVAL, "bpx_peel_decode_exact: NULL argument");
   if (N <= 0 || h <= 0 || N % 4 != 0) return fail(BPX_ERR_INVAL, "bpx_peel_decode_exact: bad N or h");
   if (!aligned(d_planes, 16) || !aligned(d_C, 16))
     return fail(BPX_ERR_INVAL, "bpx_peel_decode_exact: buffers must be 16-byte aligned");
   bpx::ExactParams P;
-  if (int rc = bpx::exact_params(c, 8, &P)) return rc;  // w, S and bits depend on sigma only
+  if (int rc = bpx::exact_params(c, K > 0 ? K : 8, &P)) return rc;  // w, S and bits depend on sigma only
+  if (K > 0) bpx::exact_pair_digits(c, &P);
   // The scales and the int64 blocks sit before every K-dependent region.
   const bpx::WsLayout L = bpx::ws_layout(c, 0, N, 8, h, BPX_EXACT);
   if (int rc = check_ws(c, ws, ws_bytes, L)) return rc;
@@ -380,8 +383,8 @@ int peel_exact_impl(const bpx_code* c, const int32_t* d_planes, int N, int h, fl
   long long* c64 = reinterpret_cast<long long*>(base + L.ex_c64);
   const int ctas = opts ? opts->peel_ctas : 0;
   stage_mark(opts, BPX_STAGE_PEEL, 0, st);
-  cudaError_t e = bpx::launch_peel_exact(p, P, d_planes, static_cast<long long>(c->num_cells) * h * N, c64, d_C,
-                                         amax, amax + h, N, h, ctas, st);
+  cudaError_t e = bpx::launch_peel_exact(p, P, c->sigma, d_planes, static_cast<long long>(c->num_cells) * h * N,
+                                         c64, d_C, amax, amax + h, N, h, ctas, st);
   stage_mark(opts, BPX_STAGE_PEEL, 1, st);
   if (e != cudaSuccess) return cuda_fail(e, "bpx_peel_decode_exact: launch");
   return BPX_OK;
@@ -552,10 +555,10 @@ extern "C" int bpx_coded_matmul(const bpx_code* c, const float* d_A, const float
   };
   if (precision == BPX_EXACT) {
     if (int rc = products_impl(c, d_A, d_B, M, N, K, h, precision, ws, ws_bytes, products, nullptr, &o, d_info,
-                               S(stream)))
+                               S(stream), true))
       return rc;
     if (int rc = join()) return rc;
-    return peel_exact_impl(c, reinterpret_cast<const int32_t*>(products), N, h, d_C, &o, ws, ws_bytes, S(stream));
+    return peel_exact_impl(c, reinterpret_cast<const int32_t*>(products), N, h, d_C, &o, ws, ws_bytes, S(stream), K);
   }
   if (int rc = products_impl(c, d_A, d_B, M, N, K, h, precision, ws, ws_bytes, products,
                              o.direct_write ? d_C : nullptr, &o, d_info, S(stream)))

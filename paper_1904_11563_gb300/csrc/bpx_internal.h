@@ -73,11 +73,21 @@ struct WsLayout {
 // K elements per exact FP32 accumulation segment, K padded to 64.
 struct ExactParams {
   int w = 0, S = 0, bits = 0, seg = 0, Kp = 0;
+  int step = 1, np = 0;  // diagonals computed: S - 1, S - 1 - step, ...: np of them (see exact_pair_digits)
 };
 
 // Fills *P for the code's sigma and K; BPX_ERR_UNSUPPORTED (with a message)
 // when the digits or the exact integer sums would not fit.
 int exact_params(const bpx_code* c, int K, ExactParams* P);
+
+// The whole path's form for narrow digits (w <= 4: codes of sigma > 16, S 6
+// or 8): B plane l holds two of B's digits, E_{l-1} 2^w + E_l (plane 0: E_0),
+// still exact in bf16 (at most 136), so that the diagonals S - 1, S - 3, ...
+// of A digits and these planes, A_i x plane d - i, hold the same kept digit
+// pairs as all S diagonals: 12 products instead of 21 (S = 6), 20 instead of
+// 36 (S = 8), and half the product planes.  Sets step 2, np = S / 2 and the
+// segment for the larger products, where the int32 diagonal sums still fit.
+void exact_pair_digits(const bpx_code* c, ExactParams* P);
 
 // Coded rows to expect from a mask of e erased columns (launch heuristics).
 inline long long rows_expected(const bpx_code* c, int h) {

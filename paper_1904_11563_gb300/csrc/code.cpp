@@ -378,7 +378,20 @@ int exact_params(const bpx_code* c, int K, ExactParams* P) {
   for (int d = 0; d < P->S; ++d) q += std::ldexp(1.0, w * (P->S - 1 - d)) * (d + 1) * P->Kp * maxprod;
   if (2.0 * q >= std::ldexp(1.0, 52))
     return fail(BPX_ERR_UNSUPPORTED, "exact-slice: K = %d too large for exact decoded integers", K);
+  P->step = 1;
+  P->np = P->S;
   return BPX_OK;
+}
+
+void exact_pair_digits(const bpx_code* c, ExactParams* P) {
+  if (P->w > 4 || P->S % 2 != 0) return;
+  const double half = std::ldexp(1.0, P->w - 1);
+  const double maxprod = std::max(1, c->sigma) * half * (half * (2.0 * half + 1.0));
+  const int seg = static_cast<int>(std::floor(std::ldexp(1.0, 23) / maxprod / 64.0)) * 64;
+  if (seg < 128 || static_cast<double>(P->S) * P->Kp * maxprod >= std::ldexp(1.0, 31)) return;
+  P->step = 2;
+  P->np = P->S / 2;
+  P->seg = seg;
 }
 
 // The line between the two FP32 forms.  Staging of B and GEMM, CUDA cores

@@ -298,8 +298,12 @@ cudaError_t launch_gemm_tc(const DevGraph& g, const DevPlan& p, const void* a_hi
 
 // Exact-slice staging (max |B| per column + B digit planes; max |A| per row
 // position + coded A digit planes), digit-product GEMM and exact peel.
-cudaError_t launch_exact_b(const float* B, int K, int N, const ExactParams& P, uint32_t* amax_b, void* bt,
-                           cudaStream_t st);
+// (launch_exact_b also clears the h words of amax_a; launch_exact_a follows it)
+cudaError_t launch_exact_b(const float* B, int K, int N, const ExactParams& P, uint32_t* amax_b, uint32_t* amax_a,
+                           int h, void* bt, cudaStream_t st);
+// max |B| per column as float bits; clears `clear` words of `cleared` besides.
+cudaError_t launch_colmax(const float* B, int K, int N, uint32_t* bmax, uint32_t* cleared, long long clear,
+                          cudaStream_t st);
 // src_digits: the workspace's int8 source-digit region (ex_src) when the
 // layout has one, else nullptr.
 cudaError_t launch_exact_a(const DevGraph& g, const DevPlan& p, const float* A, int M, int K, int h,
@@ -308,9 +312,10 @@ cudaError_t launch_exact_a(const DevGraph& g, const DevPlan& p, const float* A, 
 cudaError_t launch_gemm_exact(const DevPlan& p, const void* a_planes, const void* b_planes, int num_cells, int N,
                               int K, int h, const ExactParams& P, int32_t* planes, int config, int32_t* info_out,
                               cudaStream_t st);
-cudaError_t launch_peel_exact(const DevPlan& p, const ExactParams& P, const int32_t* planes, long long plane_stride,
-                              long long* C64, float* C, const uint32_t* amax_a, const uint32_t* amax_b, int N,
-                              int h, int ctas, cudaStream_t st);
+cudaError_t launch_peel_exact(const DevPlan& p, const ExactParams& P, int sigma,
+                              const int32_t* planes, long long plane_stride, long long* C64, float* C,
+                              const uint32_t* amax_a, const uint32_t* amax_b, int N, int h, int ctas,
+                              cudaStream_t st);
 
 // Two-dimensional scheme: operand staging (summed A blocks, summed B^T
 // blocks, bf16 hi (+ lo)), products GEMM over each cell's terms, and the peel

@@ -25,6 +25,8 @@
 //                    to FP32.
 #include <cuda_bf16.h>
 
+#include <algorithm>
+
 #include "device_common.cuh"
 #include "rn_scaled.cuh"
 
@@ -82,39 +84,31 @@ __device__ __forceinline__ float warp_max(float m) {
   return m;
 }
 
-// One warp per row of A.
+// max |A| per row position j, the max over rows s h + j of every block s: a
+// CTA takes 1 / parts of one position's rows (grid: h x parts).  One part
+// stores; more fold into the word that the B kernel has cleared.
 __global__ void __launch_bounds__(256) exact_amax_a_kernel(const float* __restrict__ A, int M, int K, int h,
                                                            uint32_t* amax) {
-  const int r = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (r >= M) return;
-  const float4* row = reinterpret_cast<const float4*>(A + static_cast<long long>(r) * K);
+  __shared__ float red[8];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float m = 0.f;
-  for (int i = lane; i < K / 4; i += 32) {
-    const float4 v = __ldg(row + i);
-    m = fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
+  for (long long r = blockIdx.x + static_cast<long long>(blockIdx.y * 8 + warp) * h; r < M;
+       r += 8LL * gridDim.y * h) {
+    const float4* row = reinterpret_cast<const float4*>(A + r * K);
+#pragma unroll 4
+    for (int i = lane; i < K / 4; i += 32) {
+      const float4 v = __ldg(row + i);
+      m = fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
+    }
   }
   m = warp_max(m);
-  if (lane == 0) atomicMax(amax + r % h, __float_as_uint(m));
-}
-
-// Thread = 4 columns of B over a 256-row slice of K.
-__global__ void __launch_bounds__(256) exact_amax_b_kernel(const float* __restrict__ B, int K, int N,
-                                                           uint32_t* amax) {
-  const int c4 = blockIdx.x * 256 + threadIdx.x;
-  if (c4 * 4 >= N) return;
-  const int k0 = blockIdx.y * 256, k1 = min(K, k0 + 256);
-  float4 m = make_float4(0.f, 0.f, 0.f, 0.f);
-  for (int k = k0; k < k1; ++k) {
-    const float4 v = __ldg(reinterpret_cast<const float4*>(B + static_cast<long long>(k) * N) + c4);
-    m.x = fmaxf(m.x, fabsf(v.x));
-    m.y = fmaxf(m.y, fabsf(v.y));
-    m.z = fmaxf(m.z, fabsf(v.z));
-    m.w = fmaxf(m.w, fabsf(v.w));
+  if (lane == 0) red[warp] = m;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) m = fmaxf(m, red[w]);
+    if (gridDim.y == 1) amax[blockIdx.x] = __float_as_uint(m);
+    else if (m > 0.f) atomicMax(amax + blockIdx.x, __float_as_uint(m));
   }
-  atomicMax(amax + 4 * c4 + 0, __float_as_uint(m.x));
-  atomicMax(amax + 4 * c4 + 1, __float_as_uint(m.y));
-  atomicMax(amax + 4 * c4 + 2, __float_as_uint(m.z));
-  atomicMax(amax + 4 * c4 + 3, __float_as_uint(m.w));
 }
 
 // B (K x N) -> digit planes of B^T through a 64 x 64 shared-memory tile
@@ -122,7 +116,7 @@ __global__ void __launch_bounds__(256) exact_amax_b_kernel(const float* __restri
 template <int S>
 __global__ void __launch_bounds__(256)
 exact_b_digits_kernel(const float* __restrict__ B, int K, int N, const uint32_t* __restrict__ amax_b, int w,
-                      int bits, int Kp, __nv_bfloat16* bt) {
+                      int bits, int Kp, bool pairs, __nv_bfloat16* bt) {
   __shared__ float tile[64][65];
   const int n0 = blockIdx.x * 64, k0 = blockIdx.y * 64;
   {
@@ -150,6 +144,12 @@ exact_b_digits_kernel(const float* __restrict__ B, int K, int N, const uint32_t*
     int dg[8][S];
 #pragma unroll
     for (int q = 0; q < 8; ++q) balanced_digits<S>(to_fixed(tile[8 * kc + q][r], f), w, dg[q]);
+    if (pairs) {  // plane l: digits l - 1 and l
+#pragma unroll
+      for (int q = 0; q < 8; ++q)
+#pragma unroll
+        for (int l = S - 1; l >= 1; --l) dg[q][l] += dg[q][l - 1] * (1 << w);
+    }
     __nv_bfloat16* dst = bt + static_cast<long long>(n) * row_len + k;
 #pragma unroll
     for (int l = 0; l < S; ++l)
@@ -314,11 +314,13 @@ exact_a_digits_src_kernel(DevGraph g, DevPlan p, const uint8_t* __restrict__ src
 // Peel on exact integers.  As in the FP32 peel, each CTA owns one slice of
 // the block's 4-element groups and walks every wave over it; __syncthreads
 // between waves is the only synchronisation.
+// S product planes, plane d weighted 2^(w (S - 1 - d)); e_base: the exponent
+// of the lowest plane.
 template <int S>
 __global__ void __launch_bounds__(256)
 exact_peel_kernel(DevPlan p, const int32_t* __restrict__ planes, long long plane_stride, long long* C64, float* C,
                   const uint32_t* __restrict__ amax_a, const uint32_t* __restrict__ amax_b, int N, int h, int w,
-                  int bits, long long nv, int chunk) {
+                  int e_base, long long nv, int chunk) {
   if (p.ctr[CTR_PLAN] != kPlanReady) {  // no schedule has planned this workspace: refuse, write nothing
     if (blockIdx.x == 0 && threadIdx.x == 0) {
       atomicExch(&p.info[BPX_INFO_DEVICE_ERR], BPX_ERR_INVAL);
@@ -331,7 +333,6 @@ exact_peel_kernel(DevPlan p, const int32_t* __restrict__ planes, long long plane
   if (v0 >= nv) return;
   const int clen = static_cast<int>(min(static_cast<long long>(chunk), nv - v0));
   const long long hN = static_cast<long long>(h) * N;
-  const int e_base = w * (S - 1) - 2 * bits;
   for (int d = 1; d <= nwaves; ++d) {
     const int o0 = p.wave_ptr[d - 1], o1 = p.wave_ptr[d];
     const int items = (o1 - o0) * clen;
@@ -391,21 +392,150 @@ exact_peel_kernel(DevPlan p, const int32_t* __restrict__ planes, long long plane
   }
 }
 
+// The same peel for codes of long supports over few columns, whose waves are
+// narrow and many: what bounds them is the chain from wave to wave.  Eight
+// lanes share one (source, 4 columns) item: a lane takes every eighth
+// subtrahend and one or two product planes, all loads at once, and the exact
+// partial sums meet by shuffles.  Everything that does not depend on earlier
+// waves -- list entries and product planes of the next, descriptors of the one
+// after -- is loaded ahead, so a wave costs one round trip of its int64 blocks,
+// the shuffles and a barrier.
+constexpr int kExLanes = 8, kExNarrowThreads = 512;
+
+template <int S, int kSubs>
+__global__ void __launch_bounds__(kExNarrowThreads, 2)
+exact_peel_narrow_kernel(DevPlan p, const int32_t* __restrict__ planes, long long plane_stride, long long* C64,
+                         float* C, const uint32_t* __restrict__ amax_a, const uint32_t* __restrict__ amax_b, int N,
+                         int h, int w, int e_base, long long nv, int chunk) {
+  if (p.ctr[CTR_PLAN] != kPlanReady) {  // no schedule has planned this workspace: refuse, write nothing
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+      atomicExch(&p.info[BPX_INFO_DEVICE_ERR], BPX_ERR_INVAL);
+      atomicExch(&p.info[BPX_INFO_STATUS], BPX_ERR_INVAL);
+    }
+    return;
+  }
+  const int nwaves = p.ctr[CTR_NWAVES];
+  const long long v0 = static_cast<long long>(blockIdx.x) * chunk;
+  if (v0 >= nv) return;
+  const int clen = static_cast<int>(min(static_cast<long long>(chunk), nv - v0));
+  const long long hN = static_cast<long long>(h) * N;
+  const int sub = threadIdx.x % kExLanes, group = threadIdx.x / kExLanes, groups = blockDim.x / kExLanes;
+  struct Head {
+    int s, r, e, e1;   // source (-1: none), resolver, the lane's next list entry, the list's end
+    long long v;       // 4-element group of the block
+  };
+  struct Item {
+    Head h;
+    int t[kSubs];      // the lane's first subtrahends (-1: none)
+    int4 plane;        // the lane's product plane (lanes below S; used only in finish, so the load stays in flight)
+  };
+  static_assert(S <= kExLanes, "a lane holds at most one plane");
+  // item `it` of the wave of order positions [o0, o1)
+  auto head = [&](int o0, int o1, int it) {
+    Head H = {-1, 0, 0, 0, 0};
+    if (it < (o1 - o0) * clen) {
+      const int jx = it / clen, i = o0 + jx;
+      H.v = v0 + (it - jx * clen);
+      H.s = p.order[i];
+      H.r = p.pl_res[i];
+      H.e = p.pl_ptr[i] + sub;
+      H.e1 = p.pl_ptr[i + 1];
+    }
+    return H;
+  };
+  auto fetch = [&](const Head& H) {
+    Item I;
+    I.h = H;
+    I.plane = make_int4(0, 0, 0, 0);
+    if (sub < S && H.s >= 0)
+      I.plane =
+          __ldg(reinterpret_cast<const int4*>(planes + sub * plane_stride + static_cast<long long>(H.r) * hN) + H.v);
+#pragma unroll
+    for (int u = 0; u < kSubs; ++u) I.t[u] = H.e + u * kExLanes < H.e1 ? p.pl_list[H.e + u * kExLanes] : -1;
+    return I;
+  };
+  const long long weight = sub < S ? 1LL << (w * (S - 1 - sub)) : 0;
+  auto finish = [&](const Item& I) {
+    longlong2 a[kSubs], b[kSubs];
+#pragma unroll
+    for (int u = 0; u < kSubs; ++u) {
+      a[u] = b[u] = make_longlong2(0, 0);
+      if (I.t[u] >= 0) {
+        const auto* src = reinterpret_cast<const longlong2*>(C64 + static_cast<long long>(I.t[u]) * hN) + 2 * I.h.v;
+        a[u] = src[0];
+        b[u] = src[1];
+      }
+    }
+    long long q[4] = {I.plane.x * weight, I.plane.y * weight, I.plane.z * weight, I.plane.w * weight};
+#pragma unroll
+    for (int u = 0; u < kSubs; ++u) {
+      q[0] -= a[u].x;
+      q[1] -= a[u].y;
+      q[2] -= b[u].x;
+      q[3] -= b[u].y;
+    }
+    for (int e = I.h.e + kSubs * kExLanes; e < I.h.e1; e += kExLanes) {
+      const auto* src =
+          reinterpret_cast<const longlong2*>(C64 + static_cast<long long>(p.pl_list[e]) * hN) + 2 * I.h.v;
+      const longlong2 x = src[0], y = src[1];
+      q[0] -= x.x;
+      q[1] -= x.y;
+      q[2] -= y.x;
+      q[3] -= y.y;
+    }
+#pragma unroll
+    for (int o = 1; o < kExLanes; o <<= 1)
+#pragma unroll
+      for (int u = 0; u < 4; ++u) q[u] += __shfl_xor_sync(0xffffffffu, q[u], o);
+    if (I.h.s >= 0 && sub < 4) {  // lane u stores element u
+      const long long own = sub == 0 ? q[0] : sub == 1 ? q[1] : sub == 2 ? q[2] : q[3];
+      const long long el = 4 * I.h.v + sub;
+      C64[static_cast<long long>(I.h.s) * hN + el] = own;
+      const int j = static_cast<int>(el / N), n = static_cast<int>(el - static_cast<long long>(j) * N);
+      C[static_cast<long long>(I.h.s) * hN + el] =
+          rn_float_scaled(own, e_base + exponent_of(amax_a[j]) + exponent_of(amax_b[n]));
+    }
+  };
+  // wave d spans order positions [o0, o1); loaded ahead: wave d + 1's list
+  // entries and planes, wave d + 2's descriptors, wave d + 3's bound
+  auto bound = [&](int d) { return p.wave_ptr[min(d, nwaves)]; };
+  int o0 = 0, o1 = bound(1), o2 = bound(2), o3 = bound(3);
+  Item next = fetch(head(o0, o1, group));
+  Head after = head(o1, o2, group);
+  for (int d = 1; d <= nwaves; ++d) {
+    const int o4 = bound(d + 3);
+    const Item cur = next;
+    const int items = (o1 - o0) * clen;
+    next = fetch(after);
+    after = head(o2, o3, group);
+    finish(cur);
+    for (int base = groups; base < items; base += groups) finish(fetch(head(o0, o1, base + group)));
+    __syncthreads();
+    o0 = o1;
+    o1 = o2;
+    o2 = o3;
+    o3 = o4;
+  }
+}
+
 }  // namespace
 
-cudaError_t launch_exact_b(const float* B, int K, int N, const ExactParams& P, uint32_t* amax_b, void* bt,
-                           cudaStream_t st) {
-  cudaError_t e = cudaMemsetAsync(amax_b, 0, sizeof(uint32_t) * N, st);
+cudaError_t launch_exact_b(const float* B, int K, int N, const ExactParams& P, uint32_t* amax_b, uint32_t* amax_a,
+                           int h, void* bt, cudaStream_t st) {
+  // (also clears the row positions' words for launch_exact_a)
+  cudaError_t e = launch_colmax(B, K, N, amax_b, amax_a, h, st);
   if (e != cudaSuccess) return e;
-  exact_amax_b_kernel<<<dim3((N / 4 + 255) / 256, (K + 255) / 256), 256, 0, st>>>(B, K, N, amax_b);
   const dim3 grid((N + 63) / 64, P.Kp / 64);
   auto* out = static_cast<__nv_bfloat16*>(bt);
+  auto go = [&](auto kern) {
+    kern<<<grid, 256, 0, st>>>(B, K, N, amax_b, P.w, P.bits, P.Kp, P.step == 2, out);
+  };
   switch (P.S) {
-    case 3: exact_b_digits_kernel<3><<<grid, 256, 0, st>>>(B, K, N, amax_b, P.w, P.bits, P.Kp, out); break;
-    case 4: exact_b_digits_kernel<4><<<grid, 256, 0, st>>>(B, K, N, amax_b, P.w, P.bits, P.Kp, out); break;
-    case 5: exact_b_digits_kernel<5><<<grid, 256, 0, st>>>(B, K, N, amax_b, P.w, P.bits, P.Kp, out); break;
-    case 6: exact_b_digits_kernel<6><<<grid, 256, 0, st>>>(B, K, N, amax_b, P.w, P.bits, P.Kp, out); break;
-    case 8: exact_b_digits_kernel<8><<<grid, 256, 0, st>>>(B, K, N, amax_b, P.w, P.bits, P.Kp, out); break;
+    case 3: go(exact_b_digits_kernel<3>); break;
+    case 4: go(exact_b_digits_kernel<4>); break;
+    case 5: go(exact_b_digits_kernel<5>); break;
+    case 6: go(exact_b_digits_kernel<6>); break;
+    case 8: go(exact_b_digits_kernel<8>); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
@@ -414,9 +544,13 @@ cudaError_t launch_exact_b(const float* B, int K, int N, const ExactParams& P, u
 cudaError_t launch_exact_a(const DevGraph& g, const DevPlan& p, const float* A, int M, int K, int h,
                            const ExactParams& P, uint32_t* amax_a, void* a_planes, cudaStream_t st,
                            void* src_digits) {
-  cudaError_t e = cudaMemsetAsync(amax_a, 0, sizeof(uint32_t) * h, st);
-  if (e != cudaSuccess) return e;
-  if (M > 0) exact_amax_a_kernel<<<(M + 7) / 8, 256, 0, st>>>(A, M, K, h, amax_a);
+  cudaError_t e;
+  // 64 row steps of a warp, 16 K-elements a lane at least, to a CTA: about four CTAs an SM in all
+  const int positions = std::min(h, std::max(M, 1));
+  const long long rows_a = (static_cast<long long>(M) + h - 1) / h;
+  const long long parts = std::max(1LL, std::min((rows_a + 7) / 8, (4LL * num_sms() + positions - 1) / positions));
+  exact_amax_a_kernel<<<dim3(h, static_cast<unsigned>(std::min(parts, 65535LL))), 256, 0, st>>>(A, M, K, h, amax_a);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
   const long long rows = static_cast<long long>(g.num_cells) * h;
   const dim3 grid(static_cast<unsigned>(enc_row_blocks(rows, P.Kp)), enc_k_chunks(P.Kp));
   auto* out = static_cast<__nv_bfloat16*>(a_planes);
@@ -464,26 +598,33 @@ cudaError_t launch_exact_a(const DevGraph& g, const DevPlan& p, const float* A, 
   return cudaGetLastError();
 }
 
-cudaError_t launch_peel_exact(const DevPlan& p, const ExactParams& P, const int32_t* planes, long long plane_stride,
-                              long long* C64, float* C, const uint32_t* amax_a, const uint32_t* amax_b, int N,
-                              int h, int ctas, cudaStream_t st) {
+cudaError_t launch_peel_exact(const DevPlan& p, const ExactParams& P, int sigma,
+                              const int32_t* planes, long long plane_stride, long long* C64, float* C,
+                              const uint32_t* amax_a, const uint32_t* amax_b, int N, int h, int ctas,
+                              cudaStream_t st) {
   const long long nv = static_cast<long long>(h) * N / 4;
   if (nv <= 0) return cudaSuccess;
-  const int chunk = peel_chunk_for(nv, ctas);
+  const int e_base = P.w * (P.S - 1) - 2 * P.bits, w = P.w * P.step;
+  // Long supports over few columns: the form of eight lanes an item, one
+  // column group a CTA while there are fewer than two CTAs an SM.  (24 x 64
+  // grid, 32 columns of supports up to 24, N = 1024: 229 -> 99 us.)
+  const bool narrow = sigma > 4 && ctas <= 0 && nv <= 8LL * num_sms();
+  const long long slots = 2LL * num_sms();
+  const int chunk = narrow ? static_cast<int>((nv + slots - 1) / slots) : peel_chunk_for(nv, ctas);
   const unsigned grid = static_cast<unsigned>((nv + chunk - 1) / chunk);
-#define BPX_PEEL_EXACT(SV)                                                                                     \
-  exact_peel_kernel<SV><<<grid, 256, 0, st>>>(p, planes, plane_stride, C64, C, amax_a, amax_b, N, h, P.w, P.bits, \
-                                              nv, chunk)
-  switch (P.S) {
-    case 3: BPX_PEEL_EXACT(3); break;
-    case 4: BPX_PEEL_EXACT(4); break;
-    case 5: BPX_PEEL_EXACT(5); break;
-    case 6: BPX_PEEL_EXACT(6); break;
-    case 8: BPX_PEEL_EXACT(8); break;
+  auto go = [&](auto kern) {
+    kern<<<grid, narrow ? kExNarrowThreads : 256, 0, st>>>(p, planes, plane_stride, C64, C, amax_a, amax_b, N, h, w,
+                                                           e_base, nv, chunk);
+    return cudaGetLastError();
+  };
+  switch (P.np) {
+    case 3: return narrow ? go(exact_peel_narrow_kernel<3, 3>) : go(exact_peel_kernel<3>);
+    case 4: return narrow ? go(exact_peel_narrow_kernel<4, 3>) : go(exact_peel_kernel<4>);
+    case 5: return narrow ? go(exact_peel_narrow_kernel<5, 3>) : go(exact_peel_kernel<5>);
+    case 6: return narrow ? go(exact_peel_narrow_kernel<6, 3>) : go(exact_peel_kernel<6>);
+    case 8: return narrow ? go(exact_peel_narrow_kernel<8, 3>) : go(exact_peel_kernel<8>);
     default: return cudaErrorInvalidValue;
   }
-#undef BPX_PEEL_EXACT
-  return cudaGetLastError();
 }
 
 }  // namespace bpx

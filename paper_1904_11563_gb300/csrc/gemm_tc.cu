@@ -63,6 +63,7 @@ struct __align__(64) TcJob {
   int32_t* planes;
   long long plane_stride;
   int ex_S, ex_Kp;
+  int ex_np, ex_step, ex_dmajor;  // diagonals S - 1, S - 1 - step, ... (np of them); their order in the tile space
   // two-dimensional scheme: every cell (in t2_order) is a list of terms (A
   // operand, B operand) over h-row A operands and w-row B^T operands; N is the
   // row stride of C; kc = the code's k (source s = z kc + l); cnt = -1 marks
@@ -119,7 +120,7 @@ __device__ __forceinline__ void raise_error(const TcJob& J, int code, volatile i
 struct TileRef {
   const TcJob* J;
   int m, n, Mc, k_blocks;
-  int d, k_steps;  // exact slices: diagonal, and k-slices over its digit pairs
+  int d, dp, k_steps;  // exact slices: diagonal, its product plane, and k-slices over its digit pairs
   int cell, tp;    // two-dimensional scheme: the tile's cell and its first term
   bool live;
 };
@@ -154,7 +155,7 @@ __device__ __forceinline__ TileRef locate(const TcJob* jobs, int njobs, long lon
     R.n = r / m_units;
     R.m = r - R.n * m_units;
     R.Mc = J.h;
-    R.d = 0;
+    R.d = R.dp = 0;
     R.tp = J.t2_ptr[R.cell];
     R.k_blocks = (J.K + bk - 1) / bk;
     R.k_steps = (J.t2_ptr[R.cell + 1] - R.tp) * R.k_blocks;
@@ -174,10 +175,18 @@ __device__ __forceinline__ TileRef locate(const TcJob* jobs, int njobs, long lon
   R.Mc = live_mc >= 0 ? live_mc : J.ctr[CTR_NSURV] * J.h;
   int m_units = live_mc >= 0 ? (live_mc + BM - 1) / BM : J.m_tiles_max;
   if (pair) m_units = (m_units + 1) / 2;
-  int d = 0, lt = lt0;
-  if (exact) {  // the diagonals of a tile are adjacent: they reuse its digit planes from L2
-    d = lt % J.ex_S;
-    lt /= J.ex_S;
+  int d = 0, dp = 0, lt = lt0;
+  if (exact) {
+    if (J.ex_dmajor) {  // few tiles: the longest diagonal of every tile first, so that the CTAs end together
+      const int per_d = m_units * J.n_tiles;
+      dp = lt / per_d;
+      lt -= dp * per_d;
+      dp = J.ex_np - 1 - dp;
+    } else {  // the diagonals of a tile are adjacent: they reuse its digit planes from L2
+      dp = lt % J.ex_np;
+      lt /= J.ex_np;
+    }
+    d = J.ex_S - 1 - J.ex_step * (J.ex_np - 1 - dp);
   }
   const int band_tiles = group * J.n_tiles;
   const int band = lt / band_tiles;
@@ -187,6 +196,7 @@ __device__ __forceinline__ TileRef locate(const TcJob* jobs, int njobs, long lon
   R.n = r / rows_in_band;
   R.k_blocks = (J.K + bk - 1) / bk;
   R.d = d;
+  R.dp = dp;
   R.cell = R.tp = 0;
   R.k_steps = exact ? (d + 1) * R.k_blocks : R.k_blocks;
   R.live = (pair ? 2 * R.m : R.m) * BM < R.Mc;
@@ -239,7 +249,7 @@ gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ t
   if (!grouped && !k2D) {
     int units = (live_mc + BM - 1) / BM;
     if (kPair) units = (units + 1) / 2;
-    total_tiles = static_cast<long long>(units) * single.n_tiles * (kExact ? single.ex_S : 1);
+    total_tiles = static_cast<long long>(units) * single.n_tiles * (kExact ? single.ex_np : 1);
   }
   const uint32_t rank = kPair ? cluster_rank() : 0u;
   const int cid = kPair ? static_cast<int>(blockIdx.x >> 1) : static_cast<int>(blockIdx.x);
@@ -528,7 +538,7 @@ gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ t
         const int cell = J.surv[ci];
         const int n0 = T.n * kBN + half * kCols;
         if constexpr (kExact) {
-          int32_t* dst = J.planes + T.d * J.plane_stride + (static_cast<long long>(cell) * J.h + j) * J.N;
+          int32_t* dst = J.planes + T.dp * J.plane_stride + (static_cast<long long>(cell) * J.h + j) * J.N;
 #pragma unroll
           for (int q = 0; q < kCols / 4; ++q) {
             const int n = n0 + 4 * q;
@@ -904,8 +914,9 @@ cudaError_t launch_gemm_f32_tc(const DevPlan& p, void* const a[3], void* const b
 }
 
 // Exact-slice digit products: a_planes = coded rows x (S Kp) bf16, b_planes =
-// N x (S Kp) bf16 (plane i of a row at column i Kp); diagonal d of cell c's
-// product goes to planes + d * num_cells h N + c h N as int32.
+// N x (S Kp) bf16 (plane i of a row at column i Kp); the i-th computed diagonal
+// (all S, or with B's digits in pairs every second one) of cell c's product
+// goes to planes + i * num_cells h N + c h N as int32.
 cudaError_t launch_gemm_exact(const DevPlan& p, const void* a_planes, const void* b_planes, int num_cells, int N,
                               int K, int h, const ExactParams& P, int32_t* planes, int config, int32_t* info_out,
                               cudaStream_t st) {
@@ -925,8 +936,11 @@ cudaError_t launch_gemm_exact(const DevPlan& p, const void* a_planes, const void
   J.plane_stride = static_cast<long long>(num_cells) * h * N;
   J.ex_S = P.S;
   J.ex_Kp = P.Kp;
+  J.ex_np = P.np;
+  J.ex_step = P.step;
   const int units = pair ? (J.m_tiles_max + 1) / 2 : J.m_tiles_max;
-  const long long tiles = static_cast<long long>(units) * J.n_tiles * P.S;
+  const long long tiles = static_cast<long long>(units) * J.n_tiles * P.np;
+  J.ex_dmajor = tiles <= 6LL * (pair ? num_sms() / 2 : num_sms());
   return dispatch_exact(bn, pair, bk, J, tiles, group, P.seg, st);
 }
 

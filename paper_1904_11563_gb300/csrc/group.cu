@@ -452,6 +452,7 @@ extern "C" int bpx_autotune(const bpx_code* c, const float* d_A, const float* d_
   if (precision == BPX_EXACT) {
     bpx::ExactParams P;
     if (int rc = bpx::exact_params(c, K, &P)) return rc;
+    bpx::exact_pair_digits(c, &P);  // as the run above staged them
     static const int kExactConfigs[] = {8080, 16080, 4080, 8089, 8081, 8082, 8085};
     if (!configs || nconfigs <= 0) {
       configs = kExactConfigs;
