@@ -256,7 +256,7 @@ int products_impl(const bpx_code* c, const float* d_A, const float* d_B, int M, 
         stage_mark(opts, BPX_STAGE_A_PREP, 1, st);
         stage_mark(opts, BPX_STAGE_GEMM, 0, st);
         if (e == cudaSuccess)
-          e = bpx::launch_gemm_f32_tc(p, a, b, c->num_cells, N, K, h, bpx::rows_expected(c, h), d_products, d_C,
+          e = bpx::launch_gemm_f32_tc(p, a, b, c->num_cells, N, K, h, bpx::rows_range(c, h), d_products, d_C,
                                       d_info, st);
         // operands the parts cannot hold (a plan counter says so): FP32 on the CUDA cores
         if (e == cudaSuccess) e = bpx::launch_encode_f32_flagged(g, p, d_A, M, K, h, a_coded, st);
@@ -268,7 +268,7 @@ int products_impl(const bpx_code* c, const float* d_A, const float* d_B, int M, 
       e = bpx::launch_encode_f32(g, p, d_A, M, K, h, a_coded, st);
       stage_mark(opts, BPX_STAGE_A_PREP, 1, st);
       stage_mark(opts, BPX_STAGE_GEMM, 0, st);
-      if (e == cudaSuccess) e = bpx::launch_gemm_f32(g, p, a_coded, d_B, N, K, h, bpx::rows_expected(c, h), d_products, d_C, st);
+      if (e == cudaSuccess) e = bpx::launch_gemm_f32(g, p, a_coded, d_B, N, K, h, bpx::rows_range(c, h).mean, d_products, d_C, st);
       stage_mark(opts, BPX_STAGE_GEMM, 1, st);
       break;
     }
@@ -291,7 +291,7 @@ int products_impl(const bpx_code* c, const float* d_A, const float* d_B, int M, 
                                    d_info, st);
       else if (e == cudaSuccess)
         e = bpx::launch_gemm_tc(g, p, a_hi, a_lo, b_hi, b_lo, c->num_cells, N, K, h, split,
-                                bpx::rows_expected(c, h), d_products, d_C, config, d_info, st);
+                                bpx::rows_range(c, h), d_products, d_C, config, d_info, st);
       stage_mark(opts, BPX_STAGE_GEMM, 1, st);
       if (e == cudaErrorNotSupported)
         return fail(BPX_ERR_UNSUPPORTED, "bf16 tensor-core path not available in this build");
@@ -313,7 +313,7 @@ int products_impl(const bpx_code* c, const float* d_A, const float* d_B, int M, 
       stage_mark(opts, BPX_STAGE_A_PREP, 1, st);
       stage_mark(opts, BPX_STAGE_GEMM, 0, st);
       if (e == cudaSuccess)
-        e = bpx::launch_gemm_tc(g, p, a_hi, a_lo, b_hi, b_lo, c->num_cells, N, K, h, true, bpx::rows_expected(c, h),
+        e = bpx::launch_gemm_tc(g, p, a_hi, a_lo, b_hi, b_lo, c->num_cells, N, K, h, true, bpx::rows_range(c, h),
                                 d_products, d_C, config, d_info, st, a_exp, b_exp);
       stage_mark(opts, BPX_STAGE_GEMM, 1, st);
       break;

@@ -89,11 +89,17 @@ int exact_params(const bpx_code* c, int K, ExactParams* P);
 // segment for the larger products, where the int32 diagonal sums still fit.
 void exact_pair_digits(const bpx_code* c, ExactParams* P);
 
-// Coded rows to expect from a mask of e erased columns (launch heuristics).
-inline long long rows_expected(const bpx_code* c, int h) {
-  const long long rows = static_cast<long long>(c->num_cells) * h;
-  return c->e > 0 && c->e < c->n ? rows * (c->n - c->e) / c->n : rows;
-}
+// Coded rows that masks of e erased columns leave (launch heuristics; the
+// mask itself is on the device): the fewest, the mean, the most.
+struct RowsRange {
+  long long least, mean, most;
+  // the mean over the range of f(rows): least, mean, most and the midpoints between
+  template <typename F>
+  double average(F f) const {
+    return (f(least) + f((least + mean) / 2) + f(mean) + f((mean + most) / 2) + f(most)) / 5.0;
+  }
+};
+RowsRange rows_range(const bpx_code* c, int h);
 
 // Whether BPX_FP32 products of this shape run on the tensor cores (three bf16
 // parts per operand, six products) rather than on the CUDA cores.

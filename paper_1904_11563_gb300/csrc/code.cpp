@@ -394,6 +394,23 @@ void exact_pair_digits(const bpx_code* c, ExactParams* P) {
   P->seg = seg;
 }
 
+RowsRange rows_range(const bpx_code* c, int h) {
+  std::vector<long long> cells;
+  for (int j = 0; j < c->n; ++j) cells.push_back(c->col_ptr[j + 1] - c->col_ptr[j]);
+  std::sort(cells.begin(), cells.end());
+  const int e = c->e > 0 && c->e < c->n ? c->e : 0;
+  const long long all = c->num_cells;
+  RowsRange r{all, all * (c->n - e) / c->n, all};
+  for (int j = 0; j < e; ++j) {
+    r.most -= cells[j];
+    r.least -= cells[c->n - 1 - j];
+  }
+  r.least *= h;
+  r.mean *= h;
+  r.most *= h;
+  return r;
+}
+
 // The line between the two FP32 forms.  Staging of B and GEMM, CUDA cores
 // against tensor cores (coded rows x K x N): 568 x 768 x 512 (0.22 G
 // multiply-adds) 27 against 37 us, 1136 x 512 x 512 (0.30 G) 27 against 32,
@@ -403,7 +420,7 @@ void exact_pair_digits(const bpx_code* c, ExactParams* P) {
 bool f32_on_tensor_cores(const bpx_code* c, int N, int K, int h) {
   if (N <= 0 || K <= 0 || h <= 0) return false;
   return K >= 128 && static_cast<long long>(N) * K > 65536 &&
-         static_cast<double>(rows_expected(c, h)) * N * K >= 4e8;
+         static_cast<double>(rows_range(c, h).mean) * N * K >= 4e8;
 }
 
 WsLayout ws_layout(const bpx_code* c, int M, int N, int K, int h, int precision, bool twod) {

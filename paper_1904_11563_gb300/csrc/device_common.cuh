@@ -268,7 +268,7 @@ cudaError_t launch_encode_f32_flagged(const DevGraph& g, const DevPlan& p, const
 cudaError_t launch_gemm_f32_flagged(const DevGraph& g, const DevPlan& p, const float* a_coded, const float* B, int N,
                                     int K, int h, float* products, float* C_direct, cudaStream_t st);
 cudaError_t launch_gemm_f32_tc(const DevPlan& p, void* const a[3], void* const b[3], int num_cells, int N, int K, int h,
-                               long long rows_est, float* products, float* C_direct, int32_t* info_out,
+                               const RowsRange& range, float* products, float* C_direct, int32_t* info_out,
                                cudaStream_t st);
 // MXFP8 staging (E4M3 data + UE8M0 scales in the GEMM's per-stage order) and GEMM.
 cudaError_t launch_encode_mx(const DevGraph& g, const DevPlan& p, const float* A, int M, int K, int h,
@@ -287,12 +287,12 @@ cudaError_t launch_gemm_f32(const DevGraph& g, const DevPlan& p, const float* a_
 cudaError_t launch_gemm_fused(const DevGraph& g, const DevPlan& p, const float* A, int M, const void* b_hi,
                               const void* b_lo, int num_cells, int N, int K, int h, bool split3, float* products,
                               float* C_direct, int config, int32_t* info_out, cudaStream_t st);
-// rows_est: the coded rows to expect (chooses the tile when config is 0).
+// range: the coded rows to expect (chooses the tile when config is 0).
 // a_exp / b_exp non-null: the split-fp16 operands of BPX_FP16X3 (a_lo and
 // b_lo required), unscaled by 2^-(a_exp[row] + b_exp[col]) in the epilogue.
 cudaError_t launch_gemm_tc(const DevGraph& g, const DevPlan& p, const void* a_hi, const void* a_lo,
                            const void* b_hi, const void* b_lo, int num_cells, int N, int K, int h,
-                           bool split3, long long rows_est, float* products, float* C_direct, int config,
+                           bool split3, const RowsRange& range, float* products, float* C_direct, int config,
                            int32_t* info_out, cudaStream_t st, const int32_t* a_exp = nullptr,
                            const int32_t* b_exp = nullptr);
 

@@ -207,7 +207,10 @@ __device__ __forceinline__ TileRef locate(const TcJob* jobs, int njobs, long lon
 // a pair with the same B tile, computed by CTA-pair MMAs (cta_group::2,
 // M = 256): each CTA loads only its own A rows and its half of the B tile,
 // so a CTA's shared memory takes a third less traffic per MMA.  kPair == 0:
-// one CTA per tile.  (No variant loads by TMA multicast.)
+// one CTA per tile.  kPair == 4: clusters of two such pairs on two adjacent
+// n-tiles of the same rows; each CTA loads half of its A rows and multicasts
+// them to its counterpart in the other pair, and a stage is free once both
+// pairs' MMAs have read it.
 // kMode == kModeExact: exact-slice digit products (plain bf16 MMAs over the
 // digit planes, k-slices of the diagonal's digit pairs in sequence; FP32
 // segments exact by construction, promoted to int32 and stored to the
@@ -225,8 +228,9 @@ gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ t
                long long total_tiles, int group, int seg_kb) {
   constexpr bool kExact = kMode == kModeExact;
   constexpr bool k2D = kMode == kMode2D;
-  static_assert(kPair == 0 || kPair == 2, "tiles are 1-CTA or CTA-pair MMAs");
-  constexpr bool k2Sm = kPair == 2;
+  static_assert(kPair == 0 || kPair == 2 || (kPair == 4 && kParts < 3), "tiles are 1-CTA or CTA-pair MMAs, alone or two pairs");
+  constexpr bool k2Sm = kPair != 0;
+  constexpr bool kQuad = kPair == 4;
   constexpr bool kSplit = kParts >= 2;
   using St = Stage<kParts, k2Sm ? kBN / 2 : kBN, kBK>;  // a CTA pair holds half the B tile each
   constexpr int kTmemCols = 2 * kBN;  // two FP32 segment accumulators
@@ -251,15 +255,19 @@ gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ t
     if (kPair) units = (units + 1) / 2;
     total_tiles = static_cast<long long>(units) * single.n_tiles * (kExact ? single.ex_np : 1);
   }
-  const uint32_t rank = kPair ? cluster_rank() : 0u;
-  const int cid = kPair ? static_cast<int>(blockIdx.x >> 1) : static_cast<int>(blockIdx.x);
-  const int nclusters = kPair ? static_cast<int>(gridDim.x >> 1) : static_cast<int>(gridDim.x);
+  constexpr int kClusterShift = kQuad ? 2 : kPair ? 1 : 0;
+  const uint32_t crank = kPair ? cluster_rank() : 0u;
+  const uint32_t rank = crank & 1u, leader = crank & ~1u;  // of the pair; its even CTA
+  const int side = static_cast<int>(crank >> 1);           // quad: which of the two n-tiles the pair takes
+  const int cid = static_cast<int>(blockIdx.x >> kClusterShift);
+  const int nclusters = static_cast<int>(gridDim.x >> kClusterShift);
+  const uint16_t pair_mask = static_cast<uint16_t>(3u << leader);
 
   if (threadIdx.x == 0) {
     abort_flag = 0;
     for (int s = 0; s < kStages; ++s) {
       mbar_init(smem_u32(&full_bar[s]), 1);
-      mbar_init(smem_u32(&empty_bar[s]), 1);
+      mbar_init(smem_u32(&empty_bar[s]), kQuad ? 2 : 1);  // quad: both pairs' MMAs have read the shared A rows
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(smem_u32(&sfull_bar[a]), 1);
@@ -309,7 +317,8 @@ gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ t
           fenced = T.J;
         }
         const int m_cta = kPair ? 2 * T.m + static_cast<int>(rank) : T.m;
-        int ya = m_cta * BM, yb = T.n * kBN, cur_term = -1;
+        const int n_tile = kQuad ? 2 * T.n + side : T.n;
+        int ya = m_cta * BM, yb = n_tile * kBN, cur_term = -1;
         for (int q = 0; q < T.k_steps; ++q, ++kb_all) {
           const int s = kb_all % kStages;
           int xa = q * kBK, xb = q * kBK;
@@ -323,7 +332,7 @@ gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ t
             if (ti != cur_term) {
               cur_term = ti;
               ya = T.J->t2_a[T.tp + ti] * T.J->h + m_cta * BM;
-              yb = T.J->t2_b[T.tp + ti] * T.J->w2 + T.n * kBN;
+              yb = T.J->t2_b[T.tp + ti] * T.J->w2 + n_tile * kBN;
             }
             xa = xb = kb * kBK;
           }
@@ -338,11 +347,18 @@ gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ t
           if constexpr (k2Sm) {
             // both CTAs' copies count on the even CTA's barrier, armed there
             // for the two stages' bytes
-            const uint32_t fb0 = mapa_rank(fb, 0);
+            const uint32_t fb0 = mapa_rank(fb, leader);
             if (rank == 0) mbar_expect_tx(fb, 2 * St::kBytes);
             const int yh = yb + static_cast<int>(rank) * (kBN / 2);
-            tma_load_2d_pair(base + St::kAhi, &T.J->map_ahi, fb0, xa, ya);
-            if (kSplit) tma_load_2d_pair(base + St::kAlo, &T.J->map_alo, fb0, xa, ya);
+            if constexpr (kQuad) {  // half of the A rows, for this CTA and its counterpart in the other pair
+              const uint16_t both = static_cast<uint16_t>(5u << rank);
+              const uint32_t half = static_cast<uint32_t>(side) * (St::kA / 2);
+              tma_load_2d_pairs(base + St::kAhi + half, &T.J->map_ahi, fb0, xa, ya + side * (BM / 2), both);
+              if (kSplit) tma_load_2d_pairs(base + St::kAlo + half, &T.J->map_alo, fb0, xa, ya + side * (BM / 2), both);
+            } else {
+              tma_load_2d_pair(base + St::kAhi, &T.J->map_ahi, fb0, xa, ya);
+              if (kSplit) tma_load_2d_pair(base + St::kAlo, &T.J->map_alo, fb0, xa, ya);
+            }
             tma_load_2d_pair(base + St::kBhi, &T.J->map_bhi, fb0, xb, yh);
             if (kSplit) tma_load_2d_pair(base + St::kBlo, &T.J->map_blo, fb0, xb, yh);
             if (kParts == 3) {
@@ -449,13 +465,13 @@ gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ t
               }
             }
             if (k2Sm)
-              umma_commit_pair(smem_u32(&empty_bar[s]));
+              umma_commit_pair(smem_u32(&empty_bar[s]), kQuad ? 15 : 3);
             else
               umma_commit(smem_u32(&empty_bar[s]));
           }
           if (!ok) break;
           if (k2Sm)
-            umma_commit_pair(smem_u32(&sfull_bar[buf]));
+            umma_commit_pair(smem_u32(&sfull_bar[buf]), pair_mask);
           else
             umma_commit(smem_u32(&sfull_bar[buf]));
         }
@@ -506,13 +522,14 @@ gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ t
         __syncwarp();
         if (lane == 0) {
           if (k2Sm)  // the even CTA's MMA thread waits for both CTAs' drains
-            mbar_arrive_cluster(mapa_rank(smem_u32(&sempty_bar[buf]), 0));
+            mbar_arrive_cluster(mapa_rank(smem_u32(&sempty_bar[buf]), leader));
           else
             mbar_arrive(smem_u32(&sempty_bar[buf]));
         }
       }
       if (!ok) break;
       const TcJob& J = *T.J;
+      const int n_tile = kQuad ? 2 * T.n + side : T.n;
       const int r = (kPair ? 2 * T.m + static_cast<int>(rank) : T.m) * BM + row;
       if (k2D) {
         if (r < J.h) {  // row r of the cell's h x w block
@@ -524,7 +541,7 @@ gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ t
           } else {
             dst = J.products + (static_cast<long long>(T.cell) * J.h + r) * J.w2;
           }
-          const int n0 = T.n * kBN + half * kCols;
+          const int n0 = n_tile * kBN + half * kCols;
 #pragma unroll
           for (int q = 0; q < kCols / 4; ++q) {
             const int n = n0 + 4 * q;
@@ -536,7 +553,7 @@ gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ t
         const int ci = r / J.h;
         const int j = r - ci * J.h;
         const int cell = J.surv[ci];
-        const int n0 = T.n * kBN + half * kCols;
+        const int n0 = n_tile * kBN + half * kCols;
         if constexpr (kExact) {
           int32_t* dst = J.planes + T.dp * J.plane_stride + (static_cast<long long>(cell) * J.h + j) * J.N;
 #pragma unroll
@@ -652,8 +669,9 @@ int tile_bk(int config) { return (config % 10) >= 5 ? 32 : 64; }
 // tile reads as much of A from shared memory per MMA.  GEMM, pair against the
 // tile chosen (coded rows x K x N): 568 x 256 x 128 16.3 -> 10.2 us, 1136 x
 // 1416 x 1100 32.8 -> 26.6, 4544 x 4096 x 512 67.5 -> 49.3; 2272 x 1992 x 2044
-// keeps pairs, 44 against 60.
-int auto_bn(int parts, long long rows, int N, int K) {
+// keeps pairs, 44 against 60.  The waves are averaged over the rows that masks
+// of the code's e erasures leave.
+int auto_bn(int parts, const RowsRange& range, int N, int K) {
   const long long sms = std::max(1, num_sms());
   const int kb = (K + BK - 1) / BK;
   const double scale = parts == 1 ? 2.0 : parts == 3 ? 0.5 : 1.0;  // drains against a k-block's MMAs
@@ -664,14 +682,35 @@ int auto_bn(int parts, long long rows, int N, int K) {
   for (int i = 0; i < 3; ++i) {
     const int m = i == 0 ? 256 : 128;
     const long long slots = i == 0 ? std::max(1LL, sms / 2) : sms;
-    const long long tiles = (rows + m - 1) / m * ((N + bn[i] - 1) / bn[i]);
-    const double t = static_cast<double>((tiles + slots - 1) / slots) * kb * step[i] + drain[i];
+    const double waves = range.average([&](long long rows) {
+      const long long tiles = (rows + m - 1) / m * ((N + bn[i] - 1) / bn[i]);
+      return static_cast<double>((tiles + slots - 1) / slots);
+    });
+    const double t = waves * kb * step[i] + drain[i];
     if (i == 0 || t < least) {
       least = t;
       best = i;
     }
   }
   return bn[best];
+}
+
+// Whether a product over 256 x 256 tiles, n_tiles of them across, runs as clusters of two CTA pairs that share their A rows by TMA
+// multicast (kPair 4): a quarter less is read from L2 per MMA.  Only as the
+// default's choice, with an even number of n-tiles (none is left out) and no
+// more waves.  Benchmark GEMM 1874 -> 1773 us (split bf16), 2093 -> 1995 (split
+// fp16); two-dimensional bf16 at 4096 cubed 291 -> 262.  The exact slices'
+// digit products keep single pairs (7128 against 6904 us at 8192 cubed), and so
+// does FP32 in three parts (the same within 0.4 %).
+bool take_quads(const RowsRange& range, int n_tiles) {
+  if (n_tiles % 2 != 0) return false;
+  const long long pairs = std::max(1, num_sms() / 2), quads = std::max(1, num_sms() / 4);
+  auto waves = [&](long long slots, int n) {
+    return range.average([&](long long rows) {
+      return static_cast<double>(((rows + 255) / 256 * n + slots - 1) / slots);
+    });
+  };
+  return waves(quads, n_tiles / 2) <= waves(pairs, n_tiles);
 }
 
 // seg_kb: k-slices of kBK per TMEM accumulation segment.
@@ -681,7 +720,7 @@ cudaError_t launch_variant(const TcJob& single, const TcJob* table, int njobs, l
   // 32-wide slices: 32 KB of slack after the stages, so that the descriptors
   // of the 64-byte swizzled layout can never reach past the allocation.
   // (a CTA of a cta_group::2 pair stages half the B tile)
-  using St = Stage<kParts, kPair == 2 ? kBN / 2 : kBN, kBK>;
+  using St = Stage<kParts, kPair != 0 ? kBN / 2 : kBN, kBK>;
   const size_t smem = static_cast<size_t>(kStages) * St::kBytes + 1024 + (kBK == 32 ? 32768 : 0);
   auto kern = gemm_tc_kernel<kParts, kStages, kBN, kPair, kBK, kMode>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
@@ -698,21 +737,22 @@ cudaError_t launch_variant(const TcJob& single, const TcJob* table, int njobs, l
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 2;
+  constexpr int kCtas = kPair == 4 ? 4 : 2;
+  attr[0].val.clusterDim.x = kCtas;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   // as many CTA pairs as can be resident at once (pairs must share a GPC)
-  cfg.gridDim = dim3(2 * (num_sms() / 2));
+  cfg.gridDim = dim3(kCtas * (num_sms() / kCtas));
   int resident = 0;
   if (cudaOccupancyMaxActiveClusters(&resident, kern, &cfg) != cudaSuccess || resident <= 0) {
     cudaGetLastError();
-    resident = num_sms() / 2;
+    resident = num_sms() / kCtas;
   }
-  resident = std::max(1, resident - (reserved_sms() + 1) / 2);
+  resident = std::max(1, resident - (reserved_sms() + kCtas - 1) / kCtas);
   const int clusters = static_cast<int>(std::min<long long>(total_tiles, resident));
-  cfg.gridDim = dim3(2 * clusters);
+  cfg.gridDim = dim3(kCtas * clusters);
   return cudaLaunchKernelEx(&cfg, kern, single, table, njobs, total_tiles, group, seg_kb);
 }
 
@@ -728,6 +768,9 @@ cudaError_t dispatch_bk(bool split3, int bn, int pair, const TcJob& single, cons
     if (bn == 64) return split3 ? BPX_LV(2, 4, 64, 0) : BPX_LV(1, 8, 64, 0);
   }
   // CTA-pair MMAs: a stage holds the CTA's A rows and half the B tile
+  if constexpr (kBK == BK) {
+    if (pair == 4) return split3 ? BPX_LV(2, 3, 256, 4) : BPX_LV(1, 6, 256, 4);
+  }
   if (pair == 2) return split3 ? BPX_LV(2, 3 * m, 256, 2) : BPX_LV(1, 6 * m, 256, 2);
   if (split3) return bn == 128 ? BPX_LV(2, 3 * m, 128, 0) : BPX_LV(2, 2 * m, 256, 0);
   return bn == 128 ? BPX_LV(1, 6 * m, 128, 0) : BPX_LV(1, 4 * m, 256, 0);
@@ -789,19 +832,20 @@ void decode_config(int config, int* group, int* seg_kb, int* bn, int* pair, int*
 namespace {
 
 bool tc_fill_job(TcJob* J, const DevPlan& p, const void* a_hi, const void* a_lo, const void* b_hi,
-                 const void* b_lo, int num_cells, int N, int K, int h, int bn, bool pair, int bk,
+                 const void* b_lo, int num_cells, int N, int K, int h, int bn, int pair, int bk,
                  float* products, float* C_direct, int32_t* info_out, const int32_t* a_exp = nullptr,
                  const int32_t* b_exp = nullptr) {
   memset(J, 0, sizeof *J);
   const long long rows = static_cast<long long>(num_cells) * h;
   const int box_b = pair ? bn / 2 : bn;  // a paired CTA loads half of the B tile
+  const int box_a = pair == 4 ? BM / 2 : BM;  // two pairs share A: each CTA loads half of its rows for both
   const bool f16 = a_exp != nullptr;
-  if (!make_map(&J->map_ahi, a_hi, rows, K, BM, bk, f16) || !make_map(&J->map_bhi, b_hi, N, K, box_b, bk, f16))
+  if (!make_map(&J->map_ahi, a_hi, rows, K, box_a, bk, f16) || !make_map(&J->map_bhi, b_hi, N, K, box_b, bk, f16))
     return false;
   J->a_exp = a_exp;
   J->b_exp = b_exp;
   if (a_lo) {
-    if (!make_map(&J->map_alo, a_lo, rows, K, BM, bk, f16) || !make_map(&J->map_blo, b_lo, N, K, box_b, bk, f16))
+    if (!make_map(&J->map_alo, a_lo, rows, K, box_a, bk, f16) || !make_map(&J->map_blo, b_lo, N, K, box_b, bk, f16))
       return false;
   } else {
     J->map_alo = J->map_ahi;
@@ -819,6 +863,7 @@ bool tc_fill_job(TcJob* J, const DevPlan& p, const void* a_hi, const void* a_lo,
   J->h = h;
   J->m_tiles_max = static_cast<int>((rows + BM - 1) / BM);
   J->n_tiles = (N + bn - 1) / bn;
+  if (pair == 4) J->n_tiles = (J->n_tiles + 1) / 2;  // counted by two
   J->tile_base = 0;
   return true;
 }
@@ -862,7 +907,7 @@ bool gemm_config_ok(int config) { return tile_valid(config); }
 
 cudaError_t launch_gemm_tc(const DevGraph& g, const DevPlan& p, const void* a_hi, const void* a_lo,
                            const void* b_hi, const void* b_lo, int num_cells, int N, int K, int h,
-                           bool split3, long long rows_est, float* products, float* C_direct, int config,
+                           bool split3, const RowsRange& range, float* products, float* C_direct, int config,
                            int32_t* info_out, cudaStream_t st, const int32_t* a_exp, const int32_t* b_exp) {
   if (!tile_valid(config)) return cudaErrorInvalidValue;
   if ((a_exp != nullptr) != (b_exp != nullptr) || (a_exp && !split3)) return cudaErrorInvalidValue;
@@ -877,8 +922,8 @@ cudaError_t launch_gemm_tc(const DevGraph& g, const DevPlan& p, const void* a_hi
   // (propagation factor 32) 256-wide segments 9.2e-6, 128-wide 7.9e-6.
   if (a_exp && config == 0) seg_kb = 2;
   if (config == 0) {
-    bn = auto_bn(split3 ? 2 : 1, rows_est, N, K);
-    pair = bn == 256 ? 2 : 0;
+    bn = auto_bn(split3 ? 2 : 1, range, N, K);
+    pair = bn < 256 ? 0 : take_quads(range, (N + bn - 1) / bn) ? 4 : 2;
   }
   TcJob J;
   if (!tc_fill_job(&J, p, a_hi, split3 ? a_lo : nullptr, b_hi, split3 ? b_lo : nullptr, num_cells, N, K, h,
@@ -897,12 +942,12 @@ cudaError_t launch_gemm_tc(const DevGraph& g, const DevPlan& p, const void* a_hi
 // directly computed block 1.3e-7 at K = 1992 against 8.0e-7, 1.7e-7 at 4096
 // against 1.1e-6.  32-wide k-slices (four stages) ran 3.73 ms.
 cudaError_t launch_gemm_f32_tc(const DevPlan& p, void* const a[3], void* const b[3], int num_cells, int N, int K, int h,
-                               long long rows_est, float* products, float* C_direct, int32_t* info_out,
+                               const RowsRange& range, float* products, float* C_direct, int32_t* info_out,
                                cudaStream_t st) {
-  const int bn = auto_bn(3, rows_est, N, K);
+  const int bn = auto_bn(3, range, N, K);
   const bool small = bn < 256;
   TcJob J;
-  if (!tc_fill_job(&J, p, a[0], a[1], b[0], b[1], num_cells, N, K, h, bn, !small, BK, products, C_direct, info_out))
+  if (!tc_fill_job(&J, p, a[0], a[1], b[0], b[1], num_cells, N, K, h, bn, small ? 0 : 2, BK, products, C_direct, info_out))
     return cudaErrorInvalidValue;
   const long long rows = static_cast<long long>(num_cells) * h;
   if (!make_map(&J.map_a3, a[2], rows, K, BM) || !make_map(&J.map_b3, b[2], N, K, bn == 64 ? 64 : 128)) return cudaErrorInvalidValue;
@@ -940,7 +985,7 @@ cudaError_t launch_gemm_exact(const DevPlan& p, const void* a_planes, const void
   J.ex_step = P.step;
   const int units = pair ? (J.m_tiles_max + 1) / 2 : J.m_tiles_max;
   const long long tiles = static_cast<long long>(units) * J.n_tiles * P.np;
-  J.ex_dmajor = tiles <= 6LL * (pair ? num_sms() / 2 : num_sms());
+  J.ex_dmajor = tiles <= 6LL * (num_sms() / (pair ? pair : 1));
   return dispatch_exact(bn, pair, bk, J, tiles, group, P.seg, st);
 }
 
@@ -957,12 +1002,14 @@ cudaError_t launch_gemm_2d(const DevGraph& g, const DevPlan& p, const void* a_hi
   decode_config(config, &group, &seg_kb, &bn, &pair, &bk);
   TcJob J;
   memset(&J, 0, sizeof J);
-  const int box_b = pair ? bn / 2 : bn;
+  const long long space = (h + 255) / 256 * 256LL * g.num_cells;  // every cell's rows, erased or not
+  if (config == 0 && take_quads({space, space, space}, (w + bn - 1) / bn)) pair = 4;
+  const int box_b = pair ? bn / 2 : bn, box_a = pair == 4 ? BM / 2 : BM;
   const long long rows_a = static_cast<long long>(g.EA) * h, rows_b = static_cast<long long>(g.EB) * w;
-  if (!make_map(&J.map_ahi, a_hi, rows_a, K, BM, bk) || !make_map(&J.map_bhi, b_hi, rows_b, K, box_b, bk))
+  if (!make_map(&J.map_ahi, a_hi, rows_a, K, box_a, bk) || !make_map(&J.map_bhi, b_hi, rows_b, K, box_b, bk))
     return cudaErrorInvalidValue;
   if (split3) {
-    if (!make_map(&J.map_alo, a_lo, rows_a, K, BM, bk) || !make_map(&J.map_blo, b_lo, rows_b, K, box_b, bk))
+    if (!make_map(&J.map_alo, a_lo, rows_a, K, box_a, bk) || !make_map(&J.map_blo, b_lo, rows_b, K, box_b, bk))
       return cudaErrorInvalidValue;
   } else {
     J.map_alo = J.map_ahi;
@@ -980,6 +1027,7 @@ cudaError_t launch_gemm_2d(const DevGraph& g, const DevPlan& p, const void* a_hi
   J.h = h;
   J.m_tiles_max = (h + BM - 1) / BM;
   J.n_tiles = (w + bn - 1) / bn;
+  if (pair == 4) J.n_tiles = (J.n_tiles + 1) / 2;
   J.t2_ptr = g.t2_ptr;
   J.t2_a = g.t2_a;
   J.t2_b = g.t2_b;

@@ -470,7 +470,7 @@ extern "C" int bpx_autotune(const bpx_code* c, const float* d_A, const float* d_
               [&](int cfg) -> int {
                 cudaError_t e = bpx::launch_gemm_tc(g, p, base + L.a_hi, split ? base + L.a_lo : nullptr,
                                                     base + L.b_hi, split ? base + L.b_lo : nullptr,
-                                                    c->num_cells, N, K, h, split, bpx::rows_expected(c, h), products,
+                                                    c->num_cells, N, K, h, split, bpx::rows_range(c, h), products,
                                                     d_C, cfg, nullptr, st, a_exp, b_exp);
                 return e == cudaSuccess ? BPX_OK : cuda_fail(e, "autotune launch");
               },

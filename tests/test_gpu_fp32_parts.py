@@ -100,3 +100,28 @@ def test_default_tile_same_bits(libbpx, M, K, N, prec, pair):
     C = [bpx.coded_matmul(code, A, B, h, bpx.PRECISIONS[prec], mask, ws, opts=bpx.default_opts(gemm_config=c))[0]
          for c in (0, pair)]
     assert torch.equal(C[0], C[1])
+
+
+# two pairs a cluster (an even number of 256-wide tiles, the default of larger
+# products) against single pairs, rows short of a tile and one wave or several
+@pytest.mark.parametrize("M,K,N", [(4000, 200, 4096), (8190, 136, 1536), (2050, 72, 2300)])
+@pytest.mark.parametrize("prec,pair", [("bf16", 8080), ("bf16x3", 8080), ("fp16x3", 8020)])
+def test_pairs_sharing_rows_same_bits(libbpx, M, K, N, prec, pair):
+    test_default_tile_same_bits(libbpx, M, K, N, prec, pair)
+
+
+@pytest.mark.parametrize("M,K,w", [(2048, 200, 512), (1000, 72, 1000), (4096, 136, 256)])
+@pytest.mark.parametrize("prec", ["bf16", "bf16x3"])
+def test_two_dimensional_default_same_bits(libbpx, M, K, w, prec):
+    bpx = libbpx
+    code = bpx.Code.systematic(4, 2, 5)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(M + K)
+    N, h, P = code.k * w, -(-M // code.b), bpx.PRECISIONS[prec]
+    A = torch.randn((M, K), generator=g, device="cuda")
+    B = torch.randn((K, N), generator=g, device="cuda")
+    ws = bpx.Workspace2D(code, M, N, K, h, P)
+    mask = torch.zeros(code.n, dtype=torch.uint8, device="cuda")
+    mask[[1, 4]] = 1
+    C = [bpx.coded_matmul_2d(code, A, B, h, P, mask, ws, opts=bpx.default_opts(gemm_config=c))[0] for c in (0, 8080)]
+    assert torch.equal(C[0], C[1])
