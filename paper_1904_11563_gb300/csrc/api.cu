@@ -24,6 +24,11 @@ int num_sms() {
   return sms;
 }
 
+bool& chain_on() {
+  thread_local bool on = false;
+  return on;
+}
+
 int& reserved_sms() {
   thread_local int r = 0;
   return r;
@@ -178,6 +183,18 @@ SideStream* side_stream() {
   return &ss;
 }
 
+// Whether a call's launches on st may be chained: not while the caller times
+// the stages (each kernel then runs alone) nor while st is being captured.
+bool may_chain(const bpx_opts& o, cudaStream_t st) {
+  if (o.stage_events) return false;
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &status) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return status == cudaStreamCaptureStatusNone;
+}
+
 struct ReserveGuard {
   explicit ReserveGuard(int n) { bpx::reserved_sms() = n; }
   ~ReserveGuard() { bpx::reserved_sms() = 0; }
@@ -218,7 +235,8 @@ namespace {
 
 int products_impl(const bpx_code* c, const float* d_A, const float* d_B, int M, int N, int K,
                   int h, int precision, void* ws, size_t ws_bytes, float* d_products, float* d_C,
-                  const bpx_opts* opts, int32_t* d_info, cudaStream_t st, bool pair_digits = false) {
+                  const bpx_opts* opts, int32_t* d_info, cudaStream_t st, bool pair_digits = false,
+                  bool after_schedule = false) {
   if (!c || (!d_A && M > 0) || !d_B || !ws || !d_products)  // A unused when M = 0
     return fail(BPX_ERR_INVAL, "bpx_coded_products: NULL argument");
   if (int rc = check_shapes(c, M, N, K, h)) return rc;
@@ -242,6 +260,7 @@ int products_impl(const bpx_code* c, const float* d_A, const float* d_B, int M, 
     return fail(BPX_ERR_INVAL, "bpx_coded_products: the fused encode needs gemm_config 0 or tile code 0 (got %d)",
                 config);
   cudaError_t e = cudaSuccess;
+  const bool early = after_schedule && bpx::chain_on();
   switch (precision) {
     case BPX_FP32: {
       float* a_coded = reinterpret_cast<float*>(base + L.a_hi);
@@ -249,7 +268,7 @@ int products_impl(const bpx_code* c, const float* d_A, const float* d_B, int M, 
         void* const a[3] = {base + L.a_hi, base + L.a_lo, base + L.a_3};
         void* const b[3] = {base + L.b_hi, base + L.b_lo, base + L.b_3};
         stage_mark(opts, BPX_STAGE_B_PREP, 0, st);
-        e = bpx::launch_b_parts(p, d_B, K, N, b, st);
+        e = bpx::launch_b_parts(p, d_B, K, N, b, st, early);
         stage_mark(opts, BPX_STAGE_B_PREP, 1, st);
         stage_mark(opts, BPX_STAGE_A_PREP, 0, st);
         if (e == cudaSuccess) e = bpx::launch_encode_parts(g, p, d_A, M, K, h, a, st);
@@ -280,7 +299,7 @@ int products_impl(const bpx_code* c, const float* d_A, const float* d_B, int M, 
       void* b_hi = base + L.b_hi;
       void* b_lo = split ? base + L.b_lo : nullptr;
       stage_mark(opts, BPX_STAGE_B_PREP, 0, st);
-      e = bpx::launch_b_split(d_B, K, N, b_hi, b_lo, st);
+      e = bpx::launch_b_split(d_B, K, N, b_hi, b_lo, st, early);
       stage_mark(opts, BPX_STAGE_B_PREP, 1, st);
       stage_mark(opts, BPX_STAGE_A_PREP, 0, st);
       if (e == cudaSuccess && !fused) e = bpx::launch_encode_split(g, p, d_A, M, K, h, a_hi, a_lo, st);
@@ -306,7 +325,7 @@ int products_impl(const bpx_code* c, const float* d_A, const float* d_B, int M, 
       uint32_t* b_max = reinterpret_cast<uint32_t*>(base + L.b_scale);
       int32_t* b_exp = reinterpret_cast<int32_t*>(b_max + N);
       stage_mark(opts, BPX_STAGE_B_PREP, 0, st);
-      e = bpx::launch_b_f16(d_B, K, N, b_hi, b_lo, b_max, b_exp, st);
+      e = bpx::launch_b_f16(g, h, d_B, K, N, b_hi, b_lo, b_max, b_exp, a_exp, st, early);
       stage_mark(opts, BPX_STAGE_B_PREP, 1, st);
       stage_mark(opts, BPX_STAGE_A_PREP, 0, st);
       if (e == cudaSuccess) e = bpx::launch_encode_f16(g, p, d_A, M, K, h, a_hi, a_lo, a_exp, st);
@@ -325,7 +344,7 @@ int products_impl(const bpx_code* c, const float* d_A, const float* d_B, int M, 
       void* sfa = base + L.a_scale;
       void* sfb = base + L.b_scale;
       stage_mark(opts, BPX_STAGE_B_PREP, 0, st);
-      e = bpx::launch_b_mx(d_B, K, N, b8, sfb, st);
+      e = bpx::launch_b_mx(d_B, K, N, b8, sfb, st, early);
       stage_mark(opts, BPX_STAGE_B_PREP, 1, st);
       stage_mark(opts, BPX_STAGE_A_PREP, 0, st);
       if (e == cudaSuccess) e = bpx::launch_encode_mx(g, p, d_A, M, K, h, a8, sfa, st);
@@ -344,7 +363,7 @@ int products_impl(const bpx_code* c, const float* d_A, const float* d_B, int M, 
       void* a_pl = base + L.a_hi;
       void* b_pl = base + L.b_hi;
       stage_mark(opts, BPX_STAGE_B_PREP, 0, st);
-      e = bpx::launch_exact_b(d_B, K, N, P, amax + h, amax, h, b_pl, st);
+      e = bpx::launch_exact_b(d_B, K, N, P, amax + h, amax, h, b_pl, st, early);
       stage_mark(opts, BPX_STAGE_B_PREP, 1, st);
       stage_mark(opts, BPX_STAGE_A_PREP, 0, st);
       if (e == cudaSuccess)
@@ -488,6 +507,7 @@ extern "C" int bpx_coded_matmul_2d(const bpx_code* c, const float* d_A, const fl
   if (!bpx::gemm_config_ok(o.gemm_config))
     return fail(BPX_ERR_INVAL, "bpx_coded_matmul_2d: gemm_config %d names no tile", o.gemm_config);
   cudaStream_t st = S(stream);
+  const bpx::ChainScope chain(may_chain(o, st));
   stage_mark(&o, BPX_STAGE_SCHEDULE, 0, st);
   if (int rc = schedule_impl(c, d_mask, o.mask_cells != 0, ws, ws_bytes, nullptr, nullptr, d_info, st)) return rc;
   stage_mark(&o, BPX_STAGE_SCHEDULE, 1, st);
@@ -501,7 +521,7 @@ extern "C" int bpx_coded_matmul_2d(const bpx_code* c, const float* d_A, const fl
   void* b_lo = split ? base + L.b_lo : nullptr;
   float* products = reinterpret_cast<float*>(base + L.products);
   stage_mark(&o, BPX_STAGE_A_PREP, 0, st);
-  cudaError_t e = bpx::launch_stage_2d(g, d_A, d_B, M, N, K, h, w, a_hi, a_lo, b_hi, b_lo, st);
+  cudaError_t e = bpx::launch_stage_2d(g, d_A, d_B, M, N, K, h, w, a_hi, a_lo, b_hi, b_lo, st, bpx::chain_on());
   stage_mark(&o, BPX_STAGE_A_PREP, 1, st);
   if (e != cudaSuccess) return cuda_fail(e, "bpx_coded_matmul_2d: staging");
   stage_mark(&o, BPX_STAGE_GEMM, 0, st);
@@ -529,6 +549,7 @@ extern "C" int bpx_coded_matmul(const bpx_code* c, const float* d_A, const float
   const bpx::WsLayout L = bpx::ws_layout(c, M, N, K, h, precision);
   if (int rc = check_ws(c, ws, ws_bytes, L)) return rc;
   SideStream* side = c->S >= kOverlapSources ? side_stream() : nullptr;
+  const bpx::ChainScope chain(!side && may_chain(o, S(stream)));
   stage_mark(&o, BPX_STAGE_SCHEDULE, 0, S(stream));
   if (!side) {
     if (int rc = schedule_impl(c, d_mask, o.mask_cells != 0, ws, ws_bytes, nullptr, nullptr, d_info, S(stream)))
@@ -555,13 +576,13 @@ extern "C" int bpx_coded_matmul(const bpx_code* c, const float* d_A, const float
   };
   if (precision == BPX_EXACT) {
     if (int rc = products_impl(c, d_A, d_B, M, N, K, h, precision, ws, ws_bytes, products, nullptr, &o, d_info,
-                               S(stream), true))
+                               S(stream), true, true))
       return rc;
     if (int rc = join()) return rc;
     return peel_exact_impl(c, reinterpret_cast<const int32_t*>(products), N, h, d_C, &o, ws, ws_bytes, S(stream), K);
   }
   if (int rc = products_impl(c, d_A, d_B, M, N, K, h, precision, ws, ws_bytes, products,
-                             o.direct_write ? d_C : nullptr, &o, d_info, S(stream)))
+                             o.direct_write ? d_C : nullptr, &o, d_info, S(stream), false, true))
     return rc;
   if (int rc = join()) return rc;
   return peel_impl(c, products, N, h, d_C, o.direct_write, &o, ws, S(stream));

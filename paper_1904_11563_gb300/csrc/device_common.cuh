@@ -128,6 +128,52 @@ struct GJob {
   int enc_sblocks;  // grouped encode: CTAs of the job (kEncGroupRows row blocks each, every k-chunk)
 };
 
+// Chained launches (programmatic dependent launch).  Inside one library call
+// each kernel may be placed as soon as the CTAs of the one before it in the
+// stream have ended, and every kernel of the chain waits for that one,
+// complete and visible, before it touches memory another kernel writes: the
+// launch and the kernel's own set-up overlap the previous one's end.  Only the
+// schedule (one CTA) lets its successor in earlier.  (Letting every successor
+// in at a kernel's start made the tiny FP32 call slower, 37 against 19 us: its
+// GEMM's CTAs then pile up on the few SMs that have room.)  Without the launch
+// attribute these are no-ops.
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// Staging that needs nothing of the schedule launched right before it (early):
+// the schedule lets it in only after its own wait, so everything older than
+// the schedule is complete; the grid's last CTA waits at its end, so that the
+// staging does not count as complete before the schedule.
+__device__ __forceinline__ void chain_begin_staging(bool early) {
+  if (!early) chain_wait();
+}
+__device__ __forceinline__ void chain_end_staging(bool early) {
+  if (early && blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1) chain_wait();
+}
+
+// Whether this thread's launches are chained (set by the entry points).
+bool& chain_on();
+struct ChainScope {
+  explicit ChainScope(bool on) : was(chain_on()) { chain_on() = on; }
+  ~ChainScope() { chain_on() = was; }
+  bool was;
+};
+
+// Launches a kernel, as the next link of a chain when one is on.
+template <typename... P, typename... A>
+cudaError_t launch(void (*kern)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = chain_on() ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
 // Index of the last entry of the ascending array bases[0 .. n) that is <= x:
 // the job of a grouped launch's CTA x.  The bases of one stage sit in a
 // dense array (8 bytes a job, cached by every SM) rather than in the job
@@ -217,8 +263,9 @@ __host__ __device__ inline float scale_pow2(float x, int e) {
 }
 cudaError_t launch_encode_f16(const DevGraph& g, const DevPlan& p, const float* A, int M, int K, int h,
                               void* a_hi, void* a_lo, int32_t* a_exp, cudaStream_t st);
-cudaError_t launch_b_f16(const float* B, int K, int N, void* b_hi, void* b_lo, uint32_t* b_max, int32_t* b_exp,
-                         cudaStream_t st);
+// (clears a_exp for the K-chunked encode of high-degree codes)
+cudaError_t launch_b_f16(const DevGraph& g, int h, const float* B, int K, int N, void* b_hi, void* b_lo,
+                         uint32_t* b_max, int32_t* b_exp, int32_t* a_exp, cudaStream_t st, bool early);
 // gemm_config is a tile configuration the GEMM kernels have (tile codes 3,
 // 4, 7 and 8 do not exist; negative values are invalid).
 bool gemm_config_ok(int config);
@@ -255,13 +302,15 @@ cudaError_t launch_encode_f32(const DevGraph& g, const DevPlan& p, const float* 
                               int h, float* out, cudaStream_t st);
 cudaError_t launch_encode_split(const DevGraph& g, const DevPlan& p, const float* A, int M, int K,
                                 int h, void* a_hi, void* a_lo, cudaStream_t st);
-cudaError_t launch_b_split(const float* B, int K, int N, void* b_hi, void* b_lo, cudaStream_t st);
+// (early, here and below: launched right after the schedule of the same call, see chain_begin_staging)
+cudaError_t launch_b_split(const float* B, int K, int N, void* b_hi, void* b_lo, cudaStream_t st, bool early);
 // FP32 operands for the tensor cores: the coded rows / B^T as three bf16
 // parts whose sum is the FP32 value; flag (a plan counter) is raised when an
 // element's parts would not hold it.
 cudaError_t launch_encode_parts(const DevGraph& g, const DevPlan& p, const float* A, int M, int K, int h,
                                 void* const a[3], cudaStream_t st);
-cudaError_t launch_b_parts(const DevPlan& p, const float* B, int K, int N, void* const b[3], cudaStream_t st);
+cudaError_t launch_b_parts(const DevPlan& p, const float* B, int K, int N, void* const b[3], cudaStream_t st,
+                           bool early);
 // The FP32 encode and GEMM on the CUDA cores when that flag is up (else both return at once).
 cudaError_t launch_encode_f32_flagged(const DevGraph& g, const DevPlan& p, const float* A, int M, int K, int h,
                                       float* out, cudaStream_t st);
@@ -273,7 +322,7 @@ cudaError_t launch_gemm_f32_tc(const DevPlan& p, void* const a[3], void* const b
 // MXFP8 staging (E4M3 data + UE8M0 scales in the GEMM's per-stage order) and GEMM.
 cudaError_t launch_encode_mx(const DevGraph& g, const DevPlan& p, const float* A, int M, int K, int h,
                              void* out, void* sfa, cudaStream_t st);
-cudaError_t launch_b_mx(const float* B, int K, int N, void* bt, void* sfb, cudaStream_t st);
+cudaError_t launch_b_mx(const float* B, int K, int N, void* bt, void* sfb, cudaStream_t st, bool early);
 cudaError_t launch_gemm_mx(const DevPlan& p, const void* a8, const void* sfa, const void* b8, const void* sfb,
                            int num_cells, int N, int K, int h, float* products, float* C_direct, int config,
                            int32_t* info_out, cudaStream_t st);
@@ -300,10 +349,10 @@ cudaError_t launch_gemm_tc(const DevGraph& g, const DevPlan& p, const void* a_hi
 // position + coded A digit planes), digit-product GEMM and exact peel.
 // (launch_exact_b also clears the h words of amax_a; launch_exact_a follows it)
 cudaError_t launch_exact_b(const float* B, int K, int N, const ExactParams& P, uint32_t* amax_b, uint32_t* amax_a,
-                           int h, void* bt, cudaStream_t st);
+                           int h, void* bt, cudaStream_t st, bool early);
 // max |B| per column as float bits; clears `clear` words of `cleared` besides.
 cudaError_t launch_colmax(const float* B, int K, int N, uint32_t* bmax, uint32_t* cleared, long long clear,
-                          cudaStream_t st);
+                          cudaStream_t st, bool early);
 // src_digits: the workspace's int8 source-digit region (ex_src) when the
 // layout has one, else nullptr.
 cudaError_t launch_exact_a(const DevGraph& g, const DevPlan& p, const float* A, int M, int K, int h,
@@ -321,7 +370,7 @@ cudaError_t launch_peel_exact(const DevPlan& p, const ExactParams& P, int sigma,
 // blocks, bf16 hi (+ lo)), products GEMM over each cell's terms, and the peel
 // over strided h x w blocks of C.
 cudaError_t launch_stage_2d(const DevGraph& g, const float* A, const float* B, int M, int N, int K, int h, int w,
-                            void* a_hi, void* a_lo, void* b_hi, void* b_lo, cudaStream_t st);
+                            void* a_hi, void* a_lo, void* b_hi, void* b_lo, cudaStream_t st, bool early);
 cudaError_t launch_gemm_2d(const DevGraph& g, const DevPlan& p, const void* a_hi, const void* a_lo, const void* b_hi,
                            const void* b_lo, int N, int K, int h, int w, bool split3, float* products,
                            float* C_direct, int config, int32_t* info_out, cudaStream_t st);

@@ -90,6 +90,7 @@ __device__ __forceinline__ float warp_max(float m) {
 __global__ void __launch_bounds__(256) exact_amax_a_kernel(const float* __restrict__ A, int M, int K, int h,
                                                            uint32_t* amax) {
   __shared__ float red[8];
+  chain_wait();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float m = 0.f;
   for (long long r = blockIdx.x + static_cast<long long>(blockIdx.y * 8 + warp) * h; r < M;
@@ -118,6 +119,7 @@ __global__ void __launch_bounds__(256)
 exact_b_digits_kernel(const float* __restrict__ B, int K, int N, const uint32_t* __restrict__ amax_b, int w,
                       int bits, int Kp, bool pairs, __nv_bfloat16* bt) {
   __shared__ float tile[64][65];
+  chain_wait();
   const int n0 = blockIdx.x * 64, k0 = blockIdx.y * 64;
   {
     const int c4 = threadIdx.x & 15, r0 = threadIdx.x >> 4;
@@ -165,6 +167,7 @@ template <int S>
 __global__ void __launch_bounds__(kExThreads)
 exact_a_digits_kernel(DevGraph g, DevPlan p, const float* __restrict__ A, int M, int K, int h,
                       const uint32_t* __restrict__ amax_a, int w, int bits, int Kp, __nv_bfloat16* out) {
+  chain_wait();
   const int tpr = enc_threads_per_row(Kp);
   const int row = blockIdx.x * (kExThreads / tpr) + threadIdx.x / tpr;
   const int nsurv = p.ctr[CTR_NSURV];
@@ -218,6 +221,7 @@ template <int S>
 __global__ void __launch_bounds__(256)
 exact_src_digits_kernel(const float* __restrict__ A, int M, int K, int h, const uint32_t* __restrict__ amax_a,
                         int w, int bits, int Kp, long long src_rows, uint8_t* out) {
+  chain_wait();
   const long long c = static_cast<long long>(blockIdx.x) * 256 + threadIdx.x;  // (row, 8-column chunk)
   const int per_row = Kp / 8;
   const long long r = c / per_row;
@@ -259,6 +263,7 @@ template <int S>
 __global__ void __launch_bounds__(kExThreads)
 exact_a_digits_src_kernel(DevGraph g, DevPlan p, const uint8_t* __restrict__ src_digits, int M, int h, int Kp,
                           int K, int w, __nv_bfloat16* out) {
+  chain_wait();
   const int tpr = enc_threads_per_row(Kp);
   const int row = blockIdx.x * (kExThreads / tpr) + threadIdx.x / tpr;
   const int nsurv = p.ctr[CTR_NSURV];
@@ -321,6 +326,7 @@ __global__ void __launch_bounds__(256)
 exact_peel_kernel(DevPlan p, const int32_t* __restrict__ planes, long long plane_stride, long long* C64, float* C,
                   const uint32_t* __restrict__ amax_a, const uint32_t* __restrict__ amax_b, int N, int h, int w,
                   int e_base, long long nv, int chunk) {
+  chain_wait();
   if (p.ctr[CTR_PLAN] != kPlanReady) {  // no schedule has planned this workspace: refuse, write nothing
     if (blockIdx.x == 0 && threadIdx.x == 0) {
       atomicExch(&p.info[BPX_INFO_DEVICE_ERR], BPX_ERR_INVAL);
@@ -407,6 +413,7 @@ __global__ void __launch_bounds__(kExNarrowThreads, 2)
 exact_peel_narrow_kernel(DevPlan p, const int32_t* __restrict__ planes, long long plane_stride, long long* C64,
                          float* C, const uint32_t* __restrict__ amax_a, const uint32_t* __restrict__ amax_b, int N,
                          int h, int w, int e_base, long long nv, int chunk) {
+  chain_wait();
   if (p.ctr[CTR_PLAN] != kPlanReady) {  // no schedule has planned this workspace: refuse, write nothing
     if (blockIdx.x == 0 && threadIdx.x == 0) {
       atomicExch(&p.info[BPX_INFO_DEVICE_ERR], BPX_ERR_INVAL);
@@ -521,24 +528,23 @@ exact_peel_narrow_kernel(DevPlan p, const int32_t* __restrict__ planes, long lon
 }  // namespace
 
 cudaError_t launch_exact_b(const float* B, int K, int N, const ExactParams& P, uint32_t* amax_b, uint32_t* amax_a,
-                           int h, void* bt, cudaStream_t st) {
+                           int h, void* bt, cudaStream_t st, bool early) {
   // (also clears the row positions' words for launch_exact_a)
-  cudaError_t e = launch_colmax(B, K, N, amax_b, amax_a, h, st);
+  cudaError_t e = launch_colmax(B, K, N, amax_b, amax_a, h, st, early);
   if (e != cudaSuccess) return e;
   const dim3 grid((N + 63) / 64, P.Kp / 64);
   auto* out = static_cast<__nv_bfloat16*>(bt);
   auto go = [&](auto kern) {
-    kern<<<grid, 256, 0, st>>>(B, K, N, amax_b, P.w, P.bits, P.Kp, P.step == 2, out);
+    return launch(kern, grid, 256, 0, st, B, K, N, amax_b, P.w, P.bits, P.Kp, P.step == 2, out);
   };
   switch (P.S) {
-    case 3: go(exact_b_digits_kernel<3>); break;
-    case 4: go(exact_b_digits_kernel<4>); break;
-    case 5: go(exact_b_digits_kernel<5>); break;
-    case 6: go(exact_b_digits_kernel<6>); break;
-    case 8: go(exact_b_digits_kernel<8>); break;
+    case 3: return go(exact_b_digits_kernel<3>);
+    case 4: return go(exact_b_digits_kernel<4>);
+    case 5: return go(exact_b_digits_kernel<5>);
+    case 6: return go(exact_b_digits_kernel<6>);
+    case 8: return go(exact_b_digits_kernel<8>);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 cudaError_t launch_exact_a(const DevGraph& g, const DevPlan& p, const float* A, int M, int K, int h,
@@ -549,8 +555,9 @@ cudaError_t launch_exact_a(const DevGraph& g, const DevPlan& p, const float* A, 
   const int positions = std::min(h, std::max(M, 1));
   const long long rows_a = (static_cast<long long>(M) + h - 1) / h;
   const long long parts = std::max(1LL, std::min((rows_a + 7) / 8, (4LL * num_sms() + positions - 1) / positions));
-  exact_amax_a_kernel<<<dim3(h, static_cast<unsigned>(std::min(parts, 65535LL))), 256, 0, st>>>(A, M, K, h, amax_a);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  e = launch(exact_amax_a_kernel, dim3(h, static_cast<unsigned>(std::min(parts, 65535LL))), 256, 0, st, A, M, K, h,
+             amax_a);
+  if (e != cudaSuccess) return e;
   const long long rows = static_cast<long long>(g.num_cells) * h;
   const dim3 grid(static_cast<unsigned>(enc_row_blocks(rows, P.Kp)), enc_k_chunks(P.Kp));
   auto* out = static_cast<__nv_bfloat16*>(a_planes);
@@ -562,40 +569,30 @@ cudaError_t launch_exact_a(const DevGraph& g, const DevPlan& p, const float* A, 
     if ((chunks + 255) / 256 > 0x7fffffffLL) return cudaErrorInvalidValue;
     const unsigned sg = static_cast<unsigned>((chunks + 255) / 256);
     auto* sd = static_cast<uint8_t*>(src_digits);
+    auto cut_sum = [&](auto cut, auto sum) {
+      const cudaError_t r = launch(cut, dim3(sg), 256, 0, st, A, M, K, h, amax_a, P.w, P.bits, P.Kp, src_rows, sd);
+      if (r != cudaSuccess) return r;
+      return launch(sum, grid, kExThreads, 0, st, g, p, sd, M, h, P.Kp, K, P.w, out);
+    };
     switch (P.S) {
-      case 4:
-        exact_src_digits_kernel<4><<<sg, 256, 0, st>>>(A, M, K, h, amax_a, P.w, P.bits, P.Kp, src_rows, sd);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        exact_a_digits_src_kernel<4><<<grid, kExThreads, 0, st>>>(g, p, sd, M, h, P.Kp, K, P.w, out);
-        break;
-      case 5:
-        exact_src_digits_kernel<5><<<sg, 256, 0, st>>>(A, M, K, h, amax_a, P.w, P.bits, P.Kp, src_rows, sd);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        exact_a_digits_src_kernel<5><<<grid, kExThreads, 0, st>>>(g, p, sd, M, h, P.Kp, K, P.w, out);
-        break;
-      case 6:
-        exact_src_digits_kernel<6><<<sg, 256, 0, st>>>(A, M, K, h, amax_a, P.w, P.bits, P.Kp, src_rows, sd);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        exact_a_digits_src_kernel<6><<<grid, kExThreads, 0, st>>>(g, p, sd, M, h, P.Kp, K, P.w, out);
-        break;
-      case 8:
-        exact_src_digits_kernel<8><<<sg, 256, 0, st>>>(A, M, K, h, amax_a, P.w, P.bits, P.Kp, src_rows, sd);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        exact_a_digits_src_kernel<8><<<grid, kExThreads, 0, st>>>(g, p, sd, M, h, P.Kp, K, P.w, out);
-        break;
+      case 4: return cut_sum(exact_src_digits_kernel<4>, exact_a_digits_src_kernel<4>);
+      case 5: return cut_sum(exact_src_digits_kernel<5>, exact_a_digits_src_kernel<5>);
+      case 6: return cut_sum(exact_src_digits_kernel<6>, exact_a_digits_src_kernel<6>);
+      case 8: return cut_sum(exact_src_digits_kernel<8>, exact_a_digits_src_kernel<8>);
       default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
   }
+  auto go = [&](auto kern) {
+    return launch(kern, grid, kExThreads, 0, st, g, p, A, M, K, h, amax_a, P.w, P.bits, P.Kp, out);
+  };
   switch (P.S) {
-    case 3: exact_a_digits_kernel<3><<<grid, kExThreads, 0, st>>>(g, p, A, M, K, h, amax_a, P.w, P.bits, P.Kp, out); break;
-    case 4: exact_a_digits_kernel<4><<<grid, kExThreads, 0, st>>>(g, p, A, M, K, h, amax_a, P.w, P.bits, P.Kp, out); break;
-    case 5: exact_a_digits_kernel<5><<<grid, kExThreads, 0, st>>>(g, p, A, M, K, h, amax_a, P.w, P.bits, P.Kp, out); break;
-    case 6: exact_a_digits_kernel<6><<<grid, kExThreads, 0, st>>>(g, p, A, M, K, h, amax_a, P.w, P.bits, P.Kp, out); break;
-    case 8: exact_a_digits_kernel<8><<<grid, kExThreads, 0, st>>>(g, p, A, M, K, h, amax_a, P.w, P.bits, P.Kp, out); break;
+    case 3: return go(exact_a_digits_kernel<3>);
+    case 4: return go(exact_a_digits_kernel<4>);
+    case 5: return go(exact_a_digits_kernel<5>);
+    case 6: return go(exact_a_digits_kernel<6>);
+    case 8: return go(exact_a_digits_kernel<8>);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 cudaError_t launch_peel_exact(const DevPlan& p, const ExactParams& P, int sigma,
@@ -613,9 +610,8 @@ cudaError_t launch_peel_exact(const DevPlan& p, const ExactParams& P, int sigma,
   const int chunk = narrow ? static_cast<int>((nv + slots - 1) / slots) : peel_chunk_for(nv, ctas);
   const unsigned grid = static_cast<unsigned>((nv + chunk - 1) / chunk);
   auto go = [&](auto kern) {
-    kern<<<grid, narrow ? kExNarrowThreads : 256, 0, st>>>(p, planes, plane_stride, C64, C, amax_a, amax_b, N, h, w,
-                                                           e_base, nv, chunk);
-    return cudaGetLastError();
+    return launch(kern, dim3(grid), narrow ? kExNarrowThreads : 256, 0, st, p, planes, plane_stride, C64, C, amax_a,
+                  amax_b, N, h, w, e_base, nv, chunk);
   };
   switch (P.np) {
     case 3: return narrow ? go(exact_peel_narrow_kernel<3, 3>) : go(exact_peel_kernel<3>);

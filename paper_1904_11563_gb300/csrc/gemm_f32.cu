@@ -164,6 +164,7 @@ __device__ __forceinline__ void gemm_f32_tile(const DevPlan& p, const float* __r
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_f32_kernel(DevPlan p, const float* __restrict__ Ac, const float* __restrict__ B, int N, int K, int h,
                 float* products, float* C_direct) {
+  chain_wait();
   const long long Mc = static_cast<long long>(p.ctr[CTR_NSURV]) * h;
   const long long m0 = static_cast<long long>(blockIdx.y) * BM;
   if (m0 < Mc) gemm_f32_tile(p, Ac, B, N, K, h, products, C_direct, Mc, m0, blockIdx.x * BN);
@@ -183,6 +184,7 @@ gemm_f32_small_kernel(DevPlan p, const float* __restrict__ Ac, const float* __re
   constexpr int kThr = (SM / TM) * (SN / 4), kLd = kSmallBK + 4;
   __shared__ __align__(16) float As[kSmallStages][SM][kLd];
   __shared__ __align__(16) float Bs[kSmallStages][kSmallBK][SN];
+  chain_wait();
   const long long Mc = static_cast<long long>(p.ctr[CTR_NSURV]) * h;
   const long long m0 = static_cast<long long>(blockIdx.y) * SM;
   if (m0 >= Mc) return;
@@ -257,8 +259,8 @@ template <int SM, int SN, int TM>
 cudaError_t launch_small(const DevPlan& p, const float* a_coded, const float* B, long long rows, int N, int K, int h,
                          float* products, float* C_direct, cudaStream_t st) {
   const dim3 grid((N + SN - 1) / SN, static_cast<unsigned>((rows + SM - 1) / SM));
-  gemm_f32_small_kernel<SM, SN, TM><<<grid, (SM / TM) * (SN / 4), 0, st>>>(p, a_coded, B, N, K, h, products, C_direct);
-  return cudaGetLastError();
+  return launch(gemm_f32_small_kernel<SM, SN, TM>, grid, (SM / TM) * (SN / 4), 0, st, p, a_coded, B, N, K, h, products,
+                C_direct);
 }
 
 // Behind the tensor-core FP32 GEMM: one CTA per SM walks the tiles when the
@@ -266,6 +268,7 @@ cudaError_t launch_small(const DevPlan& p, const float* a_coded, const float* B,
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_f32_flagged_kernel(DevPlan p, const float* __restrict__ Ac, const float* __restrict__ B, int N, int K, int h,
                         float* products, float* C_direct) {
+  chain_wait();
   if (p.ctr[CTR_F32_SIMT] == 0) return;
   const long long Mc = static_cast<long long>(p.ctr[CTR_NSURV]) * h;
   const long long n_tiles = (N + BN - 1) / BN, tiles = (Mc + BM - 1) / BM * n_tiles;
@@ -286,8 +289,8 @@ cudaError_t launch_gemm_f32_flagged(const DevGraph& g, const DevPlan& p, const f
   cudaError_t e = cudaFuncSetAttribute(gemm_f32_flagged_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(smem));
   if (e != cudaSuccess) return e;
-  gemm_f32_flagged_kernel<<<num_sms(), kThreads, smem, st>>>(p, a_coded, B, N, K, h, products, C_direct);
-  return cudaGetLastError();
+  return launch(gemm_f32_flagged_kernel, dim3(num_sms()), kThreads, smem, st, p, a_coded, B, N, K, h, products,
+                C_direct);
 }
 
 // a_coded: the FP32 coded rows of the surviving cells (encode pass output),
@@ -315,8 +318,7 @@ cudaError_t launch_gemm_f32(const DevGraph& g, const DevPlan& p, const float* a_
                                        static_cast<int>(smem));
   if (e != cudaSuccess) return e;
   dim3 grid((N + BN - 1) / BN, static_cast<unsigned>((rows + BM - 1) / BM));
-  gemm_f32_kernel<<<grid, kThreads, smem, st>>>(p, a_coded, B, N, K, h, products, C_direct);
-  return cudaGetLastError();
+  return launch(gemm_f32_kernel, grid, kThreads, smem, st, p, a_coded, B, N, K, h, products, C_direct);
 }
 
 }  // namespace bpx

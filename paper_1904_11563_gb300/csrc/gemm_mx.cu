@@ -104,10 +104,6 @@ gemm_mx_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   __shared__ uint32_t tmem_base_sh;
   __shared__ volatile int abort_flag;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int Mc = P.ctr[CTR_NSURV] * P.h;
-  const int m_tiles = (Mc + BM - 1) / BM;
-  const int m_units = m_tiles;
-  const int num_tiles = m_units * P.n_tiles;
   const int k_blocks = P.K / kMxBK;
   const int KS = k_blocks;
   const int cid = static_cast<int>(blockIdx.x);
@@ -135,6 +131,12 @@ gemm_mx_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   __syncthreads();
   fence_after();
   const uint32_t tmem_base = tmem_base_sh;
+
+  chain_wait();  // the plan and the staged operands
+  const int Mc = P.ctr[CTR_NSURV] * P.h;
+  const int m_tiles = (Mc + BM - 1) / BM;
+  const int m_units = m_tiles;
+  const int num_tiles = m_units * P.n_tiles;
 
   // (m, n) of tile t in bands of m-tiles
   auto tile_mn = [&](long long t, int& m, int& n) {
@@ -330,10 +332,6 @@ gemm_mx_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
   __shared__ uint32_t tmem_base_sh;
   __shared__ volatile int abort_flag;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int Mc = P.ctr[CTR_NSURV] * P.h;
-  const int m_tiles = (Mc + BM - 1) / BM;
-  const int m_units = (m_tiles + 1) / 2;
-  const int num_tiles = m_units * P.n_tiles;
   const int k_blocks = P.K / kMxBK;
   const int KS = k_blocks;
   const uint32_t rank = cluster_rank();
@@ -363,6 +361,12 @@ gemm_mx_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
   cluster_sync();  // the peer's barriers exist before any copy or commit lands
   fence_after();
   const uint32_t tmem_base = tmem_base_sh;
+
+  chain_wait();  // the plan and the staged operands
+  const int Mc = P.ctr[CTR_NSURV] * P.h;
+  const int m_tiles = (Mc + BM - 1) / BM;
+  const int m_units = (m_tiles + 1) / 2;
+  const int num_tiles = m_units * P.n_tiles;
 
   // (pair unit, n) of tile t in bands of pair units; this CTA's m-tile
   auto tile_mn = [&](long long t, int& m, int& n) {
@@ -589,7 +593,7 @@ cudaError_t launch_gemm_mx(const DevPlan& p, const void* a8, const void* sfa, co
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = smem2;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 2;
     attr[0].val.clusterDim.y = 1;
@@ -604,6 +608,9 @@ cudaError_t launch_gemm_mx(const DevPlan& p, const void* a8, const void* sfa, co
     }
     resident = std::max(1, resident - (reserved_sms() + 1) / 2);
     cfg.gridDim = dim3(2 * static_cast<int>(std::min<long long>(pairs, resident)));
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.numAttrs = chain_on() ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kern, ma, mb, msa, msb, P);
   }
   const size_t smem = static_cast<size_t>(kMxStages) * kMxStageBytes + 1024;
@@ -613,8 +620,7 @@ cudaError_t launch_gemm_mx(const DevPlan& p, const void* a8, const void* sfa, co
   if (e != cudaSuccess) return e;
   const int grid = static_cast<int>(std::min<long long>(tiles, std::max(1, num_sms() - reserved_sms())));
   if (grid <= 0) return cudaSuccess;
-  gemm_mx_kernel<<<grid, kThreads, smem, st>>>(ma, mb, P);
-  return cudaGetLastError();
+  return launch(gemm_mx_kernel, dim3(grid), kThreads, smem, st, ma, mb, P);
 }
 
 }  // namespace bpx

@@ -242,19 +242,9 @@ gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ t
   __shared__ uint32_t tmem_base_sh;
   __shared__ volatile int abort_flag;
 
-  // FP32 operands with an element the three parts cannot hold: the CUDA-core
-  // kernel behind this launch computes the products instead
-  if (kParts == 3 && single.ctr[CTR_F32_SIMT] != 0) return;
   const TcJob* jobs = table ? table : &single;
   const bool grouped = table != nullptr;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // A single job reads its surviving row count once and walks live tiles only.
-  const int live_mc = grouped ? -1 : single.ctr[CTR_NSURV] * single.h;
-  if (!grouped && !k2D) {
-    int units = (live_mc + BM - 1) / BM;
-    if (kPair) units = (units + 1) / 2;
-    total_tiles = static_cast<long long>(units) * single.n_tiles * (kExact ? single.ex_np : 1);
-  }
   constexpr int kClusterShift = kQuad ? 2 : kPair ? 1 : 0;
   const uint32_t crank = kPair ? cluster_rank() : 0u;
   const uint32_t rank = crank & 1u, leader = crank & ~1u;  // of the pair; its even CTA
@@ -296,6 +286,18 @@ gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ t
   if (kPair) cluster_sync();  // the peer's barriers exist before any of its copies or commits land
   fence_after();
   const uint32_t tmem_base = tmem_base_sh;
+
+  chain_wait();  // the plan and the staged operands
+  // A single job reads its surviving row count once and walks live tiles only.
+  const int live_mc = grouped ? -1 : single.ctr[CTR_NSURV] * single.h;
+  if (!grouped && !k2D) {
+    int units = (live_mc + BM - 1) / BM;
+    if (kPair) units = (units + 1) / 2;
+    total_tiles = static_cast<long long>(units) * single.n_tiles * (kExact ? single.ex_np : 1);
+    // FP32 operands with an element the three parts cannot hold: the CUDA-core
+    // kernel behind this launch computes the products instead
+    if (kParts == 3 && single.ctr[CTR_F32_SIMT] != 0) total_tiles = 0;
+  }
 
   if (warp == 0) {
     if (lane == 0) {
@@ -728,14 +730,13 @@ cudaError_t launch_variant(const TcJob& single, const TcJob* table, int njobs, l
   if (total_tiles <= 0) return cudaSuccess;
   if (kPair == 0) {
     const int grid = static_cast<int>(std::min<long long>(total_tiles, std::max(1, num_sms() - reserved_sms())));
-    kern<<<grid, kThreads, smem, st>>>(single, table, njobs, total_tiles, group, seg_kb);
-    return cudaGetLastError();
+    return launch(kern, dim3(grid), kThreads, smem, st, single, table, njobs, total_tiles, group, seg_kb);
   }
   cudaLaunchConfig_t cfg = {};
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   constexpr int kCtas = kPair == 4 ? 4 : 2;
   attr[0].val.clusterDim.x = kCtas;
@@ -753,6 +754,9 @@ cudaError_t launch_variant(const TcJob& single, const TcJob* table, int njobs, l
   resident = std::max(1, resident - (reserved_sms() + kCtas - 1) / kCtas);
   const int clusters = static_cast<int>(std::min<long long>(total_tiles, resident));
   cfg.gridDim = dim3(kCtas * clusters);
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.numAttrs = chain_on() ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kern, single, table, njobs, total_tiles, group, seg_kb);
 }
 

@@ -285,6 +285,7 @@ template <int kB, bool kGather>
 __global__ void __launch_bounds__(kPeelThreads)
 peel_kernel(DevPlan p, const float* __restrict__ P, float* C, long long nv, int chunk, int first_wave,
             int compensate_depth) {
+  chain_wait();
   if (p.ctr[CTR_PLAN] != kPlanReady) {  // no schedule has planned this workspace: refuse, write nothing
     if (blockIdx.x == 0 && threadIdx.x == 0) {
       atomicExch(&p.info[BPX_INFO_DEVICE_ERR], BPX_ERR_INVAL);
@@ -396,8 +397,8 @@ cudaError_t launch_peel(const DevGraph& g, const DevPlan& p, const float* P, flo
   };
   auto run = [&](auto kern, size_t smem, long long chunk) -> cudaError_t {
     const unsigned grid = static_cast<unsigned>((nv + chunk - 1) / chunk);
-    kern<<<grid, kPeelThreads, smem, st>>>(p, P, C, nv, static_cast<int>(chunk), first_wave, compensate_depth);
-    return cudaGetLastError();
+    return launch(kern, dim3(grid), kPeelThreads, smem, st, p, P, C, nv, static_cast<int>(chunk), first_wave,
+                  compensate_depth);
   };
   // The gathered form for tall codes, when one position's rows (at most
   // sigma) over the CTA's columns fit a round of the term buffer.

@@ -128,12 +128,14 @@ template <int kMode>
 __global__ void __launch_bounds__(kEncThreads)
 encode_kernel(DevGraph g, DevPlan p, const float* __restrict__ A, int M, int K, int h,
               float* out_f32, __nv_bfloat16* out_hi, __nv_bfloat16* out_lo) {
+  chain_wait();
   encode_body<kMode>(g, p, A, M, K, h, out_f32, out_hi, out_lo, blockIdx.x, blockIdx.y);
 }
 
 __global__ void __launch_bounds__(kEncThreads)
 encode_parts_kernel(DevGraph g, DevPlan p, const float* __restrict__ A, int M, int K, int h, __nv_bfloat16* o1,
                     __nv_bfloat16* o2, __nv_bfloat16* o3) {
+  chain_wait();
   encode_body<3>(g, p, A, M, K, h, nullptr, o1, o2, blockIdx.x, blockIdx.y, o3);
 }
 
@@ -142,6 +144,7 @@ encode_parts_kernel(DevGraph g, DevPlan p, const float* __restrict__ A, int M, i
 __global__ void __launch_bounds__(kEncThreads)
 encode_f32_flagged_kernel(DevGraph g, DevPlan p, const float* __restrict__ A, int M, int K, int h, float* out,
                           long long row_blocks, long long blocks) {
+  chain_wait();
   if (p.ctr[CTR_F32_SIMT] == 0) return;
   for (long long b = blockIdx.x; b < blocks; b += gridDim.x) {
     const long long kc = b / row_blocks;
@@ -208,13 +211,17 @@ __device__ __forceinline__ bool b_split_body(const float* __restrict__ B, int K,
 
 __global__ void __launch_bounds__(256)
 b_parts_kernel(DevPlan p, const float* __restrict__ B, int K, int N, __nv_bfloat16* o1, __nv_bfloat16* o2,
-               __nv_bfloat16* o3) {
+               __nv_bfloat16* o3, bool early) {
+  chain_begin_staging(early);
   if (b_split_body<true>(B, K, N, o1, o2, blockIdx.x, blockIdx.y, o3)) p.ctr[CTR_F32_SIMT] = 1;
+  chain_end_staging(early);
 }
 
 __global__ void __launch_bounds__(256)
-b_split_kernel(const float* __restrict__ B, int K, int N, __nv_bfloat16* bt_hi, __nv_bfloat16* bt_lo) {
+b_split_kernel(const float* __restrict__ B, int K, int N, __nv_bfloat16* bt_hi, __nv_bfloat16* bt_lo, bool early) {
+  chain_begin_staging(early);
   b_split_body(B, K, N, bt_hi, bt_lo, blockIdx.x, blockIdx.y);
+  chain_end_staging(early);
 }
 
 // Grouped launches: a flat grid over every job's CTAs; each CTA finds its job
@@ -304,6 +311,9 @@ constexpr int kF16Keep = 4;
 // Codes with at least this many sources per cell on average take the
 // K-chunked form (below).
 constexpr int kF16ChunkedDegree = 4;
+bool encode_f16_chunked(const DevGraph& g) {
+  return static_cast<long long>(g.num_edges) >= kF16ChunkedDegree * static_cast<long long>(g.num_cells);
+}
 
 __device__ __forceinline__ void coded_chunk(const DevGraph& g, const float* __restrict__ A, int M, int K, int h,
                                             int e0, int e1, int j, int k8, float (&acc)[8]) {
@@ -341,6 +351,7 @@ __global__ void __launch_bounds__(kF16Threads)
 encode_f16_kernel(DevGraph g, DevPlan p, const float* __restrict__ A, int M, int K, int h, __half* out_hi,
                   __half* out_lo, int32_t* a_exp) {
   __shared__ float red[kF16Threads / 32];
+  chain_wait();
   const int row = blockIdx.x;  // coded row, compacted order
   if (row >= p.ctr[CTR_NSURV] * h) return;
   const int ci = row / h, j = row - ci * h;
@@ -426,6 +437,7 @@ encode_f16_kernel(DevGraph g, DevPlan p, const float* __restrict__ A, int M, int
 __global__ void __launch_bounds__(kEncThreads)
 encode_f16_sum_kernel(DevGraph g, DevPlan p, const float* __restrict__ A, int M, int K, int h, uint16_t* out_hi,
                       uint16_t* out_lo, uint32_t* row_max) {
+  chain_wait();
   const int tpr = enc_threads_per_row(K);
   const int row = blockIdx.x * (kEncThreads / tpr) + threadIdx.x / tpr;
   const bool live = row < p.ctr[CTR_NSURV] * h;
@@ -454,6 +466,7 @@ encode_f16_sum_kernel(DevGraph g, DevPlan p, const float* __restrict__ A, int M,
 }
 
 __global__ void __launch_bounds__(256) encode_f16_exp_kernel(DevPlan p, int h, int32_t* a_exp) {
+  chain_wait();
   const long long row = static_cast<long long>(blockIdx.x) * 256 + threadIdx.x;
   if (row < static_cast<long long>(p.ctr[CTR_NSURV]) * h)
     a_exp[row] = f16_scale_exp(__uint_as_float(static_cast<uint32_t>(a_exp[row])));
@@ -461,6 +474,7 @@ __global__ void __launch_bounds__(256) encode_f16_exp_kernel(DevPlan p, int h, i
 
 __global__ void __launch_bounds__(256)
 encode_f16_rescale_kernel(DevPlan p, int K, int h, __half* out_hi, __half* out_lo, const int32_t* __restrict__ a_exp) {
+  chain_wait();
   const long long c = static_cast<long long>(blockIdx.x) * 256 + threadIdx.x;  // 8-element chunk
   const int per_row = K / 8;
   const long long row = c / per_row;
@@ -482,17 +496,20 @@ encode_f16_rescale_kernel(DevPlan p, int K, int h, __half* out_hi, __half* out_l
 // row phases a CTA), each CTA every eighth run of kColRows rows; the partial
 // maxima meet in the first CTA's shared memory, which stores them: no clearing
 // of the words before, no atomics.  HBM-bound when large; N = 1024, K = 4096
-// 40 -> 6 us against 16 CTAs of 256 rows each.  The first CTA of the grid also
-// clears `clear` words for a later kernel.
+// 40 -> 7 us against 16 CTAs of 256 rows each.  The grid also clears `clear`
+// words for a later kernel.
 constexpr int kColRows = 128, kColSplit = 8;
 __global__ void __cluster_dims__(1, kColSplit, 1) __launch_bounds__(256)
-b_colmax_kernel(const float* __restrict__ B, int K, int N, uint32_t* bmax, uint32_t* cleared, long long clear) {
+b_colmax_kernel(const float* __restrict__ B, int K, int N, uint32_t* bmax, uint32_t* cleared, long long clear,
+                bool early) {
   __shared__ float4 red[32][8];
   __shared__ float4 part[kColSplit][8];
+  chain_begin_staging(early);
   const int c4 = threadIdx.x & 7, ph = threadIdx.x >> 3;
   const int n = blockIdx.x * 32 + 4 * c4;
-  if (blockIdx.x == 0 && blockIdx.y == 0)
-    for (long long i = threadIdx.x; i < clear; i += 256) cleared[i] = 0;
+  for (long long i = (blockIdx.x * gridDim.y + blockIdx.y) * 256LL + threadIdx.x; i < clear;
+       i += 256LL * gridDim.x * gridDim.y)
+    cleared[i] = 0;
   float4 m = make_float4(0.f, 0.f, 0.f, 0.f);
   for (int k0 = blockIdx.y * kColRows; n < N && k0 < K; k0 += kColSplit * kColRows) {
     const int k1 = min(K, k0 + kColRows);
@@ -531,6 +548,7 @@ b_colmax_kernel(const float* __restrict__ B, int K, int N, uint32_t* bmax, uint3
     bmax[n + 2] = __float_as_uint(m.z);
     bmax[n + 3] = __float_as_uint(m.w);
   }
+  chain_end_staging(early);
 }
 
 // B (K x N) -> B^T fp16 hi / lo (N x K) under each column's 2^e, through the
@@ -540,6 +558,7 @@ __global__ void __launch_bounds__(256)
 b_split_f16_kernel(const float* __restrict__ B, int K, int N, const uint32_t* __restrict__ bmax, __half* bt_hi,
                    __half* bt_lo, int32_t* b_exp) {
   __shared__ float tile[kTile][kTile + 1];
+  chain_wait();
   const int n0 = blockIdx.x * kTile, k0 = blockIdx.y * kTile;
   {
     const int c4 = threadIdx.x & 15, r0 = threadIdx.x >> 4;
@@ -643,6 +662,7 @@ __device__ __forceinline__ void encode_mx_body(const DevGraph& g, const DevPlan&
 __global__ void __launch_bounds__(kEncThreads)
 encode_mx_kernel(DevGraph g, DevPlan p, const float* __restrict__ A, int M, int K, int h, uint8_t* out,
                  uint8_t* sfa) {
+  chain_wait();
   encode_mx_body(g, p, A, M, K, h, out, sfa, blockIdx.x, blockIdx.y);
 }
 
@@ -650,8 +670,9 @@ encode_mx_kernel(DevGraph g, DevPlan p, const float* __restrict__ A, int M, int 
 // tile and 128-wide K stage: byte 512 t + 16 l + 4 c + j holds column
 // 128 t + 32 c + l, K-run 4 s + j).
 __global__ void __launch_bounds__(256)
-b_mx_kernel(const float* __restrict__ B, int K, int N, uint8_t* bt, uint8_t* sfb) {
+b_mx_kernel(const float* __restrict__ B, int K, int N, uint8_t* bt, uint8_t* sfb, bool early) {
   __shared__ float tile[kTile][kTile + 1];
+  chain_begin_staging(early);
   const int n0 = blockIdx.x * kTile, k0 = blockIdx.y * kTile;
   {
     const int c4 = threadIdx.x & 15, r0 = threadIdx.x >> 4;
@@ -691,6 +712,7 @@ b_mx_kernel(const float* __restrict__ B, int K, int N, uint8_t* bt, uint8_t* sfb
           4 * ((nn & 127) >> 5) + kb] = static_cast<uint8_t>(sbyte);
     }
   }
+  chain_end_staging(early);
 }
 
 }  // namespace
@@ -700,16 +722,14 @@ cudaError_t launch_encode_mx(const DevGraph& g, const DevPlan& p, const float* A
   const long long rows = static_cast<long long>(g.num_cells) * h;
   if (rows == 0 || K == 0) return cudaSuccess;
   dim3 grid(static_cast<unsigned>(enc_row_blocks(rows, K)), static_cast<unsigned>(enc_k_chunks(K)));
-  encode_mx_kernel<<<grid, kEncThreads, 0, st>>>(g, p, A, M, K, h, static_cast<uint8_t*>(out),
-                                                 static_cast<uint8_t*>(sfa));
-  return cudaGetLastError();
+  return launch(encode_mx_kernel, grid, kEncThreads, 0, st, g, p, A, M, K, h, static_cast<uint8_t*>(out),
+                static_cast<uint8_t*>(sfa));
 }
 
-cudaError_t launch_b_mx(const float* B, int K, int N, void* bt, void* sfb, cudaStream_t st) {
+cudaError_t launch_b_mx(const float* B, int K, int N, void* bt, void* sfb, cudaStream_t st, bool early) {
   if (K == 0 || N == 0) return cudaSuccess;
   dim3 grid((N + kTile - 1) / kTile, (K + kTile - 1) / kTile);
-  b_mx_kernel<<<grid, 256, 0, st>>>(B, K, N, static_cast<uint8_t*>(bt), static_cast<uint8_t*>(sfb));
-  return cudaGetLastError();
+  return launch(b_mx_kernel, grid, 256, 0, st, B, K, N, static_cast<uint8_t*>(bt), static_cast<uint8_t*>(sfb), early);
 }
 
 cudaError_t launch_encode_f32(const DevGraph& g, const DevPlan& p, const float* A, int M, int K,
@@ -717,8 +737,7 @@ cudaError_t launch_encode_f32(const DevGraph& g, const DevPlan& p, const float* 
   const long long rows = static_cast<long long>(g.num_cells) * h;
   if (rows == 0 || K == 0) return cudaSuccess;
   dim3 grid(static_cast<unsigned>(enc_row_blocks(rows, K)), static_cast<unsigned>(enc_k_chunks(K)));
-  encode_kernel<0><<<grid, kEncThreads, 0, st>>>(g, p, A, M, K, h, out, nullptr, nullptr);
-  return cudaGetLastError();
+  return launch(encode_kernel<0>, grid, kEncThreads, 0, st, g, p, A, M, K, h, out, nullptr, nullptr);
 }
 
 cudaError_t launch_encode_split(const DevGraph& g, const DevPlan& p, const float* A, int M, int K,
@@ -728,11 +747,7 @@ cudaError_t launch_encode_split(const DevGraph& g, const DevPlan& p, const float
   dim3 grid(static_cast<unsigned>(enc_row_blocks(rows, K)), static_cast<unsigned>(enc_k_chunks(K)));
   auto hi = static_cast<__nv_bfloat16*>(a_hi);
   auto lo = static_cast<__nv_bfloat16*>(a_lo);
-  if (lo)
-    encode_kernel<2><<<grid, kEncThreads, 0, st>>>(g, p, A, M, K, h, nullptr, hi, lo);
-  else
-    encode_kernel<1><<<grid, kEncThreads, 0, st>>>(g, p, A, M, K, h, nullptr, hi, nullptr);
-  return cudaGetLastError();
+  return launch(lo ? encode_kernel<2> : encode_kernel<1>, grid, kEncThreads, 0, st, g, p, A, M, K, h, nullptr, hi, lo);
 }
 
 cudaError_t launch_b_split_group(const GJob* d_jobs, const long long* d_bases, int njobs, long long total_ctas,
@@ -758,45 +773,39 @@ cudaError_t launch_encode_f16(const DevGraph& g, const DevPlan& p, const float* 
   const long long rows = static_cast<long long>(g.num_cells) * h;
   if (rows == 0 || K == 0) return cudaSuccess;
   if (rows > 0x7fffffffLL) return cudaErrorInvalidValue;
-  if (static_cast<long long>(g.num_edges) >= kF16ChunkedDegree * static_cast<long long>(g.num_cells)) {
-    // high mean degree: the K-chunked form
-    cudaError_t e = cudaMemsetAsync(a_exp, 0, sizeof(int32_t) * static_cast<size_t>(rows), st);
-    if (e != cudaSuccess) return e;
+  auto* hi = static_cast<__half*>(a_hi);
+  auto* lo = static_cast<__half*>(a_lo);
+  if (encode_f16_chunked(g)) {  // high mean degree: the K-chunked form (the B staging has cleared a_exp)
     const dim3 grid(static_cast<unsigned>(enc_row_blocks(rows, K)), static_cast<unsigned>(enc_k_chunks(K)));
-    encode_f16_sum_kernel<<<grid, kEncThreads, 0, st>>>(g, p, A, M, K, h, static_cast<uint16_t*>(a_hi),
-                                                         static_cast<uint16_t*>(a_lo), reinterpret_cast<uint32_t*>(a_exp));
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    encode_f16_exp_kernel<<<static_cast<unsigned>((rows + 255) / 256), 256, 0, st>>>(p, h, a_exp);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const long long chunks = rows * (K / 8);
     if ((chunks + 255) / 256 > 0x7fffffffLL) return cudaErrorInvalidValue;
-    encode_f16_rescale_kernel<<<static_cast<unsigned>((chunks + 255) / 256), 256, 0, st>>>(
-        p, K, h, static_cast<__half*>(a_hi), static_cast<__half*>(a_lo), a_exp);
-    return cudaGetLastError();
+    cudaError_t e = launch(encode_f16_sum_kernel, grid, kEncThreads, 0, st, g, p, A, M, K, h,
+                           static_cast<uint16_t*>(a_hi), static_cast<uint16_t*>(a_lo),
+                           reinterpret_cast<uint32_t*>(a_exp));
+    if (e != cudaSuccess) return e;
+    e = launch(encode_f16_exp_kernel, dim3(static_cast<unsigned>((rows + 255) / 256)), 256, 0, st, p, h, a_exp);
+    if (e != cudaSuccess) return e;
+    return launch(encode_f16_rescale_kernel, dim3(static_cast<unsigned>((chunks + 255) / 256)), 256, 0, st, p, K, h, hi,
+                  lo, a_exp);
   }
-  if (K <= 256 * 8 * kF16Keep)
-    encode_f16_kernel<256><<<static_cast<unsigned>(rows), 256, 0, st>>>(
-        g, p, A, M, K, h, static_cast<__half*>(a_hi), static_cast<__half*>(a_lo), a_exp);
-  else
-    encode_f16_kernel<512><<<static_cast<unsigned>(rows), 512, 0, st>>>(
-        g, p, A, M, K, h, static_cast<__half*>(a_hi), static_cast<__half*>(a_lo), a_exp);
-  return cudaGetLastError();
+  const bool wide = K > 256 * 8 * kF16Keep;
+  return launch(wide ? encode_f16_kernel<512> : encode_f16_kernel<256>, dim3(static_cast<unsigned>(rows)),
+                wide ? 512 : 256, 0, st, g, p, A, M, K, h, hi, lo, a_exp);
 }
 
 cudaError_t launch_colmax(const float* B, int K, int N, uint32_t* bmax, uint32_t* cleared, long long clear,
-                          cudaStream_t st) {
-  b_colmax_kernel<<<dim3((N + 31) / 32, kColSplit), 256, 0, st>>>(B, K, N, bmax, cleared, clear);
-  return cudaGetLastError();
+                          cudaStream_t st, bool early) {
+  return launch(b_colmax_kernel, dim3((N + 31) / 32, kColSplit), 256, 0, st, B, K, N, bmax, cleared, clear, early);
 }
 
-cudaError_t launch_b_f16(const float* B, int K, int N, void* b_hi, void* b_lo, uint32_t* b_max, int32_t* b_exp,
-                         cudaStream_t st) {
+cudaError_t launch_b_f16(const DevGraph& g, int h, const float* B, int K, int N, void* b_hi, void* b_lo,
+                         uint32_t* b_max, int32_t* b_exp, int32_t* a_exp, cudaStream_t st, bool early) {
   if (K == 0 || N == 0) return cudaSuccess;
-  const cudaError_t e = launch_colmax(B, K, N, b_max, nullptr, 0, st);
+  const long long rows = encode_f16_chunked(g) ? static_cast<long long>(g.num_cells) * h : 0;
+  const cudaError_t e = launch_colmax(B, K, N, b_max, reinterpret_cast<uint32_t*>(a_exp), rows, st, early);
   if (e != cudaSuccess) return e;
-  b_split_f16_kernel<<<dim3((N + kTile - 1) / kTile, (K + kTile - 1) / kTile), 256, 0, st>>>(
-      B, K, N, b_max, static_cast<__half*>(b_hi), static_cast<__half*>(b_lo), b_exp);
-  return cudaGetLastError();
+  return launch(b_split_f16_kernel, dim3((N + kTile - 1) / kTile, (K + kTile - 1) / kTile), 256, 0, st, B, K, N, b_max,
+                static_cast<__half*>(b_hi), static_cast<__half*>(b_lo), b_exp);
 }
 
 cudaError_t launch_encode_parts(const DevGraph& g, const DevPlan& p, const float* A, int M, int K, int h,
@@ -804,18 +813,16 @@ cudaError_t launch_encode_parts(const DevGraph& g, const DevPlan& p, const float
   const long long rows = static_cast<long long>(g.num_cells) * h;
   if (rows == 0 || K == 0) return cudaSuccess;
   dim3 grid(static_cast<unsigned>(enc_row_blocks(rows, K)), static_cast<unsigned>(enc_k_chunks(K)));
-  encode_parts_kernel<<<grid, kEncThreads, 0, st>>>(g, p, A, M, K, h, static_cast<__nv_bfloat16*>(a[0]),
-                                                    static_cast<__nv_bfloat16*>(a[1]),
-                                                    static_cast<__nv_bfloat16*>(a[2]));
-  return cudaGetLastError();
+  return launch(encode_parts_kernel, grid, kEncThreads, 0, st, g, p, A, M, K, h, static_cast<__nv_bfloat16*>(a[0]),
+                static_cast<__nv_bfloat16*>(a[1]), static_cast<__nv_bfloat16*>(a[2]));
 }
 
-cudaError_t launch_b_parts(const DevPlan& p, const float* B, int K, int N, void* const b[3], cudaStream_t st) {
+cudaError_t launch_b_parts(const DevPlan& p, const float* B, int K, int N, void* const b[3], cudaStream_t st,
+                           bool early) {
   if (K == 0 || N == 0) return cudaSuccess;
   dim3 grid((N + kTile - 1) / kTile, (K + kTile - 1) / kTile);
-  b_parts_kernel<<<grid, 256, 0, st>>>(p, B, K, N, static_cast<__nv_bfloat16*>(b[0]), static_cast<__nv_bfloat16*>(b[1]),
-                                       static_cast<__nv_bfloat16*>(b[2]));
-  return cudaGetLastError();
+  return launch(b_parts_kernel, grid, 256, 0, st, p, B, K, N, static_cast<__nv_bfloat16*>(b[0]),
+                static_cast<__nv_bfloat16*>(b[1]), static_cast<__nv_bfloat16*>(b[2]), early);
 }
 
 cudaError_t launch_encode_f32_flagged(const DevGraph& g, const DevPlan& p, const float* A, int M, int K, int h,
@@ -824,16 +831,14 @@ cudaError_t launch_encode_f32_flagged(const DevGraph& g, const DevPlan& p, const
   if (rows == 0 || K == 0) return cudaSuccess;
   const long long rb = enc_row_blocks(rows, K), blocks = rb * enc_k_chunks(K);
   const unsigned grid = static_cast<unsigned>(std::min<long long>(blocks, 8LL * num_sms()));
-  encode_f32_flagged_kernel<<<grid, kEncThreads, 0, st>>>(g, p, A, M, K, h, out, rb, blocks);
-  return cudaGetLastError();
+  return launch(encode_f32_flagged_kernel, dim3(grid), kEncThreads, 0, st, g, p, A, M, K, h, out, rb, blocks);
 }
 
-cudaError_t launch_b_split(const float* B, int K, int N, void* b_hi, void* b_lo, cudaStream_t st) {
+cudaError_t launch_b_split(const float* B, int K, int N, void* b_hi, void* b_lo, cudaStream_t st, bool early) {
   if (K == 0 || N == 0) return cudaSuccess;
   dim3 grid((N + kTile - 1) / kTile, (K + kTile - 1) / kTile);
-  b_split_kernel<<<grid, 256, 0, st>>>(B, K, N, static_cast<__nv_bfloat16*>(b_hi),
-                                       static_cast<__nv_bfloat16*>(b_lo));
-  return cudaGetLastError();
+  return launch(b_split_kernel, grid, 256, 0, st, B, K, N, static_cast<__nv_bfloat16*>(b_hi),
+                static_cast<__nv_bfloat16*>(b_lo), early);
 }
 
 }  // namespace bpx

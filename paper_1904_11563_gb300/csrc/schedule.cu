@@ -315,7 +315,6 @@ __device__ __forceinline__ void schedule_body(const DevGraph& g, const DevPlan& 
     if (tid == 0) {
       p.ctr[CTR_NSURV] = nsurv;
       p.ctr[CTR_PLAN] = 0;  // the rest of the plan follows (part 2)
-      p.ctr[CTR_F32_SIMT] = 0;
       p.info[BPX_INFO_DEVICE_ERR] = 0;  // cleared before the products run
     }
     return;
@@ -470,7 +469,6 @@ __device__ __forceinline__ void schedule_body(const DevGraph& g, const DevPlan& 
     p.ctr[CTR_NWAVES] = round;
     p.ctr[CTR_NREC] = nrec;
     p.ctr[CTR_ERR] = 0;
-    if (part != 2) p.ctr[CTR_F32_SIMT] = 0;
     p.ctr[CTR_PLAN] = kPlanReady;
     int32_t inf[BPX_INFO_LEN];
     for (int i = 0; i < BPX_INFO_LEN; ++i) inf[i] = 0;
@@ -494,6 +492,7 @@ __device__ __forceinline__ void schedule_body(const DevGraph& g, const DevPlan& 
 
 // The peel list of a tall plan: a warp per position, all SMs.
 __global__ void __launch_bounds__(256) fill_list_kernel(DevGraph g, DevPlan p) {
+  chain_wait();
   const int n = p.ctr[CTR_NREC], step = gridDim.x * 8;
   for (int i = blockIdx.x * 8 + (threadIdx.x >> 5); i < n; i += step) {
     const int r = p.pl_res[i], e0 = g.cell_ptr[r];
@@ -505,6 +504,12 @@ template <bool kSmem>
 __global__ void __launch_bounds__(kThreads, 1)
 schedule_kernel(DevGraph g, DevPlan p, const uint8_t* __restrict__ mask, int32_t* peel_order,
                 uint8_t* recovered, int32_t* info_out, bool cell_mask, int part, int smem_ints, bool fill) {
+  chain_wait();
+  if (threadIdx.x == 0) {  // the staging let in here may raise this flag: it is down before
+    if (part != 2) p.ctr[CTR_F32_SIMT] = 0;
+    __threadfence();
+    chain_release();
+  }
   schedule_body<kSmem>(g, p, mask, peel_order, recovered, info_out, cell_mask, part, smem_ints, fill);
 }
 
@@ -550,15 +555,14 @@ cudaError_t launch_schedule(const DevGraph& g, const DevPlan& p, const uint8_t* 
     if ((e = cudaFuncSetAttribute(schedule_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   static_cast<int>(kSmemMax))) != cudaSuccess)
       return e;
-    schedule_kernel<true><<<1, threads, static_cast<size_t>(ints) * 4, st>>>(
-        g, p, mask, peel_order, recovered, info_out, cell_mask, part, static_cast<int>(ints), !fill_later);
+    e = launch(schedule_kernel<true>, dim3(1), threads, static_cast<size_t>(ints) * 4, st, g, p, mask, peel_order,
+               recovered, info_out, cell_mask, part, static_cast<int>(ints), !fill_later);
   } else {
-    schedule_kernel<false><<<1, threads, 0, st>>>(g, p, mask, peel_order, recovered, info_out, cell_mask, part, 0,
-                                                  !fill_later);
+    e = launch(schedule_kernel<false>, dim3(1), threads, 0, st, g, p, mask, peel_order, recovered, info_out, cell_mask,
+               part, 0, !fill_later);
   }
-  if ((e = cudaGetLastError()) != cudaSuccess || !fill_later) return e;
-  fill_list_kernel<<<std::min((g.S + 7) / 8, 4 * num_sms()), 256, 0, st>>>(g, p);
-  return cudaGetLastError();
+  if (e != cudaSuccess || !fill_later) return e;
+  return launch(fill_list_kernel, dim3(std::min((g.S + 7) / 8, 4 * num_sms())), 256, 0, st, g, p);
 }
 
 }  // namespace bpx

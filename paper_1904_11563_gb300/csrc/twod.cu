@@ -39,7 +39,9 @@ __device__ __forceinline__ void split8(const float (&x)[8], __nv_bfloat16* hi, _
 // Thread = 8 consecutive k of one operand row (the encode geometry).
 __global__ void __launch_bounds__(kThreads2)
 a_ops_split_kernel(DevGraph g, const float* __restrict__ A, int M, int K, int h, __nv_bfloat16* a_hi,
-                   __nv_bfloat16* a_lo) {
+                   __nv_bfloat16* a_lo, bool early) {
+  chain_begin_staging(early);
+  chain_end_staging(early);  // (the last CTA has no more to do than others: it waits before its work)
   const int tpr = enc_threads_per_row(K);
   const long long row = static_cast<long long>(blockIdx.x) * (kThreads2 / tpr) + threadIdx.x / tpr;
   if (row >= static_cast<long long>(g.EA) * h) return;
@@ -63,8 +65,10 @@ a_ops_split_kernel(DevGraph g, const float* __restrict__ A, int M, int K, int h,
 // 64-row slice of K.
 __global__ void __launch_bounds__(256)
 b_ops_split_kernel(DevGraph g, const float* __restrict__ B, int K, int N, int w, __nv_bfloat16* bt_hi,
-                   __nv_bfloat16* bt_lo) {
+                   __nv_bfloat16* bt_lo, bool early) {
   __shared__ float tile[64][65];
+  chain_begin_staging(early);
+  chain_end_staging(early);  // (as above)
   const int nslices = (w + 63) / 64;
   const int f = blockIdx.x / nslices;
   const int n0 = (blockIdx.x - f * nslices) * 64, k0 = blockIdx.y * 64;
@@ -120,6 +124,7 @@ template <int kB>
 __global__ void __launch_bounds__(256)
 peel_2d_kernel(DevPlan p, int kc, const float* __restrict__ P, float* C, int h, int w, long long ldc, long long nv,
                int chunk, int first_wave) {
+  chain_wait();
   const int nwaves = p.ctr[CTR_NWAVES];
   const long long v0 = static_cast<long long>(blockIdx.x) * chunk;
   if (v0 >= nv) return;
@@ -167,15 +172,15 @@ peel_2d_kernel(DevPlan p, int kc, const float* __restrict__ P, float* C, int h, 
 }  // namespace
 
 cudaError_t launch_stage_2d(const DevGraph& g, const float* A, const float* B, int M, int N, int K, int h, int w,
-                            void* a_hi, void* a_lo, void* b_hi, void* b_lo, cudaStream_t st) {
+                            void* a_hi, void* a_lo, void* b_hi, void* b_lo, cudaStream_t st, bool early) {
   const long long rows = static_cast<long long>(g.EA) * h;
   const dim3 ga(static_cast<unsigned>(enc_row_blocks(rows, K)), enc_k_chunks(K));
-  a_ops_split_kernel<<<ga, kThreads2, 0, st>>>(g, A, M, K, h, static_cast<__nv_bfloat16*>(a_hi),
-                                               static_cast<__nv_bfloat16*>(a_lo));
+  const cudaError_t e = launch(a_ops_split_kernel, ga, kThreads2, 0, st, g, A, M, K, h,
+                               static_cast<__nv_bfloat16*>(a_hi), static_cast<__nv_bfloat16*>(a_lo), early);
+  if (e != cudaSuccess) return e;
   const dim3 gb(static_cast<unsigned>(g.EB * ((w + 63) / 64)), (K + 63) / 64);
-  b_ops_split_kernel<<<gb, 256, 0, st>>>(g, B, K, N, w, static_cast<__nv_bfloat16*>(b_hi),
-                                         static_cast<__nv_bfloat16*>(b_lo));
-  return cudaGetLastError();
+  return launch(b_ops_split_kernel, gb, 256, 0, st, g, B, K, N, w, static_cast<__nv_bfloat16*>(b_hi),
+                static_cast<__nv_bfloat16*>(b_lo), early);
 }
 
 cudaError_t launch_peel_2d(const DevGraph& g, const DevPlan& p, const float* P, float* C, int N, int h, int w,
@@ -184,11 +189,8 @@ cudaError_t launch_peel_2d(const DevGraph& g, const DevPlan& p, const float* P, 
   if (nv <= 0) return cudaSuccess;
   const int chunk = peel_chunk_for(nv, ctas);
   const unsigned grid = static_cast<unsigned>((nv + chunk - 1) / chunk);
-  if (g.sigma > 5)
-    peel_2d_kernel<8><<<grid, 256, 0, st>>>(p, g.k, P, C, h, w, N, nv, chunk, first_wave);
-  else
-    peel_2d_kernel<4><<<grid, 256, 0, st>>>(p, g.k, P, C, h, w, N, nv, chunk, first_wave);
-  return cudaGetLastError();
+  return launch(g.sigma > 5 ? peel_2d_kernel<8> : peel_2d_kernel<4>, dim3(grid), 256, 0, st, p, g.k, P, C, h, w,
+                static_cast<long long>(N), nv, chunk, first_wave);
 }
 
 }  // namespace bpx
