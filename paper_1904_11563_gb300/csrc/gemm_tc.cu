@@ -138,8 +138,11 @@ enum { kModeRows = 0, kModeExact = 1, kMode2D = 2 };
 // (innermost, so that a tile's diagonals run close together); the tile then
 // walks the d + 1 digit pairs (i, d - i), all k-slices of one pair after the
 // other.
+// live_bases / live_rows: a grouped launch's jobs' first tile in the space of
+// live tiles and their surviving coded rows (shared memory), or null.
 __device__ __forceinline__ TileRef locate(const TcJob* jobs, int njobs, long long t, int group, int live_mc,
-                                          bool pair, int bk, int mode = kModeRows) {
+                                          bool pair, int bk, int mode = kModeRows, const int* live_bases = nullptr,
+                                          const int* live_rows = nullptr) {
   const bool exact = mode == kModeExact;
   if (mode == kMode2D) {
     // one job; tile space = cells (most terms first) x m-units x n-tiles,
@@ -165,13 +168,14 @@ __device__ __forceinline__ TileRef locate(const TcJob* jobs, int njobs, long lon
   int lo = 0, hi = njobs - 1;
   while (lo < hi) {  // last job with tile_base <= t
     const int mid = (lo + hi + 1) >> 1;
-    if (jobs[mid].tile_base <= t) lo = mid;
+    if ((live_bases ? live_bases[mid] : jobs[mid].tile_base) <= t) lo = mid;
     else hi = mid - 1;
   }
   TileRef R;
   R.J = &jobs[lo];
   const TcJob& J = *R.J;
-  const int lt0 = static_cast<int>(t - J.tile_base);
+  const int lt0 = static_cast<int>(t - (live_bases ? live_bases[lo] : J.tile_base));
+  if (live_rows) live_mc = live_rows[lo];
   R.Mc = live_mc >= 0 ? live_mc : J.ctr[CTR_NSURV] * J.h;
   int m_units = live_mc >= 0 ? (live_mc + BM - 1) / BM : J.m_tiles_max;
   if (pair) m_units = (m_units + 1) / 2;
@@ -288,6 +292,41 @@ gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ t
   const uint32_t tmem_base = tmem_base_sh;
 
   chain_wait();  // the plan and the staged operands
+  // A grouped launch's tile space holds the live tiles only: the tiles past a
+  // job's surviving rows (a quarter of a mixed batch's) would leave the static
+  // dealing of tiles to CTAs uneven, and each would cost its job search.
+  // 48-job batch: GEMM 1856 -> 1640 us.
+  constexpr int kLiveJobs = (kMode != kModeRows || kParts == 3) ? 1 : kBK == BK ? 1024 : 64;
+  __shared__ int live_bases[kLiveJobs + 1], live_rows[kLiveJobs];
+  const bool compact = kLiveJobs > 1 && grouped && njobs <= kLiveJobs;
+  if (compact) {
+    for (int j = threadIdx.x; j < njobs; j += kThreads) live_rows[j] = jobs[j].ctr[CTR_NSURV] * jobs[j].h;
+    __syncthreads();
+    if (warp == 0) {
+      int run = 0;
+      for (int b = 0; b < njobs; b += 32) {
+        const int j = b + lane;
+        int tiles = 0;
+        if (j < njobs) {
+          const int units = (live_rows[j] + BM - 1) / BM;
+          tiles = (kPair ? (units + 1) / 2 : units) * jobs[j].n_tiles;
+        }
+        int x = tiles;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int y = __shfl_up_sync(0xffffffffu, x, o);
+          if (lane >= o) x += y;
+        }
+        if (j < njobs) live_bases[j] = run + x - tiles;
+        run += __shfl_sync(0xffffffffu, x, 31);
+      }
+      if (lane == 0) live_bases[njobs] = run;
+    }
+    __syncthreads();
+    total_tiles = live_bases[njobs];
+  }
+  const int* lb = compact ? live_bases : nullptr;
+  const int* lr = compact ? live_rows : nullptr;
   // A single job reads its surviving row count once and walks live tiles only.
   const int live_mc = grouped ? -1 : single.ctr[CTR_NSURV] * single.h;
   if (!grouped && !k2D) {
@@ -307,7 +346,7 @@ gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ t
       for (long long j = 0; ok; ++j) {
         const long long t = snake(j, cid, nclusters);
         if (t >= total_tiles) break;
-        const TileRef T = locate(jobs, njobs, t, group, live_mc, kPair, kBK, kMode);
+        const TileRef T = locate(jobs, njobs, t, group, live_mc, kPair, kBK, kMode, lb, lr);
         if (!T.live) continue;
         if (grouped && T.J != fenced) {
           tensormap_acquire(&T.J->map_ahi);
@@ -397,7 +436,7 @@ gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ t
       for (long long j = 0; ok; ++j) {
         const long long t = snake(j, cid, nclusters);
         if (t >= total_tiles) break;
-        const TileRef T = locate(jobs, njobs, t, group, live_mc, kPair, kBK, kMode);
+        const TileRef T = locate(jobs, njobs, t, group, live_mc, kPair, kBK, kMode, lb, lr);
         if (!T.live) continue;
         const int n_segs = (T.k_steps + seg_kb - 1) / seg_kb;
         // operand format: fp16 for a split-fp16 job, else bf16
@@ -490,7 +529,7 @@ gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ t
     for (long long j = 0; ok; ++j) {
       const long long t = snake(j, cid, nclusters);
       if (t >= total_tiles) break;
-      const TileRef T = locate(jobs, njobs, t, group, live_mc, kPair, kBK, kMode);
+      const TileRef T = locate(jobs, njobs, t, group, live_mc, kPair, kBK, kMode, lb, lr);
       if (!T.live) continue;
       const int n_segs = (T.k_steps + seg_kb - 1) / seg_kb;
       float accum[kCols];
