@@ -227,7 +227,7 @@ cudaError_t launch_schedule_group(const GJob* d_jobs, int njobs, size_t max_stat
 cudaError_t launch_b_split_group(const GJob* d_jobs, const long long* d_bases, int njobs, long long total_ctas,
                                  cudaStream_t st);
 cudaError_t launch_encode_split_group(const GJob* d_jobs, const long long* d_bases, int njobs,
-                                      long long total_ctas, bool split, cudaStream_t st);
+                                      long long total_ctas, int min_K, bool split, cudaStream_t st);
 // Grouped peel: jobs d_order[0 .. ngather) in the gathered form (CTAs
 // [0, gather_ctas)), the rest on the register path (CTAs [gather_ctas,
 // total_ctas)), the latter on `side` between the events when both run;

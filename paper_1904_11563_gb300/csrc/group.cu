@@ -21,6 +21,7 @@ struct bpx_group {
   size_t gjob_off = 0, tc_off = 0, total = 0;
   size_t max_state_bytes = 0, max_want_bytes = 0;
   int max_sigma = 1;
+  int min_K = 1 << 30;
   bool sched_packable = true;  // every job's schedule state fits 32-bit cell words
   long long bsplit_total = 0, enc_total = 0, peel_total = 0, tiles_total = 0;
   void* ws = nullptr;
@@ -162,7 +163,7 @@ int run_group(bpx_group* G, const bpx_opts* o, int config, cudaStream_t st) {
       (e = cudaStreamWaitEvent(st, G->join_b, 0)) != cudaSuccess)
     return cuda_fail(e, "grouped B split join");
   mark(o, BPX_STAGE_A_PREP, 0, st);
-  if ((e = bpx::launch_encode_split_group(gj, bases(G, 1), njobs, G->enc_total, split, st)) != cudaSuccess)
+  if ((e = bpx::launch_encode_split_group(gj, bases(G, 1), njobs, G->enc_total, G->min_K, split, st)) != cudaSuccess)
     return cuda_fail(e, "grouped encode");
   mark(o, BPX_STAGE_A_PREP, 1, st);
   mark(o, BPX_STAGE_GEMM, 0, st);
@@ -207,6 +208,7 @@ extern "C" int bpx_group_create(const bpx_job* jobs, int njobs, int precision, b
     G->max_want_bytes =
         std::max(G->max_want_bytes, (static_cast<size_t>(c->num_cells) + 3 * static_cast<size_t>(c->S)) * sizeof(int32_t));
     G->max_sigma = std::max(G->max_sigma, c->sigma);
+    G->min_K = std::min(G->min_K, J.K);
     G->sched_packable = G->sched_packable && bpx::sched_packable32(c->S, c->sigma);
   }
   G->gjob_off = off;
