@@ -3,6 +3,7 @@
 // library; the host only validates, binds pointers and launches.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdio>
 #include <cstring>
 #include <vector>
@@ -590,6 +591,160 @@ extern "C" int bpx_coded_matmul(const bpx_code* c, const float* d_A, const float
 
 namespace {
 
+// The calling thread's streams and events of the pipelined host call.
+constexpr int kMaxPanels = 8;
+struct HostPipe {
+  cudaStream_t in = nullptr, out = nullptr;
+  cudaEvent_t fork = nullptr, a_in = nullptr, b_in[kMaxPanels] = {}, done[kMaxPanels] = {};
+  int device = -1;
+  bool ready = false;
+  ~HostPipe() { release(); }
+  void release() {
+    for (cudaStream_t* s : {&in, &out}) {
+      if (*s) cudaStreamDestroy(*s);
+      *s = nullptr;
+    }
+    auto drop = [](cudaEvent_t& e) {
+      if (e) cudaEventDestroy(e);
+      e = nullptr;
+    };
+    drop(fork);
+    drop(a_in);
+    for (int i = 0; i < kMaxPanels; ++i) {
+      drop(b_in[i]);
+      drop(done[i]);
+    }
+    ready = false;
+  }
+};
+
+HostPipe* host_pipe() {
+  thread_local HostPipe hp;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
+  if (hp.ready && hp.device == dev) return &hp;
+  hp.release();
+  auto event = [](cudaEvent_t* e) { return cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess; };
+  bool ok = cudaStreamCreateWithFlags(&hp.in, cudaStreamNonBlocking) == cudaSuccess &&
+            cudaStreamCreateWithFlags(&hp.out, cudaStreamNonBlocking) == cudaSuccess && event(&hp.fork) && event(&hp.a_in);
+  for (int i = 0; ok && i < kMaxPanels; ++i) ok = event(&hp.b_in[i]) && event(&hp.done[i]);
+  if (!ok) {
+    cudaGetLastError();
+    hp.release();
+    return nullptr;
+  }
+  hp.device = dev;
+  hp.ready = true;
+  return &hp;
+}
+
+// Columns of B to a panel of the pipelined host call, or 0 where the call
+// runs as one piece.  Panels of whole 256-column tiles, at most eight, of 8 MB
+// or more of B and of enough tiles for most SMs (4096 cubed: four of 1024
+// columns; eight would each fill half the GPU); only calls whose copies are
+// worth it (16 MB of B), on the tensor-core paths that take a run of columns,
+// with the schedule on the caller's stream.
+int host_panel(const bpx_code* c, int N, int K, int h, int precision, const bpx_opts& o) {
+  const bool takes = precision == BPX_BF16 || precision == BPX_BF16X3 || precision == BPX_FP16X3 ||
+                     (precision == BPX_FP32 && bpx::f32_on_tensor_cores(c, N, K, h));
+  const double bytes = 4.0 * N * K;
+  if (!takes || o.stage_events || o.fused_encode || c->S >= kOverlapSources || bytes < 16e6) return 0;
+  const long long units = std::max(1LL, (bpx::rows_range(c, h).mean + 255) / 256);
+  const long long fill = 256 * ((bpx::num_sms() * 2 / 5 + units - 1) / units);
+  const int most = static_cast<int>(std::min<double>(kMaxPanels, bytes / 8e6));
+  const int panels = static_cast<int>(std::min<long long>(most, std::max(1LL, N / std::min<long long>(N, fill))));
+  const int w = ((N + panels - 1) / panels + 255) / 256 * 256;
+  return w < N ? w : 0;
+}
+
+// The host call in panels of B's columns (the mask and A first): while a panel
+// is copied in, the one before is staged, multiplied and peeled, and the one
+// before that copied out.  Same kernels over runs of columns, the same bits,
+// the same contents of d_A, d_B and d_C.  4096 cubed, split bf16, page-locked:
+// copies in 0.64 ms, kernels 0.37, copies out 0.35 one after the other 1.35 ms,
+// in panels 0.98.
+int host_panels(const bpx_code* c, const float* h_A, const float* h_B, int M, int N, int K, int h, int precision,
+                const uint8_t* h_mask, size_t mask_bytes, float* h_C, float* d_A, float* d_B, uint8_t* d_mask,
+                float* d_C, const bpx_opts& o, void* ws, size_t ws_bytes, cudaStream_t st, HostPipe* hp, int w) {
+  const bpx::WsLayout L = bpx::ws_layout(c, M, N, K, h, precision);
+  if (int rc = check_ws(c, ws, ws_bytes, L)) return rc;
+  if (!aligned(d_A, 16) || !aligned(d_B, 16) || !aligned(d_C, 16))
+    return fail(BPX_ERR_INVAL, "bpx_coded_matmul_host: buffers must be 16-byte aligned");
+  if (!bpx::gemm_config_ok(o.gemm_config))
+    return fail(BPX_ERR_INVAL, "bpx_coded_matmul_host: gemm_config %d names no tile", o.gemm_config);
+  const bpx::DevGraph g = bpx::make_graph(c, ws, L);
+  const bpx::DevPlan p = bpx::make_plan(ws, L);
+  char* base = static_cast<char*>(ws);
+  float* products = reinterpret_cast<float*>(base + L.products);
+  const bpx::RowsRange range = bpx::rows_range(c, h);
+  const int panels = (N + w - 1) / w;
+  cudaError_t e = cudaSuccess;
+  auto ok = [&](cudaError_t x) { return (e = x) == cudaSuccess; };
+  // (the caller's buffers may still be in use by earlier work on st)
+  if (!ok(cudaEventRecord(hp->fork, st)) || !ok(cudaStreamWaitEvent(hp->in, hp->fork, 0)) ||
+      !ok(cudaMemcpyAsync(d_mask, h_mask, mask_bytes, cudaMemcpyHostToDevice, hp->in)) ||
+      !ok(cudaMemcpyAsync(d_A, h_A, sizeof(float) * M * static_cast<size_t>(K), cudaMemcpyHostToDevice, hp->in)) ||
+      !ok(cudaEventRecord(hp->a_in, hp->in)) || !ok(cudaStreamWaitEvent(st, hp->a_in, 0)))
+    return cuda_fail(e, "bpx_coded_matmul_host: copy A");
+  if (int rc = schedule_impl(c, d_mask, o.mask_cells != 0, ws, ws_bytes, nullptr, nullptr, nullptr, st)) return rc;
+  int32_t* a_exp = reinterpret_cast<int32_t*>(base + L.a_scale);
+  uint32_t* b_max = reinterpret_cast<uint32_t*>(base + L.b_scale);
+  void* const a[3] = {base + L.a_hi, base + L.a_lo, base + L.a_3};
+  const bool split = precision != BPX_BF16;
+  if (precision == BPX_FP32) {
+    ok(bpx::launch_encode_parts(g, p, d_A, M, K, h, a, st));
+  } else if (precision == BPX_FP16X3) {
+    if (ok(cudaMemsetAsync(a_exp, 0, sizeof(int32_t) * static_cast<size_t>(c->num_cells) * h, st)))
+      ok(bpx::launch_encode_f16(g, p, d_A, M, K, h, a[0], a[1], a_exp, st));
+  } else {
+    ok(bpx::launch_encode_split(g, p, d_A, M, K, h, a[0], split ? a[1] : nullptr, st));
+  }
+  if (e != cudaSuccess) return cuda_fail(e, "bpx_coded_matmul_host: encode");
+  for (int i = 0; i < panels; ++i) {
+    const int n0 = i * w, wn = std::min(w, N - n0);
+    const size_t pitch = sizeof(float) * N, width = sizeof(float) * wn;
+    if (!ok(cudaMemcpy2DAsync(d_B + n0, pitch, h_B + n0, pitch, width, K, cudaMemcpyHostToDevice, hp->in)) ||
+        !ok(cudaEventRecord(hp->b_in[i], hp->in)) || !ok(cudaStreamWaitEvent(st, hp->b_in[i], 0)))
+      return cuda_fail(e, "bpx_coded_matmul_host: copy B");
+    const size_t row0 = static_cast<size_t>(n0) * K * 2;  // the panel's rows of the staged B^T
+    char* b_hi = base + L.b_hi + row0;
+    char* b_lo = base + L.b_lo + row0;
+    float* P = products + n0;
+    float* C = o.direct_write ? d_C + n0 : nullptr;
+    if (precision == BPX_FP32) {
+      void* const b[3] = {b_hi, b_lo, base + L.b_3 + row0};
+      float* a_coded = reinterpret_cast<float*>(base + L.a_hi);
+      ok(bpx::launch_b_parts(p, d_B + n0, K, wn, b, st, false, N)) &&
+          ok(bpx::launch_gemm_f32_tc(p, a, b, c->num_cells, wn, K, h, range, P, C, nullptr, st, N)) &&
+          ok(bpx::launch_encode_f32_flagged(g, p, d_A, M, K, h, a_coded, st)) &&
+          ok(bpx::launch_gemm_f32_flagged(g, p, a_coded, d_B + n0, wn, K, h, P, C, st, N));
+    } else if (precision == BPX_FP16X3) {
+      int32_t* b_exp = reinterpret_cast<int32_t*>(b_max + N) + n0;
+      ok(bpx::launch_b_f16(g, h, d_B + n0, K, wn, b_hi, b_lo, b_max + n0, b_exp, nullptr, st, false, N)) &&
+          ok(bpx::launch_gemm_tc(g, p, a[0], a[1], b_hi, b_lo, c->num_cells, wn, K, h, true, range, P, C,
+                                 o.gemm_config, nullptr, st, a_exp, b_exp, N));
+    } else {
+      ok(bpx::launch_b_split(d_B + n0, K, wn, b_hi, split ? b_lo : nullptr, st, false, N)) &&
+          ok(bpx::launch_gemm_tc(g, p, a[0], split ? a[1] : nullptr, b_hi, split ? b_lo : nullptr, c->num_cells, wn, K,
+                                 h, split, range, P, C, o.gemm_config, nullptr, st, nullptr, nullptr, N));
+    }
+    if (e == cudaSuccess)
+      ok(bpx::launch_peel(g, p, P, d_C + n0, wn, h, o.direct_write ? 2 : 1, o.compensate_depth, o.peel_ctas, st, N));
+    if (e != cudaSuccess || !ok(cudaEventRecord(hp->done[i], st))) return cuda_fail(e, "bpx_coded_matmul_host: launch");
+  }
+  for (int i = 0; i < panels; ++i) {  // (after all copies in: from pageable memory either kind holds the host up)
+    const int n0 = i * w, wn = std::min(w, N - n0);
+    const size_t pitch = sizeof(float) * N, width = sizeof(float) * wn;
+    if (!ok(cudaStreamWaitEvent(hp->out, hp->done[i], 0)) ||
+        (M > 0 && !ok(cudaMemcpy2DAsync(h_C + n0, pitch, d_C + n0, pitch, width, M, cudaMemcpyDeviceToHost, hp->out))))
+      return cuda_fail(e, "bpx_coded_matmul_host: copy C");
+  }
+  // st ends after the copies
+  if (!ok(cudaEventRecord(hp->fork, hp->out)) || !ok(cudaStreamWaitEvent(st, hp->fork, 0)))
+    return cuda_fail(e, "bpx_coded_matmul_host: join");
+  return BPX_OK;
+}
+
 // Copies in, the whole path, copies out; synchronizes at the end when `sync`.
 int host_impl(const bpx_code* c, const float* h_A, const float* h_B, int M, int N, int K, int h, int precision,
               const uint8_t* h_mask, float* h_C, float* d_A, float* d_B, uint8_t* d_mask, float* d_C,
@@ -598,17 +753,36 @@ int host_impl(const bpx_code* c, const float* h_A, const float* h_B, int M, int 
     return fail(BPX_ERR_INVAL, "bpx_coded_matmul_host: NULL argument");
   if (int rc = check_shapes(c, M, N, K, h)) return rc;
   cudaError_t e;
+  const size_t mask_bytes = (opts && opts->mask_cells) ? static_cast<size_t>(c->num_cells) : static_cast<size_t>(c->n);
+  const bpx::WsLayout L = bpx::ws_layout(c, M, N, K, h, precision);
+  int32_t* d_info = reinterpret_cast<int32_t*>(static_cast<char*>(ws) + L.p_info);
+  const bpx_opts o = opts ? *opts : bpx_default_opts();
+  if (const int w = sync ? host_panel(c, N, K, h, precision, o) : 0) {
+    if (HostPipe* hp = host_pipe()) {
+      const int rc = host_panels(c, h_A, h_B, M, N, K, h, precision, h_mask, mask_bytes, h_C, d_A, d_B, d_mask, d_C, o,
+                                 ws, ws_bytes, st, hp, w);
+      if (rc) {  // let what was enqueued end before the caller takes its buffers back
+        cudaStreamSynchronize(hp->in);
+        cudaStreamSynchronize(st);
+        cudaStreamSynchronize(hp->out);
+        return rc;
+      }
+      if ((e = cudaMemcpyAsync(h_info, d_info, sizeof(int32_t) * BPX_INFO_LEN, cudaMemcpyDeviceToHost, st)) !=
+          cudaSuccess)
+        return cuda_fail(e, "copy info");
+      if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_fail(e, "sync");
+      if (h_info[BPX_INFO_DEVICE_ERR] != 0) return h_info[BPX_INFO_DEVICE_ERR];
+      return h_info[BPX_INFO_STATUS];
+    }
+  }
   if ((e = cudaMemcpyAsync(d_A, h_A, sizeof(float) * M * static_cast<size_t>(K),
                            cudaMemcpyHostToDevice, st)) != cudaSuccess)
     return cuda_fail(e, "copy A");
   if ((e = cudaMemcpyAsync(d_B, h_B, sizeof(float) * K * static_cast<size_t>(N),
                            cudaMemcpyHostToDevice, st)) != cudaSuccess)
     return cuda_fail(e, "copy B");
-  const size_t mask_bytes = (opts && opts->mask_cells) ? static_cast<size_t>(c->num_cells) : static_cast<size_t>(c->n);
   if ((e = cudaMemcpyAsync(d_mask, h_mask, mask_bytes, cudaMemcpyHostToDevice, st)) != cudaSuccess)
     return cuda_fail(e, "copy mask");
-  const bpx::WsLayout L = bpx::ws_layout(c, M, N, K, h, precision);
-  int32_t* d_info = reinterpret_cast<int32_t*>(static_cast<char*>(ws) + L.p_info);
   if (int rc = bpx_coded_matmul(c, d_A, d_B, M, N, K, h, precision, d_mask, d_C, opts, ws, ws_bytes,
                                 nullptr, st))
     return rc;

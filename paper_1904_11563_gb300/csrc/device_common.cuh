@@ -263,9 +263,9 @@ __host__ __device__ inline float scale_pow2(float x, int e) {
 }
 cudaError_t launch_encode_f16(const DevGraph& g, const DevPlan& p, const float* A, int M, int K, int h,
                               void* a_hi, void* a_lo, int32_t* a_exp, cudaStream_t st);
-// (clears a_exp for the K-chunked encode of high-degree codes)
+// (clears a_exp, unless null, for the K-chunked encode of high-degree codes)
 cudaError_t launch_b_f16(const DevGraph& g, int h, const float* B, int K, int N, void* b_hi, void* b_lo,
-                         uint32_t* b_max, int32_t* b_exp, int32_t* a_exp, cudaStream_t st, bool early);
+                         uint32_t* b_max, int32_t* b_exp, int32_t* a_exp, cudaStream_t st, bool early, int ldb = 0);
 // gemm_config is a tile configuration the GEMM kernels have (tile codes 3,
 // 4, 7 and 8 do not exist; negative values are invalid).
 bool gemm_config_ok(int config);
@@ -297,28 +297,30 @@ cudaError_t launch_schedule(const DevGraph& g, const DevPlan& p, const uint8_t* 
 // set by the entry points for the duration of a launch.
 int& reserved_sms();
 cudaError_t launch_peel(const DevGraph& g, const DevPlan& p, const float* P, float* C, int N, int h,
-                        int first_wave, int compensate_depth, int ctas, cudaStream_t st);
+                        int first_wave, int compensate_depth, int ctas, cudaStream_t st, int ld = 0);
 cudaError_t launch_encode_f32(const DevGraph& g, const DevPlan& p, const float* A, int M, int K,
                               int h, float* out, cudaStream_t st);
 cudaError_t launch_encode_split(const DevGraph& g, const DevPlan& p, const float* A, int M, int K,
                                 int h, void* a_hi, void* a_lo, cudaStream_t st);
 // (early, here and below: launched right after the schedule of the same call, see chain_begin_staging)
-cudaError_t launch_b_split(const float* B, int K, int N, void* b_hi, void* b_lo, cudaStream_t st, bool early);
+// ldb, here and below: B's row stride where N is a run of its columns (0: N)
+cudaError_t launch_b_split(const float* B, int K, int N, void* b_hi, void* b_lo, cudaStream_t st, bool early,
+                           int ldb = 0);
 // FP32 operands for the tensor cores: the coded rows / B^T as three bf16
 // parts whose sum is the FP32 value; flag (a plan counter) is raised when an
 // element's parts would not hold it.
 cudaError_t launch_encode_parts(const DevGraph& g, const DevPlan& p, const float* A, int M, int K, int h,
                                 void* const a[3], cudaStream_t st);
 cudaError_t launch_b_parts(const DevPlan& p, const float* B, int K, int N, void* const b[3], cudaStream_t st,
-                           bool early);
+                           bool early, int ldb = 0);
 // The FP32 encode and GEMM on the CUDA cores when that flag is up (else both return at once).
 cudaError_t launch_encode_f32_flagged(const DevGraph& g, const DevPlan& p, const float* A, int M, int K, int h,
                                       float* out, cudaStream_t st);
 cudaError_t launch_gemm_f32_flagged(const DevGraph& g, const DevPlan& p, const float* a_coded, const float* B, int N,
-                                    int K, int h, float* products, float* C_direct, cudaStream_t st);
+                                    int K, int h, float* products, float* C_direct, cudaStream_t st, int ld = 0);
 cudaError_t launch_gemm_f32_tc(const DevPlan& p, void* const a[3], void* const b[3], int num_cells, int N, int K, int h,
                                const RowsRange& range, float* products, float* C_direct, int32_t* info_out,
-                               cudaStream_t st);
+                               cudaStream_t st, int ld = 0);
 // MXFP8 staging (E4M3 data + UE8M0 scales in the GEMM's per-stage order) and GEMM.
 cudaError_t launch_encode_mx(const DevGraph& g, const DevPlan& p, const float* A, int M, int K, int h,
                              void* out, void* sfa, cudaStream_t st);
@@ -343,7 +345,7 @@ cudaError_t launch_gemm_tc(const DevGraph& g, const DevPlan& p, const void* a_hi
                            const void* b_hi, const void* b_lo, int num_cells, int N, int K, int h,
                            bool split3, const RowsRange& range, float* products, float* C_direct, int config,
                            int32_t* info_out, cudaStream_t st, const int32_t* a_exp = nullptr,
-                           const int32_t* b_exp = nullptr);
+                           const int32_t* b_exp = nullptr, int ld = 0);
 
 // Exact-slice staging (max |B| per column + B digit planes; max |A| per row
 // position + coded A digit planes), digit-product GEMM and exact peel.
@@ -352,7 +354,7 @@ cudaError_t launch_exact_b(const float* B, int K, int N, const ExactParams& P, u
                            int h, void* bt, cudaStream_t st, bool early);
 // max |B| per column as float bits; clears `clear` words of `cleared` besides.
 cudaError_t launch_colmax(const float* B, int K, int N, uint32_t* bmax, uint32_t* cleared, long long clear,
-                          cudaStream_t st, bool early);
+                          cudaStream_t st, bool early, int ldb = 0);
 // src_digits: the workspace's int8 source-digit region (ex_src) when the
 // layout has one, else nullptr.
 cudaError_t launch_exact_a(const DevGraph& g, const DevPlan& p, const float* A, int M, int K, int h,

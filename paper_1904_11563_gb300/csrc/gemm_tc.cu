@@ -55,7 +55,8 @@ struct __align__(64) TcJob {
   int32_t* info_out;      // caller's info words, or null
   float* products;
   float* C_direct;
-  int N, K, h;
+  int N, K, h;  // N: row stride of the products and of C
+  int nw;       // columns computed
   int m_tiles_max, n_tiles;
   long long tile_base;    // first tile of this job in the launch's tile space
   // exact slices: int32 diagonal planes (plane d at planes + d plane_stride),
@@ -600,7 +601,7 @@ gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ t
 #pragma unroll
           for (int q = 0; q < kCols / 4; ++q) {
             const int n = n0 + 4 * q;
-            if (n < J.N)
+            if (n < J.nw)
               *reinterpret_cast<int4*>(dst + n) = make_int4(iacc[4 * q], iacc[4 * q + 1], iacc[4 * q + 2], iacc[4 * q + 3]);
           }
         } else {
@@ -612,7 +613,7 @@ gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ t
 #pragma unroll
             for (int q = 0; q < kCols / 4; ++q) {
               const int n = n0 + 4 * q;
-              if (n < J.N) {
+              if (n < J.nw) {
                 const int4 eb = *reinterpret_cast<const int4*>(J.b_exp + n);
                 accum[4 * q] = ldexpf(accum[4 * q], -(ea + eb.x));
                 accum[4 * q + 1] = ldexpf(accum[4 * q + 1], -(ea + eb.y));
@@ -624,7 +625,7 @@ gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ t
 #pragma unroll
           for (int q = 0; q < kCols / 4; ++q) {
             const int n = n0 + 4 * q;
-            if (n < J.N)
+            if (n < J.nw)
               st_cs4(dst + n, accum[4 * q], accum[4 * q + 1], accum[4 * q + 2], accum[4 * q + 3]);
           }
         }
@@ -877,7 +878,7 @@ namespace {
 bool tc_fill_job(TcJob* J, const DevPlan& p, const void* a_hi, const void* a_lo, const void* b_hi,
                  const void* b_lo, int num_cells, int N, int K, int h, int bn, int pair, int bk,
                  float* products, float* C_direct, int32_t* info_out, const int32_t* a_exp = nullptr,
-                 const int32_t* b_exp = nullptr) {
+                 const int32_t* b_exp = nullptr, int ld = 0) {
   memset(J, 0, sizeof *J);
   const long long rows = static_cast<long long>(num_cells) * h;
   const int box_b = pair ? bn / 2 : bn;  // a paired CTA loads half of the B tile
@@ -901,7 +902,8 @@ bool tc_fill_job(TcJob* J, const DevPlan& p, const void* a_hi, const void* a_lo,
   J->info_out = info_out;
   J->products = products;
   J->C_direct = C_direct;
-  J->N = N;
+  J->N = ld ? ld : N;
+  J->nw = N;
   J->K = K;
   J->h = h;
   J->m_tiles_max = static_cast<int>((rows + BM - 1) / BM);
@@ -951,7 +953,7 @@ bool gemm_config_ok(int config) { return tile_valid(config); }
 cudaError_t launch_gemm_tc(const DevGraph& g, const DevPlan& p, const void* a_hi, const void* a_lo,
                            const void* b_hi, const void* b_lo, int num_cells, int N, int K, int h,
                            bool split3, const RowsRange& range, float* products, float* C_direct, int config,
-                           int32_t* info_out, cudaStream_t st, const int32_t* a_exp, const int32_t* b_exp) {
+                           int32_t* info_out, cudaStream_t st, const int32_t* a_exp, const int32_t* b_exp, int ld) {
   if (!tile_valid(config)) return cudaErrorInvalidValue;
   if ((a_exp != nullptr) != (b_exp != nullptr) || (a_exp && !split3)) return cudaErrorInvalidValue;
   (void)g;
@@ -970,7 +972,7 @@ cudaError_t launch_gemm_tc(const DevGraph& g, const DevPlan& p, const void* a_hi
   }
   TcJob J;
   if (!tc_fill_job(&J, p, a_hi, split3 ? a_lo : nullptr, b_hi, split3 ? b_lo : nullptr, num_cells, N, K, h,
-                   bn, pair, bk, products, C_direct, info_out, a_exp, b_exp))
+                   bn, pair, bk, products, C_direct, info_out, a_exp, b_exp, ld))
     return cudaErrorInvalidValue;
   const int units = pair ? (J.m_tiles_max + 1) / 2 : J.m_tiles_max;
   const long long tiles = static_cast<long long>(units) * J.n_tiles;
@@ -986,11 +988,11 @@ cudaError_t launch_gemm_tc(const DevGraph& g, const DevPlan& p, const void* a_hi
 // against 1.1e-6.  32-wide k-slices (four stages) ran 3.73 ms.
 cudaError_t launch_gemm_f32_tc(const DevPlan& p, void* const a[3], void* const b[3], int num_cells, int N, int K, int h,
                                const RowsRange& range, float* products, float* C_direct, int32_t* info_out,
-                               cudaStream_t st) {
+                               cudaStream_t st, int ld) {
   const int bn = auto_bn(3, range, N, K);
   const bool small = bn < 256;
   TcJob J;
-  if (!tc_fill_job(&J, p, a[0], a[1], b[0], b[1], num_cells, N, K, h, bn, small ? 0 : 2, BK, products, C_direct, info_out))
+  if (!tc_fill_job(&J, p, a[0], a[1], b[0], b[1], num_cells, N, K, h, bn, small ? 0 : 2, BK, products, C_direct, info_out, nullptr, nullptr, ld))
     return cudaErrorInvalidValue;
   const long long rows = static_cast<long long>(num_cells) * h;
   if (!make_map(&J.map_a3, a[2], rows, K, BM) || !make_map(&J.map_b3, b[2], N, K, bn == 64 ? 64 : 128)) return cudaErrorInvalidValue;

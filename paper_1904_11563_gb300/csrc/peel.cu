@@ -58,6 +58,7 @@ __device__ __forceinline__ float4 two_sum_round(const float4& s, const float4& c
 
 // One (source, float4) item: C_s[v] = P_r[v] - sum of the listed blocks,
 // subtracted in ascending source id.
+// nv: float4s from one block to the next.
 template <bool kComp, int kBatch>
 __device__ __forceinline__ void peel_item(const DevPlan& p, const float4* P4, float4* C4, long long nv,
                                           int i, long long v) {
@@ -158,12 +159,21 @@ __device__ __forceinline__ void stage_wave(const DevPlan& p, const WaveDesc& w, 
   for (int t = threadIdx.x; t < nl; t += blockDim.x) cp_async4(w.list + t, p.pl_list + l0 + t);
 }
 
+// rows: how the nv float4s of a block's columns lie -- whole blocks (w4 = 0),
+// or a run of w4 float4s of each of its rows, ld4 apart (P and C point at the
+// run's first column; bs = float4s from one block to the next).
+struct Rows {
+  int w4, ld4;
+  long long bs;
+  __device__ __forceinline__ long long at(long long v) const { return w4 == 0 ? v : v / w4 * ld4 + v % w4; }
+};
+
 // kGather: the launch provides gather_smem(kCap) bytes of dynamic shared
 // memory, and sigma * chunk <= kCap (one position's rows fit a round).
 template <int kB, bool kGather, int kCap = kTermCap>
 __device__ __forceinline__ void peel_body(const DevPlan& p, const float* __restrict__ P, float* C,
                                           long long nv, int chunk, int first_wave,
-                                          int compensate_depth, long long cta) {
+                                          int compensate_depth, long long cta, const Rows& rows) {
   extern __shared__ __align__(16) uint8_t peel_smem[];
   const int nwaves = p.ctr[CTR_NWAVES];
   const long long v0 = cta * chunk;
@@ -178,11 +188,11 @@ __device__ __forceinline__ void peel_body(const DevPlan& p, const float* __restr
       const bool comp = compensate_depth >= 0 && d > compensate_depth;
       for (int it = threadIdx.x; it < items; it += blockDim.x) {
         const int j = it / clen;
-        const long long v = v0 + (it - j * clen);
+        const long long v = rows.at(v0 + (it - j * clen));
         if (comp)
-          peel_item<true, kB>(p, P4, C4, nv, o0 + j, v);
+          peel_item<true, kB>(p, P4, C4, rows.bs, o0 + j, v);
         else
-          peel_item<false, kB>(p, P4, C4, nv, o0 + j, v);
+          peel_item<false, kB>(p, P4, C4, rows.bs, o0 + j, v);
       }
       __syncthreads();
     }
@@ -193,6 +203,7 @@ __device__ __forceinline__ void peel_body(const DevPlan& p, const float* __restr
   // this thread's column and its first position / entry (stride G)
   const int col = threadIdx.x % clen, g0 = threadIdx.x / clen;
   const int G = static_cast<int>(blockDim.x) / clen;
+  const long long vcol = rows.at(v0 + col);
   const int cap = kCap / clen;  // block rows of one round
   auto fits = [&](int np, int nl) {
     return clen <= static_cast<int>(blockDim.x) && np <= kPosCap && nl <= kListCap;
@@ -227,10 +238,10 @@ __device__ __forceinline__ void peel_body(const DevPlan& p, const float* __restr
         // terms [0, tp): products; list entry e at tp + (e - e0) clen + column
         if (g0 < G) {
           for (int j = j0 + g0; j < j1; j += G)
-            cp_async16(s_term + (j - j0) * clen + col, P4 + static_cast<long long>(w.res[j]) * nv + v0 + col);
+            cp_async16(s_term + (j - j0) * clen + col, P4 + static_cast<long long>(w.res[j]) * rows.bs + vcol);
           for (int e = e0 + g0; e < e1; e += G)
             cp_async16(s_term + tp + (e - e0) * clen + col,
-                       C4 + static_cast<long long>(w.list[e - l0]) * nv + v0 + col);
+                       C4 + static_cast<long long>(w.list[e - l0]) * rows.bs + vcol);
         }
         if (round == 0 && nfit) stage_wave(p, desc(buf ^ 1), o1, o2, l1, l2);  // with the copies
         asm volatile("cp.async.wait_all;" ::: "memory");  // commit + wait for every copy issued
@@ -249,7 +260,7 @@ __device__ __forceinline__ void peel_body(const DevPlan& p, const float* __restr
               for (int e = f0; e < f1; ++e) two_sub4(r, err, t[e * clen]);
               r = two_sum_round(r, err);
             }
-            C4[static_cast<long long>(w.src[j]) * nv + v0 + col] = r;
+            C4[static_cast<long long>(w.src[j]) * rows.bs + vcol] = r;
           }
         }
         __syncthreads();
@@ -260,11 +271,11 @@ __device__ __forceinline__ void peel_body(const DevPlan& p, const float* __restr
       const int items = (o1 - o0) * clen;
       for (int it = threadIdx.x; it < items; it += blockDim.x) {
         const int j = it / clen;
-        const long long v = v0 + (it - j * clen);
+        const long long v = rows.at(v0 + (it - j * clen));
         if (comp)
-          peel_item<true, kB>(p, P4, C4, nv, o0 + j, v);
+          peel_item<true, kB>(p, P4, C4, rows.bs, o0 + j, v);
         else
-          peel_item<false, kB>(p, P4, C4, nv, o0 + j, v);
+          peel_item<false, kB>(p, P4, C4, rows.bs, o0 + j, v);
       }
       asm volatile("cp.async.wait_all;" ::: "memory");  // commit + wait for every copy issued
       __syncthreads();
@@ -284,7 +295,7 @@ __device__ __forceinline__ void peel_body(const DevPlan& p, const float* __restr
 template <int kB, bool kGather>
 __global__ void __launch_bounds__(kPeelThreads)
 peel_kernel(DevPlan p, const float* __restrict__ P, float* C, long long nv, int chunk, int first_wave,
-            int compensate_depth) {
+            int compensate_depth, Rows rows) {
   chain_wait();
   if (p.ctr[CTR_PLAN] != kPlanReady) {  // no schedule has planned this workspace: refuse, write nothing
     if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -293,7 +304,7 @@ peel_kernel(DevPlan p, const float* __restrict__ P, float* C, long long nv, int 
     }
     return;
   }
-  peel_body<kB, kGather>(p, P, C, nv, chunk, first_wave, compensate_depth, blockIdx.x);
+  peel_body<kB, kGather>(p, P, C, nv, chunk, first_wave, compensate_depth, blockIdx.x, rows);
 }
 
 // A grouped peel launch over the jobs order[0 .. n): their CTA ranges lie
@@ -308,7 +319,7 @@ peel_group_kernel(const GJob* __restrict__ jobs, const int32_t* __restrict__ ord
   const GJob& J = jobs[order[i]];
   const long long nv = static_cast<long long>(J.h) * J.N / 4;
   peel_body<kB, kGather, kTermCapGroup>(J.p, J.products, J.C, nv, J.peel_chunk, first_wave, compensate_depth,
-                                        b - __ldg(bases + i));
+                                        b - __ldg(bases + i), Rows{0, 0, nv});
 }
 
 int batch_for(int sigma) { return sigma > 9 ? 16 : (sigma > 5 ? 8 : 4); }
@@ -371,9 +382,10 @@ cudaError_t launch_peel_group(const GJob* d_jobs, const int32_t* d_order, const 
 }
 
 cudaError_t launch_peel(const DevGraph& g, const DevPlan& p, const float* P, float* C, int N, int h,
-                        int first_wave, int compensate_depth, int ctas, cudaStream_t st) {
+                        int first_wave, int compensate_depth, int ctas, cudaStream_t st, int ld) {
   const long long nv = static_cast<long long>(h) * N / 4;
   if (nv <= 0) return cudaSuccess;
+  const Rows rows = ld == 0 || ld == N ? Rows{0, 0, nv} : Rows{N / 4, ld / 4, static_cast<long long>(h) * ld / 4};
   // Every CTA walks every wave, so the grid never exceeds the CTAs that can
   // be resident at once (a CTA waiting for a slot would repeat the chain).
   // The CTA count: the hint's (default 4 per SM), capped at the CTAs that
@@ -398,7 +410,7 @@ cudaError_t launch_peel(const DevGraph& g, const DevPlan& p, const float* P, flo
   auto run = [&](auto kern, size_t smem, long long chunk) -> cudaError_t {
     const unsigned grid = static_cast<unsigned>((nv + chunk - 1) / chunk);
     return launch(kern, dim3(grid), kPeelThreads, smem, st, p, P, C, nv, static_cast<int>(chunk), first_wave,
-                  compensate_depth);
+                  compensate_depth, rows);
   };
   // The gathered form for tall codes, when one position's rows (at most
   // sigma) over the CTA's columns fit a round of the term buffer.

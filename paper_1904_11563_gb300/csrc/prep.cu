@@ -156,7 +156,7 @@ encode_f32_flagged_kernel(DevGraph g, DevPlan p, const float* __restrict__ A, in
 // shared-memory tile: float4 reads along N, 16-byte bf16 writes along K.
 constexpr int kTile = 64;
 template <bool kParts3 = false>
-__device__ __forceinline__ bool b_split_body(const float* __restrict__ B, int K, int N,
+__device__ __forceinline__ bool b_split_body(const float* __restrict__ B, int K, int N, int ldb,
                                              __nv_bfloat16* bt_hi, __nv_bfloat16* bt_lo, int bx,
                                              int by, __nv_bfloat16* bt_3 = nullptr) {
   bool unfit = false;
@@ -169,7 +169,7 @@ __device__ __forceinline__ bool b_split_body(const float* __restrict__ B, int K,
     for (int i = 0; i < 4; ++i) {
       const int r = r0 + 16 * i, k = k0 + r, n = n0 + 4 * c4;
       float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (k < K && n < N) v = __ldg(reinterpret_cast<const float4*>(B + static_cast<long long>(k) * N + n));
+      if (k < K && n < N) v = __ldg(reinterpret_cast<const float4*>(B + static_cast<long long>(k) * ldb + n));
       tile[r][4 * c4 + 0] = v.x;
       tile[r][4 * c4 + 1] = v.y;
       tile[r][4 * c4 + 2] = v.z;
@@ -210,17 +210,18 @@ __device__ __forceinline__ bool b_split_body(const float* __restrict__ B, int K,
 }
 
 __global__ void __launch_bounds__(256)
-b_parts_kernel(DevPlan p, const float* __restrict__ B, int K, int N, __nv_bfloat16* o1, __nv_bfloat16* o2,
+b_parts_kernel(DevPlan p, const float* __restrict__ B, int K, int N, int ldb, __nv_bfloat16* o1, __nv_bfloat16* o2,
                __nv_bfloat16* o3, bool early) {
   chain_begin_staging(early);
-  if (b_split_body<true>(B, K, N, o1, o2, blockIdx.x, blockIdx.y, o3)) p.ctr[CTR_F32_SIMT] = 1;
+  if (b_split_body<true>(B, K, N, ldb, o1, o2, blockIdx.x, blockIdx.y, o3)) p.ctr[CTR_F32_SIMT] = 1;
   chain_end_staging(early);
 }
 
 __global__ void __launch_bounds__(256)
-b_split_kernel(const float* __restrict__ B, int K, int N, __nv_bfloat16* bt_hi, __nv_bfloat16* bt_lo, bool early) {
+b_split_kernel(const float* __restrict__ B, int K, int N, int ldb, __nv_bfloat16* bt_hi, __nv_bfloat16* bt_lo,
+               bool early) {
   chain_begin_staging(early);
-  b_split_body(B, K, N, bt_hi, bt_lo, blockIdx.x, blockIdx.y);
+  b_split_body(B, K, N, ldb, bt_hi, bt_lo, blockIdx.x, blockIdx.y);
   chain_end_staging(early);
 }
 
@@ -233,7 +234,7 @@ b_split_group_kernel(const GJob* __restrict__ jobs, const long long* __restrict_
   const GJob& J = jobs[j];
   const uint32_t local = static_cast<uint32_t>(b - __ldg(bases + j));  // < 2^31: one launch's CTAs
   const uint32_t gx = (J.N + kTile - 1) / kTile, by = local / gx;
-  b_split_body(J.B, J.K, J.N, static_cast<__nv_bfloat16*>(J.b_hi), static_cast<__nv_bfloat16*>(J.b_lo),
+  b_split_body(J.B, J.K, J.N, J.N, static_cast<__nv_bfloat16*>(J.b_hi), static_cast<__nv_bfloat16*>(J.b_lo),
                static_cast<int>(local - by * gx), static_cast<int>(by));
 }
 
@@ -531,8 +532,8 @@ encode_f16_rescale_kernel(DevPlan p, int K, int h, __half* out_hi, __half* out_l
 // words for a later kernel.
 constexpr int kColRows = 128, kColSplit = 8;
 __global__ void __cluster_dims__(1, kColSplit, 1) __launch_bounds__(256)
-b_colmax_kernel(const float* __restrict__ B, int K, int N, uint32_t* bmax, uint32_t* cleared, long long clear,
-                bool early) {
+b_colmax_kernel(const float* __restrict__ B, int K, int N, int ldb, uint32_t* bmax, uint32_t* cleared,
+                long long clear, bool early) {
   __shared__ float4 red[32][8];
   __shared__ float4 part[kColSplit][8];
   chain_begin_staging(early);
@@ -546,7 +547,7 @@ b_colmax_kernel(const float* __restrict__ B, int K, int N, uint32_t* bmax, uint3
     const int k1 = min(K, k0 + kColRows);
 #pragma unroll 4
     for (int k = k0 + ph; k < k1; k += 32) {
-      const float4 v = __ldg(reinterpret_cast<const float4*>(B + static_cast<long long>(k) * N + n));
+      const float4 v = __ldg(reinterpret_cast<const float4*>(B + static_cast<long long>(k) * ldb + n));
       m.x = fmaxf(m.x, fabsf(v.x));
       m.y = fmaxf(m.y, fabsf(v.y));
       m.z = fmaxf(m.z, fabsf(v.z));
@@ -586,8 +587,8 @@ b_colmax_kernel(const float* __restrict__ B, int K, int N, uint32_t* bmax, uint3
 // same 64 x 64 shared-memory transpose as b_split; the first k-tile's CTAs
 // also record each column's exponent for the GEMM epilogue.
 __global__ void __launch_bounds__(256)
-b_split_f16_kernel(const float* __restrict__ B, int K, int N, const uint32_t* __restrict__ bmax, __half* bt_hi,
-                   __half* bt_lo, int32_t* b_exp) {
+b_split_f16_kernel(const float* __restrict__ B, int K, int N, int ldb, const uint32_t* __restrict__ bmax,
+                   __half* bt_hi, __half* bt_lo, int32_t* b_exp) {
   __shared__ float tile[kTile][kTile + 1];
   chain_wait();
   const int n0 = blockIdx.x * kTile, k0 = blockIdx.y * kTile;
@@ -597,7 +598,7 @@ b_split_f16_kernel(const float* __restrict__ B, int K, int N, const uint32_t* __
     for (int i = 0; i < 4; ++i) {
       const int r = r0 + 16 * i, k = k0 + r, n = n0 + 4 * c4;
       float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (k < K && n < N) v = __ldg(reinterpret_cast<const float4*>(B + static_cast<long long>(k) * N + n));
+      if (k < K && n < N) v = __ldg(reinterpret_cast<const float4*>(B + static_cast<long long>(k) * ldb + n));
       tile[r][4 * c4 + 0] = v.x;
       tile[r][4 * c4 + 1] = v.y;
       tile[r][4 * c4 + 2] = v.z;
@@ -828,18 +829,19 @@ cudaError_t launch_encode_f16(const DevGraph& g, const DevPlan& p, const float* 
 }
 
 cudaError_t launch_colmax(const float* B, int K, int N, uint32_t* bmax, uint32_t* cleared, long long clear,
-                          cudaStream_t st, bool early) {
-  return launch(b_colmax_kernel, dim3((N + 31) / 32, kColSplit), 256, 0, st, B, K, N, bmax, cleared, clear, early);
+                          cudaStream_t st, bool early, int ldb) {
+  return launch(b_colmax_kernel, dim3((N + 31) / 32, kColSplit), 256, 0, st, B, K, N, ldb ? ldb : N, bmax, cleared,
+                clear, early);
 }
 
 cudaError_t launch_b_f16(const DevGraph& g, int h, const float* B, int K, int N, void* b_hi, void* b_lo,
-                         uint32_t* b_max, int32_t* b_exp, int32_t* a_exp, cudaStream_t st, bool early) {
+                         uint32_t* b_max, int32_t* b_exp, int32_t* a_exp, cudaStream_t st, bool early, int ldb) {
   if (K == 0 || N == 0) return cudaSuccess;
-  const long long rows = encode_f16_chunked(g) ? static_cast<long long>(g.num_cells) * h : 0;
-  const cudaError_t e = launch_colmax(B, K, N, b_max, reinterpret_cast<uint32_t*>(a_exp), rows, st, early);
+  const long long rows = a_exp && encode_f16_chunked(g) ? static_cast<long long>(g.num_cells) * h : 0;
+  const cudaError_t e = launch_colmax(B, K, N, b_max, reinterpret_cast<uint32_t*>(a_exp), rows, st, early, ldb);
   if (e != cudaSuccess) return e;
-  return launch(b_split_f16_kernel, dim3((N + kTile - 1) / kTile, (K + kTile - 1) / kTile), 256, 0, st, B, K, N, b_max,
-                static_cast<__half*>(b_hi), static_cast<__half*>(b_lo), b_exp);
+  return launch(b_split_f16_kernel, dim3((N + kTile - 1) / kTile, (K + kTile - 1) / kTile), 256, 0, st, B, K, N,
+                ldb ? ldb : N, b_max, static_cast<__half*>(b_hi), static_cast<__half*>(b_lo), b_exp);
 }
 
 cudaError_t launch_encode_parts(const DevGraph& g, const DevPlan& p, const float* A, int M, int K, int h,
@@ -852,10 +854,10 @@ cudaError_t launch_encode_parts(const DevGraph& g, const DevPlan& p, const float
 }
 
 cudaError_t launch_b_parts(const DevPlan& p, const float* B, int K, int N, void* const b[3], cudaStream_t st,
-                           bool early) {
+                           bool early, int ldb) {
   if (K == 0 || N == 0) return cudaSuccess;
   dim3 grid((N + kTile - 1) / kTile, (K + kTile - 1) / kTile);
-  return launch(b_parts_kernel, grid, 256, 0, st, p, B, K, N, static_cast<__nv_bfloat16*>(b[0]),
+  return launch(b_parts_kernel, grid, 256, 0, st, p, B, K, N, ldb ? ldb : N, static_cast<__nv_bfloat16*>(b[0]),
                 static_cast<__nv_bfloat16*>(b[1]), static_cast<__nv_bfloat16*>(b[2]), early);
 }
 
@@ -868,10 +870,11 @@ cudaError_t launch_encode_f32_flagged(const DevGraph& g, const DevPlan& p, const
   return launch(encode_f32_flagged_kernel, dim3(grid), kEncThreads, 0, st, g, p, A, M, K, h, out, rb, blocks);
 }
 
-cudaError_t launch_b_split(const float* B, int K, int N, void* b_hi, void* b_lo, cudaStream_t st, bool early) {
+cudaError_t launch_b_split(const float* B, int K, int N, void* b_hi, void* b_lo, cudaStream_t st, bool early,
+                           int ldb) {
   if (K == 0 || N == 0) return cudaSuccess;
   dim3 grid((N + kTile - 1) / kTile, (K + kTile - 1) / kTile);
-  return launch(b_split_kernel, grid, 256, 0, st, B, K, N, static_cast<__nv_bfloat16*>(b_hi),
+  return launch(b_split_kernel, grid, 256, 0, st, B, K, N, ldb ? ldb : N, static_cast<__nv_bfloat16*>(b_hi),
                 static_cast<__nv_bfloat16*>(b_lo), early);
 }
 
