@@ -455,7 +455,7 @@ WsLayout ws_layout(const bpx_code* c, int M, int N, int K, int h, int precision,
   L.p_surv = take(C * i32);
   L.p_direct = take(C * i32);
   L.p_front0 = take(C * i32);
-  L.p_front1 = take(C * i32);
+  L.p_pos = take(std::max(C, S) * i32);
   L.p_word = take(C * sizeof(unsigned long long));
   L.p_depth = take(S * i32);
   L.p_resolver = take(S * i32);

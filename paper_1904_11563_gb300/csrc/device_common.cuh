@@ -30,6 +30,10 @@ struct DevGraph {
   int affine;     // the plan holds an affine cell table (bpx_code::affine)
 };
 
+// Codes this tall peel in hundreds of waves: their lists are filled by a
+// second launch, and their peels copy ahead of the wave at hand.
+constexpr int kTallSources = 1024;
+
 // Peel plan written by the schedule kernel.
 struct DevPlan {
   int32_t* info;      // BPX_INFO_LEN
@@ -38,7 +42,7 @@ struct DevPlan {
   int32_t* surv;      // surviving cells, ascending
   int32_t* direct;    // per cell: the source it resolves at depth 1, or -1
   int32_t* front0;    // frontier scratch
-  int32_t* front1;
+  int32_t* pos;       // per source: its index in `order` (tall codes)
   unsigned long long* word;  // per cell: sum of the unknown sources' ids + 1 << 32 | their count (large
                              // codes; else 32-bit initial words, uploaded with the graph)
   int32_t* depth;     // per source: round of recovery (0 = not recovered)
@@ -92,7 +96,7 @@ inline DevPlan make_plan(const void* ws, const WsLayout& L) {
   p.surv = at(L.p_surv);
   p.direct = at(L.p_direct);
   p.front0 = at(L.p_front0);
-  p.front1 = at(L.p_front1);
+  p.pos = at(L.p_pos);
   p.word = reinterpret_cast<unsigned long long*>(base + L.p_word);
   p.depth = at(L.p_depth);
   p.resolver = at(L.p_resolver);

@@ -116,7 +116,6 @@ constexpr int kTermCap = 5632;       // float4 block elements of one round (88 K
 constexpr int kTermCapGroup = 3200;  // grouped launches (50 KB): three CTAs per SM for the many chains
 constexpr int kListCap = 2048;  // subtrahend list entries of one wave
 constexpr int kPosCap = 256;    // order positions of one wave
-constexpr int kGatherMinSources = 1024;  // codes this tall peel in hundreds of waves
 constexpr int kDescInts = kListCap + 3 * kPosCap + 1;  // one descriptor buffer
 // dynamic shared memory of the gathered form: 110 KB for one job (two CTAs
 // per SM), 72 KB for grouped launches (three)
@@ -292,6 +291,232 @@ __device__ __forceinline__ void peel_body(const DevPlan& p, const float* __restr
   }
 }
 
+// Tall codes, pipelined (one job): the plan's positions are walked in rounds
+// of one wave's positions, at most kRoundPos of them and as many block rows
+// (products and subtrahends) as a slot holds.  While a round is computed, the
+// rows of the next kLook rounds are in flight to their slots, so a round
+// costs its issue and its sums, not a global round trip.  A subtrahend that
+// is recovered too late to be copied that early (about one in ten: its order
+// position is not below the first of the rounds still open when the copy
+// would start) is read from a ring of the newest results by its position.
+// Four roles by warp: kSumThreads sum, a float4 column of a position each;
+// kCopyThreads copy and, a row of a round's words each, bring the plan's words
+// ahead of the copies -- the resolvers and list entries, two rounds on the
+// entries' positions, two rounds on where each row comes from and lies --; the
+// last warp cuts the waves into rounds.  One barrier a round.  The sums run
+// in the list's order, as in the other forms: the same bits.
+//
+// Bound by the chain of a round's instructions (about 0.65 us) up to 8
+// float4s a CTA, from there by what an SM copies and sums.  One CTA an SM and
+// 16 float4s (two lines a row) at N = 8192: the fixed work of a round, which
+// is per row, serves twice the bytes of two CTAs of 8 (1.70 ms against 2.01);
+// 14 float4s on 147 SMs cut the lines, 1.79.  Sums in batches of 12 rows, 3 or
+// 4 rounds ahead, or all threads in one role: no faster to 60 % slower.
+// n = 32, k = 24, b = 683 (16392 rows, 725 waves), against the gathered form:
+// N = 8192 2.50 -> 1.70 ms, N = 4096 2.26 -> 1.20 ms, N = 256 1.90 -> 1.19 ms;
+// n = 12, k = 9, b = 340, N = 8192 555 -> 244 us.
+constexpr int kLook = 2;         // rounds in flight beyond the computed one
+constexpr int kSlot = 4096;      // float4s of one round's rows (64 KB)
+constexpr int kRing = 1024;      // float4s of the newest results (16 KB)
+constexpr int kRoundPos = 32;    // positions of one round: the planner's lanes
+constexpr int kSumThreads = 256, kCopyThreads = 256, kTallThreads = kSumThreads + kCopyThreads + 32;
+constexpr int kTallColumns = 32;   // a CTA's float4 columns at most
+constexpr int kWords = kLook + 4;  // rounds whose rows' words are held at once
+constexpr int kEnds = kLook + 6;   // rounds whose positions' words are (a power of two)
+constexpr int kRounds = 16;        // rounds whose bounds are held (a power of two)
+static_assert(kLook == 2, "words two rounds on have landed: wait_group leaves kLook - 1 groups open");
+static_assert((kEnds & (kEnds - 1)) == 0 && kRounds > kLook + 7, "the rounds' tables");
+struct TallSmem {
+  float4 row[(kLook + 1) * kSlot + kRing];  // the slots, then the ring
+  const float4* from[2][kCopyThreads];      // per row of a round: what to copy (its first float4), null: in the ring
+  int block[kWords][kCopyThreads];  // per row: its resolver or its source
+  int at[kWords][kCopyThreads];     // per row: its source's position, then its place from row[0], in bytes
+  int end[kEnds][kRoundPos];        // per position: its entries' end in the peel list
+  int src[kEnds][kRoundPos];        // per position: its source
+  int4 round[kRounds];              // positions [x, y), list entries [z, w)
+  int deep[kRounds];                // its wave is past the compensation depth
+};
+
+__global__ void __launch_bounds__(kTallThreads, 1)
+peel_tall_kernel(DevPlan p, const float* __restrict__ P, float* C, long long nv, int chunk, int first_wave,
+                 int compensate_depth, Rows rows) {
+  chain_wait();
+  if (p.ctr[CTR_PLAN] != kPlanReady) {  // no schedule has planned this workspace: refuse, write nothing
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+      atomicExch(&p.info[BPX_INFO_DEVICE_ERR], BPX_ERR_INVAL);
+      atomicExch(&p.info[BPX_INFO_STATUS], BPX_ERR_INVAL);
+    }
+    return;
+  }
+  extern __shared__ __align__(16) uint8_t peel_smem[];
+  TallSmem& S = *reinterpret_cast<TallSmem*>(peel_smem);
+  auto tall_sync = [] { asm volatile("bar.sync 1, %0;" ::"n"(kTallThreads) : "memory"); };
+  const int nwaves = p.ctr[CTR_NWAVES];
+  const long long v0 = static_cast<long long>(blockIdx.x) * chunk;
+  if (v0 >= nv || first_wave > nwaves) return;
+  const int clen = static_cast<int>(min(static_cast<long long>(chunk), nv - v0));
+  const int lane = threadIdx.x & 31;
+  // the ring's rows, a power of two: the positions of kLook + 1 rounds
+  const int ring_mask = (1 << (31 - __clz(kRing / clen))) - 1;
+  const int start = p.wave_ptr[first_wave - 1], end = p.wave_ptr[nwaves];
+  constexpr int kFirst = -(kLook + 6);                // the iteration that plans round 0
+  constexpr int kRingAt = (kLook + 1) * kSlot * 16;   // bytes
+  if (threadIdx.x < kRounds) {  // the rounds before 0: nothing
+    const int l = p.pl_ptr[start];
+    S.round[threadIdx.x] = make_int4(start, start, l, l);
+  }
+
+  if (threadIdx.x < kSumThreads) {
+    const int col = threadIdx.x % clen, g0 = threadIdx.x / clen, G = kSumThreads / clen;
+    float4* C4 = reinterpret_cast<float4*>(C) + rows.at(v0 + col);
+    uint8_t* x = reinterpret_cast<uint8_t*>(S.row + col);
+    auto row = [&](int at) { return *reinterpret_cast<const float4*>(x + at); };
+    tall_sync();
+    for (int k = kFirst; k < 0; ++k) tall_sync();
+    for (uint32_t k = 0;; ++k) {
+      tall_sync();  // round k's rows are in, round k - 1's results out
+      const int4 d = S.round[k % kRounds];
+      if (d.y == d.x) break;
+      const int np = g0 < G ? d.y - d.x : 0;
+      const int* at = S.at[k % kWords] + (d.y - d.x) - d.z;  // by list entry
+      for (int j = g0; j < np; j += G) {
+        const int e1 = S.end[k % kEnds][j], s = S.src[k % kEnds][j];
+        int e = j > 0 ? S.end[k % kEnds][j - 1] : d.z;
+        float4 r = row(k % (kLook + 1) * (kSlot * 16) + j * clen * 16);
+        float4 y[8];
+        if (S.deep[k % kRounds] == 0) {
+          for (; e + 8 <= e1; e += 8) {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) y[u] = row(at[e + u]);
+#pragma unroll
+            for (int u = 0; u < 8; ++u) sub4(r, y[u]);
+          }
+          if (e < e1) {
+#pragma unroll
+            for (int u = 0; u < 7; ++u)
+              if (e + u < e1) y[u] = row(at[e + u]);
+#pragma unroll
+            for (int u = 0; u < 7; ++u)
+              if (e + u < e1) sub4(r, y[u]);
+          }
+        } else {
+          float4 err = make_float4(0.f, 0.f, 0.f, 0.f);
+          for (; e < e1; ++e) two_sub4(r, err, row(at[e]));
+          r = two_sum_round(r, err);
+        }
+        C4[static_cast<long long>(s) * rows.bs] = r;
+        *reinterpret_cast<float4*>(x + kRingAt + ((d.x + j) & ring_mask) * clen * 16) = r;
+      }
+    }
+    return;
+  }
+
+  if (threadIdx.x >= kSumThreads + kCopyThreads) {
+    // the planner: the next round starts at position pj, list entry pe, in
+    // wave pd, whose positions end at pw (the next wave's: pw2)
+    const int cap = min(kCopyThreads, kSlot / clen);
+    const int max_pos = min(kRoundPos, (ring_mask + 1) / (kLook + 1));
+    int pj = start, pe = p.pl_ptr[start], pd = first_wave;
+    int pw = p.wave_ptr[first_wave], pw2 = first_wave < nwaves ? p.wave_ptr[first_wave + 1] : pw;
+    // list ends of the positions from pb on, 32 a register, the last ahead of its use
+    int pb = start;
+    auto ends = [&](int from) { return p.pl_ptr[min(from + 1 + lane, end)]; };
+    int l0 = ends(pb), l1 = ends(pb + 32), l2 = ends(pb + 64);
+    tall_sync();
+    for (int k = kFirst;; ++k) {
+      tall_sync();
+      if (k >= 0) {
+        const int4 d = S.round[k % kRounds];
+        if (d.y == d.x) break;
+      }
+      const int i = pj - pb + lane;  // < 64
+      const int w0 = __shfl_sync(0xffffffffu, l0, i & 31), w1 = __shfl_sync(0xffffffffu, l1, i & 31);
+      const int pv = i < 32 ? w0 : w1;
+      const bool in = lane < max_pos && pj + lane < pw && lane + 1 + pv - pe <= cap;
+      const int c = __popc(__ballot_sync(0xffffffffu, in));  // a run of the wave's next positions
+      const int ne = __shfl_sync(0xffffffffu, pv, max(c - 1, 0));
+      if (lane == 0) {
+        const int to = (k + kLook + 6) % kRounds;
+        S.round[to] = make_int4(pj, pj + c, pe, c > 0 ? ne : pe);
+        S.deep[to] = compensate_depth >= 0 && pd > compensate_depth;
+      }
+      if (c > 0) pe = ne;
+      pj += c;
+      if (pj - pb >= 32) {
+        pb += 32;
+        l0 = l1;
+        l1 = l2;
+        l2 = ends(pb + 64);
+      }
+      if (pj == pw && pd < nwaves) {
+        ++pd;
+        pw = pw2;
+        pw2 = pd < nwaves ? p.wave_ptr[pd + 1] : pw;
+      }
+    }
+    return;
+  }
+
+  const int tid = threadIdx.x - kSumThreads;
+  const int col = tid % clen, g0 = tid / clen, G = kCopyThreads / clen;
+  const long long vcol = rows.at(v0 + col), bs = rows.bs;
+  const float4* P4 = reinterpret_cast<const float4*>(P);
+  const float4* C4 = reinterpret_cast<const float4*>(C);
+  const uint32_t to0 = static_cast<uint32_t>(__cvta_generic_to_shared(S.row + g0 * clen + col));
+  const uint32_t step = static_cast<uint32_t>(G * clen * 16);
+  tall_sync();
+  for (int k = kFirst;; ++k) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kLook - 1) : "memory");
+    tall_sync();  // round k's rows are in, round k - 1's results out
+    // unsigned: negative rounds' entries are empty
+    const uint32_t rc = k + kLook, rm = rc + 1, rp = rc + 3, rw = rc + 5;
+    const int4 dk = S.round[static_cast<uint32_t>(k) % kRounds], dc = S.round[rc % kRounds];
+    const int4 dm = S.round[rm % kRounds], dp = S.round[rp % kRounds], dw = S.round[rw % kRounds];
+    const int open = S.round[(rm - kLook) % kRounds].x;
+    if (k >= 0 && dk.x == dk.y) break;
+    if (g0 < G) {  // round k + kLook starts on its way
+      const int n = dc.y - dc.x + dc.w - dc.z;
+      uint32_t to = to0 + rc % (kLook + 1) * (kSlot * 16);
+      const float4* const* from = S.from[rc & 1];
+      for (int i = g0; i < n; i += 4 * G, to += 4 * step) {
+        const float4* b[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) b[u] = i + u * G < n ? from[i + u * G] : nullptr;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (b[u])
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to + u * step), "l"(b[u] + vcol)
+                         : "memory");
+      }
+    }
+    {  // a round's rows: their words ...
+      const int np = dw.y - dw.x;
+      if (tid < np) {
+        cp_async4(&S.block[rw % kWords][tid], p.pl_res + dw.x + tid);
+        cp_async4(&S.end[rw % kEnds][tid], p.pl_ptr + dw.x + tid + 1);
+        cp_async4(&S.src[rw % kEnds][tid], p.order + dw.x + tid);
+      } else if (tid < np + dw.w - dw.z) {
+        cp_async4(&S.block[rw % kWords][tid], p.pl_list + dw.z + tid - np);
+      }
+    }
+    {  // ... two rounds on, the entries' positions ...
+      const int np = dp.y - dp.x;
+      if (tid >= np && tid < np + dp.w - dp.z) cp_async4(&S.at[rp % kWords][tid], p.pos + S.block[rp % kWords][tid]);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    {  // ... and two on, what to copy and where each will be
+      const int np = dm.y - dm.x;
+      if (tid < np + dm.w - dm.z) {
+        const int q = S.at[rm % kWords][tid];
+        const bool fresh = tid >= np && q >= open;
+        S.from[rm & 1][tid] = fresh ? nullptr : (tid < np ? P4 : C4) + S.block[rm % kWords][tid] * bs;
+        S.at[rm % kWords][tid] = fresh ? kRingAt + (q & ring_mask) * clen * 16
+                                       : static_cast<int>(rm % (kLook + 1)) * (kSlot * 16) + tid * clen * 16;
+      }
+    }
+  }
+}
+
 template <int kB, bool kGather>
 __global__ void __launch_bounds__(kPeelThreads)
 peel_kernel(DevPlan p, const float* __restrict__ P, float* C, long long nv, int chunk, int first_wave,
@@ -333,7 +558,7 @@ int peel_chunk_for(long long nv, int ctas_hint) {
 }
 
 bool peel_gather_ok(int S, int sigma, long long chunk) {
-  return S >= kGatherMinSources && chunk <= kPeelThreads &&
+  return S >= kTallSources && chunk <= kPeelThreads &&
          static_cast<long long>(std::max(1, sigma)) * chunk <= kTermCapGroup;
 }
 
@@ -390,14 +615,14 @@ cudaError_t launch_peel(const DevGraph& g, const DevPlan& p, const float* P, flo
   // be resident at once (a CTA waiting for a slot would repeat the chain).
   // The CTA count: the hint's (default 4 per SM), capped at the CTAs that
   // can be resident at once for the kernel's shared memory.
-  auto chunk_for = [&](auto kern, size_t smem, long long* chunk) -> cudaError_t {
+  auto chunk_for = [&](auto kern, size_t smem, long long* chunk, int threads = kPeelThreads) -> cudaError_t {
     if (smem) {
       const cudaError_t e =
           cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
       if (e != cudaSuccess) return e;
     }
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kPeelThreads, smem) != cudaSuccess ||
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem) != cudaSuccess ||
         per_sm <= 0) {
       cudaGetLastError();
       per_sm = 1;
@@ -407,17 +632,31 @@ cudaError_t launch_peel(const DevGraph& g, const DevPlan& p, const float* P, flo
     if ((nv + *chunk - 1) / *chunk > slots) *chunk = (nv + slots - 1) / slots;
     return cudaSuccess;
   };
-  auto run = [&](auto kern, size_t smem, long long chunk) -> cudaError_t {
+  auto run = [&](auto kern, size_t smem, long long chunk, int threads = kPeelThreads) -> cudaError_t {
     const unsigned grid = static_cast<unsigned>((nv + chunk - 1) / chunk);
-    return launch(kern, dim3(grid), kPeelThreads, smem, st, p, P, C, nv, static_cast<int>(chunk), first_wave,
+    return launch(kern, dim3(grid), threads, smem, st, p, P, C, nv, static_cast<int>(chunk), first_wave,
                   compensate_depth, rows);
   };
-  // The gathered form for tall codes, when one position's rows (at most
-  // sigma) over the CTA's columns fit a round of the term buffer.
+  // Tall codes, pipelined: slices of whole 128-byte lines, up to
+  // kTallColumns float4s, and supports of which a round holds eight (its rows
+  // are the threads that copy).  Beyond either the waves are wide enough for
+  // the forms below to be bound by their bytes: measured against them, n = 32,
+  // k = 24, b = 60, blocks of 8192 columns x 1 / 2 / 3 rows 79 / 140 / 242 us
+  // (the last in two walks) against 139 / 166 / 217, supports of 60 44 / 77
+  // against 43 / 69.
+  if (g.S >= kTallSources && 8 * g.sigma <= kCopyThreads) {
+    long long chunk = 0;
+    cudaError_t e = chunk_for(peel_tall_kernel, sizeof(TallSmem), &chunk, kTallThreads);
+    if (e != cudaSuccess) return e;
+    chunk = (chunk + 7) / 8 * 8;
+    if (chunk <= kTallColumns) return run(peel_tall_kernel, sizeof(TallSmem), chunk, kTallThreads);
+  }
+  // The gathered form, when one position's rows over the CTA's columns fit a
+  // round of the term buffer.
   auto go = [&](auto gather_kern, auto reg_kern) -> cudaError_t {
     long long chunk = 0;
     cudaError_t e;
-    if (g.S >= kGatherMinSources) {
+    if (g.S >= kTallSources) {
       if ((e = chunk_for(gather_kern, kGatherSmem, &chunk)) != cudaSuccess) return e;
       if (static_cast<long long>(std::max(1, g.sigma)) * chunk <= kTermCap) return run(gather_kern, kGatherSmem, chunk);
     }

@@ -50,8 +50,6 @@ constexpr int kThreads = 1024;
 constexpr size_t kSmemMax = 224 * 1024;  // dynamic shared memory of a plan's CTA (state + ready lists)
 constexpr size_t kSmemSmall = 16 * 1024;  // the same for the 256-thread CTA of small codes
 
-// Codes at least this tall have their peel lists filled by a second launch.
-constexpr int kFillSources = 1024;
 constexpr int kAffineMax = 64;   // columns of the affine table kept in shared memory
 constexpr int kRankMax = 256;    // sources of a round ordered by one warp comparing each with all
 
@@ -387,6 +385,7 @@ __device__ __forceinline__ void schedule_body(const DevGraph& g, const DevPlan& 
       p.order[i] = s;
       p.pl_res[i] = r;
       p.pl_ptr[i] = at;
+      if (S >= kTallSources) p.pos[s] = i;
       fill_position(cell_src + e0, deg, s, p.pl_list + at, 0, 1);
     }
   } else {
@@ -430,6 +429,7 @@ __device__ __forceinline__ void schedule_body(const DevGraph& g, const DevPlan& 
       if (i < i1) {
         const int r = p.pl_res[i];
         s = ord[i];
+        if (S >= kTallSources) p.pos[s] = i;
         e0 = cell_ptr[r];
         deg = cell_ptr[r + 1] - e0;
       }
@@ -496,7 +496,9 @@ __global__ void __launch_bounds__(256) fill_list_kernel(DevGraph g, DevPlan p) {
   const int n = p.ctr[CTR_NREC], step = gridDim.x * 8;
   for (int i = blockIdx.x * 8 + (threadIdx.x >> 5); i < n; i += step) {
     const int r = p.pl_res[i], e0 = g.cell_ptr[r];
-    fill_position(g.cell_src + e0, g.cell_ptr[r + 1] - e0, p.order[i], p.pl_list + p.pl_ptr[i], threadIdx.x & 31, 32);
+    const int s = p.order[i];
+    if ((threadIdx.x & 31) == 0) p.pos[s] = i;
+    fill_position(g.cell_src + e0, g.cell_ptr[r + 1] - e0, s, p.pl_list + p.pl_ptr[i], threadIdx.x & 31, 32);
   }
 }
 
@@ -548,7 +550,7 @@ cudaError_t launch_schedule(const DevGraph& g, const DevPlan& p, const uint8_t* 
   const bool small = state <= 4096;
   const int threads = small ? 256 : kThreads;
   const long long room = static_cast<long long>((small ? kSmemSmall : kSmemMax) / 4);
-  const bool fill_later = g.S >= kFillSources && part != 1;
+  const bool fill_later = g.S >= kTallSources && part != 1;
   cudaError_t e;
   if (sched_packable32(g.S, g.sigma) && state <= room) {
     const long long ints = sched_local(g, room) ? sched_local_ints(g) : std::min(room, state + 2LL * g.S);
