@@ -4,10 +4,11 @@
 // The subtraction is elementwise over the h x N block, so element i of C_s
 // depends only on element i of the blocks it reads.  Each CTA therefore owns
 // one contiguous slice of the block's float4 index range and walks the whole
-// schedule over that slice: a __syncthreads between waves is the only
-// synchronisation, with no grid barrier, flag or spin-wait.  Within a wave
-// the (source, float4) items of the slice are spread over the CTA's threads,
-// consecutive threads on consecutive float4s (128-bit coalesced accesses).
+// schedule over that slice: a barrier of the CTA between waves (or parts of
+// a wave) is the only synchronisation, with no grid barrier, flag or
+// spin-wait.  Within a wave the (source, float4) items of the slice are
+// spread over the CTA's threads, consecutive threads on consecutive float4s
+// (128-bit coalesced accesses).
 #include <algorithm>
 
 #include "device_common.cuh"
@@ -96,8 +97,8 @@ __device__ __forceinline__ void peel_item(const DevPlan& p, const float4* P4, fl
   C4[static_cast<long long>(s) * nv + v] = kComp ? two_sum_round(acc, err) : acc;
 }
 
-// Gathered waves (tall codes with thin blocks: hundreds of deep, narrow
-// waves).  The CTA copies every block element a wave reads -- each
+// Gathered waves (tall codes: hundreds of deep, narrow waves; those of a group,
+// and those past the limits of the pipelined form below).  The CTA copies every block element a wave reads -- each
 // position's product and all its subtrahends over the CTA's columns -- with
 // cp.async into shared memory at once, so that the wave costs one global
 // round trip instead of one per batch of kB subtrahends, with no registers

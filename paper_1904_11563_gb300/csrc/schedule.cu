@@ -86,8 +86,9 @@ __device__ __forceinline__ void fill_position(const int32_t* support, int degree
 }
 
 // kSmem: the per-cell words and per-source depths (the state every round
-// reads and updates) live in shared memory, followed by the ready ring (and, when the launch's smem_ints allow, the graph, the resolvers and the
-// order); otherwise in the plan's global arrays.
+// reads and updates) live in shared memory, followed by the ready ring (and,
+// when the launch's smem_ints allow, the graph, the resolvers and the order);
+// otherwise in the plan's global arrays.
 // cell_mask: the mask has one byte per cell (a processor whose output is
 // missing) instead of one per column (a node).
 // part: 0 = the whole plan; 1 = what the products need (surviving cells,
