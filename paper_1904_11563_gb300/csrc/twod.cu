@@ -73,25 +73,38 @@ b_ops_split_kernel(DevGraph g, const float* __restrict__ B, int K, int N, int w,
   const int f = blockIdx.x / nslices;
   const int n0 = (blockIdx.x - f * nslices) * 64, k0 = blockIdx.y * 64;
   {
+    // block by block, a thread's four rows in flight: with a row's blocks
+    // summed before the next row's loads this pass waited for each (4096 x
+    // 4096, 9 operands: 34.2 -> 24.4 us, floor 15.5; two blocks in flight, at
+    // 80 registers, 26.6)
     const int c4 = threadIdx.x & 15, r0 = threadIdx.x >> 4;
+    const int n = n0 + 4 * c4, rows = n < w ? min(64, K - k0) : 0;
+    const float* src = B + static_cast<long long>(k0 + r0) * N + n;
+    float4 v[4], x[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int j = g.b2_ptr[f]; j < g.b2_ptr[f + 1]; ++j) {
+      const float* from = src + static_cast<long long>(__ldg(g.b2_blk + j)) * w;
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (r0 + 16 * i < rows)
+          x[i] = __ldg(reinterpret_cast<const float4*>(from + static_cast<long long>(16 * i) * N));
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (r0 + 16 * i < rows) {
+          v[i].x += x[i].x;
+          v[i].y += x[i].y;
+          v[i].z += x[i].z;
+          v[i].w += x[i].w;
+        }
+    }
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const int r = r0 + 16 * i, k = k0 + r, n = n0 + 4 * c4;
-      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (k < K && n < w) {
-        for (int j = g.b2_ptr[f]; j < g.b2_ptr[f + 1]; ++j) {
-          const long long col = static_cast<long long>(__ldg(g.b2_blk + j)) * w + n;
-          const float4 x = __ldg(reinterpret_cast<const float4*>(B + static_cast<long long>(k) * N + col));
-          v.x += x.x;
-          v.y += x.y;
-          v.z += x.z;
-          v.w += x.w;
-        }
-      }
-      tile[r][4 * c4 + 0] = v.x;
-      tile[r][4 * c4 + 1] = v.y;
-      tile[r][4 * c4 + 2] = v.z;
-      tile[r][4 * c4 + 3] = v.w;
+      const int r = r0 + 16 * i;
+      tile[r][4 * c4 + 0] = v[i].x;
+      tile[r][4 * c4 + 1] = v[i].y;
+      tile[r][4 * c4 + 2] = v[i].z;
+      tile[r][4 * c4 + 3] = v[i].w;
     }
   }
   __syncthreads();
