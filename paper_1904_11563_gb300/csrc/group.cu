@@ -272,7 +272,6 @@ extern "C" int bpx_group_init(bpx_group* G, void* ws, size_t ws_bytes, bpx_strea
     g.bsplit_base = bs;
     bs += bpx::bsplit_ctas(J.N, J.K);
     g.enc_base = en;
-    g.enc_sblocks = static_cast<int>(bpx::enc_group_sblocks(static_cast<long long>(c->num_cells) * J.h, J.K));
     en += bpx::encode_group_ctas(static_cast<long long>(c->num_cells) * J.h, J.K);
     bpx::TcSpec& sp = G->specs[j];
     sp.p = g.p;
