@@ -536,6 +536,9 @@ b_colmax_kernel(const float* __restrict__ B, int K, int N, int ldb, uint32_t* bm
                 long long clear, bool early) {
   __shared__ float4 red[32][8];
   __shared__ float4 part[kColSplit][8];
+  // another CTA's shared memory may be stored to once that CTA has started:
+  // arrived here, waited for before the store, behind the column loads
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
   chain_begin_staging(early);
   const int c4 = threadIdx.x & 7, ph = threadIdx.x >> 3;
   const int n = blockIdx.x * 32 + 4 * c4;
@@ -562,6 +565,7 @@ b_colmax_kernel(const float* __restrict__ B, int K, int N, int ldb, uint32_t* bm
   };
   red[ph][c4] = m;
   __syncthreads();
+  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
   if (ph == 0) {
 #pragma unroll
     for (int q = 1; q < 32; ++q) more(red[q][c4]);
