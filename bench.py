@@ -495,8 +495,6 @@ def run_ours(args, wl):
             cfg = 0
             if prec in ("bf16x3", "bf16", "exact", "fp16x3"):
                 cfg, _tuned_ms = bpx.autotune(code, A, Bm, h, P, masks[0], ws, C=C)
-        if cfg == 0 and world > 1 and not fused:  # replicas: no TMA multicast (the named pair tiles)
-            cfg = {"fp16x3": 8020, "mxfp8": 16009}.get(prec, 8080)
         tuned[prec] = cfg
         opts = bpx.default_opts(gemm_config=cfg, compensate_depth=args.compensate_depth, fused_encode=fused)
         try:

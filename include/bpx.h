@@ -519,10 +519,8 @@ int bpx_group_autotune(bpx_group* group, const int* configs, int nconfigs, bpx_s
  * one CTA for products that fill few CTA pairs.  Precisions BPX_BF16,
  * BPX_BF16X3 and BPX_EXACT (which uses the tile shape, pairing, k-slice and
  * band, with its own exact segment length; its default is also 8080).
- * Tile codes 3, 4, 7 and 8 name no kernel (BPX_ERR_INVAL).  Only the default
- * (gemm_config 0) may load by TMA multicast, where two CTA pairs of a cluster
- * share rows of A; a caller that must not multicast names a configuration.
- * Synchronizes. */
+ * Tile codes 3, 4, 7 and 8 name no kernel (BPX_ERR_INVAL).  No kernel loads
+ * by TMA multicast.  Synchronizes. */
 int bpx_autotune(const bpx_code* code, const float* d_A, const float* d_B, int M, int N, int K, int h,
                  int precision, const uint8_t* d_erasure_mask, float* d_C, void* d_ws, size_t ws_bytes,
                  const int* configs, int nconfigs, bpx_stream stream, int* best_config, float* best_ms);

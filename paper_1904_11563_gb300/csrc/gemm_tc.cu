@@ -212,10 +212,7 @@ __device__ __forceinline__ TileRef locate(const TcJob* jobs, int njobs, long lon
 // a pair with the same B tile, computed by CTA-pair MMAs (cta_group::2,
 // M = 256): each CTA loads only its own A rows and its half of the B tile,
 // so a CTA's shared memory takes a third less traffic per MMA.  kPair == 0:
-// one CTA per tile.  kPair == 4: clusters of two such pairs on two adjacent
-// n-tiles of the same rows; each CTA loads half of its A rows and multicasts
-// them to its counterpart in the other pair, and a stage is free once both
-// pairs' MMAs have read it.
+// one CTA per tile.  (No variant loads by TMA multicast.)
 // kMode == kModeExact: exact-slice digit products (plain bf16 MMAs over the
 // digit planes, k-slices of the diagonal's digit pairs in sequence; FP32
 // segments exact by construction, promoted to int32 and stored to the
@@ -233,9 +230,8 @@ gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ t
                long long total_tiles, int group, int seg_kb) {
   constexpr bool kExact = kMode == kModeExact;
   constexpr bool k2D = kMode == kMode2D;
-  static_assert(kPair == 0 || kPair == 2 || (kPair == 4 && kParts < 3), "tiles are 1-CTA or CTA-pair MMAs, alone or two pairs");
-  constexpr bool k2Sm = kPair != 0;
-  constexpr bool kQuad = kPair == 4;
+  static_assert(kPair == 0 || kPair == 2, "tiles are 1-CTA or CTA-pair MMAs");
+  constexpr bool k2Sm = kPair == 2;
   constexpr bool kSplit = kParts >= 2;
   using St = Stage<kParts, k2Sm ? kBN / 2 : kBN, kBK>;  // a CTA pair holds half the B tile each
   constexpr int kTmemCols = 2 * kBN;  // two FP32 segment accumulators
@@ -250,19 +246,15 @@ gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ t
   const TcJob* jobs = table ? table : &single;
   const bool grouped = table != nullptr;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  constexpr int kClusterShift = kQuad ? 2 : kPair ? 1 : 0;
-  const uint32_t crank = kPair ? cluster_rank() : 0u;
-  const uint32_t rank = crank & 1u, leader = crank & ~1u;  // of the pair; its even CTA
-  const int side = static_cast<int>(crank >> 1);           // quad: which of the two n-tiles the pair takes
-  const int cid = static_cast<int>(blockIdx.x >> kClusterShift);
-  const int nclusters = static_cast<int>(gridDim.x >> kClusterShift);
-  const uint16_t pair_mask = static_cast<uint16_t>(3u << leader);
+  const uint32_t rank = kPair ? cluster_rank() : 0u;
+  const int cid = kPair ? static_cast<int>(blockIdx.x >> 1) : static_cast<int>(blockIdx.x);
+  const int nclusters = kPair ? static_cast<int>(gridDim.x >> 1) : static_cast<int>(gridDim.x);
 
   if (threadIdx.x == 0) {
     abort_flag = 0;
     for (int s = 0; s < kStages; ++s) {
       mbar_init(smem_u32(&full_bar[s]), 1);
-      mbar_init(smem_u32(&empty_bar[s]), kQuad ? 2 : 1);  // quad: both pairs' MMAs have read the shared A rows
+      mbar_init(smem_u32(&empty_bar[s]), 1);
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(smem_u32(&sfull_bar[a]), 1);
@@ -359,8 +351,7 @@ gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ t
           fenced = T.J;
         }
         const int m_cta = kPair ? 2 * T.m + static_cast<int>(rank) : T.m;
-        const int n_tile = kQuad ? 2 * T.n + side : T.n;
-        int ya = m_cta * BM, yb = n_tile * kBN, cur_term = -1;
+        int ya = m_cta * BM, yb = T.n * kBN, cur_term = -1;
         for (int q = 0; q < T.k_steps; ++q, ++kb_all) {
           const int s = kb_all % kStages;
           int xa = q * kBK, xb = q * kBK;
@@ -374,7 +365,7 @@ gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ t
             if (ti != cur_term) {
               cur_term = ti;
               ya = T.J->t2_a[T.tp + ti] * T.J->h + m_cta * BM;
-              yb = T.J->t2_b[T.tp + ti] * T.J->w2 + n_tile * kBN;
+              yb = T.J->t2_b[T.tp + ti] * T.J->w2 + T.n * kBN;
             }
             xa = xb = kb * kBK;
           }
@@ -389,18 +380,11 @@ gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ t
           if constexpr (k2Sm) {
             // both CTAs' copies count on the even CTA's barrier, armed there
             // for the two stages' bytes
-            const uint32_t fb0 = mapa_rank(fb, leader);
+            const uint32_t fb0 = mapa_rank(fb, 0);
             if (rank == 0) mbar_expect_tx(fb, 2 * St::kBytes);
             const int yh = yb + static_cast<int>(rank) * (kBN / 2);
-            if constexpr (kQuad) {  // half of the A rows, for this CTA and its counterpart in the other pair
-              const uint16_t both = static_cast<uint16_t>(5u << rank);
-              const uint32_t half = static_cast<uint32_t>(side) * (St::kA / 2);
-              tma_load_2d_pairs(base + St::kAhi + half, &T.J->map_ahi, fb0, xa, ya + side * (BM / 2), both);
-              if (kSplit) tma_load_2d_pairs(base + St::kAlo + half, &T.J->map_alo, fb0, xa, ya + side * (BM / 2), both);
-            } else {
-              tma_load_2d_pair(base + St::kAhi, &T.J->map_ahi, fb0, xa, ya);
-              if (kSplit) tma_load_2d_pair(base + St::kAlo, &T.J->map_alo, fb0, xa, ya);
-            }
+            tma_load_2d_pair(base + St::kAhi, &T.J->map_ahi, fb0, xa, ya);
+            if (kSplit) tma_load_2d_pair(base + St::kAlo, &T.J->map_alo, fb0, xa, ya);
             tma_load_2d_pair(base + St::kBhi, &T.J->map_bhi, fb0, xb, yh);
             if (kSplit) tma_load_2d_pair(base + St::kBlo, &T.J->map_blo, fb0, xb, yh);
             if (kParts == 3) {
@@ -507,13 +491,13 @@ gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ t
               }
             }
             if (k2Sm)
-              umma_commit_pair(smem_u32(&empty_bar[s]), kQuad ? 15 : 3);
+              umma_commit_pair(smem_u32(&empty_bar[s]));
             else
               umma_commit(smem_u32(&empty_bar[s]));
           }
           if (!ok) break;
           if (k2Sm)
-            umma_commit_pair(smem_u32(&sfull_bar[buf]), pair_mask);
+            umma_commit_pair(smem_u32(&sfull_bar[buf]));
           else
             umma_commit(smem_u32(&sfull_bar[buf]));
         }
@@ -564,14 +548,13 @@ gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ t
         __syncwarp();
         if (lane == 0) {
           if (k2Sm)  // the even CTA's MMA thread waits for both CTAs' drains
-            mbar_arrive_cluster(mapa_rank(smem_u32(&sempty_bar[buf]), leader));
+            mbar_arrive_cluster(mapa_rank(smem_u32(&sempty_bar[buf]), 0));
           else
             mbar_arrive(smem_u32(&sempty_bar[buf]));
         }
       }
       if (!ok) break;
       const TcJob& J = *T.J;
-      const int n_tile = kQuad ? 2 * T.n + side : T.n;
       const int r = (kPair ? 2 * T.m + static_cast<int>(rank) : T.m) * BM + row;
       if (k2D) {
         if (r < J.h) {  // row r of the cell's h x w block
@@ -583,7 +566,7 @@ gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ t
           } else {
             dst = J.products + (static_cast<long long>(T.cell) * J.h + r) * J.w2;
           }
-          const int n0 = n_tile * kBN + half * kCols;
+          const int n0 = T.n * kBN + half * kCols;
 #pragma unroll
           for (int q = 0; q < kCols / 4; ++q) {
             const int n = n0 + 4 * q;
@@ -595,7 +578,7 @@ gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ t
         const int ci = r / J.h;
         const int j = r - ci * J.h;
         const int cell = J.surv[ci];
-        const int n0 = n_tile * kBN + half * kCols;
+        const int n0 = T.n * kBN + half * kCols;
         if constexpr (kExact) {
           int32_t* dst = J.planes + T.dp * J.plane_stride + (static_cast<long long>(cell) * J.h + j) * J.N;
 #pragma unroll
@@ -737,24 +720,6 @@ int auto_bn(int parts, const RowsRange& range, int N, int K) {
   return bn[best];
 }
 
-// Whether a product over 256 x 256 tiles, n_tiles of them across, runs as clusters of two CTA pairs that share their A rows by TMA
-// multicast (kPair 4): a quarter less is read from L2 per MMA.  Only as the
-// default's choice, with an even number of n-tiles (none is left out) and no
-// more waves.  Benchmark GEMM 1874 -> 1773 us (split bf16), 2093 -> 1995 (split
-// fp16); two-dimensional bf16 at 4096 cubed 291 -> 262.  The exact slices'
-// digit products keep single pairs (7128 against 6904 us at 8192 cubed), and so
-// does FP32 in three parts (the same within 0.4 %).
-bool take_quads(const RowsRange& range, int n_tiles) {
-  if (n_tiles % 2 != 0) return false;
-  const long long pairs = std::max(1, num_sms() / 2), quads = std::max(1, num_sms() / 4);
-  auto waves = [&](long long slots, int n) {
-    return range.average([&](long long rows) {
-      return static_cast<double>(((rows + 255) / 256 * n + slots - 1) / slots);
-    });
-  };
-  return waves(quads, n_tiles / 2) <= waves(pairs, n_tiles);
-}
-
 // seg_kb: k-slices of kBK per TMEM accumulation segment.
 template <int kParts, int kStages, int kBN, int kPair, int kBK, int kMode = kModeRows>
 cudaError_t launch_variant(const TcJob& single, const TcJob* table, int njobs, long long total_tiles,
@@ -762,7 +727,7 @@ cudaError_t launch_variant(const TcJob& single, const TcJob* table, int njobs, l
   // 32-wide slices: 32 KB of slack after the stages, so that the descriptors
   // of the 64-byte swizzled layout can never reach past the allocation.
   // (a CTA of a cta_group::2 pair stages half the B tile)
-  using St = Stage<kParts, kPair != 0 ? kBN / 2 : kBN, kBK>;
+  using St = Stage<kParts, kPair == 2 ? kBN / 2 : kBN, kBK>;
   const size_t smem = static_cast<size_t>(kStages) * St::kBytes + 1024 + (kBK == 32 ? 32768 : 0);
   auto kern = gemm_tc_kernel<kParts, kStages, kBN, kPair, kBK, kMode>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
@@ -778,22 +743,21 @@ cudaError_t launch_variant(const TcJob& single, const TcJob* table, int njobs, l
   cfg.stream = st;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  constexpr int kCtas = kPair == 4 ? 4 : 2;
-  attr[0].val.clusterDim.x = kCtas;
+  attr[0].val.clusterDim.x = 2;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   // as many CTA pairs as can be resident at once (pairs must share a GPC)
-  cfg.gridDim = dim3(kCtas * (num_sms() / kCtas));
+  cfg.gridDim = dim3(2 * (num_sms() / 2));
   int resident = 0;
   if (cudaOccupancyMaxActiveClusters(&resident, kern, &cfg) != cudaSuccess || resident <= 0) {
     cudaGetLastError();
-    resident = num_sms() / kCtas;
+    resident = num_sms() / 2;
   }
-  resident = std::max(1, resident - (reserved_sms() + kCtas - 1) / kCtas);
+  resident = std::max(1, resident - (reserved_sms() + 1) / 2);
   const int clusters = static_cast<int>(std::min<long long>(total_tiles, resident));
-  cfg.gridDim = dim3(kCtas * clusters);
+  cfg.gridDim = dim3(2 * clusters);
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.numAttrs = chain_on() ? 2 : 1;
@@ -812,9 +776,6 @@ cudaError_t dispatch_bk(bool split3, int bn, int pair, const TcJob& single, cons
     if (bn == 64) return split3 ? BPX_LV(2, 4, 64, 0) : BPX_LV(1, 8, 64, 0);
   }
   // CTA-pair MMAs: a stage holds the CTA's A rows and half the B tile
-  if constexpr (kBK == BK) {
-    if (pair == 4) return split3 ? BPX_LV(2, 3, 256, 4) : BPX_LV(1, 6, 256, 4);
-  }
   if (pair == 2) return split3 ? BPX_LV(2, 3 * m, 256, 2) : BPX_LV(1, 6 * m, 256, 2);
   if (split3) return bn == 128 ? BPX_LV(2, 3 * m, 128, 0) : BPX_LV(2, 2 * m, 256, 0);
   return bn == 128 ? BPX_LV(1, 6 * m, 128, 0) : BPX_LV(1, 4 * m, 256, 0);
@@ -876,20 +837,19 @@ void decode_config(int config, int* group, int* seg_kb, int* bn, int* pair, int*
 namespace {
 
 bool tc_fill_job(TcJob* J, const DevPlan& p, const void* a_hi, const void* a_lo, const void* b_hi,
-                 const void* b_lo, int num_cells, int N, int K, int h, int bn, int pair, int bk,
+                 const void* b_lo, int num_cells, int N, int K, int h, int bn, bool pair, int bk,
                  float* products, float* C_direct, int32_t* info_out, const int32_t* a_exp = nullptr,
                  const int32_t* b_exp = nullptr, int ld = 0) {
   memset(J, 0, sizeof *J);
   const long long rows = static_cast<long long>(num_cells) * h;
   const int box_b = pair ? bn / 2 : bn;  // a paired CTA loads half of the B tile
-  const int box_a = pair == 4 ? BM / 2 : BM;  // two pairs share A: each CTA loads half of its rows for both
   const bool f16 = a_exp != nullptr;
-  if (!make_map(&J->map_ahi, a_hi, rows, K, box_a, bk, f16) || !make_map(&J->map_bhi, b_hi, N, K, box_b, bk, f16))
+  if (!make_map(&J->map_ahi, a_hi, rows, K, BM, bk, f16) || !make_map(&J->map_bhi, b_hi, N, K, box_b, bk, f16))
     return false;
   J->a_exp = a_exp;
   J->b_exp = b_exp;
   if (a_lo) {
-    if (!make_map(&J->map_alo, a_lo, rows, K, box_a, bk, f16) || !make_map(&J->map_blo, b_lo, N, K, box_b, bk, f16))
+    if (!make_map(&J->map_alo, a_lo, rows, K, BM, bk, f16) || !make_map(&J->map_blo, b_lo, N, K, box_b, bk, f16))
       return false;
   } else {
     J->map_alo = J->map_ahi;
@@ -908,7 +868,6 @@ bool tc_fill_job(TcJob* J, const DevPlan& p, const void* a_hi, const void* a_lo,
   J->h = h;
   J->m_tiles_max = static_cast<int>((rows + BM - 1) / BM);
   J->n_tiles = (N + bn - 1) / bn;
-  if (pair == 4) J->n_tiles = (J->n_tiles + 1) / 2;  // counted by two
   J->tile_base = 0;
   return true;
 }
@@ -968,7 +927,7 @@ cudaError_t launch_gemm_tc(const DevGraph& g, const DevPlan& p, const void* a_hi
   if (a_exp && config == 0) seg_kb = 2;
   if (config == 0) {
     bn = auto_bn(split3 ? 2 : 1, range, N, K);
-    pair = bn < 256 ? 0 : take_quads(range, (N + bn - 1) / bn) ? 4 : 2;
+    pair = bn < 256 ? 0 : 2;
   }
   TcJob J;
   if (!tc_fill_job(&J, p, a_hi, split3 ? a_lo : nullptr, b_hi, split3 ? b_lo : nullptr, num_cells, N, K, h,
@@ -1047,14 +1006,12 @@ cudaError_t launch_gemm_2d(const DevGraph& g, const DevPlan& p, const void* a_hi
   decode_config(config, &group, &seg_kb, &bn, &pair, &bk);
   TcJob J;
   memset(&J, 0, sizeof J);
-  const long long space = (h + 255) / 256 * 256LL * g.num_cells;  // every cell's rows, erased or not
-  if (config == 0 && take_quads({space, space, space}, (w + bn - 1) / bn)) pair = 4;
-  const int box_b = pair ? bn / 2 : bn, box_a = pair == 4 ? BM / 2 : BM;
+  const int box_b = pair ? bn / 2 : bn;
   const long long rows_a = static_cast<long long>(g.EA) * h, rows_b = static_cast<long long>(g.EB) * w;
-  if (!make_map(&J.map_ahi, a_hi, rows_a, K, box_a, bk) || !make_map(&J.map_bhi, b_hi, rows_b, K, box_b, bk))
+  if (!make_map(&J.map_ahi, a_hi, rows_a, K, BM, bk) || !make_map(&J.map_bhi, b_hi, rows_b, K, box_b, bk))
     return cudaErrorInvalidValue;
   if (split3) {
-    if (!make_map(&J.map_alo, a_lo, rows_a, K, box_a, bk) || !make_map(&J.map_blo, b_lo, rows_b, K, box_b, bk))
+    if (!make_map(&J.map_alo, a_lo, rows_a, K, BM, bk) || !make_map(&J.map_blo, b_lo, rows_b, K, box_b, bk))
       return cudaErrorInvalidValue;
   } else {
     J.map_alo = J.map_ahi;
@@ -1072,7 +1029,6 @@ cudaError_t launch_gemm_2d(const DevGraph& g, const DevPlan& p, const void* a_hi
   J.h = h;
   J.m_tiles_max = (h + BM - 1) / BM;
   J.n_tiles = (w + bn - 1) / bn;
-  if (pair == 4) J.n_tiles = (J.n_tiles + 1) / 2;
   J.t2_ptr = g.t2_ptr;
   J.t2_a = g.t2_a;
   J.t2_b = g.t2_b;

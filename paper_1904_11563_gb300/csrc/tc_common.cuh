@@ -230,18 +230,6 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap
       : "memory");
 }
 
-// The same into every CTA of `mask` (a cluster of two pairs): the tile lands
-// at dst's offset in each, and each copy's bytes count on the barrier at
-// cluster_bar's offset in that CTA's own pair's even CTA.
-__device__ __forceinline__ void tma_load_2d_pairs(uint32_t dst, const CUtensorMap* map, uint32_t cluster_bar, int x,
-                                                  int y, uint16_t mask) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-      ".multicast::cluster [%0], [%1, {%2, %3}], [%4], %5;" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(cluster_bar), "h"(mask)
-      : "memory");
-}
-
 // kind::f16, M = 256 (128 rows in each CTA of the pair), N = kBN.
 template <int kBN>
 __host__ __device__ constexpr uint32_t idesc_bf16_pair() {
@@ -271,11 +259,10 @@ __device__ __forceinline__ void umma_bf16_pair(uint32_t tmem_d, uint64_t a, uint
       "l"(a), "l"(b), "r"(idesc_bf16_pair<kBN>()), "r"(acc));
 }
 
-// Arrives on the barrier in every CTA of `mask` (default: a cluster that is one pair).
-__device__ __forceinline__ void umma_commit_pair(uint32_t bar, uint16_t mask = 3) {
+__device__ __forceinline__ void umma_commit_pair(uint32_t bar) {
   asm volatile(
       "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
-      "h"(mask)
+      "h"(static_cast<uint16_t>(3))
       : "memory");
 }
 
