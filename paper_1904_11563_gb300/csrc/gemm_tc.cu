@@ -130,6 +130,13 @@ struct TileRef {
 // digit products, and the two-dimensional scheme's per-cell term products.
 enum { kModeRows = 0, kModeExact = 1, kMode2D = 2 };
 
+// Dynamic shared memory past a kernel's stages: 32-wide slices take 32 KB of
+// slack, so that the descriptors of the 64-byte swizzled layout can never
+// reach past the allocation; a grouped launch of at most live_jobs jobs takes
+// its table of live tiles.
+constexpr int slack_bytes(int bk) { return bk == 32 ? 32768 : 0; }
+constexpr int live_jobs(int bk) { return bk == BK ? 1024 : 64; }
+
 // live_mc >= 0: a single job whose surviving row count is already known; its
 // tile space then holds the live m-tiles only (no skipped tiles inside the
 // rasterisation bands).  pair: the tile space counts pairs of vertically
@@ -141,9 +148,9 @@ enum { kModeRows = 0, kModeExact = 1, kMode2D = 2 };
 // other.
 // live_bases / live_rows: a grouped launch's jobs' first tile in the space of
 // live tiles and their surviving coded rows (shared memory), or null.
+template <bool kGrouped>
 __device__ __forceinline__ TileRef locate(const TcJob* jobs, int njobs, long long t, int group, int live_mc,
-                                          bool pair, int bk, int mode = kModeRows, const int* live_bases = nullptr,
-                                          const int* live_rows = nullptr) {
+                                          bool pair, int bk, int mode, const int* live_bases, const int* live_rows) {
   const bool exact = mode == kModeExact;
   if (mode == kMode2D) {
     // one job; tile space = cells (most terms first) x m-units x n-tiles,
@@ -166,17 +173,23 @@ __device__ __forceinline__ TileRef locate(const TcJob* jobs, int njobs, long lon
     R.live = J.cnt[R.cell] >= 0;
     return R;
   }
-  int lo = 0, hi = njobs - 1;
-  while (lo < hi) {  // last job with tile_base <= t
-    const int mid = (lo + hi + 1) >> 1;
-    if ((live_bases ? live_bases[mid] : jobs[mid].tile_base) <= t) lo = mid;
-    else hi = mid - 1;
+  int lo = 0;
+  if constexpr (kGrouped) {  // last job with tile_base <= t
+    int hi = njobs - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if ((live_bases ? live_bases[mid] : jobs[mid].tile_base) <= t) lo = mid;
+      else hi = mid - 1;
+    }
   }
   TileRef R;
   R.J = &jobs[lo];
   const TcJob& J = *R.J;
-  const int lt0 = static_cast<int>(t - (live_bases ? live_bases[lo] : J.tile_base));
-  if (live_rows) live_mc = live_rows[lo];
+  int lt0 = static_cast<int>(t);
+  if constexpr (kGrouped) {
+    lt0 = static_cast<int>(t - (live_bases ? live_bases[lo] : J.tile_base));
+    if (live_rows) live_mc = live_rows[lo];
+  }
   R.Mc = live_mc >= 0 ? live_mc : J.ctr[CTR_NSURV] * J.h;
   int m_units = live_mc >= 0 ? (live_mc + BM - 1) / BM : J.m_tiles_max;
   if (pair) m_units = (m_units + 1) / 2;
@@ -224,7 +237,11 @@ __device__ __forceinline__ TileRef locate(const TcJob* jobs, int njobs, long lon
 // a3 b1), the five small ones of a segment before a1 b1, so that only a
 // segment's few a1 b1 adds truncate at the accumulator's full magnitude.  The
 // dropped products are below 2^-25 of a b each, half an FP32 rounding.
-template <int kParts, int kStages, int kBN, int kPair, int kBK, int kMode = kModeRows>
+// kGrouped: a table of jobs instead of `single`.  A kernel of its own: with the
+// table of live tiles in the same kernel a single plain bf16 product of 8192
+// cubed took 966 us, as two kernels 888 (the registers and the code of the
+// loops change with it; split operands, 2130, do not show it).
+template <int kParts, int kStages, int kBN, int kPair, int kBK, int kMode, bool kGrouped>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ table, int njobs,
                long long total_tiles, int group, int seg_kb) {
@@ -243,8 +260,8 @@ gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ t
   __shared__ uint32_t tmem_base_sh;
   __shared__ volatile int abort_flag;
 
-  const TcJob* jobs = table ? table : &single;
-  const bool grouped = table != nullptr;
+  static_assert(!kGrouped || (kMode == kModeRows && kParts < 3), "groups take the coded GEMM of one or two parts");
+  const TcJob* jobs = kGrouped ? table : &single;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = kPair ? cluster_rank() : 0u;
   const int cid = kPair ? static_cast<int>(blockIdx.x >> 1) : static_cast<int>(blockIdx.x);
@@ -285,44 +302,45 @@ gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ t
   const uint32_t tmem_base = tmem_base_sh;
 
   chain_wait();  // the plan and the staged operands
-  // A grouped launch's tile space holds the live tiles only: the tiles past a
-  // job's surviving rows (a quarter of a mixed batch's) would leave the static
-  // dealing of tiles to CTAs uneven, and each would cost its job search.
-  // 48-job batch: GEMM 1856 -> 1640 us.
-  constexpr int kLiveJobs = (kMode != kModeRows || kParts == 3) ? 1 : kBK == BK ? 1024 : 64;
-  __shared__ int live_bases[kLiveJobs + 1], live_rows[kLiveJobs];
-  const bool compact = kLiveJobs > 1 && grouped && njobs <= kLiveJobs;
-  if (compact) {
-    for (int j = threadIdx.x; j < njobs; j += kThreads) live_rows[j] = jobs[j].ctr[CTR_NSURV] * jobs[j].h;
-    __syncthreads();
-    if (warp == 0) {
-      int run = 0;
-      for (int b = 0; b < njobs; b += 32) {
-        const int j = b + lane;
-        int tiles = 0;
-        if (j < njobs) {
-          const int units = (live_rows[j] + BM - 1) / BM;
-          tiles = (kPair ? (units + 1) / 2 : units) * jobs[j].n_tiles;
-        }
-        int x = tiles;
+  int* live_bases = nullptr;
+  int* live_rows = nullptr;
+  int live_mc = -1;
+  if constexpr (kGrouped) {
+    // The tile space of up to live_jobs jobs holds the live tiles only: the
+    // tiles past a job's surviving rows (a quarter of a mixed batch's) would
+    // leave the static dealing of tiles to CTAs uneven, and each would cost its
+    // job search.  48-job batch: GEMM 1856 -> 1640 us.
+    if (njobs <= live_jobs(kBK)) {
+      live_rows = reinterpret_cast<int*>(smem + kStages * St::kBytes + slack_bytes(kBK));
+      live_bases = live_rows + njobs;
+      for (int j = threadIdx.x; j < njobs; j += kThreads) live_rows[j] = jobs[j].ctr[CTR_NSURV] * jobs[j].h;
+      __syncthreads();
+      if (warp == 0) {
+        int run = 0;
+        for (int b = 0; b < njobs; b += 32) {
+          const int j = b + lane;
+          int tiles = 0;
+          if (j < njobs) {
+            const int units = (live_rows[j] + BM - 1) / BM;
+            tiles = (kPair ? (units + 1) / 2 : units) * jobs[j].n_tiles;
+          }
+          int x = tiles;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int y = __shfl_up_sync(0xffffffffu, x, o);
-          if (lane >= o) x += y;
+          for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+          }
+          if (j < njobs) live_bases[j] = run + x - tiles;
+          run += __shfl_sync(0xffffffffu, x, 31);
         }
-        if (j < njobs) live_bases[j] = run + x - tiles;
-        run += __shfl_sync(0xffffffffu, x, 31);
+        if (lane == 0) live_bases[njobs] = run;
       }
-      if (lane == 0) live_bases[njobs] = run;
+      __syncthreads();
+      total_tiles = live_bases[njobs];
     }
-    __syncthreads();
-    total_tiles = live_bases[njobs];
-  }
-  const int* lb = compact ? live_bases : nullptr;
-  const int* lr = compact ? live_rows : nullptr;
-  // A single job reads its surviving row count once and walks live tiles only.
-  const int live_mc = grouped ? -1 : single.ctr[CTR_NSURV] * single.h;
-  if (!grouped && !k2D) {
+  } else if constexpr (!k2D) {
+    // A single job reads its surviving row count once and walks live tiles only.
+    live_mc = single.ctr[CTR_NSURV] * single.h;
     int units = (live_mc + BM - 1) / BM;
     if (kPair) units = (units + 1) / 2;
     total_tiles = static_cast<long long>(units) * single.n_tiles * (kExact ? single.ex_np : 1);
@@ -339,9 +357,9 @@ gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ t
       for (long long j = 0; ok; ++j) {
         const long long t = snake(j, cid, nclusters);
         if (t >= total_tiles) break;
-        const TileRef T = locate(jobs, njobs, t, group, live_mc, kPair, kBK, kMode, lb, lr);
+        const TileRef T = locate<kGrouped>(jobs, njobs, t, group, live_mc, kPair, kBK, kMode, live_bases, live_rows);
         if (!T.live) continue;
-        if (grouped && T.J != fenced) {
+        if (kGrouped && T.J != fenced) {
           tensormap_acquire(&T.J->map_ahi);
           tensormap_acquire(&T.J->map_bhi);
           if (kSplit) {
@@ -421,7 +439,7 @@ gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ t
       for (long long j = 0; ok; ++j) {
         const long long t = snake(j, cid, nclusters);
         if (t >= total_tiles) break;
-        const TileRef T = locate(jobs, njobs, t, group, live_mc, kPair, kBK, kMode, lb, lr);
+        const TileRef T = locate<kGrouped>(jobs, njobs, t, group, live_mc, kPair, kBK, kMode, live_bases, live_rows);
         if (!T.live) continue;
         const int n_segs = (T.k_steps + seg_kb - 1) / seg_kb;
         // operand format: fp16 for a split-fp16 job, else bf16
@@ -514,7 +532,7 @@ gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ t
     for (long long j = 0; ok; ++j) {
       const long long t = snake(j, cid, nclusters);
       if (t >= total_tiles) break;
-      const TileRef T = locate(jobs, njobs, t, group, live_mc, kPair, kBK, kMode, lb, lr);
+      const TileRef T = locate<kGrouped>(jobs, njobs, t, group, live_mc, kPair, kBK, kMode, live_bases, live_rows);
       if (!T.live) continue;
       const int n_segs = (T.k_steps + seg_kb - 1) / seg_kb;
       float accum[kCols];
@@ -721,16 +739,17 @@ int auto_bn(int parts, const RowsRange& range, int N, int K) {
 }
 
 // seg_kb: k-slices of kBK per TMEM accumulation segment.
-template <int kParts, int kStages, int kBN, int kPair, int kBK, int kMode = kModeRows>
+template <int kParts, int kStages, int kBN, int kPair, int kBK, int kMode = kModeRows, bool kGrouped = false>
 cudaError_t launch_variant(const TcJob& single, const TcJob* table, int njobs, long long total_tiles,
                            int group, int seg_kb, cudaStream_t st) {
-  // 32-wide slices: 32 KB of slack after the stages, so that the descriptors
-  // of the 64-byte swizzled layout can never reach past the allocation.
   // (a CTA of a cta_group::2 pair stages half the B tile)
   using St = Stage<kParts, kPair == 2 ? kBN / 2 : kBN, kBK>;
-  const size_t smem = static_cast<size_t>(kStages) * St::kBytes + 1024 + (kBK == 32 ? 32768 : 0);
-  auto kern = gemm_tc_kernel<kParts, kStages, kBN, kPair, kBK, kMode>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  auto table_bytes = [](int n) { return (2 * static_cast<size_t>(n) + 1) * sizeof(int); };
+  size_t smem = static_cast<size_t>(kStages) * St::kBytes + 1024 + slack_bytes(kBK);
+  const size_t most = smem + (kGrouped ? table_bytes(live_jobs(kBK)) : 0);  // (one value for every thread's launches)
+  if (kGrouped && njobs <= live_jobs(kBK)) smem += table_bytes(njobs);
+  auto kern = gemm_tc_kernel<kParts, kStages, kBN, kPair, kBK, kMode, kGrouped>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(most));
   if (e != cudaSuccess) return e;
   if (total_tiles <= 0) return cudaSuccess;
   if (kPair == 0) {
@@ -764,15 +783,15 @@ cudaError_t launch_variant(const TcJob& single, const TcJob* table, int njobs, l
   return cudaLaunchKernelEx(&cfg, kern, single, table, njobs, total_tiles, group, seg_kb);
 }
 
-template <int kBK, int kMode = kModeRows>
+template <int kBK, int kMode = kModeRows, bool kGrouped = false>
 cudaError_t dispatch_bk(bool split3, int bn, int pair, const TcJob& single, const TcJob* table, int njobs,
                         long long total_tiles, int group, int seg_kb, cudaStream_t st) {
   constexpr int m = BK / kBK;  // stages scale up as slices shrink
   seg_kb *= m;                 // configs count segments in 64-wide k-blocks
 #define BPX_LV(PARTS, STAGES, BN, PAIR) \
-  launch_variant<PARTS, STAGES, BN, PAIR, kBK, kMode>(single, table, njobs, total_tiles, group, seg_kb, st)
+  launch_variant<PARTS, STAGES, BN, PAIR, kBK, kMode, kGrouped>(single, table, njobs, total_tiles, group, seg_kb, st)
   // (64-wide tiles: only as the default's choice for a small product)
-  if constexpr (kBK == BK && kMode == kModeRows) {
+  if constexpr (kBK == BK && kMode == kModeRows && !kGrouped) {
     if (bn == 64) return split3 ? BPX_LV(2, 4, 64, 0) : BPX_LV(1, 8, 64, 0);
   }
   // CTA-pair MMAs: a stage holds the CTA's A rows and half the B tile
@@ -807,6 +826,11 @@ cudaError_t dispatch(bool split3, int bn, int pair, int bk, const TcJob& single,
     if (bk == 32)
       return dispatch_bk<32, kMode2D>(split3, bn, pair, single, table, njobs, total_tiles, group, seg_kb, st);
     return dispatch_bk<64, kMode2D>(split3, bn, pair, single, table, njobs, total_tiles, group, seg_kb, st);
+  }
+  if (table) {
+    if (bk == 32)
+      return dispatch_bk<32, kModeRows, true>(split3, bn, pair, single, table, njobs, total_tiles, group, seg_kb, st);
+    return dispatch_bk<64, kModeRows, true>(split3, bn, pair, single, table, njobs, total_tiles, group, seg_kb, st);
   }
   if (bk == 32) return dispatch_bk<32>(split3, bn, pair, single, table, njobs, total_tiles, group, seg_kb, st);
   return dispatch_bk<64>(split3, bn, pair, single, table, njobs, total_tiles, group, seg_kb, st);
