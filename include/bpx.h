@@ -357,6 +357,11 @@ int bpx_peel_decode(const bpx_code* code, const float* d_products, const uint8_t
  * FP64 decoded integers could lose exactness. */
 int bpx_exact_params(const bpx_code* code, int K, int32_t* out);
 
+/* The form that the products of this shape take when gemm_config is 0 (host
+ * only): *tile = 0 for the CUDA cores (small BPX_FP32 products), else the
+ * width of a tensor-core tile: 256 (CTA pairs), 128 or 64. */
+int bpx_default_tile(const bpx_code* code, int precision, int N, int K, int h, int32_t* tile);
+
 /* a4 for BPX_EXACT: d_planes = the S int32 product planes written by
  * bpx_coded_products(..., BPX_EXACT, ...) (plane d at d_planes + d num_cells h N,
  * each num_cells h N, row-major h x N per cell); the scales and an int64 copy

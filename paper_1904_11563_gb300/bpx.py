@@ -90,6 +90,7 @@ def lib():
                                    ct.POINTER(Opts), vp]),
         "bpx_peel_decode": (i, [vp, f32p, vp, i, i, f32p, i, ct.POINTER(Opts), vp, sz, vp, vp]),
         "bpx_exact_params": (i, [vp, i, ct.POINTER(ct.c_int32)]),
+        "bpx_default_tile": (i, [vp, i, i, i, i, ct.POINTER(ct.c_int32)]),
         "bpx_peel_decode_exact": (i, [vp, vp, vp, i, i, f32p, ct.POINTER(Opts), vp, sz, vp, vp]),
         "bpx_coded_matmul": (i, [vp, f32p, f32p, i, i, i, i, i, vp, f32p, ct.POINTER(Opts),
                                  vp, sz, vp, vp]),
@@ -367,6 +368,14 @@ def first_decodable(code: Code, order):
     _check(lib().bpx_first_decodable(code.handle, order.ctypes.data_as(ct.c_void_p), len(order),
                                      rec.ctypes.data_as(ct.c_void_p), ct.byref(first)))
     return int(first.value), rec
+
+
+def default_tile(code: Code, precision, N, K, h) -> int:
+    """The products' form at gemm_config 0 (host only): 0 = CUDA cores, else
+    the width of a tensor-core tile."""
+    tile = ct.c_int32()
+    _check(lib().bpx_default_tile(code.handle, precision, N, K, h, ct.byref(tile)))
+    return tile.value
 
 
 def exact_params(code: Code, K) -> dict:

@@ -83,6 +83,23 @@ extern "C" size_t bpx_workspace_info_offset(const bpx_code* c) {
   return bpx::ws_layout(c, 0, 0, 0, 1, BPX_FP32).p_info;
 }
 
+extern "C" int bpx_default_tile(const bpx_code* c, int precision, int N, int K, int h, int32_t* tile) {
+  bpx::clear_error();
+  if (!c || !tile) return fail(BPX_ERR_INVAL, "bpx_default_tile: NULL argument");
+  if (int rc = check_shapes(c, 0, N, K, h)) return rc;
+  const bpx::RowsRange range = bpx::rows_range(c, h);
+  switch (precision) {
+    case BPX_FP32: *tile = bpx::f32_on_tensor_cores(c, N, K, h) ? bpx::auto_bn(bpx::kTileF32, range, N, K) : 0; break;
+    case BPX_BF16: *tile = bpx::auto_bn(bpx::kTileBf16, range, N, K); break;
+    case BPX_BF16X3: *tile = bpx::auto_bn(bpx::kTileBf16x3, range, N, K); break;
+    case BPX_FP16X3: *tile = bpx::auto_bn(bpx::kTileF16x3, range, N, K); break;
+    case BPX_MXFP8:
+    case BPX_EXACT: *tile = 256; break;
+    default: return fail(BPX_ERR_INVAL, "bpx_default_tile: precision %d", precision);
+  }
+  return BPX_OK;
+}
+
 extern "C" int bpx_workspace_init(const bpx_code* c, void* ws, size_t ws_bytes, bpx_stream stream) {
   bpx::clear_error();
   const bpx::WsLayout L = bpx::ws_layout(c ? c : nullptr, 0, 0, 0, 1, BPX_FP32);

@@ -31,6 +31,7 @@ struct bpx_code {
   // + j] z + affine[2 n + j] l -- that table (else empty).
   std::vector<uint32_t> word0;
   std::vector<int32_t> affine;
+  int32_t live_cells[8] = {};  // cells that masks of e erased columns leave: eight quantiles over the masks
 };
 
 namespace bpx {
@@ -90,20 +91,19 @@ int exact_params(const bpx_code* c, int K, ExactParams* P);
 void exact_pair_digits(const bpx_code* c, ExactParams* P);
 
 // Coded rows that masks of e erased columns leave (launch heuristics; the
-// mask itself is on the device): the fewest, the mean, the most.
+// mask itself is on the device): the mean, and eight quantiles over the masks.
 struct RowsRange {
-  long long least, mean, most;
-  // the mean over the range of f(rows): least, mean, most and the midpoints between
-  template <typename F>
-  double average(F f) const {
-    return (f(least) + f((least + mean) / 2) + f(mean) + f((mean + most) / 2) + f(most)) / 5.0;
-  }
+  long long mean, rows[8];
 };
 RowsRange rows_range(const bpx_code* c, int h);
 
 // Whether BPX_FP32 products of this shape run on the tensor cores (three bf16
 // parts per operand, six products) rather than on the CUDA cores.
 bool f32_on_tensor_cores(const bpx_code* c, int N, int K, int h);
+
+// The tile that a product takes when its caller names none (gemm_tc.cu).
+enum TileKind { kTileBf16 = 0, kTileBf16x3, kTileF32, kTileF16x3 };
+int auto_bn(TileKind kind, const RowsRange& range, int N, int K);
 
 // twod: the two-dimensional scheme (products are h x (N / k) blocks, operand
 // staging holds the summed A and B operands of the code's factored cells).
@@ -137,6 +137,9 @@ constexpr int sched_count_bits(int sigma) { return sched_id_bits(sigma) + 1; }
 
 // Fills the code's schedule tables (word0, affine).
 void build_schedule_tables(bpx_code* c);
+
+// Fills live_cells.
+void count_live_cells(bpx_code* c);
 
 // Factors every cell for the two-dimensional scheme (fills the t2_* / a2_* /
 // b2_* arrays of the code).

@@ -77,6 +77,46 @@ void finish_code(bpx_code* c, const std::vector<std::vector<int32_t>>& cells,
   c->eps = static_cast<double>(tot) / (static_cast<double>(c->k) * c->b) - 1.0;
   build_terms_2d(c);
   build_schedule_tables(c);
+  count_live_cells(c);
+}
+
+// Every mask of e erased columns where there are at most kMasks, else kMasks
+// drawn ones (a fixed sequence: the same code always gives the same counts).
+void count_live_cells(bpx_code* c) {
+  constexpr int kMasks = 4096;
+  const int n = c->n, e = c->e > 0 && c->e < c->n ? c->e : 0;
+  auto height = [&](int j) { return c->col_ptr[j + 1] - c->col_ptr[j]; };
+  double masks = 1.0;
+  for (int i = 0; i < e; ++i) masks = masks * (n - i) / (i + 1);
+  std::vector<int32_t> left, pick(n);
+  for (int j = 0; j < n; ++j) pick[j] = j;
+  if (masks < kMasks + 0.5) {
+    std::vector<int> at(e);
+    for (int i = 0; i < e; ++i) at[i] = i;
+    for (;;) {
+      int cells = c->num_cells;
+      for (int j : at) cells -= height(j);
+      left.push_back(cells);
+      int i = e - 1;
+      while (i >= 0 && at[i] == n - e + i) --i;
+      if (i < 0) break;
+      ++at[i];
+      for (++i; i < e; ++i) at[i] = at[i - 1] + 1;
+    }
+  } else {
+    uint64_t x = 1;
+    for (int m = 0; m < kMasks; ++m) {
+      int cells = c->num_cells;
+      for (int i = 0; i < e; ++i) {
+        x = x * 6364136223846793005ull + 1442695040888963407ull;
+        std::swap(pick[i], pick[i + static_cast<int>((x >> 33) % static_cast<uint64_t>(n - i))]);
+        cells -= height(pick[i]);
+      }
+      left.push_back(cells);
+    }
+  }
+  std::sort(left.begin(), left.end());
+  for (int q = 0; q < 8; ++q) c->live_cells[q] = left[(2 * q + 1) * left.size() / 16];
 }
 
 // word0 and affine (see bpx_code).
@@ -395,19 +435,10 @@ void exact_pair_digits(const bpx_code* c, ExactParams* P) {
 }
 
 RowsRange rows_range(const bpx_code* c, int h) {
-  std::vector<long long> cells;
-  for (int j = 0; j < c->n; ++j) cells.push_back(c->col_ptr[j + 1] - c->col_ptr[j]);
-  std::sort(cells.begin(), cells.end());
   const int e = c->e > 0 && c->e < c->n ? c->e : 0;
-  const long long all = c->num_cells;
-  RowsRange r{all, all * (c->n - e) / c->n, all};
-  for (int j = 0; j < e; ++j) {
-    r.most -= cells[j];
-    r.least -= cells[c->n - 1 - j];
-  }
-  r.least *= h;
-  r.mean *= h;
-  r.most *= h;
+  RowsRange r;
+  r.mean = static_cast<long long>(c->num_cells) * (c->n - e) / c->n * h;
+  for (int q = 0; q < 8; ++q) r.rows[q] = static_cast<long long>(c->live_cells[q]) * h;
   return r;
 }
 

@@ -703,41 +703,6 @@ int tile_pair(int config) {
 }
 int tile_bk(int config) { return (config % 10) >= 5 ? 32 : 64; }
 
-// The tile of a product whose caller names none (gemm_config 0): 256 x 256 of
-// a CTA pair, or 128 x 128 / 128 x 64 of one CTA where the pairs would leave
-// SMs idle (the same K segments, so the same bits).  Time = waves x k-blocks x
-// time per k-block + the last tile's drain, in units of a pair tile's
-// k-block.  Measured, split bf16, us per k-block of one tile on every SM and
-// drain: 1.03 and 8 (pair), 0.675 and 5.5 (128), 0.67 and 3.5 (64): a narrower
-// tile reads as much of A from shared memory per MMA.  GEMM, pair against the
-// tile chosen (coded rows x K x N): 568 x 256 x 128 16.3 -> 10.2 us, 1136 x
-// 1416 x 1100 32.8 -> 26.6, 4544 x 4096 x 512 67.5 -> 49.3; 2272 x 1992 x 2044
-// keeps pairs, 44 against 60.  The waves are averaged over the rows that masks
-// of the code's e erasures leave.
-int auto_bn(int parts, const RowsRange& range, int N, int K) {
-  const long long sms = std::max(1, num_sms());
-  const int kb = (K + BK - 1) / BK;
-  const double scale = parts == 1 ? 2.0 : parts == 3 ? 0.5 : 1.0;  // drains against a k-block's MMAs
-  const int bn[3] = {256, 128, 64};
-  const double step[3] = {1.0, 0.655, parts == 1 ? 0.68 : 0.65}, drain[3] = {7.8 * scale, 5.3 * scale, 3.4 * scale};
-  int best = 0;
-  double least = 0.0;
-  for (int i = 0; i < 3; ++i) {
-    const int m = i == 0 ? 256 : 128;
-    const long long slots = i == 0 ? std::max(1LL, sms / 2) : sms;
-    const double waves = range.average([&](long long rows) {
-      const long long tiles = (rows + m - 1) / m * ((N + bn[i] - 1) / bn[i]);
-      return static_cast<double>((tiles + slots - 1) / slots);
-    });
-    const double t = waves * kb * step[i] + drain[i];
-    if (i == 0 || t < least) {
-      least = t;
-      best = i;
-    }
-  }
-  return bn[best];
-}
-
 // seg_kb: k-slices of kBK per TMEM accumulation segment.
 template <int kParts, int kStages, int kBN, int kPair, int kBK, int kMode = kModeRows, bool kGrouped = false>
 cudaError_t launch_variant(const TcJob& single, const TcJob* table, int njobs, long long total_tiles,
@@ -933,6 +898,53 @@ size_t tc_job_bytes() { return sizeof(TcJob); }
 
 bool gemm_config_ok(int config) { return tile_valid(config); }
 
+// The tile of a product whose caller names none (gemm_config 0): 256 x 256 of
+// a CTA pair, or 128 x 128 / 128 x 64 of one CTA where the pairs would leave
+// SMs idle (the same K segments, so the same bits).  Time = waves x (k-blocks x
+// time per k-block + drain), the times fitted to 470 products each of 64 to
+// 4096 columns, K 128 to 8192, 500 to 7300 coded rows (relative residual 8 %
+// on pairs, 4 % on the others).  The rows depend on the mask, which is on the
+// device: the least mean over eight quantiles of the code's masks, and no form
+// that at one of them takes a tenth longer than pairs would (two waves of
+// narrow tiles at the mask's rows, where another mask leaves one).
+// GEMM, pair against the tile chosen (coded rows x K x N, split bf16): 568 x
+// 256 x 128 16.3 -> 10.2 us, 1136 x 1416 x 1100 32.8 -> 26.6, 4544 x 4096 x 512
+// 67.5 -> 49.3.  2496 x 8192 x 1024 keeps pairs: 117 us against 156 (128 x 128,
+// two waves; 122 against 184 in split fp16, 230 against 328 in FP32).
+int auto_bn(TileKind kind, const RowsRange& range, int N, int K) {
+  struct Cost {
+    double drain, step;  // us a wave, us a k-block of 64
+  };
+  static constexpr Cost kCost[4][3] = {{{6.8, 0.337}, {2.4, 0.323}, {1.1, 0.313}},    // bf16
+                                       {{5.7, 0.800}, {2.8, 0.556}, {1.1, 0.504}},    // split bf16
+                                       {{6.0, 1.625}, {2.4, 1.205}, {1.0, 1.040}},    // FP32 in three parts
+                                       {{13.0, 0.816}, {4.8, 0.648}, {2.1, 0.608}}};  // split fp16 (128-wide segments)
+  const long long sms = std::max(1, num_sms());
+  const int kb = (K + BK - 1) / BK;
+  const int bn[3] = {256, 128, 64};
+  auto time = [&](int i, long long rows) {
+    const long long m = i == 0 ? 256 : 128, slots = i == 0 ? std::max(1LL, sms / 2) : sms;
+    const long long tiles = (rows + m - 1) / m * ((N + bn[i] - 1) / bn[i]);
+    return static_cast<double>((tiles + slots - 1) / slots) * (kCost[kind][i].drain + kb * kCost[kind][i].step);
+  };
+  int best = 0;
+  double least = 0.0;
+  for (int i = 0; i < 3; ++i) {
+    double sum = 0.0;
+    bool ok = true;
+    for (long long rows : range.rows) {
+      const double t = time(i, rows);
+      sum += t;
+      ok = ok && t <= 1.1 * time(0, rows);
+    }
+    if (i == 0 || (ok && sum < least)) {
+      least = sum;
+      best = i;
+    }
+  }
+  return bn[best];
+}
+
 cudaError_t launch_gemm_tc(const DevGraph& g, const DevPlan& p, const void* a_hi, const void* a_lo,
                            const void* b_hi, const void* b_lo, int num_cells, int N, int K, int h,
                            bool split3, const RowsRange& range, float* products, float* C_direct, int config,
@@ -950,7 +962,7 @@ cudaError_t launch_gemm_tc(const DevGraph& g, const DevPlan& p, const void* a_hi
   // (propagation factor 32) 256-wide segments 9.2e-6, 128-wide 7.9e-6.
   if (a_exp && config == 0) seg_kb = 2;
   if (config == 0) {
-    bn = auto_bn(split3 ? 2 : 1, range, N, K);
+    bn = auto_bn(a_exp ? kTileF16x3 : split3 ? kTileBf16x3 : kTileBf16, range, N, K);
     pair = bn < 256 ? 0 : 2;
   }
   TcJob J;
@@ -972,7 +984,7 @@ cudaError_t launch_gemm_tc(const DevGraph& g, const DevPlan& p, const void* a_hi
 cudaError_t launch_gemm_f32_tc(const DevPlan& p, void* const a[3], void* const b[3], int num_cells, int N, int K, int h,
                                const RowsRange& range, float* products, float* C_direct, int32_t* info_out,
                                cudaStream_t st, int ld) {
-  const int bn = auto_bn(3, range, N, K);
+  const int bn = auto_bn(kTileF32, range, N, K);
   const bool small = bn < 256;
   TcJob J;
   if (!tc_fill_job(&J, p, a[0], a[1], b[0], b[1], num_cells, N, K, h, bn, small ? 0 : 2, BK, products, C_direct, info_out, nullptr, nullptr, ld))
