@@ -81,18 +81,25 @@ int ensure_table(bpx_group* G, int config, cudaStream_t st) {
 void plan_peel(bpx_group* G) {
   const int njobs = static_cast<int>(G->host_jobs.size());
   // Every CTA walks its job's whole chain of waves, so a batch's CTAs are
-  // shared out: 24 an SM in all, an eighth of an SM count to 4 x the SM count a
-  // job.  Peel of 48 jobs, 608 CTAs a job against 76: 391 -> 265 us; 12 jobs,
-  // 304: the same 185; 48 jobs of at most 1024, 172 -> 94 with 16.
+  // shared out.  Up to 31 jobs: 12 an SM in all, at most 1.5 x the SM count a
+  // job, so that a job's chain is short.  From 32 jobs on the CTAs' number is
+  // what counts: 24 an SM, an eighth of the SM count a job at least, and chunks
+  // of 64 columns.  Peel, geometric means over nine batches each of 256 to
+  // 4096 rows, against 608 CTAs a job: 4 jobs 0.84 (wide chunks 1.86), 8 jobs
+  // 0.88 (1.59), 12 jobs 0.83 (1.24), 16 jobs 0.74 (0.95), 24 jobs 0.75 (0.85),
+  // 32 jobs 0.77 (0.73), 48 jobs 0.79 (0.74).
   const int sms = bpx::num_sms();
-  const int target = G->peel_target > 0 ? G->peel_target : std::min(4 * sms, std::max(sms / 8, 24 * sms / njobs));
+  const bool many = njobs >= 32;
+  const int target = G->peel_target > 0 ? G->peel_target
+                     : many             ? std::max(sms / 8, 24 * sms / njobs)
+                                        : std::min(3 * sms / 2, 12 * sms / njobs);
   std::vector<int32_t> gat, reg;
   for (int j = 0; j < njobs; ++j) {
     auto& g = G->host_jobs[j];
     const long long nv = static_cast<long long>(g.h) * g.N / 4;
     g.peel_chunk = bpx::peel_chunk_for(nv, target);
-    // without a tuned target: no chunk under 64 columns while the job has 16
-    if (G->peel_target <= 0 && g.peel_chunk < 64)
+    // (no chunk under 64 columns while the job has 16)
+    if (G->peel_target <= 0 && many && g.peel_chunk < 64)
       g.peel_chunk = static_cast<int>(std::max<long long>(g.peel_chunk, std::min<long long>(64, (nv / 16 + 7) / 8 * 8)));
     const bpx_code* c = G->jobs[j].code;
     (bpx::peel_gather_ok(c->S, c->sigma, g.peel_chunk) ? gat : reg).push_back(j);
