@@ -36,7 +36,10 @@
 // barrier); n = 12, b = 120 153 -> 77; n = 8, b = 300 258 -> 177; n = 16,
 // b = 2800 with its state in global memory 7050 -> 4280.  Taking four sources
 // a warp at once made the rounds slower (550 -> 760 us: their claims queue),
-// and so did swapping without a look first (630).
+// and so did swapping without a look first (630).  Codes of few, wide rounds
+// (n = 27, b = 12: one of 252 sources) 16.6 -> 14.6, n = 32, b = 24 28.9 ->
+// 22.9; with rounds of up to 256 ordered by one warp, an element at a time,
+// and a warp copying each position's list, these took 49 and 40.
 #include <algorithm>
 #include <climits>
 #include <mutex>
@@ -51,7 +54,7 @@ constexpr size_t kSmemMax = 224 * 1024;  // dynamic shared memory of a plan's CT
 constexpr size_t kSmemSmall = 16 * 1024;  // the same for the 256-thread CTA of small codes
 
 constexpr int kAffineMax = 64;   // columns of the affine table kept in shared memory
-constexpr int kRankMax = 256;    // sources of a round ordered by one warp comparing each with all
+constexpr int kRankMax = 128;    // sources of a round ordered by one warp, four a lane, comparing each with all
 
 // The per-cell word: 32 bits in shared memory (when count and sum fit), 64
 // bits in the plan otherwise.
@@ -79,9 +82,13 @@ __host__ __device__ inline bool sched_local(const DevGraph& g, long long smem_in
 // One position of the peel list: its resolver's sources but s, ascending.
 __device__ __forceinline__ void fill_position(const int32_t* support, int degree, int s, int32_t* list, int first,
                                               int step) {
-  for (int e = first; e < degree; e += step) {
-    const int t = support[e];  // ascending: the entries past s move up by one
-    if (t != s) list[e - (t > s ? 1 : 0)] = t;
+  for (int e = first; e < degree; e += 8 * step) {
+    int t[8];  // eight loads in flight (the stores could alias them)
+#pragma unroll
+    for (int u = 0; u < 8; ++u) t[u] = e + u * step < degree ? support[e + u * step] : s;
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (t[u] != s) list[e + u * step - (t[u] > s ? 1 : 0)] = t[u];  // ascending: those past s move up by one
   }
 }
 
@@ -339,16 +346,25 @@ __device__ __forceinline__ void schedule_body(const DevGraph& g, const DevPlan& 
           for (int t = 0; t < n; ++t) below += __shfl_sync(0xffffffffu, x, t) < x ? 1 : 0;
           if (lane < n) ord[w0 + below] = x;
         } else if (n <= kRankMax) {
-          for (int i = 0; i < n; i += 32) {
-            const int xi = i + lane < n ? claimed[w0 + i + lane] : INT_MAX;
-            int below = 0;
-            for (int j = 0; j < n; j += 32) {
-              const int y = j + lane < n ? claimed[w0 + j + lane] : INT_MAX;
-#pragma unroll 8
-              for (int t = 0; t < 32; ++t) below += __shfl_sync(0xffffffffu, y, t) < xi ? 1 : 0;
-            }
-            if (i + lane < n) ord[w0 + below] = xi;
+          int v[kRankMax / 32], below[kRankMax / 32];
+#pragma unroll
+          for (int u = 0; u < kRankMax / 32; ++u) {
+            v[u] = 32 * u + lane < n ? claimed[w0 + 32 * u + lane] : INT_MAX;
+            below[u] = 0;
           }
+#pragma unroll
+          for (int j = 0; j < kRankMax / 32; ++j) {
+            if (32 * j >= n) break;
+#pragma unroll 8
+            for (int t = 0; t < 32; ++t) {
+              const int y = __shfl_sync(0xffffffffu, v[j], t);
+#pragma unroll
+              for (int u = 0; u < kRankMax / 32; ++u) below[u] += y < v[u] ? 1 : 0;
+            }
+          }
+#pragma unroll
+          for (int u = 0; u < kRankMax / 32; ++u)
+            if (32 * u + lane < n) ord[w0 + below[u]] = v[u];
         }
         w0 = w1;
         w1 = w2;
@@ -368,7 +384,7 @@ __device__ __forceinline__ void schedule_body(const DevGraph& g, const DevPlan& 
   // then the runs' totals, then the entries.
   int i0, i1, list_len;
   run_of(nrec, i0, i1);
-  if (nrec <= nt && fill && (local || g.sigma <= 8)) {  // a position a thread: no pass over the plan in between
+  if (nrec <= nt && fill) {  // a position a thread: no pass over the plan in between
     const int i = i0 + lane;
     const bool in = i < i1;
     const int s = in ? ord[i] : 0, r = in ? res[s] : 0;
@@ -419,41 +435,13 @@ __device__ __forceinline__ void schedule_body(const DevGraph& g, const DevPlan& 
     if (lane == 0) s_warp[warp] = run;
     __syncthreads();
     const int list0 = warp_base(&list_len);
-    for (int b = i0; b < i1; b += 32) {
-      const int i = b + lane;
-      int s = 0, o = 0, e0 = 0, deg = 0;
-      if (i < i1) {
-        o = list0 + p.pl_ptr[i];
-        p.pl_ptr[i] = o;
-      }
+    for (int i = i0 + lane; i < i1; i += 32) {
+      const int at = list0 + p.pl_ptr[i];
+      p.pl_ptr[i] = at;
       if (!fill) continue;
-      if (i < i1) {
-        const int r = p.pl_res[i];
-        s = ord[i];
-        if (S >= kTallSources) p.pos[s] = i;
-        e0 = cell_ptr[r];
-        deg = cell_ptr[r + 1] - e0;
-      }
-      if (local || g.sigma <= 8) {
-        if (i < i1) fill_position(cell_src + e0, deg, s, p.pl_list + o, 0, 1);
-      } else {  // long supports: the warp copies four positions at a time
-        for (int q = 0; q < min(32, i1 - b); q += 4) {
-          int t[4], at[4], n[4], x[4], from[4];
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {  // (lanes past the run hold degree 0)
-            from[u] = __shfl_sync(0xffffffffu, e0, q + u);
-            n[u] = __shfl_sync(0xffffffffu, deg, q + u);
-            x[u] = __shfl_sync(0xffffffffu, s, q + u);
-            at[u] = __shfl_sync(0xffffffffu, o, q + u);
-            t[u] = lane < n[u] ? cell_src[from[u] + lane] : x[u];
-          }
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            if (t[u] != x[u]) p.pl_list[at[u] + lane - (t[u] > x[u] ? 1 : 0)] = t[u];
-            if (n[u] > 32) fill_position(cell_src + from[u], n[u], x[u], p.pl_list + at[u], lane + 32, 32);
-          }
-        }
-      }
+      const int r = p.pl_res[i], x = ord[i], e0 = cell_ptr[r];
+      if (S >= kTallSources) p.pos[x] = i;
+      fill_position(cell_src + e0, cell_ptr[r + 1] - e0, x, p.pl_list + at, 0, 1);
     }
   }
   if (tid == 0) p.pl_ptr[nrec] = list_len;
