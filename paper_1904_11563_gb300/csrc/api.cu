@@ -154,14 +154,15 @@ extern "C" int bpx_workspace_init(const bpx_code* c, void* ws, size_t ws_bytes, 
 namespace {
 
 int schedule_impl(const bpx_code* c, const uint8_t* d_mask, bool cell_mask, void* ws, size_t ws_bytes,
-                  int32_t* d_peel_order, uint8_t* d_recovered, int32_t* d_info, cudaStream_t st, int part = 0) {
+                  int32_t* d_peel_order, uint8_t* d_recovered, int32_t* d_info, cudaStream_t st, int part = 0,
+                  bool clear_f32 = false) {
   if (!c) return fail(BPX_ERR_INVAL, "bpx_schedule: code is NULL");
   const bpx::WsLayout L = bpx::ws_layout(c, 0, 0, 0, 1, BPX_FP32);
   if (int rc = check_ws(c, ws, ws_bytes, L)) return rc;
   if (!d_mask) return fail(BPX_ERR_INVAL, "bpx_schedule: erasure mask is NULL");
   const bpx::DevGraph g = bpx::make_graph(c, ws, L);
   const bpx::DevPlan p = bpx::make_plan(ws, L);
-  cudaError_t e = bpx::launch_schedule(g, p, d_mask, d_peel_order, d_recovered, d_info, st, cell_mask, part);
+  cudaError_t e = bpx::launch_schedule(g, p, d_mask, d_peel_order, d_recovered, d_info, st, cell_mask, part, clear_f32);
   if (e != cudaSuccess) return cuda_fail(e, "bpx_schedule: launch");
   return BPX_OK;
 }
@@ -286,7 +287,9 @@ int products_impl(const bpx_code* c, const float* d_A, const float* d_B, int M, 
         void* const a[3] = {base + L.a_hi, base + L.a_lo, base + L.a_3};
         void* const b[3] = {base + L.b_hi, base + L.b_lo, base + L.b_3};
         stage_mark(opts, BPX_STAGE_B_PREP, 0, st);
-        e = bpx::launch_b_parts(p, d_B, K, N, b, st, early);
+        if (!early)  // (early: the schedule has cleared it)
+          e = cudaMemsetAsync(p.ctr + bpx::CTR_F32_SIMT, 0, sizeof(int32_t), st);
+        if (e == cudaSuccess) e = bpx::launch_b_parts(p, d_B, K, N, b, st, early);
         stage_mark(opts, BPX_STAGE_B_PREP, 1, st);
         stage_mark(opts, BPX_STAGE_A_PREP, 0, st);
         if (e == cudaSuccess) e = bpx::launch_encode_parts(g, p, d_A, M, K, h, a, st);
@@ -570,7 +573,8 @@ extern "C" int bpx_coded_matmul(const bpx_code* c, const float* d_A, const float
   const bpx::ChainScope chain(!side && may_chain(o, S(stream)));
   stage_mark(&o, BPX_STAGE_SCHEDULE, 0, S(stream));
   if (!side) {
-    if (int rc = schedule_impl(c, d_mask, o.mask_cells != 0, ws, ws_bytes, nullptr, nullptr, d_info, S(stream)))
+    if (int rc = schedule_impl(c, d_mask, o.mask_cells != 0, ws, ws_bytes, nullptr, nullptr, d_info, S(stream), 0,
+                               precision == BPX_FP32 && bpx::chain_on()))
       return rc;
     stage_mark(&o, BPX_STAGE_SCHEDULE, 1, S(stream));
   } else {
@@ -709,7 +713,8 @@ int host_panels(const bpx_code* c, const float* h_A, const float* h_B, int M, in
   void* const a[3] = {base + L.a_hi, base + L.a_lo, base + L.a_3};
   const bool split = precision != BPX_BF16;
   if (precision == BPX_FP32) {
-    ok(bpx::launch_encode_parts(g, p, d_A, M, K, h, a, st));
+    ok(cudaMemsetAsync(p.ctr + bpx::CTR_F32_SIMT, 0, sizeof(int32_t), st)) &&
+        ok(bpx::launch_encode_parts(g, p, d_A, M, K, h, a, st));
   } else if (precision == BPX_FP16X3) {
     if (ok(cudaMemsetAsync(a_exp, 0, sizeof(int32_t) * static_cast<size_t>(c->num_cells) * h, st)))
       ok(bpx::launch_encode_f16(g, p, d_A, M, K, h, a[0], a[1], a_exp, st));

@@ -160,7 +160,7 @@ enum {
   CTR_NNEW,       // sources recovered this round (scratch)
   CTR_ERR,        // device error code raised by a kernel self-check
   CTR_PLAN,       // kPlanReady once a whole plan is in place (zeroed by bpx_workspace_init)
-  CTR_F32_SIMT,   // FP32 operands hold an element the tensor-core parts cannot (cleared by every schedule)
+  CTR_F32_SIMT,   // FP32 operands hold an element the tensor-core parts cannot (cleared by every call's products)
   CTR_LEN = 16
 };
 constexpr int32_t kPlanReady = 0x504C414E;  // "PLAN"

@@ -290,9 +290,10 @@ cudaError_t tc_build_table(const TcSpec* specs, int n, bool split3, int config, 
                            long long* total_tiles, cudaStream_t st);
 // cell_mask: the mask has one byte per cell instead of one per column.
 // part: 0 = whole plan, 1 = survivors + depth-1 direct map, 2 = the rest.
+// clear_f32: also clears CTR_F32_SIMT, before a chained launch may start.
 cudaError_t launch_schedule(const DevGraph& g, const DevPlan& p, const uint8_t* mask,
                             int32_t* peel_order, uint8_t* recovered, int32_t* info_out,
-                            cudaStream_t st, bool cell_mask = false, int part = 0);
+                            cudaStream_t st, bool cell_mask = false, int part = 0, bool clear_f32 = false);
 
 // SMs the persistent GEMMs leave free (for a schedule running beside them);
 // set by the entry points for the duration of a launch.

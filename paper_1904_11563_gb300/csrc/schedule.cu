@@ -494,11 +494,14 @@ __global__ void __launch_bounds__(256) fill_list_kernel(DevGraph g, DevPlan p) {
 template <bool kSmem>
 __global__ void __launch_bounds__(kThreads, 1)
 schedule_kernel(DevGraph g, DevPlan p, const uint8_t* __restrict__ mask, int32_t* peel_order,
-                uint8_t* recovered, int32_t* info_out, bool cell_mask, int part, int smem_ints, bool fill) {
+                uint8_t* recovered, int32_t* info_out, bool cell_mask, int part, int smem_ints, bool fill,
+                bool clear_f32) {
   chain_wait();
-  if (threadIdx.x == 0) {  // the staging let in here may raise this flag: it is down before
-    if (part != 2) p.ctr[CTR_F32_SIMT] = 0;
-    __threadfence();
+  if (threadIdx.x == 0) {
+    if (clear_f32) {  // the staging let in here may raise this flag: it is down before
+      p.ctr[CTR_F32_SIMT] = 0;
+      __threadfence();
+    }
     chain_release();
   }
   schedule_body<kSmem>(g, p, mask, peel_order, recovered, info_out, cell_mask, part, smem_ints, fill);
@@ -531,7 +534,7 @@ cudaError_t launch_schedule_group(const GJob* d_jobs, int njobs, size_t max_stat
 
 cudaError_t launch_schedule(const DevGraph& g, const DevPlan& p, const uint8_t* mask,
                             int32_t* peel_order, uint8_t* recovered, int32_t* info_out,
-                            cudaStream_t st, bool cell_mask, int part) {
+                            cudaStream_t st, bool cell_mask, int part, bool clear_f32) {
   const long long state = static_cast<long long>(g.num_cells) + g.S;  // int32 words
   // Small codes take a 256-thread block with at most 16 KB of shared memory:
   // it fits beside a resident GEMM CTA, so the schedule of one
@@ -547,10 +550,10 @@ cudaError_t launch_schedule(const DevGraph& g, const DevPlan& p, const uint8_t* 
                                   static_cast<int>(kSmemMax))) != cudaSuccess)
       return e;
     e = launch(schedule_kernel<true>, dim3(1), threads, static_cast<size_t>(ints) * 4, st, g, p, mask, peel_order,
-               recovered, info_out, cell_mask, part, static_cast<int>(ints), !fill_later);
+               recovered, info_out, cell_mask, part, static_cast<int>(ints), !fill_later, clear_f32);
   } else {
     e = launch(schedule_kernel<false>, dim3(1), threads, 0, st, g, p, mask, peel_order, recovered, info_out, cell_mask,
-               part, 0, !fill_later);
+               part, 0, !fill_later, clear_f32);
   }
   if (e != cudaSuccess || !fill_later) return e;
   return launch(fill_list_kernel, dim3(std::min((g.S + 7) / 8, 4 * num_sms())), 256, 0, st, g, p);
