@@ -71,10 +71,15 @@ enum bpx_variant {
 /* Arithmetic of the coded products.  FP32 accumulation in every case. */
 enum bpx_precision {
   BPX_FP32 = 0,   /* FP32: every operand the exact sum of three bf16 parts, six tcgen05 products
-                     accumulated in FP32 (errors below an FFMA chain's at every K); on the CUDA
-                     cores (FP32 encode pass, then an FFMA GEMM) for small products and for
-                     operands with elements the parts cannot hold: infinities, NaN, nonzero
-                     magnitudes below 2^-102 or from 2^127 */
+                     accumulated in FP32; on the CUDA cores (FP32 encode pass, then an FFMA GEMM)
+                     for small products, for operands with elements the parts cannot hold
+                     (infinities, NaN, nonzero magnitudes below 2^-102 or from 2^127) and for
+                     products whose sums could leave FP32's range: K max(|coded A|, 2^32)
+                     max(|B|, 2^32) from 2^126.  Such a call takes as long as the FFMA GEMM
+                     and the staging of the parts before it.  Error against 64 bits, relative
+                     to sum |a||b|, on dense operands (normal, uniform, magnitudes spread over
+                     e^20): a quarter to a seventh of an FFMA chain's at K 1024 to 8192; an
+                     element with one dominant term may be off by twice an FFMA's last bit */
   BPX_BF16 = 1,   /* coded A and B rounded to bf16, one tcgen05 MMA per k-step */
   BPX_BF16X3 = 2, /* split bf16: a = a_hi + a_lo; hi*hi + hi*lo + lo*hi on tcgen05 */
   BPX_MXFP8 = 3,  /* E4M3 with one UE8M0 scale per 32 K-elements (tcgen05 block-scaled) */

@@ -287,8 +287,8 @@ int products_impl(const bpx_code* c, const float* d_A, const float* d_B, int M, 
         void* const a[3] = {base + L.a_hi, base + L.a_lo, base + L.a_3};
         void* const b[3] = {base + L.b_hi, base + L.b_lo, base + L.b_3};
         stage_mark(opts, BPX_STAGE_B_PREP, 0, st);
-        if (!early)  // (early: the schedule has cleared it)
-          e = cudaMemsetAsync(p.ctr + bpx::CTR_F32_SIMT, 0, sizeof(int32_t), st);
+        if (!early)  // (early: the schedule has cleared them)
+          e = cudaMemsetAsync(p.ctr + bpx::CTR_F32_SIMT, 0, bpx::kF32Words * sizeof(int32_t), st);
         if (e == cudaSuccess) e = bpx::launch_b_parts(p, d_B, K, N, b, st, early);
         stage_mark(opts, BPX_STAGE_B_PREP, 1, st);
         stage_mark(opts, BPX_STAGE_A_PREP, 0, st);
@@ -298,7 +298,7 @@ int products_impl(const bpx_code* c, const float* d_A, const float* d_B, int M, 
         if (e == cudaSuccess)
           e = bpx::launch_gemm_f32_tc(p, a, b, c->num_cells, N, K, h, bpx::rows_range(c, h), d_products, d_C,
                                       d_info, st);
-        // operands the parts cannot hold (a plan counter says so): FP32 on the CUDA cores
+        // operands the parts cannot hold or sum (plan counters say so): FP32 on the CUDA cores
         if (e == cudaSuccess) e = bpx::launch_encode_f32_flagged(g, p, d_A, M, K, h, a_coded, st);
         if (e == cudaSuccess) e = bpx::launch_gemm_f32_flagged(g, p, a_coded, d_B, N, K, h, d_products, d_C, st);
         stage_mark(opts, BPX_STAGE_GEMM, 1, st);
@@ -713,7 +713,7 @@ int host_panels(const bpx_code* c, const float* h_A, const float* h_B, int M, in
   void* const a[3] = {base + L.a_hi, base + L.a_lo, base + L.a_3};
   const bool split = precision != BPX_BF16;
   if (precision == BPX_FP32) {
-    ok(cudaMemsetAsync(p.ctr + bpx::CTR_F32_SIMT, 0, sizeof(int32_t), st)) &&
+    ok(cudaMemsetAsync(p.ctr + bpx::CTR_F32_SIMT, 0, bpx::kF32Words * sizeof(int32_t), st)) &&
         ok(bpx::launch_encode_parts(g, p, d_A, M, K, h, a, st));
   } else if (precision == BPX_FP16X3) {
     if (ok(cudaMemsetAsync(a_exp, 0, sizeof(int32_t) * static_cast<size_t>(c->num_cells) * h, st)))

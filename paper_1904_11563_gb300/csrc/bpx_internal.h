@@ -160,9 +160,16 @@ enum {
   CTR_NNEW,       // sources recovered this round (scratch)
   CTR_ERR,        // device error code raised by a kernel self-check
   CTR_PLAN,       // kPlanReady once a whole plan is in place (zeroed by bpx_workspace_init)
-  CTR_F32_SIMT,   // FP32 operands hold an element the tensor-core parts cannot (cleared by every call's products)
+  // FP32 on the tensor cores (cleared by every call's products): an operand
+  // holds an element that the parts cannot; the float bits of the largest
+  // magnitude of the coded rows and of B (kF32Plain and below: not noted)
+  CTR_F32_SIMT,
+  CTR_F32_AMAX,
+  CTR_F32_BMAX,
   CTR_LEN = 16
 };
 constexpr int32_t kPlanReady = 0x504C414E;  // "PLAN"
+constexpr int kF32Words = CTR_F32_BMAX - CTR_F32_SIMT + 1;
+constexpr float kF32Plain = 4294967296.f;  // 2^32
 
 }  // namespace bpx

@@ -161,6 +161,17 @@ struct ChainScope {
   bool was;
 };
 
+// Whether an FP32 product staged for the tensor cores is left to the CUDA
+// cores: an element that three bf16 parts cannot hold, or operands so large
+// that a partial sum of the parts' products could leave FP32's range where the
+// sum itself stays in it, or leave it with the other sign.  In whatever order,
+// sums of the six products stay below 1.03 K max|A| max|B|.
+__device__ __forceinline__ bool f32_on_cuda_cores(const int32_t* ctr, int K) {
+  const float a = fmaxf(kF32Plain, __int_as_float(ctr[CTR_F32_AMAX]));
+  const float b = fmaxf(kF32Plain, __int_as_float(ctr[CTR_F32_BMAX]));
+  return ctr[CTR_F32_SIMT] != 0 || !(static_cast<float>(K) * (a * b) < 0x1p126f);
+}
+
 // Launches a kernel, as the next link of a chain when one is on.
 template <typename... P, typename... A>
 cudaError_t launch(void (*kern)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, A&&... args) {
@@ -290,7 +301,7 @@ cudaError_t tc_build_table(const TcSpec* specs, int n, bool split3, int config, 
                            long long* total_tiles, cudaStream_t st);
 // cell_mask: the mask has one byte per cell instead of one per column.
 // part: 0 = whole plan, 1 = survivors + depth-1 direct map, 2 = the rest.
-// clear_f32: also clears CTR_F32_SIMT, before a chained launch may start.
+// clear_f32: also clears the CTR_F32 words, before a chained launch may start.
 cudaError_t launch_schedule(const DevGraph& g, const DevPlan& p, const uint8_t* mask,
                             int32_t* peel_order, uint8_t* recovered, int32_t* info_out,
                             cudaStream_t st, bool cell_mask = false, int part = 0, bool clear_f32 = false);
@@ -309,13 +320,13 @@ cudaError_t launch_encode_split(const DevGraph& g, const DevPlan& p, const float
 cudaError_t launch_b_split(const float* B, int K, int N, void* b_hi, void* b_lo, cudaStream_t st, bool early,
                            int ldb = 0);
 // FP32 operands for the tensor cores: the coded rows / B^T as three bf16
-// parts whose sum is the FP32 value; flag (a plan counter) is raised when an
-// element's parts would not hold it.
+// parts whose sum is the FP32 value; the CTR_F32 words note elements that the
+// parts would not hold, and the largest magnitudes.
 cudaError_t launch_encode_parts(const DevGraph& g, const DevPlan& p, const float* A, int M, int K, int h,
                                 void* const a[3], cudaStream_t st);
 cudaError_t launch_b_parts(const DevPlan& p, const float* B, int K, int N, void* const b[3], cudaStream_t st,
                            bool early, int ldb = 0);
-// The FP32 encode and GEMM on the CUDA cores when that flag is up (else both return at once).
+// The FP32 encode and GEMM on the CUDA cores when those words say so (else both return at once).
 cudaError_t launch_encode_f32_flagged(const DevGraph& g, const DevPlan& p, const float* A, int M, int K, int h,
                                       float* out, cudaStream_t st);
 cudaError_t launch_gemm_f32_flagged(const DevGraph& g, const DevPlan& p, const float* a_coded, const float* B, int N,

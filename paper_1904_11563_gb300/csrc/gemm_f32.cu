@@ -264,12 +264,12 @@ cudaError_t launch_small(const DevPlan& p, const float* a_coded, const float* B,
 }
 
 // Behind the tensor-core FP32 GEMM: one CTA per SM walks the tiles when the
-// staging raised the flag, else returns at once.
+// staged operands are left to the CUDA cores, else returns at once.
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_f32_flagged_kernel(DevPlan p, const float* __restrict__ Ac, const float* __restrict__ B, int N, int ld, int K,
                         int h, float* products, float* C_direct) {
   chain_wait();
-  if (p.ctr[CTR_F32_SIMT] == 0) return;
+  if (!f32_on_cuda_cores(p.ctr, K)) return;
   const long long Mc = static_cast<long long>(p.ctr[CTR_NSURV]) * h;
   const long long n_tiles = (N + BN - 1) / BN, tiles = (Mc + BM - 1) / BM * n_tiles;
   for (long long t = blockIdx.x; t < tiles; t += gridDim.x) {

@@ -36,14 +36,31 @@ __device__ __forceinline__ bool parts_unfit(float x) {
   const uint32_t u = __float_as_uint(x) & 0x7fffffffu;
   return u != 0u && u - (25u << 23) >= (254u - 25u) << 23;
 }
+// Notes an unfit element, and the largest magnitude (as float bits) in
+// ctr[word] where it is above kF32Plain: ordinary operands then cost no
+// traffic; of others a warp reads the word and raises it if need be (all
+// operands above it: 62 -> 67 us on 1000 x 1416 x 1100, 665 -> 688 at 4096 cubed).
+__device__ __forceinline__ void note_parts(const DevPlan& p, int word, uint32_t most, bool unfit) {
+  if (unfit) {
+    p.ctr[CTR_F32_SIMT] = 1;
+  } else if (most > __float_as_uint(kF32Plain)) {
+    const unsigned lanes = __activemask();
+    most = __reduce_max_sync(lanes, most);
+    auto* at = reinterpret_cast<uint32_t*>(p.ctr + word);
+    if ((threadIdx.x & 31) == __ffs(lanes) - 1 && *reinterpret_cast<volatile uint32_t*>(at) < most)
+      atomicMax(at, most);
+  }
+}
+// most: raised to the largest magnitude of the eight; returns whether one is unfit.
 __device__ __forceinline__ bool parts_split8(const float (&v)[8], __nv_bfloat16* o1, __nv_bfloat16* o2,
-                                             __nv_bfloat16* o3) {
+                                             __nv_bfloat16* o3, uint32_t& most) {
   uint32_t w1[4], w2[4], w3[4];
   bool unfit = false;
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const float x0 = v[2 * q], x1 = v[2 * q + 1];
     unfit |= parts_unfit(x0) | parts_unfit(x1);
+    most = max(most, max(__float_as_uint(fabsf(x0)), __float_as_uint(fabsf(x1))));
     const __nv_bfloat162 p1 = __floats2bfloat162_rn(x0, x1);
     const float2 f1 = __bfloat1622float2(p1);
     const float r0 = x0 - f1.x, r1 = x1 - f1.y;
@@ -106,7 +123,9 @@ __device__ __forceinline__ void encode_body(const DevGraph& g, const DevPlan& p,
     d[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
     d[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
   } else if constexpr (kMode == 3) {
-    if (parts_split8(acc, out_hi + o, out_lo + o, out_3 + o)) p.ctr[CTR_F32_SIMT] = 1;
+    uint32_t most = 0;
+    const bool unfit = parts_split8(acc, out_hi + o, out_lo + o, out_3 + o, most);
+    note_parts(p, CTR_F32_AMAX, most, unfit);
   } else {
     uint32_t hv[4], lv[4];
 #pragma unroll
@@ -140,12 +159,13 @@ encode_parts_kernel(DevGraph g, DevPlan p, const float* __restrict__ A, int M, i
 }
 
 // The FP32 encode behind the tensor-core FP32 GEMM: a fixed grid walks the
-// (row block, k-chunk) blocks when the staging raised the flag.
+// (row block, k-chunk) blocks when the staged operands are left to the CUDA
+// cores.
 __global__ void __launch_bounds__(kEncThreads)
 encode_f32_flagged_kernel(DevGraph g, DevPlan p, const float* __restrict__ A, int M, int K, int h, float* out,
                           long long row_blocks, long long blocks) {
   chain_wait();
-  if (p.ctr[CTR_F32_SIMT] == 0) return;
+  if (!f32_on_cuda_cores(p.ctr, K)) return;
   for (long long b = blockIdx.x; b < blocks; b += gridDim.x) {
     const long long kc = b / row_blocks;
     encode_body<0>(g, p, A, M, K, h, out, nullptr, nullptr, static_cast<int>(b - kc * row_blocks), static_cast<int>(kc));
@@ -158,7 +178,7 @@ constexpr int kTile = 64;
 template <bool kParts3 = false>
 __device__ __forceinline__ bool b_split_body(const float* __restrict__ B, int K, int N, int ldb,
                                              __nv_bfloat16* bt_hi, __nv_bfloat16* bt_lo, int bx,
-                                             int by, __nv_bfloat16* bt_3 = nullptr) {
+                                             int by, __nv_bfloat16* bt_3 = nullptr, uint32_t* most = nullptr) {
   bool unfit = false;
   __shared__ float tile[kTile][kTile + 1];
   const int n0 = bx * kTile, k0 = by * kTile;
@@ -189,7 +209,7 @@ __device__ __forceinline__ bool b_split_body(const float* __restrict__ B, int K,
 #pragma unroll
       for (int q = 0; q < 8; ++q) v[q] = tile[8 * kc + q][r];
       const long long o = static_cast<long long>(n) * K + k;
-      unfit |= parts_split8(v, bt_hi + o, bt_lo + o, bt_3 + o);
+      unfit |= parts_split8(v, bt_hi + o, bt_lo + o, bt_3 + o, *most);
     } else {
       uint32_t hv[4], lv[4];
 #pragma unroll
@@ -213,7 +233,9 @@ __global__ void __launch_bounds__(256)
 b_parts_kernel(DevPlan p, const float* __restrict__ B, int K, int N, int ldb, __nv_bfloat16* o1, __nv_bfloat16* o2,
                __nv_bfloat16* o3, bool early) {
   chain_begin_staging(early);
-  if (b_split_body<true>(B, K, N, ldb, o1, o2, blockIdx.x, blockIdx.y, o3)) p.ctr[CTR_F32_SIMT] = 1;
+  uint32_t most = 0;
+  const bool unfit = b_split_body<true>(B, K, N, ldb, o1, o2, blockIdx.x, blockIdx.y, o3, &most);
+  note_parts(p, CTR_F32_BMAX, most, unfit);
   chain_end_staging(early);
 }
 

@@ -498,8 +498,8 @@ schedule_kernel(DevGraph g, DevPlan p, const uint8_t* __restrict__ mask, int32_t
                 bool clear_f32) {
   chain_wait();
   if (threadIdx.x == 0) {
-    if (clear_f32) {  // the staging let in here may raise this flag: it is down before
-      p.ctr[CTR_F32_SIMT] = 0;
+    if (clear_f32) {  // the staging let in here may raise these words: they are down before
+      for (int i = 0; i < kF32Words; ++i) p.ctr[CTR_F32_SIMT + i] = 0;
       __threadfence();
     }
     chain_release();
