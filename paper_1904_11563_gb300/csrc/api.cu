@@ -681,7 +681,10 @@ int host_panel(const bpx_code* c, int N, int K, int h, int precision, const bpx_
 // The host call in panels of B's columns (the mask and A first): while a panel
 // is copied in, the one before is staged, multiplied and peeled, and the one
 // before that copied out.  Same kernels over runs of columns, the same bits,
-// the same contents of d_A, d_B and d_C.  4096 cubed, split bf16, page-locked:
+// the same contents of d_A, d_B and d_C.  (FP32 operands that turn out to be
+// for the CUDA cores: any panel may show that, so the caller looks at the
+// CTR_F32 words at the end and runs the call over, the operands being in
+// place.)  4096 cubed, split bf16, page-locked:
 // copies in 0.64 ms, kernels 0.37, copies out 0.35 one after the other 1.35 ms,
 // in panels 0.98.
 int host_panels(const bpx_code* c, const float* h_A, const float* h_B, int M, int N, int K, int h, int precision,
@@ -735,11 +738,8 @@ int host_panels(const bpx_code* c, const float* h_A, const float* h_B, int M, in
     float* C = o.direct_write ? d_C + n0 : nullptr;
     if (precision == BPX_FP32) {
       void* const b[3] = {b_hi, b_lo, base + L.b_3 + row0};
-      float* a_coded = reinterpret_cast<float*>(base + L.a_hi);
       ok(bpx::launch_b_parts(p, d_B + n0, K, wn, b, st, false, N)) &&
-          ok(bpx::launch_gemm_f32_tc(p, a, b, c->num_cells, wn, K, h, range, P, C, nullptr, st, N)) &&
-          ok(bpx::launch_encode_f32_flagged(g, p, d_A, M, K, h, a_coded, st)) &&
-          ok(bpx::launch_gemm_f32_flagged(g, p, a_coded, d_B + n0, wn, K, h, P, C, st, N));
+          ok(bpx::launch_gemm_f32_tc(p, a, b, c->num_cells, wn, K, h, range, P, C, nullptr, st, N));
     } else if (precision == BPX_FP16X3) {
       int32_t* b_exp = reinterpret_cast<int32_t*>(b_max + N) + n0;
       ok(bpx::launch_b_f16(g, h, d_B + n0, K, wn, b_hi, b_lo, b_max + n0, b_exp, nullptr, st, false, N)) &&
@@ -779,6 +779,7 @@ int host_impl(const bpx_code* c, const float* h_A, const float* h_B, int M, int 
   const bpx::WsLayout L = bpx::ws_layout(c, M, N, K, h, precision);
   int32_t* d_info = reinterpret_cast<int32_t*>(static_cast<char*>(ws) + L.p_info);
   const bpx_opts o = opts ? *opts : bpx_default_opts();
+  bool staged = false;  // A, B and the mask are on the device
   if (const int w = sync ? host_panel(c, N, K, h, precision, o) : 0) {
     if (HostPipe* hp = host_pipe()) {
       const int rc = host_panels(c, h_A, h_B, M, N, K, h, precision, h_mask, mask_bytes, h_C, d_A, d_B, d_mask, d_C, o,
@@ -792,19 +793,27 @@ int host_impl(const bpx_code* c, const float* h_A, const float* h_B, int M, int 
       if ((e = cudaMemcpyAsync(h_info, d_info, sizeof(int32_t) * BPX_INFO_LEN, cudaMemcpyDeviceToHost, st)) !=
           cudaSuccess)
         return cuda_fail(e, "copy info");
+      int32_t words[bpx::kF32Words] = {};
+      if (precision == BPX_FP32 &&
+          (e = cudaMemcpyAsync(words, bpx::make_plan(ws, L).ctr + bpx::CTR_F32_SIMT, sizeof words,
+                               cudaMemcpyDeviceToHost, st)) != cudaSuccess)
+        return cuda_fail(e, "copy FP32 words");
       if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_fail(e, "sync");
       if (h_info[BPX_INFO_DEVICE_ERR] != 0) return h_info[BPX_INFO_DEVICE_ERR];
-      return h_info[BPX_INFO_STATUS];
+      if (precision != BPX_FP32 || !bpx::f32_on_cuda_cores(words, K)) return h_info[BPX_INFO_STATUS];
+      staged = true;
     }
   }
-  if ((e = cudaMemcpyAsync(d_A, h_A, sizeof(float) * M * static_cast<size_t>(K),
-                           cudaMemcpyHostToDevice, st)) != cudaSuccess)
-    return cuda_fail(e, "copy A");
-  if ((e = cudaMemcpyAsync(d_B, h_B, sizeof(float) * K * static_cast<size_t>(N),
-                           cudaMemcpyHostToDevice, st)) != cudaSuccess)
-    return cuda_fail(e, "copy B");
-  if ((e = cudaMemcpyAsync(d_mask, h_mask, mask_bytes, cudaMemcpyHostToDevice, st)) != cudaSuccess)
-    return cuda_fail(e, "copy mask");
+  if (!staged) {
+    if ((e = cudaMemcpyAsync(d_A, h_A, sizeof(float) * M * static_cast<size_t>(K),
+                             cudaMemcpyHostToDevice, st)) != cudaSuccess)
+      return cuda_fail(e, "copy A");
+    if ((e = cudaMemcpyAsync(d_B, h_B, sizeof(float) * K * static_cast<size_t>(N),
+                             cudaMemcpyHostToDevice, st)) != cudaSuccess)
+      return cuda_fail(e, "copy B");
+    if ((e = cudaMemcpyAsync(d_mask, h_mask, mask_bytes, cudaMemcpyHostToDevice, st)) != cudaSuccess)
+      return cuda_fail(e, "copy mask");
+  }
   if (int rc = bpx_coded_matmul(c, d_A, d_B, M, N, K, h, precision, d_mask, d_C, opts, ws, ws_bytes,
                                 nullptr, st))
     return rc;

@@ -166,10 +166,14 @@ struct ChainScope {
 // that a partial sum of the parts' products could leave FP32's range where the
 // sum itself stays in it, or leave it with the other sign.  In whatever order,
 // sums of the six products stay below 1.03 K max|A| max|B|.
-__device__ __forceinline__ bool f32_on_cuda_cores(const int32_t* ctr, int K) {
-  const float a = fmaxf(kF32Plain, __int_as_float(ctr[CTR_F32_AMAX]));
-  const float b = fmaxf(kF32Plain, __int_as_float(ctr[CTR_F32_BMAX]));
-  return ctr[CTR_F32_SIMT] != 0 || !(static_cast<float>(K) * (a * b) < 0x1p126f);
+// words: the CTR_F32 words (on the host: a copy of them).
+__host__ __device__ __forceinline__ bool f32_on_cuda_cores(const int32_t* words, int K) {
+  float a, b;
+  memcpy(&a, words + (CTR_F32_AMAX - CTR_F32_SIMT), sizeof a);
+  memcpy(&b, words + (CTR_F32_BMAX - CTR_F32_SIMT), sizeof b);
+  a = a > kF32Plain ? a : kF32Plain;
+  b = b > kF32Plain ? b : kF32Plain;
+  return words[0] != 0 || !(static_cast<float>(K) * (a * b) < 0x1p126f);
 }
 
 // Launches a kernel, as the next link of a chain when one is on.
@@ -330,7 +334,7 @@ cudaError_t launch_b_parts(const DevPlan& p, const float* B, int K, int N, void*
 cudaError_t launch_encode_f32_flagged(const DevGraph& g, const DevPlan& p, const float* A, int M, int K, int h,
                                       float* out, cudaStream_t st);
 cudaError_t launch_gemm_f32_flagged(const DevGraph& g, const DevPlan& p, const float* a_coded, const float* B, int N,
-                                    int K, int h, float* products, float* C_direct, cudaStream_t st, int ld = 0);
+                                    int K, int h, float* products, float* C_direct, cudaStream_t st);
 cudaError_t launch_gemm_f32_tc(const DevPlan& p, void* const a[3], void* const b[3], int num_cells, int N, int K, int h,
                                const RowsRange& range, float* products, float* C_direct, int32_t* info_out,
                                cudaStream_t st, int ld = 0);

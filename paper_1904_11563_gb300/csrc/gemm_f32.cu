@@ -37,7 +37,7 @@ __device__ __forceinline__ void cp_async_wait() {
 }
 
 __device__ __forceinline__ void gemm_f32_tile(const DevPlan& p, const float* __restrict__ Ac,
-                                              const float* __restrict__ B, int N, int ld, int K, int h, float* products,
+                                              const float* __restrict__ B, int N, int K, int h, float* products,
                                               float* C_direct, long long Mc, long long m0, int n0) {
 
   extern __shared__ __align__(16) float smem_f[];
@@ -79,7 +79,7 @@ __device__ __forceinline__ void gemm_f32_tile(const DevPlan& p, const float* __r
     for (int q = 0; q < 4; ++q) {
       const int n = n0 + b_n + 64 * q;
       const bool v = k < K && n < N;
-      const float* src = v ? B + static_cast<long long>(k) * ld + n : B;
+      const float* src = v ? B + static_cast<long long>(k) * N + n : B;
       cp_async16(&Bs[buf][b_k][b_n + 64 * q], src, v);
     }
   };
@@ -147,8 +147,8 @@ __device__ __forceinline__ void gemm_f32_tile(const DevPlan& p, const float* __r
     const int j = static_cast<int>(r - static_cast<long long>(ci) * h);
     const int cell = p.surv[ci];
     const int ds = C_direct ? p.direct[cell] : -1;
-    float* dst = ds >= 0 ? C_direct + (static_cast<long long>(ds) * h + j) * ld
-                         : products + (static_cast<long long>(cell) * h + j) * ld;
+    float* dst = ds >= 0 ? C_direct + (static_cast<long long>(ds) * h + j) * N
+                         : products + (static_cast<long long>(cell) * h + j) * N;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const int n = n0 + tx * 4 + 64 * q;
@@ -167,7 +167,7 @@ gemm_f32_kernel(DevPlan p, const float* __restrict__ Ac, const float* __restrict
   chain_wait();
   const long long Mc = static_cast<long long>(p.ctr[CTR_NSURV]) * h;
   const long long m0 = static_cast<long long>(blockIdx.y) * BM;
-  if (m0 < Mc) gemm_f32_tile(p, Ac, B, N, N, K, h, products, C_direct, Mc, m0, blockIdx.x * BN);
+  if (m0 < Mc) gemm_f32_tile(p, Ac, B, N, K, h, products, C_direct, Mc, m0, blockIdx.x * BN);
 }
 
 // Small products: BM x BN tiles, TM x 4 outputs a thread, so that a few
@@ -266,15 +266,15 @@ cudaError_t launch_small(const DevPlan& p, const float* a_coded, const float* B,
 // Behind the tensor-core FP32 GEMM: one CTA per SM walks the tiles when the
 // staged operands are left to the CUDA cores, else returns at once.
 __global__ void __launch_bounds__(kThreads, 1)
-gemm_f32_flagged_kernel(DevPlan p, const float* __restrict__ Ac, const float* __restrict__ B, int N, int ld, int K,
+gemm_f32_flagged_kernel(DevPlan p, const float* __restrict__ Ac, const float* __restrict__ B, int N, int K,
                         int h, float* products, float* C_direct) {
   chain_wait();
-  if (!f32_on_cuda_cores(p.ctr, K)) return;
+  if (!f32_on_cuda_cores(p.ctr + CTR_F32_SIMT, K)) return;
   const long long Mc = static_cast<long long>(p.ctr[CTR_NSURV]) * h;
   const long long n_tiles = (N + BN - 1) / BN, tiles = (Mc + BM - 1) / BM * n_tiles;
   for (long long t = blockIdx.x; t < tiles; t += gridDim.x) {
     const long long m = t / n_tiles;
-    gemm_f32_tile(p, Ac, B, N, ld, K, h, products, C_direct, Mc, m * BM, static_cast<int>(t - m * n_tiles) * BN);
+    gemm_f32_tile(p, Ac, B, N, K, h, products, C_direct, Mc, m * BM, static_cast<int>(t - m * n_tiles) * BN);
     __syncthreads();  // the tile's last shared-memory reads before the next tile's copies
   }
 }
@@ -282,15 +282,15 @@ gemm_f32_flagged_kernel(DevPlan p, const float* __restrict__ Ac, const float* __
 }  // namespace
 
 cudaError_t launch_gemm_f32_flagged(const DevGraph& g, const DevPlan& p, const float* a_coded, const float* B, int N,
-                                    int K, int h, float* products, float* C_direct, cudaStream_t st, int ld) {
+                                    int K, int h, float* products, float* C_direct, cudaStream_t st) {
   const long long rows = static_cast<long long>(g.num_cells) * h;
   if (rows == 0 || N == 0) return cudaSuccess;
   const size_t smem = sizeof(float) * kStages * BK * ((BM + APAD) + BN);
   cudaError_t e = cudaFuncSetAttribute(gemm_f32_flagged_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(smem));
   if (e != cudaSuccess) return e;
-  return launch(gemm_f32_flagged_kernel, dim3(num_sms()), kThreads, smem, st, p, a_coded, B, N, ld ? ld : N, K, h,
-                products, C_direct);
+  return launch(gemm_f32_flagged_kernel, dim3(num_sms()), kThreads, smem, st, p, a_coded, B, N, K, h, products,
+                C_direct);
 }
 
 // a_coded: the FP32 coded rows of the surviving cells (encode pass output),

@@ -346,7 +346,7 @@ gemm_tc_kernel(const __grid_constant__ TcJob single, const TcJob* __restrict__ t
     total_tiles = static_cast<long long>(units) * single.n_tiles * (kExact ? single.ex_np : 1);
     // FP32 operands the three parts cannot hold or sum: the CUDA-core kernel
     // behind this launch computes the products instead
-    if (kParts == 3 && f32_on_cuda_cores(single.ctr, single.K)) total_tiles = 0;
+    if (kParts == 3 && f32_on_cuda_cores(single.ctr + CTR_F32_SIMT, single.K)) total_tiles = 0;
   }
 
   if (warp == 0) {

@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(kEncThreads)
 encode_f32_flagged_kernel(DevGraph g, DevPlan p, const float* __restrict__ A, int M, int K, int h, float* out,
                           long long row_blocks, long long blocks) {
   chain_wait();
-  if (!f32_on_cuda_cores(p.ctr, K)) return;
+  if (!f32_on_cuda_cores(p.ctr + CTR_F32_SIMT, K)) return;
   for (long long b = blockIdx.x; b < blocks; b += gridDim.x) {
     const long long kc = b / row_blocks;
     encode_body<0>(g, p, A, M, K, h, out, nullptr, nullptr, static_cast<int>(b - kc * row_blocks), static_cast<int>(kc));
