@@ -780,7 +780,13 @@ int host_impl(const bpx_code* c, const float* h_A, const float* h_B, int M, int 
   int32_t* d_info = reinterpret_cast<int32_t*>(static_cast<char*>(ws) + L.p_info);
   const bpx_opts o = opts ? *opts : bpx_default_opts();
   bool staged = false;  // A, B and the mask are on the device
-  if (const int w = sync ? host_panel(c, N, K, h, precision, o) : 0) {
+  // (a panel of C is written before the last of B is read: not where they share memory)
+  auto apart = [](const float* x, size_t nx, const float* y, size_t ny) { return x + nx <= y || y + ny <= x; };
+  const size_t a_len = static_cast<size_t>(M) * K, b_len = static_cast<size_t>(K) * N;
+  const size_t c_len = static_cast<size_t>(c->S) * h * N;
+  const bool panels = sync && apart(h_C, static_cast<size_t>(M) * N, h_B, b_len) && apart(d_C, c_len, d_B, b_len) &&
+                      apart(d_C, c_len, d_A, a_len);
+  if (const int w = panels ? host_panel(c, N, K, h, precision, o) : 0) {
     if (HostPipe* hp = host_pipe()) {
       const int rc = host_panels(c, h_A, h_B, M, N, K, h, precision, h_mask, mask_bytes, h_C, d_A, d_B, d_mask, d_C, o,
                                  ws, ws_bytes, st, hp, w);
