@@ -526,8 +526,9 @@ int bpx_group_autotune(bpx_group* group, const int* configs, int nconfigs, bpx_s
  * the B tile) with 64- / 32-wide k-slices; seg_kb = k-blocks of 64 per TMEM
  * accumulation segment, band = m-tiles (or m-tile pairs) per rasterisation
  * band.  gemm_config 0 = the default: 8080, or 128-wide or narrower tiles of
- * one CTA for products that fill few CTA pairs.  Precisions BPX_BF16,
- * BPX_BF16X3 and BPX_EXACT (which uses the tile shape, pairing, k-slice and
+ * one CTA for products that fill few CTA pairs (bpx_default_tile); the
+ * built-in list (NULL / 0) starts with it.  Precisions BPX_BF16, BPX_BF16X3,
+ * BPX_FP16X3 and BPX_EXACT (which uses the tile shape, pairing, k-slice and
  * band, with its own exact segment length; its default is also 8080).
  * Tile codes 3, 4, 7 and 8 name no kernel (BPX_ERR_INVAL).  No kernel loads
  * by TMA multicast.  Synchronizes. */
@@ -537,10 +538,11 @@ int bpx_autotune(const bpx_code* code, const float* d_A, const float* d_B, int M
 
 /* Peel-schedule autotuner of a group: times the grouped numeric peel (a4)
  * with each job's float4 columns cut so that the job gets about `targets[i]`
- * CTAs (NULL / 0 = a built-in list from 1/8 to 8 x the SM count; the default
- * plan aims at 4 x the SM count), on the group's own plans and products (one full
- * run first), keeps the fastest plan for later runs and graph launches, and
- * reports it.  Synchronizes; not capturable. */
+ * CTAs (NULL / 0 = a built-in list: the default plan, which goes by the
+ * number of jobs and is reported as target 0, and 1/8 to 8 x the SM count), on
+ * the group's own plans and products (one full run first), keeps the fastest
+ * plan for later runs and graph launches, and reports it.  Synchronizes; not
+ * capturable. */
 int bpx_group_autotune_peel(bpx_group* group, const int* targets, int ntargets, bpx_stream stream,
                             int* best_target, float* best_ms);
 

@@ -31,7 +31,7 @@ struct bpx_group {
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   int graph_key[5] = {0, 0, 0, 0, 0};
-  int peel_target = 0;                // peel CTAs aimed at per job (0 = 4 x the SM count)
+  int peel_target = 0;                // peel CTAs aimed at per job (0 = by the batch's size)
   std::vector<bpx::GJob> host_jobs;   // the device job table's host copy (re-planned peels)
   // peel launch order: the jobs in the gathered form first, then the rest
   size_t order_off = 0;
@@ -483,6 +483,12 @@ extern "C" int bpx_autotune(const bpx_code* c, const float* d_A, const float* d_
                 },
                 best_config, best_ms);
   }
+  // (the default first: its narrower tiles have no name)
+  static const int kRowsConfigs[] = {0, 8080, 16080, 4080, 8089, 16089, 8085, 16041, 8086, 16042};
+  if (!configs || nconfigs <= 0) {
+    configs = kRowsConfigs;
+    nconfigs = static_cast<int>(sizeof(kRowsConfigs) / sizeof(kRowsConfigs[0]));
+  }
   return tune(configs, nconfigs, st,
               [&](int cfg) -> int {
                 cudaError_t e = bpx::launch_gemm_tc(g, p, base + L.a_hi, split ? base + L.a_lo : nullptr,
@@ -500,14 +506,15 @@ extern "C" int bpx_group_autotune_peel(bpx_group* G, const int* targets, int nta
   if (!G || !G->ws) return fail(BPX_ERR_INVAL, "bpx_group_autotune_peel: group not initialised");
   cudaStream_t st = S(stream);
   const int sms = bpx::num_sms();
-  const int defaults[] = {std::max(1, sms / 8), std::max(1, sms / 4), std::max(1, sms / 2), sms, 2 * sms, 4 * sms,
-                          8 * sms};
+  // (0: the default plan, by the batch's size)
+  const int defaults[] = {0,       std::max(1, sms / 8), std::max(1, sms / 4), std::max(1, sms / 2), sms,
+                          2 * sms, 4 * sms,              8 * sms};
+  for (int i = 0; targets && i < ntargets; ++i)
+    if (targets[i] < 1) return fail(BPX_ERR_INVAL, "bpx_group_autotune_peel: targets must be >= 1");
   if (!targets || ntargets <= 0) {
     targets = defaults;
     ntargets = static_cast<int>(sizeof(defaults) / sizeof(defaults[0]));
   }
-  for (int i = 0; i < ntargets; ++i)
-    if (targets[i] < 1) return fail(BPX_ERR_INVAL, "bpx_group_autotune_peel: targets must be >= 1");
   // one full run so that every job's plan, products and direct blocks exist;
   // re-running the peel alone then recomputes the same C
   if (int rc = run_group(G, nullptr, G->tuned_config, st)) return rc;
