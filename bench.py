@@ -265,6 +265,45 @@ def _exact_mult(bpx, code, K):
     return S * (S + 1) // 2
 
 
+def _on_cuda_cores(bpx, code, prec, N, K, h):
+    """FP32 products too small for the tensor cores."""
+    return prec == "fp32" and bpx.default_tile(code, bpx.FP32, N, K, h) == 0
+
+
+def _gemm_unit(bpx, code, prec, N, K, h, peaks, sms):
+    """What the coded GEMM runs on: (operations a useful coded flop, peak
+    TFLOP/s, the peak's source, bound, kernel).  Tensor-core paths: the MMA
+    flops executed (split terms, FP32's six products, or the exact path's
+    digit products) against the measured bf16 peak (FP8: times the nominal
+    fp8 / bf16 ratio of 2); small FP32 products: FFMA."""
+    if _on_cuda_cores(bpx, code, prec, N, K, h):
+        mhz = peaks.get("sm_max_mhz", 2070.0)
+        return (1, sms * 128 * 2 * mhz * 1e6 / 1e12, f"FFMA: {sms} SMs x 128 lanes x 2 x {mhz:.0f} MHz", "alu",
+                "coded FP32 SIMT GEMM")
+    mx = prec == "mxfp8"
+    mult = _exact_mult(bpx, code, K) if prec == "exact" else MMA_MULT[prec]
+    src = "measured bf16 burst (MEASURED_PEAKS.json)" if peaks else "fallback"
+    return (mult, peaks.get("bf16_tflops", 1900.0) * (2.0 if mx else 1.0),
+            src + (" x 2 (nominal fp8/bf16)" if mx else ""), "tensor",
+            "coded tcgen05 GEMM" + (" (block-scaled MXFP8)" if mx else ""))
+
+
+def _launches(bpx, code, prec, N, K, h):
+    """Kernels of one coded multiplication: the plan, B's staging, the encode,
+    the GEMM, the peel; split fp16 and exact slices also scan B's columns,
+    exact slices A's rows; FP32 on the tensor cores is followed by the CUDA-core
+    encode and GEMM, which return at once for ordinary operands."""
+    n = {"bf16x3": 5, "bf16": 5, "mxfp8": 5, "fp32": 7, "exact": 7, "fp16x3": 6, "bf16x3-fused": 4}[prec]
+    if _on_cuda_cores(bpx, code, prec, N, K, h):
+        n = 4
+    if prec == "fp16x3" and len(code.cell_src) >= 4 * code.num_cells:
+        n += 2  # the K-chunked encode of high-degree codes: three kernels instead of one
+    if prec == "exact" and bpx.exact_params(code, K)["S"] >= 4 and len(code.cell_src) >= 4 * code.num_cells:
+        n += 1  # each source row's digits cut once
+    S = code.num_sources
+    return n + (S >= 1024) + (S >= 4096)  # tall codes: the peel list, and the plan in two parts
+
+
 def _propagation(code, order, Ah, Bh, h, sources, ncols=256, kappa=None):
     """nu_s = sqrt(sum_c coef_{s,c}^2 ||P_c||^2) / ||C_s|| for the sampled
     sources: coef from the peel recurrence over the library's plan (each
@@ -641,22 +680,13 @@ def run_ours(args, wl):
     gemm_ms = R["stage"]["gemm"]
     rows_mean = sum(R["rows"]) / len(R["rows"])
     clk = R["clocks"].get("sm_mhz") or 0
-    # tensor-core paths: MMA flops executed per launch (split terms, or the
-    # exact path's digit-pair products) against the measured bf16 peak (FP8:
-    # times the nominal fp8 / bf16 ratio of 2)
-    if head == "exact":
-        mult = _exact_mult(bpx, code, K)
-    else:
-        mult = MMA_MULT[head]
-    flops = 2.0 * rows_mean * N * K * mult
-    achieved = flops / (gemm_ms * 1e-3) / 1e12
-    peak = peaks.get("bf16_tflops", 1900.0) * (2.0 if head == "mxfp8" else 1.0)
-    src = "measured bf16 burst (MEASURED_PEAKS.json)" if peaks else "fallback"
-    roof = {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+    sms = torch.cuda.get_device_properties(dev).multi_processor_count
+    mult, peak, src, bound, kernel = _gemm_unit(bpx, code, head, N, K, h, peaks, sms)
+    achieved = 2.0 * rows_mean * N * K * mult / (gemm_ms * 1e-3) / 1e12
+    roof = {"bound": bound, "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
             "frac": achieved / peak, "traffic": _traffic(wl["name"], head, tuned.get(head)),
-            "peak_source": src + (" x 2 (nominal fp8/bf16)" if head == "mxfp8" else ""),
-            "kernel": "coded tcgen05 GEMM" + (" (block-scaled MXFP8)" if head == "mxfp8" else ""),
-            "work_per_launch": "2 x coded rows x N x K x %d MMA flops" % mult}
+            "peak_source": src, "kernel": kernel,
+            "work_per_launch": "2 x coded rows x N x K" + (" x %d MMA flops" % mult if bound == "tensor" else "")}
     # decode GB/s: compulsory bytes of the peel (read each non-direct
     # resolver's product and every other block it subtracts, write C_s)
     peel_ms = R["stage"]["peel"]
@@ -706,12 +736,7 @@ def run_ours(args, wl):
         rows_m = sum(r["rows"]) / len(r["rows"])
         if gm <= 0:
             continue
-        if prec == "exact":
-            mult = _exact_mult(bpx, code, K)
-        else:
-            mult = MMA_MULT[prec]
-        pk = peaks.get("bf16_tflops", 1900.0) * (2.0 if prec == "mxfp8" else 1.0)
-        unit = "measured bf16 burst" + (" x 2 (nominal fp8/bf16)" if prec == "mxfp8" else "")
+        mult, pk, unit, _bound, _kernel = _gemm_unit(bpx, code, prec, N, K, h, peaks, sms)
         work = 2.0 * rows_m * N * K * mult
         ach = work / (gm * 1e-3) / 1e12
         gr[prec] = {"achieved_tflops": ach, "peak_tflops": pk, "frac": ach / pk, "peak": unit, "gemm_ms": gm}
@@ -724,24 +749,21 @@ def run_ours(args, wl):
                       "bytes_def": "sum over non-direct sources of (deg(resolver)+1) h N 4"}
     # the HBM-bound staging stages against their compulsory bytes: the
     # encode reads A once and writes the coded rows (bf16 hi + lo: 4 B per
-    # element, or FP32 in three bf16 parts: 6 B), the B split reads B and writes B^T hi + lo
+    # element, FP32: 4 B, or in three bf16 parts 6 B), the B split reads B and writes B^T hi + lo
     def _hbm(nbytes, ms, what):
         gbs = nbytes / (ms * 1e-3) / 1e9 if ms and ms > 0 else None
         return {"bytes_per_step": nbytes, "ms": ms, "gbs": gbs, "frac_hbm": gbs / hbm if gbs else None,
                 "bytes_def": what}
     st_ = R["stage"]
     if head in ("bf16x3", "bf16", "fp32"):
-        out_b = {"bf16x3": 4, "fp32": 6}.get(head, 2)
+        out_b = {"bf16x3": 4, "bf16": 2, "fp32": 4 if _on_cuda_cores(bpx, code, head, N, K, h) else 6}[head]
         line["encode"] = _hbm(4.0 * M * K + out_b * rows_mean * K, st_.get("a_prep", 0.0),
                               "read A once (4 M K) + write the coded rows (%d B per element)" % out_b)
     if head in ("bf16x3", "bf16"):
         line["b_split"] = _hbm(4.0 * K * N + (4 if head == "bf16x3" else 2) * K * N, st_.get("b_prep", 0.0),
                                "read B (4 K N) + write B^T hi (+ lo) bf16")
     line["clocks"] = R["clocks"]
-    per_step = {"bf16x3": 5, "bf16": 5, "mxfp8": 5, "fp32": 7, "exact": 7, "fp16x3": 7, "bf16x3-fused": 4}[head]
-    if head == "fp16x3" and len(code.cell_src) >= 4 * code.num_cells:
-        per_step += 2  # the K-chunked encode of high-degree codes: three kernels instead of one
-    line["gpu_launches"] = per_step * steps
+    line["gpu_launches"] = _launches(bpx, code, head, N, K, h) * steps
 
     # end to end through the host entry points (pinned host buffers): every
     # step copies its A, B and mask in and its C and info words out inside the
@@ -1112,17 +1134,14 @@ def run_straggler(args, wl):
     timed = plans[warm:]
     useful = 2.0 * M * N * K
     rows = [int((p_["mask"] == 0).sum().item()) * h for p_ in timed]
-    if prec == "exact":
-        mult = _exact_mult(bpx, code, K)
-    else:
-        mult = {"bf16x3": 3, "fp16x3": 3, "bf16": 1, "fp32": 6}[prec]
     peaks = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json"))) if os.path.exists(
         os.path.join(ROOT, "MEASURED_PEAKS.json")) else {}
+    mult, pk, _src, bound, kernel = _gemm_unit(bpx, code, prec, N, K, h, peaks,
+                                               torch.cuda.get_device_properties(0).multi_processor_count)
     ach = 2.0 * float(np.mean(rows)) * N * K * mult / (stage["gemm"] * 1e-3) / 1e12
-    pk = peaks.get("bf16_tflops", 1900.0)
-    roof = {"bound": "tensor", "achieved": ach, "peak": pk, "unit": "TFLOP/s", "frac": ach / pk,
-            "traffic": None, "kernel": "coded tcgen05 GEMM",
-            "work_per_launch": "2 x coded rows x N x K x %d MMA flops" % mult}
+    roof = {"bound": bound, "achieved": ach, "peak": pk, "unit": "TFLOP/s", "frac": ach / pk,
+            "traffic": None, "kernel": kernel,
+            "work_per_launch": "2 x coded rows x N x K" + (" x %d MMA flops" % mult if bound == "tensor" else "")}
     H = sum(1.0 / j for j in range(1, code.num_cells + 1))
     # How much of the peel could have overlapped the products (outside the
     # timed region, on the first timed steps): the decodable set's arrivals in
@@ -1163,8 +1182,7 @@ def run_straggler(args, wl):
                       "units": "1 / mu; T_c = sigma_c X_c"},
             "computed_cells_mean": float(np.mean(rows)) / h,
             "roofline": roof, "clocks": ck,
-            "gpu_launches": ({"bf16x3": 5, "bf16": 5, "fp16x3": 7, "fp32": 7, "exact": 7}[prec]
-                             + (2 if prec == "fp16x3" and len(code.cell_src) >= 4 * code.num_cells else 0)) * steps}
+            "gpu_launches": _launches(bpx, code, prec, N, K, h) * steps}
     print(json.dumps(line), flush=True)
 
 
