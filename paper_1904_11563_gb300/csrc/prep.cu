@@ -32,35 +32,22 @@ constexpr int kEncVec = 8;  // consecutive K elements per thread (two float4 loa
 // - p2, whose sum is x exactly (8 significand bits each) while x lies in
 // [2^-102, 2^127): p1 does not round up to infinity and p3's last bit is a
 // normal bf16.  Zero is exact too; any other value is reported.
-__device__ __forceinline__ bool parts_unfit(float x) {
+
+// |x| lies outside [2^-102, 2^(top - 127)) and is not zero.
+template <uint32_t top>
+__device__ __forceinline__ bool parts_outside(float x) {
   const uint32_t u = __float_as_uint(x) & 0x7fffffffu;
-  return u != 0u && u - (25u << 23) >= (254u - 25u) << 23;
+  return u != 0u && u - (25u << 23) >= (top - 25u) << 23;
 }
-// Notes an unfit element, and the largest magnitude (as float bits) in
-// ctr[word] where it is above kF32Plain: ordinary operands then cost no
-// traffic; of others a warp reads the word and raises it if need be (all
-// operands above it: 62 -> 67 us on 1000 x 1416 x 1100, 665 -> 688 at 4096 cubed).
-__device__ __forceinline__ void note_parts(const DevPlan& p, int word, uint32_t most, bool unfit) {
-  if (unfit) {
-    p.ctr[CTR_F32_SIMT] = 1;
-  } else if (most > __float_as_uint(kF32Plain)) {
-    const unsigned lanes = __activemask();
-    most = __reduce_max_sync(lanes, most);
-    auto* at = reinterpret_cast<uint32_t*>(p.ctr + word);
-    if ((threadIdx.x & 31) == __ffs(lanes) - 1 && *reinterpret_cast<volatile uint32_t*>(at) < most)
-      atomicMax(at, most);
-  }
-}
-// most: raised to the largest magnitude of the eight; returns whether one is unfit.
+// Splits eight elements; returns whether one is outside [2^-102, 2^32).
 __device__ __forceinline__ bool parts_split8(const float (&v)[8], __nv_bfloat16* o1, __nv_bfloat16* o2,
-                                             __nv_bfloat16* o3, uint32_t& most) {
+                                             __nv_bfloat16* o3) {
   uint32_t w1[4], w2[4], w3[4];
-  bool unfit = false;
+  bool odd = false;
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const float x0 = v[2 * q], x1 = v[2 * q + 1];
-    unfit |= parts_unfit(x0) | parts_unfit(x1);
-    most = max(most, max(__float_as_uint(fabsf(x0)), __float_as_uint(fabsf(x1))));
+    odd |= parts_outside<127 + 32>(x0) | parts_outside<127 + 32>(x1);
     const __nv_bfloat162 p1 = __floats2bfloat162_rn(x0, x1);
     const float2 f1 = __bfloat1622float2(p1);
     const float r0 = x0 - f1.x, r1 = x1 - f1.y;
@@ -74,7 +61,34 @@ __device__ __forceinline__ bool parts_split8(const float (&v)[8], __nv_bfloat16*
   *reinterpret_cast<uint4*>(o1) = make_uint4(w1[0], w1[1], w1[2], w1[3]);
   *reinterpret_cast<uint4*>(o2) = make_uint4(w2[0], w2[1], w2[2], w2[3]);
   *reinterpret_cast<uint4*>(o3) = make_uint4(w3[0], w3[1], w3[2], w3[3]);
-  return unfit;
+  return odd;
+}
+// Of eight elements with one outside that range: notes an element that the
+// parts cannot hold, else raises ctr[word] to their largest magnitude (float
+// bits).  Ordinary operands come here never; where all are large a warp reads
+// the word every time (1000 x 1416 x 1100 62 -> 67 us, 4096 cubed 665 -> 688).
+static_assert(kF32Plain == 0x1p32f, "magnitudes below are not noted");
+__device__ __noinline__ void note_parts8(int32_t* ctr, int word, const float4 a, const float4 b) {
+  const float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+  bool unfit = false;
+  uint32_t most = 0;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    unfit |= parts_outside<254>(v[q]);
+    most = max(most, __float_as_uint(fabsf(v[q])));
+  }
+  if (unfit) {
+    ctr[CTR_F32_SIMT] = 1;
+    return;
+  }
+  const unsigned lanes = __activemask();
+  most = __reduce_max_sync(lanes, most);
+  auto* at = reinterpret_cast<uint32_t*>(ctr + word);
+  if ((threadIdx.x & 31) == __ffs(lanes) - 1 && *reinterpret_cast<volatile uint32_t*>(at) < most)
+    atomicMax(at, most);
+}
+__device__ __forceinline__ void note_parts8(int32_t* ctr, int word, const float (&v)[8]) {
+  note_parts8(ctr, word, make_float4(v[0], v[1], v[2], v[3]), make_float4(v[4], v[5], v[6], v[7]));
 }
 
 // A CTA covers `rows` coded rows x `cols` columns (cols = min(1024, K rounded
@@ -123,9 +137,7 @@ __device__ __forceinline__ void encode_body(const DevGraph& g, const DevPlan& p,
     d[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
     d[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
   } else if constexpr (kMode == 3) {
-    uint32_t most = 0;
-    const bool unfit = parts_split8(acc, out_hi + o, out_lo + o, out_3 + o, most);
-    note_parts(p, CTR_F32_AMAX, most, unfit);
+    if (parts_split8(acc, out_hi + o, out_lo + o, out_3 + o)) note_parts8(p.ctr, CTR_F32_AMAX, acc);
   } else {
     uint32_t hv[4], lv[4];
 #pragma unroll
@@ -176,10 +188,9 @@ encode_f32_flagged_kernel(DevGraph g, DevPlan p, const float* __restrict__ A, in
 // shared-memory tile: float4 reads along N, 16-byte bf16 writes along K.
 constexpr int kTile = 64;
 template <bool kParts3 = false>
-__device__ __forceinline__ bool b_split_body(const float* __restrict__ B, int K, int N, int ldb,
+__device__ __forceinline__ void b_split_body(const float* __restrict__ B, int K, int N, int ldb,
                                              __nv_bfloat16* bt_hi, __nv_bfloat16* bt_lo, int bx,
-                                             int by, __nv_bfloat16* bt_3 = nullptr, uint32_t* most = nullptr) {
-  bool unfit = false;
+                                             int by, __nv_bfloat16* bt_3 = nullptr, int32_t* ctr = nullptr) {
   __shared__ float tile[kTile][kTile + 1];
   const int n0 = bx * kTile, k0 = by * kTile;
   {
@@ -209,7 +220,7 @@ __device__ __forceinline__ bool b_split_body(const float* __restrict__ B, int K,
 #pragma unroll
       for (int q = 0; q < 8; ++q) v[q] = tile[8 * kc + q][r];
       const long long o = static_cast<long long>(n) * K + k;
-      unfit |= parts_split8(v, bt_hi + o, bt_lo + o, bt_3 + o, *most);
+      if (parts_split8(v, bt_hi + o, bt_lo + o, bt_3 + o)) note_parts8(ctr, CTR_F32_BMAX, v);
     } else {
       uint32_t hv[4], lv[4];
 #pragma unroll
@@ -226,16 +237,13 @@ __device__ __forceinline__ bool b_split_body(const float* __restrict__ B, int K,
       if (bt_lo) *reinterpret_cast<uint4*>(bt_lo + o) = make_uint4(lv[0], lv[1], lv[2], lv[3]);
     }
   }
-  return unfit;
 }
 
 __global__ void __launch_bounds__(256)
 b_parts_kernel(DevPlan p, const float* __restrict__ B, int K, int N, int ldb, __nv_bfloat16* o1, __nv_bfloat16* o2,
                __nv_bfloat16* o3, bool early) {
   chain_begin_staging(early);
-  uint32_t most = 0;
-  const bool unfit = b_split_body<true>(B, K, N, ldb, o1, o2, blockIdx.x, blockIdx.y, o3, &most);
-  note_parts(p, CTR_F32_BMAX, most, unfit);
+  b_split_body<true>(B, K, N, ldb, o1, o2, blockIdx.x, blockIdx.y, o3, p.ctr);
   chain_end_staging(early);
 }
 
