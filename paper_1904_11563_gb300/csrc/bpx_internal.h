@@ -155,10 +155,6 @@ enum {
   CTR_NSURV = 0,  // surviving cells
   CTR_NWAVES,     // rounds
   CTR_NREC,       // recovered sources
-  CTR_NF,         // frontier size (scratch)
-  CTR_NNEXT,      // next frontier size (scratch)
-  CTR_NNEW,       // sources recovered this round (scratch)
-  CTR_ERR,        // device error code raised by a kernel self-check
   CTR_PLAN,       // kPlanReady once a whole plan is in place (zeroed by bpx_workspace_init)
   // FP32 on the tensor cores (cleared by every call's products): an operand
   // holds an element that the parts cannot; the float bits of the largest

@@ -457,7 +457,6 @@ __device__ __forceinline__ void schedule_body(const DevGraph& g, const DevPlan& 
     p.ctr[CTR_NSURV] = nsurv;
     p.ctr[CTR_NWAVES] = round;
     p.ctr[CTR_NREC] = nrec;
-    p.ctr[CTR_ERR] = 0;
     p.ctr[CTR_PLAN] = kPlanReady;
     int32_t inf[BPX_INFO_LEN];
     for (int i = 0; i < BPX_INFO_LEN; ++i) inf[i] = 0;
