@@ -52,8 +52,8 @@ CODE_TEXT = {
 # precision, config and the SHA-256 of the GEMM sources it was taken with: a
 # changed kernel reports null until it is captured again.
 TRAFFIC = {
-    ("sysmoj_8192", "bf16x3", 0): ("b653608ba7325866b23c715fd20a2f60acb16d7b16b30ed9f30d539d646aa41b",
-                                   2741324288 + 301022720),
+    ("sysmoj_8192", "bf16x3", 0): ("99335bd29497d34fdff7542c74c1d9fb0eb4c1f64fee3b38f4d23d40ad3320d9",
+                                   2848139520 + 296659200),
 }
 
 

@@ -977,10 +977,11 @@ cudaError_t launch_gemm_tc(const DevGraph& g, const DevPlan& p, const void* a_hi
 // FP32 operands in three bf16 parts (a[i], b[i]), the tile by auto_bn; 64-wide
 // segments (24 MMAs each, so a drain is as rare as with hi + lo operands).
 // Tensor-bound: 96 KB staged per 24 MMAs and CTA, 32 B a clock.  Benchmark
-// workload (9088 coded rows, 8192 x 8192): 3.67 ms, 2.0 PFLOP/s of MMA work,
-// against 19.1 ms for the CUDA-core GEMM (FFMA-bound); relative error of a
-// directly computed block 1.3e-7 at K = 1992 against 8.0e-7, 1.7e-7 at 4096
-// against 1.1e-6.  32-wide k-slices (four stages) ran 3.73 ms.
+// workload (9088 to 9984 coded rows by mask, 8192 x 8192): 3.82 ms, 2.06
+// PFLOP/s of MMA work, against 19.1 ms for the CUDA-core GEMM (FFMA-bound);
+// relative error of a directly computed block 1.3e-7 at K = 1992 against
+// 8.0e-7, 1.7e-7 at 4096 against 1.1e-6.  32-wide k-slices (four stages) ran
+// 2 % longer.
 cudaError_t launch_gemm_f32_tc(const DevPlan& p, void* const a[3], void* const b[3], int num_cells, int N, int K, int h,
                                const RowsRange& range, float* products, float* C_direct, int32_t* info_out,
                                cudaStream_t st, int ld) {
