@@ -39,7 +39,8 @@
 // and so did swapping without a look first (630).  Codes of few, wide rounds
 // (n = 27, b = 12: one of 252 sources) 16.6 -> 14.6, n = 32, b = 24 28.9 ->
 // 22.9; with rounds of up to 256 ordered by one warp, an element at a time,
-// and a warp copying each position's list, these took 49 and 40.
+// and a warp copying each position's list, these took 49 and 40.  (Four a lane,
+// up to 128 sources, cost every plan of many rounds 1 %: registers.)
 #include <algorithm>
 #include <climits>
 #include <mutex>
@@ -54,7 +55,7 @@ constexpr size_t kSmemMax = 224 * 1024;  // dynamic shared memory of a plan's CT
 constexpr size_t kSmemSmall = 16 * 1024;  // the same for the 256-thread CTA of small codes
 
 constexpr int kAffineMax = 64;   // columns of the affine table kept in shared memory
-constexpr int kRankMax = 128;    // sources of a round ordered by one warp, four a lane, comparing each with all
+constexpr int kRankMax = 96;     // sources of a round ordered by one warp, three a lane, comparing each with all
 
 // The per-cell word: 32 bits in shared memory (when count and sum fit), 64
 // bits in the plan otherwise.
