@@ -605,6 +605,7 @@ b_colmax_kernel(const float* __restrict__ B, int K, int N, int ldb, uint32_t* bm
     asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(to), "f"(m.x), "f"(m.y), "f"(m.z), "f"(m.w)
                  : "memory");
   }
+  __syncwarp();  // (aligned: whole warps arrive)
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
   if (blockIdx.y % kColSplit == 0 && ph == 0 && n < N) {
 #pragma unroll
