@@ -397,8 +397,10 @@ int bpx_coded_matmul(const bpx_code* code, const float* d_A, const float* d_B, i
  * Host buffers should be page-locked for full copy bandwidth.  A call of 16 MB
  * of B or more runs in panels of B's columns on two streams of the calling
  * thread beside `stream` (which waits for them): copies in, kernels and copies
- * out of different panels overlap; same bits.  Not for BPX_MXFP8, BPX_EXACT,
- * fused_encode, stage_events or codes of 4096 sources or more. */
+ * out of different panels overlap; same bits (BPX_FP32 operands that turn out
+ * to be for the CUDA cores: the call is run over, in one piece).  Not for
+ * BPX_MXFP8, BPX_EXACT, fused_encode, stage_events, codes of 4096 sources or
+ * more, or where C shares memory with B (h_C with h_B, d_C with d_B or d_A). */
 int bpx_coded_matmul_host(const bpx_code* code, const float* h_A, const float* h_B, int M, int N,
                           int K, int h, int precision, const uint8_t* h_erasure_mask, float* h_C,
                           float* d_A, float* d_B, uint8_t* d_mask, float* d_C, const bpx_opts* opts,

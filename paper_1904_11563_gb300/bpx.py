@@ -573,7 +573,8 @@ class Group:
         return best.value, ms.value
 
     def autotune_peel(self, targets=None):
-        """Peel-schedule autotuner: (CTAs per job aimed at, ms of the grouped peel)."""
+        """Peel-schedule autotuner: (CTAs per job aimed at, 0 = the default plan,
+        ms of the grouped peel)."""
         best, ms = ct.c_int(), ct.c_float()
         arr = (ct.c_int * len(targets))(*targets) if targets else None
         _check(lib().bpx_group_autotune_peel(self._h, arr, len(targets) if targets else 0, _stream(),
